@@ -587,6 +587,8 @@ int do_tree_density(sph_ctx* c, const double* x, const double* y, const double* 
   d.tgt = c->tgt;
   d.leaves = c->leaves;
   d.n_leaves = c->n_leaves;
+  d.flag = c->flag;
+  d.leaf_of = c->leaf_of;
   d.ranges = c->ranges;
   d.fine = c->fine;
   d.rel = c->rel;

@@ -346,6 +346,7 @@ struct TreeDensityArgs {
   const int32_t* tgt;  // target order -> source index
   const sphk::TreeLeaf* leaves;
   const int32_t* n_leaves;
+  const int32_t *flag, *leaf_of;  // target order: first of its leaf; leaves that begin before it
   const sphk::TreeRange* ranges;
   const int4* fine;
   const float4 *rel, *vel4;

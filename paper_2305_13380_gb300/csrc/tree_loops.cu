@@ -9,15 +9,18 @@
 // the integer part exact, so FP32 keeps the sub-cell scale's precision
 // however wide the top cells are.
 //
-// Density, one warp per leaf, kTreeTpp lanes per target:
-//   1. the 27 ranges are staged in chunks relative to the leaf corner;
-//   2. each target keeps, in per-lane lists, the sources closer than its list
-//      radius R_i = min(leaf side, kTreeListReach * starting support);
-//   3. Newton-Raphson passes read r^2 from the lists; a target whose support
-//      outgrows R_i (or whose list overflows) leaves its group for the
-//      per-target kernel (k_tree_density_fb at its own level: a warp per
-//      target over its 27 cells), so that its round-mates do not wait;
-//   4. the final pass at the converged h gathers the sources from memory and
+// Density, a warp per round of kTPer targets of one leaf, kTreeTpp lanes per
+// target (k_tree_density):
+//   1. filter: the children of the 27 cells that some target of the round
+//      reaches, as segments of source order, 32 sources at a time, one per
+//      lane, each tested against the round's targets in turn.  The sources
+//      closer than a target's list radius R_i = min(leaf side, kTreeListReach *
+//      starting support) are kept in shared memory and listed per lane;
+//   2. Newton-Raphson passes walk the lists; a target whose support outgrows
+//      R_i (or whose list overflows) leaves its round for the per-target kernel
+//      (k_tree_density_fb at its own level: a warp per target over its 27
+//      cells), so that its round-mates do not wait;
+//   3. the final pass at the converged h gathers the sources from memory and
 //      publishes the lists for the force loop.
 // A force pair needs r < max(H_i, H_j).  The list of i holds every j with
 // r < R_i >= H_i; a j with H_j > r >= R_i is only in j's own reach, so the
@@ -31,35 +34,56 @@
 // own leaf frame with the same arithmetic as the density filter, so no pair is
 // counted twice or dropped at the boundary; emission uses a margin so that the
 // reverse pairs are a superset.
-#include <type_traits>
-
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "tree.cuh"
 
 namespace sphk {
 
-constexpr int kTWarps = 4;       // warps per CTA
-#ifndef SPH_TREE_TCAP
-#define SPH_TREE_TCAP 384
-#endif
-constexpr int kTCap = SPH_TREE_TCAP;  // staged sources per warp and chunk
-constexpr int kTRows = kTreeList + 1;  // + one scratch row for the branch-free append
+constexpr int kTWarps = 4;             // warps per CTA
+constexpr int kTCap = 384;             // staged sources per warp and chunk (per-target kernel)
 constexpr int kTPer = 32 / kTreeTpp;   // targets per round
-constexpr int kTChildren = 27 * 8;      // children of the 27 neighbour cells
+constexpr int kTChildren = 27 * 8;     // children of the 27 neighbour cells
 
-// Pruning tables of a warp's group (groups that do not fit one staging chunk).
-struct TPrune {
-  int32_t cv[kTChildren + 4];    // virtual start of each child (Morton order), + end
-  int32_t hoff[kTChildren + 4];  // offsets of the round's hit children, + total
-  uint8_t hch[kTChildren];       // the round's hit children, in order
+// Tables of a warp's leaf.
+struct TTab {
+  int32_t cv[kTChildren + 1];          // virtual start of each child (Morton order), + end
   int32_t rlo[28], rcum[28], rsc[28];  // per neighbour range: first source, virtual start, shift
   uint32_t cact[(kTChildren + 31) / 32];  // masked loops: children holding a masked source
 };
+// ... and of the per-target kernel.
+struct TPrune : TTab {
+  int32_t hoff[kTChildren + 4];  // offsets of the target's hit children, + total
+  uint8_t hch[kTChildren];       // the hit children, in order
+};
 constexpr size_t kTPruneBytes = (sizeof(TPrune) + 15) / 16 * 16;
-constexpr size_t kTWarpSmem = (size_t)kTCap * (sizeof(float4) + sizeof(uint32_t)) +
-                              (size_t)kTRows * 32 * (sizeof(float) + sizeof(uint32_t)) + kTPruneBytes;
-constexpr size_t kTDensSmem = kTWarps * kTWarpSmem;
+constexpr size_t kTFbWarpSmem = (size_t)kTCap * (sizeof(float4) + sizeof(uint32_t)) + kTPruneBytes;
+constexpr size_t kTFbSmem = kTWarps * kTFbWarpSmem;
+static_assert(kTFbWarpSmem % 16 == 0, "per-warp regions keep float4 alignment");
+
+// A density warp's shared memory.  Only the sources that some target of the
+// round lists are kept (about 90 of the ~305 it tests), as a position and a
+// packed index, and a list entry is one byte, the slot.
+constexpr int kTKept = 256;
+constexpr int kTWhole = 384;           // a leaf with at most this many sources is taken whole
+constexpr int kTSegs = 27 * 4 + 4;     // runs of hit children: at most four per range
+constexpr int kTWin = 2 * kTPer;       // targets per window (k_tree_density)
+constexpr int kTDensBlocks = 6;        // resident CTAs per SM the registers are sized for
+struct TRound {
+  float4 pos[kTKept];                  // position from the leaf corner; packed index and shift
+  float4 tgt[kTPer];                   // the targets' positions and R^2
+  int2 seg[kTSegs];                    // segments: virtual start; first source and shift
+  TTab tab;
+  uint8_t list[kTreeList + 1][32];     // + one scratch row for an overflowing append
+};
+constexpr size_t kTRoundBytes = (sizeof(TRound) + 15) / 16 * 16;
+constexpr size_t kTDensSmem = kTWarps * kTRoundBytes;
+static_assert(kTDensBlocks * (kTDensSmem + 1024) <= 228 * 1024, "resident density CTAs per SM");
+static_assert(kTKept <= 256 && kTreeTpp * kTreeList <= kTKept, "a slot is a byte; one target's list fits");
+// the sources of lane sub among 32: bits sub, sub + kTreeTpp, ...
+constexpr uint32_t kTLanes = 0x01010101u;
+constexpr uint32_t kTGroup = (1u << kTreeTpp) - 1u;  // the lanes of one target
+static_assert(kTreeTpp == 8 && kTreeList == 32, "one byte per target in a ballot, one mark bit per entry");
 constexpr int kNoShift = 1 | (1 << 2) | (1 << 4);
 // list_cnt marker: the target is solved by the per-target kernels
 constexpr uint16_t kListFallback = 0xfffe;
@@ -70,7 +94,6 @@ constexpr uint16_t kListFallback = 0xfffe;
 constexpr int32_t kFbOwnLevel = 1 << 30;
 constexpr int32_t kFbPassive = 1 << 29;
 constexpr int32_t kFbIndex = kFbPassive - 1;
-static_assert(kTWarpSmem % 16 == 0, "per-warp regions keep float4 alignment");
 static_assert(kTreeList <= kTreeListRegion, "published lists fit their regions");
 // a target's published list: its lanes' lists packed one after another in a
 // region of kTreeTpp * kTreeListRegion entries, the count in list_cnt[target]
@@ -262,8 +285,8 @@ __device__ __forceinline__ TRanges load_ranges(const TreeRange* __restrict__ ran
 // start and shift, and the virtual start of each of its 8 children (which
 // are contiguous in Morton order; a cell of the deepest level has one).
 // Lanes 0..26 search their range's keys.  Called by the whole warp.
-__device__ __forceinline__ void prune_tables(const uint64_t* __restrict__ skey, const TRanges& R, int depth,
-                                             int lane, TPrune* pr, const int32_t* __restrict__ act_pre = nullptr) {
+__device__ __noinline__ void prune_tables(const uint64_t* __restrict__ skey, TRanges R, int depth,
+                                          int lane, TTab* pr, const int32_t* __restrict__ act_pre = nullptr) {
   const int32_t cum_next = __shfl_down_sync(0xffffffffu, R.cum, 1);
   if (act_pre != nullptr) {
     if (lane < (kTChildren + 31) / 32) pr->cact[lane] = 0u;
@@ -288,6 +311,7 @@ __device__ __forceinline__ void prune_tables(const uint64_t* __restrict__ skey, 
         lo[c] = R.lo;
         hi[c] = R.lo + len;
       }
+#pragma unroll 1
       for (bool more = true; more;) {
         more = false;
 #pragma unroll
@@ -336,111 +360,34 @@ __device__ __forceinline__ float child_dist2(int ch, float side, float cside, co
   return fmaf(ex, ex, fmaf(ey, ey, ez * ez));
 }
 
-// The children any target of the round can reach: each target's lanes test
-// 27 children each (ch = sub + 8 m) against its list radius, the union over
-// the round's targets is compacted in child order with the offsets of their
-// sources.  Returns the union's source count.  Called by the whole warp.
-// lane sub owns children sub + kTreeTpp k (k < kCh) of every neighbour cell:
-// bit m kCh + k of a lane's child mask
-constexpr int kCh = 8 / kTreeTpp;
-using ChMask = std::conditional_t<(27 * kCh > 32), unsigned long long, uint32_t>;
-
-__device__ __forceinline__ int union_round(ChMask mine, int lane, TPrune* pr, int& nh);
-
-__device__ __forceinline__ int prune_round(bool valid, int sub, int lane, const float3& pi, float Rb2,
-                                           float side, float cside, TPrune* pr, int& nh, bool need_act = false) {
-  using Mask = ChMask;
-  Mask mine = 0;
-  if (valid) {
-    for (int m = 0; m < 27; ++m) {
-#pragma unroll
-      for (int k = 0; k < kCh; ++k) {
-        const int ch = 8 * m + sub + kTreeTpp * k;
-        // a target outside the mask reaches only the children with a masked
-        // source (its list serves only reverse pairs to those)
-        if (pr->cv[ch] < pr->cv[ch + 1] && (!need_act || ((pr->cact[ch >> 5] >> (ch & 31)) & 1u)) &&
-            child_dist2(ch, side, cside, pi) < Rb2)
-          mine |= (Mask)1 << (m * kCh + k);
-      }
-    }
-  }
-  return union_round(mine, lane, pr, nh);
-}
-
-// The lane's candidate children of a group (bits as above): those holding a
-// source, and (mask_only) a masked one.  Called once per group, after
-// prune_tables.
-__device__ __forceinline__ ChMask group_candidates(int sub, const TPrune* pr, bool mask_only) {
-  ChMask c = 0;
+// The children that a target at pi reaches within Rb2 (the per-target kernel):
+// lane sub of each eight tests child sub of the 27 cells; the hit children are
+// compacted in child order with the offsets of their sources.  Returns their
+// number and their sources.  Called by the whole warp.
+__device__ __noinline__ int2 prune_round(int lane, float3 pi, float Rb2, float side, float cside, TPrune* pr) {
+  uint32_t mine = 0;
+  const int sub = lane % kTreeTpp;
+#pragma unroll 1
   for (int m = 0; m < 27; ++m) {
-#pragma unroll
-    for (int k = 0; k < kCh; ++k) {
-      const int ch = 8 * m + sub + kTreeTpp * k;
-      if (pr->cv[ch] < pr->cv[ch + 1] && (!mask_only || ((pr->cact[ch >> 5] >> (ch & 31)) & 1u)))
-        c |= (ChMask)1 << (m * kCh + k);
-    }
+    const int ch = 8 * m + sub;
+    if (pr->cv[ch] < pr->cv[ch + 1] && child_dist2(ch, side, cside, pi) < Rb2) mine |= 1u << m;
   }
-  return c;
-}
-
-// prune_round with the candidates precomputed per group and the box
-// distances taken per axis: along each axis a lane's child boxes take three
-// positions (the neighbour offset, its child bit fixed), so nine squared
-// distances give all 27 (the sum's rounding lies far inside the margin of
-// Rb2).
-__device__ __forceinline__ int prune_round_fast(bool valid, int sub, int lane, const float3& pi, float Rb2,
-                                                float side, float cside, TPrune* pr, int& nh, ChMask cand) {
-  ChMask mine = 0;
-  if (valid) {
-#pragma unroll
-    for (int k = 0; k < kCh; ++k) {
-      const int c = sub + kTreeTpp * k;
-      const float cx = (float)(c & 1) * cside, cy = (float)((c >> 1) & 1) * cside, cz = (float)(c >> 2) * cside;
-      float ex[3], ey[3], ez[3];
-#pragma unroll
-      for (int o = 0; o < 3; ++o) {
-        const float b0 = (float)(o - 1) * side;
-        const float dx = fmaxf(fmaxf(b0 + cx - pi.x, pi.x - (b0 + cx + cside)), 0.0f);
-        const float dy = fmaxf(fmaxf(b0 + cy - pi.y, pi.y - (b0 + cy + cside)), 0.0f);
-        const float dz = fmaxf(fmaxf(b0 + cz - pi.z, pi.z - (b0 + cz + cside)), 0.0f);
-        ex[o] = dx * dx;
-        ey[o] = dy * dy;
-        ez[o] = dz * dz;
-      }
-#pragma unroll
-      for (int m = 0; m < 27; ++m) {
-        const ChMask bit = (ChMask)1 << (m * kCh + k);
-        if ((cand & bit) && ex[m % 3] + ey[(m / 3) % 3] + ez[m / 9] < Rb2) mine |= bit;
-      }
-    }
-  }
-  return union_round(mine, lane, pr, nh);
-}
-
-// The union over the round's targets of their children, compacted in child
-// order with the offsets of their sources; returns the union's source count.
-// Called by the whole warp.
-__device__ __forceinline__ int union_round(ChMask mine, int lane, TPrune* pr, int& nh) {
-#pragma unroll
-  for (int o = kTreeTpp; o < 32; o <<= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, o);
-  // lanes 0..kTreeTpp-1 hold the union; compacted in child order
-  nh = 0;
+  int nh = 0;
+#pragma unroll 1
   for (int m = 0; m < 27; ++m) {
-#pragma unroll
-    for (int k = 0; k < kCh; ++k) {
-      const bool hb = lane < kTreeTpp && ((mine >> (m * kCh + k)) & 1u);
-      const unsigned b = __ballot_sync(0xffffffffu, hb);
-      if (hb) {
-        const int ch = 8 * m + kTreeTpp * k + lane;
-        const int idx = nh + __popc(b & ((1u << lane) - 1u));
-        pr->hch[idx] = (uint8_t)ch;
-        pr->hoff[idx] = pr->cv[ch + 1] - pr->cv[ch];
-      }
-      nh += __popc(b);
+    const bool hb = lane < kTreeTpp && ((mine >> m) & 1u);
+    const unsigned b = __ballot_sync(0xffffffffu, hb);
+    if (hb) {
+      const int ch = 8 * m + lane;
+      const int idx = nh + __popc(b & ((1u << lane) - 1u));
+      pr->hch[idx] = (uint8_t)ch;
+      pr->hoff[idx] = pr->cv[ch + 1] - pr->cv[ch];
     }
+    nh += __popc(b);
   }
   __syncwarp();
   int run = 0;
+#pragma unroll 1
   for (int k0 = 0; k0 < nh; k0 += 32) {
     const int k = k0 + lane;
     const int v = k < nh ? pr->hoff[k] : 0;
@@ -455,18 +402,97 @@ __device__ __forceinline__ int union_round(ChMask mine, int lane, TPrune* pr, in
   }
   if (lane == 0) pr->hoff[nh] = run;
   __syncwarp();
-  return run;
+  return make_int2(nh, run);
 }
 
-// Stages cnt sources into spos / sidx [0, cnt) relative to the group corner
-// (w: the mass, or the mask bit of masked loops); item u is source map(u) (its
-// index and shift code).  A lane takes its items four at a time and issues
-// their loads together, so that four L2 latencies overlap instead of running
-// one after another.  Called by the whole warp.
+// The lane's candidate children of a leaf (child sub of range m: bit m): those
+// holding a source, and (mask_only) a masked one (a target outside the mask
+// lists only those).  Called once per leaf, after prune_tables.
+__device__ __forceinline__ uint32_t group_candidates(int sub, const TTab* pr, bool mask_only) {
+  uint32_t c = 0;
+#pragma unroll 3
+  for (int m = 0; m < 27; ++m) {
+    const int ch = 8 * m + sub;
+    if (pr->cv[ch] < pr->cv[ch + 1] && (!mask_only || ((pr->cact[ch >> 5] >> (ch & 31)) & 1u))) c |= 1u << m;
+  }
+  return c;
+}
+
+// The segments of a round: the union over its targets of the candidate
+// children that they reach, in child order, adjacent children of a range
+// (contiguous in source order) as one segment: virtual start and packed first
+// source.  The box distances are taken per axis: along each axis a lane's
+// child boxes take three positions (the neighbour offset, its child bit
+// fixed), so nine squared distances give all 27 (the sum's rounding lies far
+// inside the margin of Rb2).  Lane r < 27 then collects the hit children of
+// range r from the lanes' masks.  Returns the segments and their sources.  Called
+// by the whole warp.
+__device__ __noinline__ int2 prune_round_fast(bool valid, int sub, int lane, float3 pi, float Rb2, float side,
+                                              float cside, const TTab* pr, uint32_t cand, int2* seg) {
+  uint32_t mine = 0;
+  if (valid) {
+    const float cx = (float)(sub & 1) * cside, cy = (float)((sub >> 1) & 1) * cside, cz = (float)(sub >> 2) * cside;
+    float ex[3], ey[3], ez[3];
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      const float b0 = (float)(o - 1) * side;
+      const float dx = fmaxf(fmaxf(b0 + cx - pi.x, pi.x - (b0 + cx + cside)), 0.0f);
+      const float dy = fmaxf(fmaxf(b0 + cy - pi.y, pi.y - (b0 + cy + cside)), 0.0f);
+      const float dz = fmaxf(fmaxf(b0 + cz - pi.z, pi.z - (b0 + cz + cside)), 0.0f);
+      ex[o] = dx * dx;
+      ey[o] = dy * dy;
+      ez[o] = dz * dz;
+    }
+#pragma unroll
+    for (int m = 0; m < 27; ++m)
+      if (((cand >> m) & 1u) && ex[m % 3] + ey[(m / 3) % 3] + ez[m / 9] < Rb2) mine |= 1u << m;
+  }
+#pragma unroll
+  for (int o = kTreeTpp; o < 32; o <<= 1) mine |= __shfl_xor_sync(0xffffffffu, mine, o);
+  uint32_t hit = 0;
+#pragma unroll
+  for (int c = 0; c < kTreeTpp; ++c) hit |= ((__shfl_sync(0xffffffffu, mine, c) >> lane) & 1u) << c;
+  const int r = lane < 27 ? lane : 0;
+  if (lane >= 27) hit = 0;
+  const int32_t* cv = pr->cv + 8 * r;
+  int len = 0;
+#pragma unroll 1
+  for (uint32_t b = hit; b != 0u;) {  // the runs of hit children
+    const int c0 = __ffs((int)b) - 1, c1 = c0 + __ffs((int)~(b >> c0)) - 1;
+    len += cv[c1] - cv[c0];
+    b &= b + (1u << c0);
+  }
+  const int ns = __popc(hit & ~(hit << 1));
+  int il = len, in = ns;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int ul = __shfl_up_sync(0xffffffffu, il, o), un = __shfl_up_sync(0xffffffffu, in, o);
+    if (lane >= o) {
+      il += ul;
+      in += un;
+    }
+  }
+  const int2 out = make_int2(__shfl_sync(0xffffffffu, in, 31), __shfl_sync(0xffffffffu, il, 31));
+  il -= len;
+  in -= ns;
+#pragma unroll 1
+  for (uint32_t b = hit; b != 0u; ++in) {
+    const int c0 = __ffs((int)b) - 1, c1 = c0 + __ffs((int)~(b >> c0)) - 1;
+    seg[in] = make_int2(il, (int)pack_js(pr->rlo[r] + (cv[c0] - pr->rcum[r]), pr->rsc[r]));
+    il += cv[c1] - cv[c0];
+    b &= b + (1u << c0);
+  }
+  return out;
+}
+
+// Stages cnt sources into spos / sidx [0, cnt) relative to the group corner (w:
+// the mass); item u is source map(u) (its index and shift code).  A lane takes
+// its items four at a time and issues their loads together, so that four L2
+// latencies overlap instead of running one after another.  Called by the whole
+// warp.
 template <class Map>
 __device__ __forceinline__ void tstage_items(int cnt, int lane, const TGeo& g, const float4* __restrict__ rel,
-                                             const int4* __restrict__ fine, float4* spos, uint32_t* sidx,
-                                             const uint8_t* __restrict__ act, Map map) {
+                                             const int4* __restrict__ fine, float4* spos, uint32_t* sidx, Map map) {
   for (int u0 = lane; u0 < cnt; u0 += 4 * 32) {
     int32_t j[4];
     int sc[4];
@@ -478,16 +504,13 @@ __device__ __forceinline__ void tstage_items(int cnt, int lane, const TGeo& g, c
     }
     float4 rj[4];
     int4 fj[4];
-    float aw[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       rj[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       fj[i] = make_int4(0, 0, 0, 0);
-      aw[i] = 0.0f;
       if (u0 + 32 * i < cnt) {
         rj[i] = rel[j[i]];
         fj[i] = fine[j[i]];
-        if (act != nullptr) aw[i] = (float)act[j[i]];
       }
     }
 #pragma unroll
@@ -495,7 +518,7 @@ __device__ __forceinline__ void tstage_items(int cnt, int lane, const TGeo& g, c
       const int u = u0 + 32 * i;
       if (u < cnt) {
         const float3 p = rel_to(g, rj[i], fj[i], sc[i]);
-        spos[u] = make_float4(p.x, p.y, p.z, act != nullptr ? aw[i] : rj[i].w);
+        spos[u] = make_float4(p.x, p.y, p.z, rj[i].w);
         sidx[u] = pack_js(j[i], sc[i]);
       }
     }
@@ -505,12 +528,11 @@ __device__ __forceinline__ void tstage_items(int cnt, int lane, const TGeo& g, c
 
 // Stages sources [u0, u0 + kTCap) of the round's hit children (flattened)
 // relative to the group corner.  Called by the whole warp.
-__device__ __forceinline__ int tstage_union(int u0, int total, int nh, const TPrune* pr, int lane,
+__device__ __noinline__ int tstage_union(int u0, int total, int nh, const TPrune* pr, int lane,
                                             const TGeo& g, const float4* __restrict__ rel,
-                                            const int4* __restrict__ fine, float4* spos, uint32_t* sidx,
-                                            const uint8_t* __restrict__ act = nullptr) {
+                                            const int4* __restrict__ fine, float4* spos, uint32_t* sidx) {
   const int cnt = min(kTCap, total - u0);
-  tstage_items(cnt, lane, g, rel, fine, spos, sidx, act, [&](int u, int32_t& j, int& sc) {
+  tstage_items(cnt, lane, g, rel, fine, spos, sidx, [&](int u, int32_t& j, int& sc) {
     const int uu = u0 + u;
     int lo = 0, hi = nh - 1;
     while (lo < hi) {
@@ -522,34 +544,6 @@ __device__ __forceinline__ int tstage_union(int u0, int total, int nh, const TPr
     const int r = ch >> 3;
     j = pr->rlo[r] + (vv - pr->rcum[r]);
     sc = pr->rsc[r];
-  });
-  return cnt;
-}
-
-// Stages sources [v0, v0 + kTCap) of the concatenated ranges relative to the
-// leaf corner (the ranges' first sources, starts and shifts go to pr first).
-// Called by the whole warp.
-__device__ __forceinline__ int tstage(int v0, const TRanges& R, int lane, const TGeo& g,
-                                      const float4* __restrict__ rel, const int4* __restrict__ fine, float4* spos,
-                                      uint32_t* sidx, TPrune* pr, const uint8_t* __restrict__ act = nullptr) {
-  const int cnt = min(kTCap, R.nsrc - v0);
-  if (lane < 28) {
-    pr->rlo[lane] = R.lo;
-    pr->rcum[lane] = R.cum;  // lane 27 (an empty range): the total
-    pr->rsc[lane] = R.sc;
-  }
-  __syncwarp();
-  tstage_items(cnt, lane, g, rel, fine, spos, sidx, act, [&](int u, int32_t& j, int& sc) {
-    const int v = v0 + u;
-    // the last range starting at or before v (an empty range shares its
-    // start with the next one)
-    int lo = 0, hi = 26;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (pr->rcum[mid] <= v) lo = mid; else hi = mid - 1;
-    }
-    j = pr->rlo[lo] + (v - pr->rcum[lo]);
-    sc = pr->rsc[lo];
   });
   return cnt;
 }
@@ -594,43 +588,43 @@ __device__ __forceinline__ uint64_t reverse_rec(int32_t j, int32_t ti, int sc) {
 }
 
 // Appends the list entries marked in each lane's mask wm (bit e: entry e of
-// the lane's column in lje): one counter atomic for the warp, then every
-// lane writes its records at its offset.  Called by all 32 lanes.
-// one mask bit per list entry
-using TMark = std::conditional_t<(kTreeList > 32), unsigned long long, uint32_t>;
-__device__ __forceinline__ int tmark_popc(uint32_t m) { return __popc(m); }
-__device__ __forceinline__ int tmark_popc(unsigned long long m) { return __popcll(m); }
-__device__ __forceinline__ int tmark_ffs(uint32_t m) { return __ffs((int)m); }
-__device__ __forceinline__ int tmark_ffs(unsigned long long m) { return __ffsll((long long)m); }
-
-__device__ __forceinline__ void emit_marked(const sphh::TreeDensityArgs& a, TMark wm, const uint32_t* lje,
-                                            int32_t ti, int lane) {
-  static_assert(kTreeList <= 64, "one mask bit per list entry");
-  const int my = tmark_popc(wm);
+// the lane's list): one counter atomic for the warp, then every lane writes its
+// records at its offset.  Called by all 32 lanes.  (Not inlined: expanded in
+// place it made the kernel 40 % longer, and instruction fetches are a part of
+// its time.)
+struct TEmit {
+  unsigned long long* count;
+  uint64_t* raw;
+  int32_t* start;
+  int64_t cap;
+  int32_t* status;
+};
+__device__ __noinline__ void emit_marked(TEmit o, uint32_t wm, const TRound& S, int32_t ti, int lane) {
+  const int my = __popc(wm);
   int incl = my;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += v;
+  for (int d = 1; d < 32; d <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += v;
   }
   const int total = __shfl_sync(0xffffffffu, incl, 31);
-  if (total == 0) return;
-  unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(a.rev_count, (unsigned long long)total);
-  unsigned long long k = __shfl_sync(0xffffffffu, base, 0) + (unsigned long long)(incl - my);
-  while (wm) {
-    const int e = tmark_ffs(wm) - 1;
-    wm &= wm - 1u;
-    const uint32_t je = lje[e * 32 + lane];
-    const int32_t j = unpack_j(je);
-    if (k < (unsigned long long)a.rev_cap) {
-      a.rev_raw[k] = reverse_rec(j, ti, unpack_s(je));
-      atomicAdd(&a.rev_start[j], 1);
-    } else {
-      atomicOr(a.status, SPH_ST_CAPACITY);
+  if (total != 0) {
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(o.count, (unsigned long long)total);
+    unsigned long long k = __shfl_sync(0xffffffffu, base, 0) + (unsigned long long)(incl - my);
+#pragma unroll 1
+    for (; wm != 0u; wm &= wm - 1u, ++k) {
+      const uint32_t je = __float_as_uint(S.pos[S.list[__ffs((int)wm) - 1][lane]].w);
+      const int32_t j = unpack_j(je);
+      if (k < (unsigned long long)o.cap) {
+        o.raw[k] = reverse_rec(j, ti, unpack_s(je));
+        atomicAdd(&o.start[j], 1);
+      } else {
+        atomicOr(o.status, SPH_ST_CAPACITY);
+      }
     }
-    ++k;
   }
+  __syncwarp();
 }
 
 // Outputs of target ti (source index) from its sums at h (Sec. 3.1 and the
@@ -661,211 +655,300 @@ __device__ __forceinline__ void tdens_write(const sphh::TreeDensityArgs& a, cons
   if (noconv) atomicOr(a.status, SPH_ST_H_NOCONV);
 }
 
+// A warp takes windows of kTWin consecutive targets from a counter: of each
+// leaf the rounds (kTPer targets from the leaf's first one on) that begin in
+// the window, so that a leaf's rounds, and with them the order of every sum, do
+// not depend on the windows nor on what else the pool holds.
+//
+// Bound by instruction issue and fetch: 24 warps per SM, 1,670 warp
+// instructions per particle.  On the 2M clustered box the call (build, density,
+// force) went from 11.10 to 7.13 ms and the kernel from 7.9 to 4.1 ms; before,
+// every round staged the ~290 sources of its children in shared memory (18.6 KB
+// per warp, 12 warps per SM) and filtered them from there.  What counted: the
+// filter on sources held in registers, keeping only the ~90 listed ones (11.1
+// -> 9.8 ms with windows of 32 targets); the loops and warp functions that are
+// not expanded in place, as fetch stalls were the largest (63 -> 43 KB of code,
+// 10.0 -> 7.3 ms); windows of two rounds, as a round beside a dense core tests
+// up to 23,000 sources (32 targets 7.32 ms, 12 7.02, 8 7.13, 4 7.61; but the
+// pool of 48 uneven boxes 4.45, 3.73, 3.64 and 3.59 ms).
+//
 // kMask: the masked loops (a.act, a.act_pre set); the plain instance carries
 // none of their tests.
 template <int K, bool kMask>
-__global__ void __launch_bounds__(kTWarps * 32) k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
+__global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
   const NewtonConst nwt = newton_const<K>(ph);
-  unsigned char* base = tsm + (size_t)warp * kTWarpSmem;
-  float4* spos = reinterpret_cast<float4*>(base);
-  uint32_t* sidx = reinterpret_cast<uint32_t*>(spos + kTCap);
-  float* lr2 = reinterpret_cast<float*>(sidx + kTCap);
-  uint32_t* lje = reinterpret_cast<uint32_t*>(lr2 + kTRows * 32);
-  TPrune* pr = reinterpret_cast<TPrune*>(lje + kTRows * 32);
+  TRound& S = *reinterpret_cast<TRound*>(tsm + (size_t)(threadIdx.x >> 5) * kTRoundBytes);
   const int t = lane / kTreeTpp, sub = lane % kTreeTpp;
   const int32_t nl = *a.n_leaves;
+  const int64_t n = a.n_total;
   unsigned long long pair_acc = 0, free_acc = 0;
-  for (int32_t li = next_group(a.work, lane); li < nl; li = next_group(a.work, lane)) {
-    const TreeLeaf Lf = a.leaves[li];
-    const int32_t t_lo = Lf.start, n_t = a.leaves[li + 1].start - Lf.start;
-    const GridDev G = a.grid[sim_of_cell(a.grid, a.n_sims, Lf.cell)];
-    const TGeo g = leaf_geo(Lf, G);
-    const TRanges R = load_ranges(a.ranges, li, lane);
-    if (kMask) {
-      // masked loops: a group without a masked particle in its 27 cells has
-      // no masked target and no masked receiver of a reverse pair
+  for (int64_t w0 = (int64_t)next_group(a.work, lane) * kTWin; w0 < n; w0 = (int64_t)next_group(a.work, lane) * kTWin) {
+    const int32_t w1 = (int32_t)(w0 + kTWin < n ? w0 + kTWin : n);
+    for (int32_t li = a.leaf_of[w0] + a.flag[w0] - 1; li < nl; ++li) {
+      const TreeLeaf Lf = a.leaves[li];
+      if (Lf.start >= w1) break;
+      const int32_t t_hi = a.leaves[li + 1].start;
+      const int32_t first =
+          Lf.start >= (int32_t)w0 ? Lf.start : Lf.start + (((int32_t)w0 - Lf.start + kTPer - 1) / kTPer) * kTPer;
+      if (first >= t_hi || first >= w1) continue;  // no round of this leaf begins here
+      const GridDev G = a.grid[sim_of_cell(a.grid, a.n_sims, Lf.cell)];
+      const TGeo g = leaf_geo(Lf, G);
+      const TRanges R = load_ranges(a.ranges, li, lane);
       const int32_t cum_next = __shfl_down_sync(0xffffffffu, R.cum, 1);
-      const int32_t na = lane < 27 ? a.act_pre[R.lo + (cum_next - R.cum)] - a.act_pre[R.lo] : 0;
-      if (!__any_sync(0xffffffffu, na > 0)) continue;
-    }
-    const int nsrc = R.nsrc;
-    const float hcap = h_cap<K>(g.side_d, g.L);
-    const bool one_chunk = nsrc <= kTCap;
-    // children are half the cell (a cell at the deepest level has one child)
-    const float cside = Lf.depth < kTreeDepth ? 0.5f * g.side : g.side;
-    // (masked loops: the staged w is 1 for a masked source, else 0)
-    ChMask cand_all = 0, cand_act = 0;
-    if (one_chunk) {
-      tstage(0, R, lane, g, a.rel, a.fine, spos, sidx, pr, kMask ? a.act : nullptr);
-    } else {
-      prune_tables(a.skey, R, Lf.depth, lane, pr, kMask ? a.act_pre : nullptr);
-      cand_all = group_candidates(sub, pr, false);
-      if (kMask) cand_act = group_candidates(sub, pr, true);
-    }
-    for (int32_t t0 = 0; t0 < n_t; t0 += kTPer) {
-      const bool valid = t0 + t < n_t;
-      const int32_t ti = a.tgt[t_lo + (valid ? t0 + t : 0)];
-      // masked loops: a target outside the mask keeps its h and outputs; its
-      // list at its current support only sends reverse pairs to the masked
-      // particles (whose forces need every pair within either support)
-      const bool on = valid && (!kMask || a.act[ti] != 0);
-      const float4 reli = a.rel[ti];
-      const int4 fi = a.fine[ti];
-      const float3 pi = rel_to(g, reli, fi, kNoShift);
-      const float4 vi = a.vel4[ti];
-      const float Ri = a.lrad[ti];
-      const float R2 = Ri * Ri;
-      // (a target outside the mask lists the masked sources only)
-      const bool all_src = !kMask || on;
-      // 1. filter: sources with r < R_i into this lane's list.  A group that
-      // does not fit one staging chunk stages, per round, only the children
-      // of its 27 cells that some target of the round reaches: a child whose
-      // box lies beyond R_i (with a margin far above the rounding of r) holds
-      // no list entry of that target.
-      int cnt = 0;
-      if (one_chunk) {
-        if (valid) {
-          for (int k = sub; k < nsrc; k += kTreeTpp) {
-            const float4 sk = spos[k];
-            const float r2 = r2_of(pi, sk);
-            const int at = min(cnt, kTreeList) * 32 + lane;
-            lr2[at] = r2;
-            lje[at] = sidx[k];
-            cnt += r2 < R2 && (all_src || sk.w != 0.0f);
-          }
-        }
+      if (kMask) {
+        // masked loops: a leaf without a masked particle in its 27 cells has
+        // no masked target and no masked receiver of a reverse pair
+        const int32_t na = lane < 27 ? a.act_pre[R.lo + (cum_next - R.cum)] - a.act_pre[R.lo] : 0;
+        if (!__any_sync(0xffffffffu, na > 0)) continue;
+      }
+      const float hcap = h_cap<K>(g.side_d, g.L);
+      // few sources: the 27 ranges whole; else the children of the ranges
+      // that some target of the round reaches (children are half the cell; a
+      // cell at the deepest level has one child)
+      const bool whole = R.nsrc <= kTWhole;
+      const bool shifted = __any_sync(0xffffffffu, R.sc != kNoShift);
+      const float cside = Lf.depth < kTreeDepth ? 0.5f * g.side : g.side;
+      uint32_t cand_all = 0, cand_act = 0;
+      int nseg = 0, total = 0;
+      if (whole) {
+        __syncwarp();
+        const bool some = lane < 27 && cum_next > R.cum;
+        const unsigned bm = __ballot_sync(0xffffffffu, some);
+        if (some) S.seg[__popc(bm & lt)] = make_int2(R.cum, (int)pack_js(R.lo, R.sc));
+        nseg = __popc(bm);
+        total = R.nsrc;
+        __syncwarp();
       } else {
-        int nh = 0;
-        const int total = prune_round_fast(valid, sub, lane, pi, R2 * (1.0f + 0x1p-10f), g.side, cside, pr, nh,
-                                           all_src ? cand_all : cand_act);
-        for (int u0 = 0; u0 < total; u0 += kTCap) {
-          const int c = tstage_union(u0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx, kMask ? a.act : nullptr);
-          if (valid) {
-            for (int k = sub; k < c; k += kTreeTpp) {
-              const float4 sk = spos[k];
-              const float r2 = r2_of(pi, sk);
-              const int at = min(cnt, kTreeList) * 32 + lane;
-              lr2[at] = r2;
-              lje[at] = sidx[k];
-              cnt += r2 < R2 && (all_src || sk.w != 0.0f);
+        prune_tables(a.skey, R, Lf.depth, lane, &S.tab, kMask ? a.act_pre : nullptr);
+        cand_all = group_candidates(sub, &S.tab, false);
+        if (kMask) cand_act = group_candidates(sub, &S.tab, true);
+      }
+#pragma unroll 1
+      for (int32_t t0 = first; t0 < t_hi && t0 < w1; t0 += kTPer) {
+        const bool valid = t0 + t < t_hi;
+        const int32_t ti = a.tgt[t0 + (valid ? t : 0)];
+        // masked loops: a target outside the mask keeps its h and outputs; its
+        // list, of masked sources, only sends reverse pairs to them (their
+        // forces need every pair within either support)
+        const bool on = valid && (!kMask || a.act[ti] != 0);
+        const float4 reli = a.rel[ti];
+        const int4 fi = a.fine[ti];
+        const float3 pi = rel_to(g, reli, fi, kNoShift);
+        const float4 vi = a.vel4[ti];
+        const float Ri = a.lrad[ti];
+        const float R2 = Ri * Ri;
+        const float h_start = a.hs[ti];
+        __syncwarp();  // the previous round is done with the shared arrays
+        if (sub == 0) S.tgt[t] = make_float4(pi.x, pi.y, pi.z, valid ? R2 : -1.0f);
+        if (!whole) {
+          const int2 st = prune_round_fast(valid, sub, lane, pi, R2 * (1.0f + 0x1p-10f), g.side, cside, &S.tab,
+                                           !kMask || on ? cand_all : cand_act, S.seg);
+          nseg = st.x;
+          total = st.y;
+        }
+        __syncwarp();
+        // masked loops: which targets are in the mask (bit 8 q: target q)
+        const unsigned on_mask = kMask ? __ballot_sync(0xffffffffu, on) : 0xffffffffu;
+        int nq = 0;  // the sources the lane's target lists, once more were kept than fit
+#pragma unroll 1
+        for (unsigned todo = (1u << kTPer) - 1u; todo != 0u;) {
+          // the round's targets, or as many of them as are known to fit
+          unsigned now = 0u;
+          for (int q = 0, sum = 0; q < kTPer; ++q) {
+            sum += ((todo >> q) & 1u) ? __shfl_sync(0xffffffffu, nq, q * kTreeTpp) : 0;
+            if (((todo >> q) & 1u) && (now == 0u || sum <= kTKept)) now |= 1u << q;
+          }
+          // 1. filter: the sources 32 at a time, one per lane; the round's
+          // targets test each in turn.  Those within some target's list radius
+          // are kept; lane sub of a target lists the kept slots of its own
+          // sources, every kTreeTpp-th of the segments' sequence, in order.
+          // A target whose list overflows (it leaves for the per-target kernel)
+          // stops listing, so that a round beside a dense core does not go on
+          // collecting the core.
+          unsigned live = now;
+          int cnt = 0, kept = 0, seg0 = 0;
+#pragma unroll 1
+          for (int u0 = 0; u0 < total; u0 += 64) {
+            const unsigned over = __ballot_sync(0xffffffffu, cnt > kTreeList);
+            if (over != 0u) {
+#pragma unroll
+              for (int q = 0; q < kTPer; ++q)
+                if ((over >> (q * kTreeTpp)) & kTGroup) live &= ~(1u << q);
+              if (live == 0u) break;
+            }
+            float4 rj[2];
+            int4 fj[2];
+            uint32_t je[2];
+            bool aj[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              // the segment of source u: the starts that fall into these 32
+              // sources, as a bit mask, count up to lane
+              const int ub = u0 + 32 * i, u = ub + lane, s = seg0 + 1 + lane;
+              const int st = s < nseg ? S.seg[s].x - ub : 32;
+              const unsigned bits = __reduce_or_sync(0xffffffffu, st < 32 ? 1u << st : 0u);
+              const int2 sg = S.seg[seg0 + __popc(bits & (lt | (1u << lane)))];
+              seg0 += __popc(bits);
+              je[i] = (uint32_t)sg.y + (uint32_t)(u - sg.x);
+              const int32_t j = u < total ? unpack_j(je[i]) : ti;
+              rj[i] = a.rel[j];
+              fj[i] = a.fine[j];
+              aj[i] = kMask ? a.act[j] != 0 : true;
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              const float3 p = shifted ? rel_to(g, rj[i], fj[i], unpack_s(je[i])) : rel_to(g, rj[i], fj[i], kNoShift);
+              const bool in = u0 + 32 * i + lane < total;
+              unsigned any = 0u, own = 0u;
+#pragma unroll
+              for (int q = 0; q < kTPer; ++q) {
+                const float4 T = S.tgt[q];
+                // (a target outside the mask lists the masked sources only)
+                const bool is = in && r2_of(make_float3(T.x, T.y, T.z), make_float4(p.x, p.y, p.z, 0.f)) < T.w &&
+                                (!kMask || aj[i] || ((on_mask >> (q * kTreeTpp)) & 1u));
+                const unsigned hit = ((live >> q) & 1u) ? __ballot_sync(0xffffffffu, is) : 0u;
+                any |= hit;
+                if (q == t) own = hit;
+              }
+              if ((any >> lane) & 1u) {
+                const int at = kept + __popc(any & lt);
+                if (at < kTKept) S.pos[at] = make_float4(p.x, p.y, p.z, __uint_as_float(je[i]));
+              }
+#pragma unroll 1
+              for (unsigned m = (own >> sub) & kTLanes; m != 0u; m &= m - 1u) {
+                const int b = __ffs((int)m) - 1 + sub;
+                S.list[min(cnt, kTreeList)][lane] = (uint8_t)(kept + __popc(any & ((1u << b) - 1u)));
+                ++cnt;
+              }
+              kept += __popc(any);
+            }
+          }
+          __syncwarp();
+          if (kept > kTKept && live != 0u && (live != now || (live & (live - 1u)) != 0u)) {
+            // too many sources are near some target: fewer targets at a time
+            // (one target's list of up to kTreeTpp * kTreeList sources fits);
+            // those that left are done
+            const int nt = gsumi(cnt);
+            if ((now >> t) & 1u) nq = nt;
+            now &= ~live;
+          }
+          if (now == 0u) continue;
+          todo &= ~now;
+          const bool act_now = valid && ((now >> t) & 1u), on_now = act_now && on;
+          // a target whose list overflowed, or whose support outgrows R_i, leaves
+          // the round: it is queued for the per-target kernel, which solves it at
+          // its own level with all 32 lanes of a warp over its 27 cells (so the
+          // other targets of its round do not wait for it).  The flag is shared
+          // by the target's lanes.
+          bool queued = group_any(cnt > kTreeList, lane);
+          // 2. Newton-Raphson passes
+          float h = valid ? h_start : hcap;
+          if (on) {
+            if (!(h > 0.0f)) h = 0.5f * hcap;
+            if (h > hcap) h = hcap;
+          }
+          if (valid && KernT<K>::gamma * h > Ri) queued = true;
+          float hlo = 0.0f, hhi = INFINITY;
+          bool done = !on_now || queued, atcap = false, conv = false;
+          int it = 0, passes = 0;
+#pragma unroll 1
+          while (__any_sync(0xffffffffu, !done)) {
+            const float H = KernT<K>::gamma * h;
+            const float Hinv = 1.0f / H;
+            float Sw = 0.f, Sdw = 0.f;
+            if (!done)
+#pragma unroll 1
+              for (int e = 0; e < cnt; ++e) tnewton_pair<K>(r2_of(pi, S.pos[S.list[e][lane]]), H, Hinv, Sw, Sdw);
+            Sw = gsum(Sw);
+            Sdw = gsum(Sdw);
+            if (!done) {
+              passes = it + 1;
+              if (newton_update(Sw, Sdw, nwt, hcap, h, hlo, hhi, it, atcap, conv)) done = true;
+            }
+            // the list holds r < R_i: a support beyond it is queued
+            if (act_now && !queued && !atcap && KernT<K>::gamma * h > Ri) {
+              queued = true;
+              done = true;
+            }
+          }
+          // 3. final pass at h; the list's reverse pairs are marked on the way
+          // (bit e: entry e), with j's threshold read with its fine position
+          const float H = KernT<K>::gamma * h;
+          const float Hinv = 1.0f / H;
+          const float H2 = H * H;
+          TDSums s;
+          tds_zero(s);
+          uint32_t wm = 0;
+          if (on_now && !queued) {
+#pragma unroll 1
+            for (int e = 0; e < cnt; ++e) {
+              const float4 pk = S.pos[S.list[e][lane]];
+              const uint32_t je = __float_as_uint(pk.w);
+              const int32_t j = unpack_j(je);
+              const float4 rj = a.rel[j];
+              const int4 fj = a.fine[j];
+              const float3 d = pair_vec(g, reli, fi, rj, fj, unpack_s(je));
+              tdens_pair<K>(d.x, d.y, d.z, vi, a.vel4[j], rj.w, H, Hinv, s);
+              if (!atcap && want_reverse_t(__int_as_float(fj.w), ti, j, r2_of(pi, pk), H2, H, g.side) &&
+                  (!kMask || a.act[j] != 0))
+                wm |= 1u << e;
+            }
+          } else if (kMask && act_now && !queued) {
+            // outside the mask: the reverse pairs to its listed (masked) sources
+#pragma unroll 1
+            for (int e = 0; e < cnt; ++e) {
+              const float4 pk = S.pos[S.list[e][lane]];
+              if (want_reverse(a, ti, unpack_j(__float_as_uint(pk.w)), r2_of(pi, pk), H2, H, g.side)) wm |= 1u << e;
+            }
+          }
+          // reverse pairs from the lists: the warp takes one slot range for the
+          // whole round
+          emit_marked(TEmit{a.rev_count, a.rev_raw, a.rev_start, a.rev_cap, a.status}, wm, S, ti, lane);
+          tcombine(s);
+          // 4. publish the list for the force loop: the target's lanes' lists
+          // packed one after another (lane sub's entries after those of the
+          // lanes below it), so that the force reads them in whole sectors
+          {
+            int incl = on_now && !queued ? cnt : 0;
+#pragma unroll
+            for (int o = 1; o < kTreeTpp; o <<= 1) {
+              const int v = __shfl_up_sync(0xffffffffu, incl, o, kTreeTpp);
+              if (sub >= o) incl += v;
+            }
+            const int all = __shfl_sync(0xffffffffu, incl, kTreeTpp - 1, kTreeTpp);
+            if (on_now) {
+              if (sub == 0) a.list_cnt[ti] = (uint16_t)(atcap || queued ? kListFallback : all);
+              if (!queued) {
+                uint32_t* dst = a.lists + (int64_t)ti * kTreeListTarget + (incl - cnt);
+#pragma unroll 1
+                for (int e = 0; e < cnt; ++e) dst[e] = __float_as_uint(S.pos[S.list[e][lane]].w);
+              }
+            }
+          }
+          if (act_now && sub == 0) {
+            if (queued) {
+              // solved at its own level by the per-target kernel
+              const int32_t k = atomicAdd(a.fb_count, 1);
+              if (k < a.n_total) a.fb_list[k] = ti | kFbOwnLevel | (on ? 0 : kFbPassive);
+              free_acc += on ? 1ull : 0ull;
+            } else if (on) {
+              tdens_write<K>(a, ph, ti, h, s, vi.w, passes, !conv && !atcap);
+              if (atcap) {
+                // the support outgrew this level: re-solved at a coarser one
+                const int32_t k = atomicAdd(a.fb_count, 1);
+                if (k < a.n_total) a.fb_list[k] = ti;
+              } else {
+                pair_acc += (unsigned long long)s.npair;
+              }
             }
           }
           __syncwarp();
         }
       }
-      // a target whose list overflowed, or whose support outgrows R_i, leaves
-      // the group: it is queued for the per-target kernel, which solves it at
-      // its own level with all 32 lanes of a warp over its 27 cells (so the
-      // other targets of its round do not wait for it).  The flag is shared by
-      // the target's lanes.
-      bool queued = group_any(cnt > kTreeList, lane);
-      // 2. Newton-Raphson passes
-      float h = valid ? a.hs[ti] : hcap;
-      if (on) {
-        if (!(h > 0.0f)) h = 0.5f * hcap;
-        if (h > hcap) h = hcap;
-      }
-      {
-        // evaluated by every lane (a ballot), then merged
-        const bool outgrown = group_any(valid && KernT<K>::gamma * h > Ri, lane);
-        queued = queued || outgrown;
-      }
-      float hlo = 0.0f, hhi = INFINITY;
-      bool done = !on || queued, atcap = false, conv = false;
-      int it = 0, passes = 0;
-      while (__any_sync(0xffffffffu, !done)) {
-        const float H = KernT<K>::gamma * h;
-        const float Hinv = 1.0f / H;
-        float Sw = 0.f, Sdw = 0.f;
-        if (!done)
-          for (int e = 0; e < cnt; ++e) tnewton_pair<K>(lr2[e * 32 + lane], H, Hinv, Sw, Sdw);
-        Sw = gsum(Sw);
-        Sdw = gsum(Sdw);
-        if (!done) {
-          passes = it + 1;
-          if (newton_update(Sw, Sdw, nwt, hcap, h, hlo, hhi, it, atcap, conv)) done = true;
-        }
-        // the list holds r < R_i: a support beyond it is queued
-        const bool outgrown = group_any(valid && !queued && !atcap && KernT<K>::gamma * h > Ri, lane);
-        if (outgrown) {
-          queued = true;
-          done = true;
-        }
-      }
-      // 3. final pass at h
-      const float H = KernT<K>::gamma * h;
-      const float Hinv = 1.0f / H;
-      const float H2 = H * H;
-      TDSums s;
-      tds_zero(s);
-      // the list's reverse pairs are marked on the way (bit e: entry e; a
-      // list holds at most kTreeList = 32), with j's threshold read with its
-      // fine position
-      TMark wm = 0;
-      if (on && !queued) {
-        for (int e = 0; e < cnt; ++e) {
-          const uint32_t je = lje[e * 32 + lane];
-          const int32_t j = unpack_j(je);
-          const float4 rj = a.rel[j];
-          const int4 fj = a.fine[j];
-          const float3 d = pair_vec(g, reli, fi, rj, fj, unpack_s(je));
-          tdens_pair<K>(d.x, d.y, d.z, vi, a.vel4[j], rj.w, H, Hinv, s);
-          if (!atcap && want_reverse_t(__int_as_float(fj.w), ti, j, lr2[e * 32 + lane], H2, H, g.side) &&
-              (!kMask || a.act[j] != 0))
-            wm |= (TMark)1 << e;
-        }
-      } else if (kMask && valid && !queued) {
-        // outside the mask: the reverse pairs to its listed (masked) sources
-        for (int e = 0; e < cnt; ++e) {
-          const int32_t j = unpack_j(lje[e * 32 + lane]);
-          if (want_reverse(a, ti, j, lr2[e * 32 + lane], H2, H, g.side)) wm |= (TMark)1 << e;
-        }
-      }
-      // reverse pairs from the lists: the warp takes one slot range for the
-      // whole round
-      emit_marked(a, wm, lje, ti, lane);
-      tcombine(s);
-      // 4. publish the list for the force loop: the target's lanes' lists
-      // packed one after another (lane sub's entries after those of the
-      // lanes below it), so that the force reads them in whole sectors
-      {
-        int incl = on && !queued ? cnt : 0;
-#pragma unroll
-        for (int o = 1; o < kTreeTpp; o <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, incl, o, kTreeTpp);
-          if (sub >= o) incl += v;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, kTreeTpp - 1, kTreeTpp);
-        if (on) {
-          if (sub == 0) a.list_cnt[ti] = (uint16_t)(atcap || queued ? kListFallback : total);
-          if (!queued) {
-            uint32_t* dst = a.lists + (int64_t)ti * kTreeListTarget + (incl - cnt);
-            for (int e = 0; e < cnt; ++e) dst[e] = lje[e * 32 + lane];
-          }
-        }
-      }
-      if (valid && sub == 0) {
-        if (queued) {
-          // solved at its own level by the per-target kernel
-          const int32_t k = atomicAdd(a.fb_count, 1);
-          if (k < a.n_total) a.fb_list[k] = ti | kFbOwnLevel | (on ? 0 : kFbPassive);
-          free_acc += on ? 1ull : 0ull;
-        } else if (on) {
-          tdens_write<K>(a, ph, ti, h, s, vi.w, passes, !conv && !atcap);
-          if (atcap) {
-            // the support outgrew this level: re-solved at a coarser one
-            const int32_t k = atomicAdd(a.fb_count, 1);
-            if (k < a.n_total) a.fb_list[k] = ti;
-          } else {
-            pair_acc += (unsigned long long)s.npair;
-          }
-        }
-      }
-      __syncwarp();
     }
-    __syncwarp();
   }
   if (ph.count_pairs) {
     unsigned long long v = pair_acc, w = free_acc;
@@ -1238,10 +1321,10 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
   extern __shared__ __align__(16) unsigned char tsm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const NewtonConst nwt = newton_const<K>(ph);
-  unsigned char* base = tsm + (size_t)warp * kTWarpSmem;
+  unsigned char* base = tsm + (size_t)warp * kTFbWarpSmem;
   float4* spos = reinterpret_cast<float4*>(base);
   uint32_t* sidx = reinterpret_cast<uint32_t*>(spos + kTCap);
-  TPrune* pr = reinterpret_cast<TPrune*>(sidx + kTCap + kTRows * 32 * 2);
+  TPrune* pr = reinterpret_cast<TPrune*>(sidx + kTCap);
   const int32_t nq = min(*a.fb_count, (int32_t)a.n_total);
   unsigned long long pair_acc = 0;
   for (int32_t q = next_group(a.fb_work, lane); q < nq; q = next_group(a.fb_work, lane)) {
@@ -1272,8 +1355,8 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
       prune_tables(a.skey, Rr, Lp.depth, lane, pr);
       const float cs = Lp.depth < kTreeDepth ? 0.5f * gp.side : gp.side;
       const float H2 = H * H;
-      int nhp = 0;
-      const int tot = prune_round(true, lane % kTreeTpp, lane, pp, H2 * (1.0f + 0x1p-10f), gp.side, cs, pr, nhp);
+      const int2 hp2 = prune_round(lane, pp, H2 * (1.0f + 0x1p-10f), gp.side, cs, pr);
+      const int nhp = hp2.x, tot = hp2.y;
       for (int v0 = 0; v0 < tot; v0 += kTCap) {
         const int c = tstage_union(v0, tot, nhp, pr, lane, gp, a.rel, a.fine, spos, sidx);
         for (int k0 = 0; k0 < c; k0 += 32) {
@@ -1323,7 +1406,9 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
 #define TREE_FB_SELECT(Hsup)                                                                                   \
   if ((Hsup) > Rp) {                                                                                           \
     Rp = fminf(g.side, 1.25f * (Hsup));                                                                        \
-    total = prune_round(true, lane % kTreeTpp, lane, pi, Rp * Rp * (1.0f + 0x1p-10f), g.side, cside, pr, nh); \
+    const int2 hit = prune_round(lane, pi, Rp * Rp * (1.0f + 0x1p-10f), g.side, cside, pr);                     \
+    nh = hit.x;                                                                                                \
+    total = hit.y;                                                                                             \
     one_chunk = total <= kTCap;                                                                                \
     if (one_chunk) tstage_union(0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx);                         \
   }
@@ -1531,18 +1616,22 @@ static int tree_blocks(int64_t n) {
 
 template <int K>
 static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev& ph, cudaStream_t st) {
-  static int bps = 0;
+  static int bps = 0, bps_fb = 0;
   if (!bps) {
+    int b = 0;
     cudaError_t e = cudaFuncSetAttribute(k_tree_density<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kTDensSmem);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k_tree_density<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTDensSmem);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_tree_density_fb<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTDensSmem);
+      e = cudaFuncSetAttribute(k_tree_density_fb<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTFbSmem);
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_tree_density<K, false>, kTWarps * 32, kTDensSmem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tree_density<K, false>, kTWarps * 32, kTDensSmem);
     if (e != cudaSuccess) return e;
-    if (bps < 1) bps = 1;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_fb, k_tree_density_fb<K>, kTWarps * 32, kTFbSmem);
+    if (e != cudaSuccess) return e;
+    if (bps_fb < 1) bps_fb = 1;
+    bps = b < 1 ? 1 : b;
   }
   const int64_t n = a.n_total;
   cudaError_t e = cudaMemsetAsync(a.rev_count, 0, sizeof(unsigned long long), st);
@@ -1553,11 +1642,13 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_fill, 0, sizeof(int32_t) * (n > 0 ? n : 1), st);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
+  const int64_t want = (n + (int64_t)kTWin * kTWarps - 1) / ((int64_t)kTWin * kTWarps);
+  const int blocks = (int)(want < (int64_t)a.num_sms * bps ? want : (int64_t)a.num_sms * bps);
   if (a.act != nullptr)
-    k_tree_density<K, true><<<a.num_sms * bps, kTWarps * 32, kTDensSmem, st>>>(a, ph);
+    k_tree_density<K, true><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
   else
-    k_tree_density<K, false><<<a.num_sms * bps, kTWarps * 32, kTDensSmem, st>>>(a, ph);
-  k_tree_density_fb<K><<<a.num_sms * bps, kTWarps * 32, kTDensSmem, st>>>(a, ph);
+    k_tree_density<K, false><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
+  k_tree_density_fb<K><<<a.num_sms * bps_fb, kTWarps * 32, kTFbSmem, st>>>(a, ph);
   e = scan_exclusive_host_n(a.rev_start, n + 1, a.scan_tmp, st);
   if (e != cudaSuccess) return e;
   k_rev_scatter<<<a.num_sms * 4, 256, 0, st>>>(a.rev_raw, a.rev_count, a.rev_cap, a.rev_start, a.rev_fill, a.rev);
