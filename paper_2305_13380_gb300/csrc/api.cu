@@ -53,8 +53,8 @@ struct sph_ctx {
   // nested-grid scratch (SPH_FLAG_TREE), grown separately
   int64_t cap_tree = 0;
   int64_t rev_cap = 0;
-  uint64_t *key64 = nullptr, *key64_b = nullptr, *key64_c = nullptr, *skey = nullptr;
-  int32_t *tgt = nullptr, *flag = nullptr, *leaf_of = nullptr, *n_leaves = nullptr;
+  uint64_t *key64 = nullptr, *key64_b = nullptr, *skey = nullptr;
+  int32_t *tgt = nullptr, *leaf_of = nullptr, *n_leaves = nullptr;
   int8_t *level = nullptr, *fb_level = nullptr;
   int32_t* fb_list = nullptr;
   sphk::TreeLeaf* leaves = nullptr;
@@ -162,13 +162,11 @@ void free_grown(sph_ctx* c) {
 void free_tree(sph_ctx* c) {
   dfree(c->key64);
   dfree(c->key64_b);
-  dfree(c->key64_c);
   dfree(c->skey);
   dfree(c->tgt);
   dfree(c->level);
   dfree(c->fb_level);
   dfree(c->fb_list);
-  dfree(c->flag);
   dfree(c->leaf_of);
   dfree(c->n_leaves);
   dfree(c->leaves);
@@ -205,8 +203,8 @@ int ensure_tree(sph_ctx* c, int64_t n, int64_t rev_need) {
   if (rc < rev_need) rc = rev_need;
   if (rc < rev_old) rc = rev_old;
   if (rc > INT32_MAX) rc = INT32_MAX;
-  bool ok = dalloc(c->key64, cn) && dalloc(c->key64_b, cn) && dalloc(c->key64_c, cn) &&
-            dalloc(c->skey, cn) && dalloc(c->tgt, cn) && dalloc(c->flag, cn) && dalloc(c->level, cn) &&
+  bool ok = dalloc(c->key64, cn) && dalloc(c->key64_b, cn) && dalloc(c->skey, cn) && dalloc(c->tgt, cn) &&
+            dalloc(c->level, cn) &&
             dalloc(c->fb_level, cn) && dalloc(c->fb_list, cn) && dalloc(c->leaf_of, cn) && dalloc(c->n_leaves, 1) &&
             dalloc(c->leaves, cn + 1) && dalloc(c->ranges, 27 * cn) && dalloc(c->leaf_side, cn) &&
             dalloc(c->lrad, cn) && dalloc(c->fine, cn) && dalloc(c->rel, cn) && dalloc(c->trec, 4 * cn) &&
@@ -240,8 +238,8 @@ int ensure(sph_ctx* c, int64_t n, int n_sims, int cells_per_particle = 8) {
   const int64_t cc = (cells_per_particle > 8 ? cells_per_particle : 8) * cn + 216 * (int64_t)cs;
   bool ok = dalloc(c->grid, cs) && dalloc(c->key, cn) && dalloc(c->slot, cn) &&
             dalloc(c->count, cc + 1) && dalloc(c->cell_start, cc + 1) &&
-            dalloc(c->scan_sums, cc / 1024 + 2) && dalloc(c->perm, cn) &&
-            dalloc(c->rk, cn) && dalloc(c->rv, cn) && dalloc(c->rhist, sphh::radix_hist_words(cn)) &&
+            dalloc(c->scan_sums, sphh::scan_words(cc + 1)) && dalloc(c->perm, cn) &&
+            dalloc(c->rk, cn) && dalloc(c->rv, cn) && dalloc(c->rhist, sphh::radix_words(cn, (c->p.flags & SPH_FLAG_TREE) ? 8 : 4)) &&
             dalloc(c->overflow, (8 * cn + 216 * (int64_t)cs) / 3 + 2) && dalloc(c->pos4, cn) &&
             dalloc(c->vel4, cn) && dalloc(c->th4, cn) && dalloc(c->hs, cn) && dalloc(c->fD, cn) &&
             dalloc(c->dt_bits, cs) && dalloc(c->dt_f, 2 * cs) && dalloc(c->hmax_bits, cs) &&
@@ -426,6 +424,7 @@ int cuda_code(cudaError_t e) { return e == cudaSuccess ? SPH_OK : SPH_E_CUDA; }
 
 // Maps device status bits to the most severe return code.
 int code_of_status(int32_t s) {
+  if (s & SPH_ST_TIMEOUT) return SPH_E_TIMEOUT;
   if (s & SPH_ST_BOX) return SPH_E_BOX;
   if (s & SPH_ST_CAPACITY) return SPH_E_CAPACITY;
   if (s & SPH_ST_REBUILD) return SPH_E_REBUILD;
@@ -519,15 +518,15 @@ int do_build(sph_ctx* c, int n_sims, int64_t n_total, const int64_t* off, const 
     t.cell_start = c->cell_start;
     t.key64 = c->key64;
     t.key64_b = c->key64_b;
-    t.key64_c = c->key64_c;
     t.skey = c->skey;
     t.perm = c->perm;
     t.tgt = c->tgt;
     t.rv = c->rv;
     t.hist = c->rhist;
-    t.flag = c->flag;
     t.leaf_of = c->leaf_of;
     t.scan_tmp = c->scan_sums;
+    t.status = c->misc + sphk::kStatus;
+    t.num_sms = c->num_sms;
     t.leaves = c->leaves;
     t.n_leaves = c->n_leaves;
     t.ranges = c->ranges;
@@ -587,7 +586,6 @@ int do_tree_density(sph_ctx* c, const double* x, const double* y, const double* 
   d.tgt = c->tgt;
   d.leaves = c->leaves;
   d.n_leaves = c->n_leaves;
-  d.flag = c->flag;
   d.leaf_of = c->leaf_of;
   d.ranges = c->ranges;
   d.fine = c->fine;
@@ -630,7 +628,8 @@ int do_tree_density(sph_ctx* c, const double* x, const double* y, const double* 
     // masked loops: the mask in tree order
     const int rc = ensure_act(c, c->built_n);
     if (rc != SPH_OK) return rc;
-    if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, c->act_pre, c->scan_sums, c->st) !=
+    if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, c->act_pre, c->scan_sums,
+                               c->misc + sphk::kStatus, c->num_sms, c->st) !=
         cudaSuccess)
       return SPH_E_CUDA;
     d.act = c->act_s;
@@ -884,7 +883,7 @@ int do_force(sph_ctx* c, const double* x, const double* y, const double* z, cons
     if (active) {
       const int rc = ensure_act(c, c->built_n);
       if (rc != SPH_OK) return rc;
-      if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, nullptr, nullptr, c->st) != cudaSuccess)
+      if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, nullptr, nullptr, nullptr, 0, c->st) != cudaSuccess)
         return SPH_E_CUDA;
       a.act = c->act_s;
     }
@@ -1510,7 +1509,7 @@ int hier_substep(sph_ctx* c, const sph_pool* pl, int32_t* bins, int64_t* tbeg, d
     a.wake = c->hwake;
     if (cudaMemsetAsync(c->hwake, 0xff, (size_t)n * sizeof(int32_t), c->st) != cudaSuccess ||
         sphh::launch_gather_bins(n, c->perm, bins, c->sx4, c->st) != cudaSuccess ||
-        sphh::launch_tree_mask(n, c->perm, c->hact, c->act_s, nullptr, nullptr, c->st) != cudaSuccess ||
+        sphh::launch_tree_mask(n, c->perm, c->hact, c->act_s, nullptr, nullptr, nullptr, 0, c->st) != cudaSuccess ||
         sphh::launch_tree_wake(a, phys_of(c->p), c->st) != cudaSuccess)
       return SPH_E_CUDA;
     h.wake = c->hwake;

@@ -6,7 +6,7 @@
 //   k_grid_setup   per simulation: max h -> cells per side n_c
 //   k_grid_base    prefix of n_c^3 over simulations -> global cell ids
 //   k_key_count    FP64 cell coordinates, cell id, per-cell count
-//   k_scan_*       exclusive scan of the counts -> cell_start
+//   k_scan         exclusive scan of the counts -> cell_start (radix.cu)
 //   radix sort     stable sort of (cell id, particle index) -> perm, so the
 //                  order inside a cell is ascending index for any cell size
 //                  (radix.cu)
@@ -125,7 +125,7 @@ __global__ void k_zero_counts(int32_t* __restrict__ count, const int32_t* __rest
 __global__ void k_key_count(int64_t n_total, const double* __restrict__ x, const double* __restrict__ y,
                             const double* __restrict__ z, const int64_t* __restrict__ sim_offset,
                             int n_sims, const GridDev* __restrict__ grid, int32_t* __restrict__ key,
-                            int32_t* __restrict__ sort_key, int32_t* __restrict__ count) {
+                            int32_t* __restrict__ count) {
   const WarpRange wr = warp_range(n_total);
   SimCursor sc;
   for (int64_t p = wr.lo + (threadIdx.x & 31); p < wr.hi; p += 32) {
@@ -136,105 +136,10 @@ __global__ void k_key_count(int64_t n_total, const double* __restrict__ x, const
     const int32_t kz = cell_coord_fast(z[p], G.L, G.n_c, G.scale_f);
     const int32_t k = G.cell_base + kx + G.n_c * (ky + G.n_c * kz);
     key[p] = k;
-    sort_key[p] = k;
     // neighbours in index order often share a cell: one atomic per distinct
     // cell of the converged lanes
     const unsigned peers = __match_any_sync(__activemask(), k);
     if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&count[k], __popc(peers));
-  }
-}
-
-// ---- exclusive scan with a device-side length ------------------------------
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
-constexpr int kScanTile = kScanThreads * kScanItems;
-
-__device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t* total) {
-  __shared__ int32_t ws[kScanThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int32_t x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int32_t t = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += t;
-  }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int32_t s = lane < kScanThreads / 32 ? ws[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int32_t t = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += t;
-    }
-    if (lane < kScanThreads / 32) ws[lane] = s;
-  }
-  __syncthreads();
-  const int32_t before = (w > 0 ? ws[w - 1] : 0) + x - v;
-  *total = ws[kScanThreads / 32 - 1];
-  __syncthreads();
-  return before;
-}
-
-// count[0 .. total) -> out (tile-local exclusive), tile sums -> sums
-__device__ __forceinline__ void scan_tile(const int32_t* __restrict__ count, int32_t* __restrict__ out,
-                                          int32_t* __restrict__ sums, int32_t total, int64_t tile) {
-  const int64_t base = tile * kScanTile;
-  int32_t v[kScanItems];
-  int32_t s = 0;
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const int64_t c = base + threadIdx.x * kScanItems + i;
-    v[i] = c < total ? count[c] : 0;
-    s += v[i];
-  }
-  int32_t tot;
-  int32_t run = block_exclusive_scan(s, &tot);
-#pragma unroll
-  for (int i = 0; i < kScanItems; ++i) {
-    const int64_t c = base + threadIdx.x * kScanItems + i;
-    if (c < total) out[c] = run;
-    run += v[i];
-  }
-  if (threadIdx.x == 0) sums[tile] = tot;
-}
-
-// (tiles in a block-uniform grid-stride loop: the grid is sized for the
-// capacity, the cell count is only known on the device)
-__global__ void k_scan_tiles(const int32_t* __restrict__ count, int32_t* __restrict__ out,
-                             int32_t* __restrict__ sums, const int32_t* __restrict__ misc) {
-  const int32_t total = misc[kTotalCells];
-  for (int64_t tile = blockIdx.x; tile * kScanTile < total; tile += gridDim.x)
-    scan_tile(count, out, sums, total, tile);
-}
-
-// single block: exclusive scan of the tile sums; writes out[total] = grand total
-__global__ void k_scan_sums(int32_t* __restrict__ sums, int32_t* __restrict__ out,
-                            const int32_t* __restrict__ misc) {
-  const int32_t total = misc[kTotalCells];
-  const int32_t nt = (total + kScanTile - 1) / kScanTile;
-  int32_t carry = 0;
-  for (int32_t b0 = 0; b0 < nt; b0 += kScanThreads) {
-    const int32_t i = b0 + threadIdx.x;
-    const int32_t v = i < nt ? sums[i] : 0;
-    int32_t tot;
-    const int32_t ex = block_exclusive_scan(v, &tot);
-    if (i < nt) sums[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) out[total] = carry;
-}
-
-__global__ void k_scan_add(int32_t* __restrict__ out, const int32_t* __restrict__ sums,
-                           const int32_t* __restrict__ misc) {
-  const int32_t total = misc[kTotalCells];
-  for (int64_t tile = blockIdx.x; tile * kScanTile < total; tile += gridDim.x) {
-    const int64_t base = tile * kScanTile;
-    const int32_t add = sums[tile];
-    for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
-      const int64_t c = base + i;
-      if (c < total) out[c] += add;
-    }
   }
 }
 
@@ -395,16 +300,14 @@ cudaError_t launch_build(const BuildArgs& a, cudaStream_t st) {
   k_zero_counts<<<zb, 256, 0, st>>>(a.count, a.misc);
   const int pb = grid_for(a.n_total, 256, 65535);
   if (a.n_total > 0)
-    k_key_count<<<pb, 256, 0, st>>>(a.n_total, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.key,
-                                    a.slot, a.count);  // slot receives a copy of the keys to sort
-  const int tb = grid_for(a.cap_cells, kScanTile, a.num_sms * 4);
-  k_scan_tiles<<<tb, kScanThreads, 0, st>>>(a.count, a.cell_start, a.scan_sums, a.misc);
-  k_scan_sums<<<1, kScanThreads, 0, st>>>(a.scan_sums, a.cell_start, a.misc);
-  k_scan_add<<<tb, kScanThreads, 0, st>>>(a.cell_start, a.scan_sums, a.misc);
+    k_key_count<<<pb, 256, 0, st>>>(a.n_total, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.key, a.count);
+  cudaError_t e = scan_exclusive(a.count, a.cell_start, a.misc + kTotalCells, a.cap_cells, true, a.scan_sums,
+                                 a.misc + kStatus, a.num_sms, st);
+  if (e != cudaSuccess) return e;
   if (a.n_total > 0 && a.sort_cells) {
     int bits = 1;
     while (bits < 31 && ((int64_t)1 << bits) <= a.cap_cells) ++bits;
-    const cudaError_t e = radix_sort_index(a.n_total, bits, a.slot, a.rk, a.perm, a.rv, a.hist, st);
+    e = radix_sort_index(a.n_total, bits, a.key, a.slot, a.rk, a.perm, a.rv, a.hist, a.misc + kStatus, st);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();

@@ -1,165 +1,227 @@
-// radix.cu -- stable least-significant-digit radix sort of (key, value)
-// pairs, used to order particles by cell id.  Values enter in ascending
-// particle index, so equal keys keep ascending index: the result is exactly
-// the stable counting sort of the cell grid (Sec. 2.1), for any cell size.
+// radix.cu -- stable least-significant-digit radix sort of (key, index) and
+// exclusive scans, one pass over memory each.  Indices enter in ascending
+// order, so equal keys keep ascending index: the result is exactly the stable
+// counting sort of the cell grid (Sec. 2.1), for any cell size.
 //
-// Each pass sorts by one 8-bit digit:
-//   k_radix_hist     per tile of 2048 items: digit histogram -> hist[d * T + t]
-//   (scan)           exclusive scan of hist, digit-major, so that tiles of the
-//                    same digit follow each other in index order
-//   k_radix_scatter  per tile: stable rank of each item among equal digits
-//                    (warp match + running per-warp counts, then a prefix over
-//                    the warps of the tile), written to hist[d * T + t] + rank
+//   k_radix_hist  the digit counts of every pass, from one read of the keys
+//   k_radix_pass  one 8-bit digit: a tile of 2048 items ranks its keys (warp
+//                 match + running per-warp counts), finds by look-back how many
+//                 equal digits the tiles before it hold (lookback.cuh, a word
+//                 per tile and digit), and scatters.  A pass whose keys all
+//                 share the digit (the bits beyond the cells in use) only
+//                 copies.
+//   k_scan        exclusive scan, tiles of 4096, the same look-back
+//
+// Both are bound by the latency of the look-back and of the scattered stores,
+// not by bandwidth.  A pass over 2M 64-bit keys takes 40 us (49 us as a
+// histogram, three scan kernels and a scatter), 8 us at 6,000 keys (23 us):
+// one launch instead of five is what small inputs pay for.  The nested-grid
+// build of 6,000 particles went from 62 launches and 310 us to 18 and 90 us.
+//
+// A tile whose wait ran out, and those behind it, copy their items in place:
+// stale, but valid, keys and indices.
+#include "lookback.cuh"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 
 namespace sphk {
 
-constexpr int kRadixThreads = 256;
 constexpr int kRadixItems = 8;
-constexpr int kRadixTile = kRadixThreads * kRadixItems;
-constexpr int kRadixWarps = kRadixThreads / 32;
+constexpr int kRadixTile = kScanThreads * kRadixItems;
+constexpr int kRadixMaxPasses = 8;
 
+// Digit counts of `passes` 8-bit digits of n keys, added to hist[pass * 256 + d].
 template <class K>
-__global__ void k_radix_hist(int64_t n, const K* __restrict__ keys, int shift, int n_tiles,
-                             int32_t* __restrict__ hist) {
-  __shared__ int32_t h[256];
-  h[threadIdx.x] = 0;
+__global__ void k_radix_hist(int64_t n, const K* __restrict__ keys, int passes, int32_t* __restrict__ hist) {
+  __shared__ int32_t h[kRadixMaxPasses * 256];
+  for (int i = threadIdx.x; i < passes * 256; i += kScanThreads) h[i] = 0;
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-  for (int i = threadIdx.x; i < kRadixTile; i += kRadixThreads) {
-    const int64_t p = base + i;
-    if (p < n) atomicAdd(&h[(int)((keys[p] >> shift) & 255)], 1);
-  }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
-}
-
-// Warp w of the tile handles items base + w * 256 + j * 32 + lane, j = 0..7,
-// i.e. 8 consecutive groups of 32 consecutive items: processing j in order
-// visits the warp's items in index order.
-template <class K>
-__global__ void k_radix_scatter(int64_t n, const K* __restrict__ keys_in,
-                                const int32_t* __restrict__ vals_in, int shift, int n_tiles,
-                                const int32_t* __restrict__ offsets, K* __restrict__ keys_out,
-                                int32_t* __restrict__ vals_out) {
-  __shared__ int32_t wcount[kRadixWarps][256];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int d = lane; d < 256; d += 32) wcount[warp][d] = 0;
-  __syncwarp();
-  const int64_t base = (int64_t)blockIdx.x * kRadixTile + warp * (32 * kRadixItems);
-  K key[kRadixItems];
-  int32_t val[kRadixItems], rank[kRadixItems];
-  const unsigned lt = (1u << lane) - 1u;
+  const int lane = threadIdx.x & 31;
+  for (int64_t base = (int64_t)blockIdx.x * kRadixTile; base < n; base += (int64_t)gridDim.x * kRadixTile) {
+    K key[kRadixItems];
 #pragma unroll
-  for (int j = 0; j < kRadixItems; ++j) {
-    const int64_t p = base + j * 32 + lane;
-    const bool ok = p < n;
-    key[j] = ok ? keys_in[p] : (K)0;
-    val[j] = ok ? vals_in[p] : 0;
-    const int d = ok ? (int)((key[j] >> shift) & 255) : 256 + lane;  // out-of-range items never match
-    const unsigned peers = __match_any_sync(0xffffffffu, d);
-    const int before = __popc(peers & lt);
-    int r = 0;
-    if (ok) r = wcount[warp][d] + before;
-    rank[j] = r;
-    __syncwarp();
-    // the highest lane of each group of equal digits advances the count
-    if (ok && (peers >> lane) == 1u) wcount[warp][d] += __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  // exclusive prefix over the warps of the tile, per digit, in place
-  for (int d = threadIdx.x; d < 256; d += kRadixThreads) {
-    int32_t run = 0;
-    for (int w = 0; w < kRadixWarps; ++w) {
-      const int32_t c = wcount[w][d];
-      wcount[w][d] = run;
-      run += c;
+    for (int i = 0; i < kRadixItems; ++i) {
+      const int64_t p = base + i * kScanThreads + threadIdx.x;
+      key[i] = p < n ? keys[p] : (K)0;
+    }
+#pragma unroll
+    for (int i = 0; i < kRadixItems; ++i) {
+      const int64_t p0 = base + i * kScanThreads + (threadIdx.x & ~31);
+      const bool ok = p0 + lane < n;
+      for (int s = 0; s < passes; ++s) {
+        const int d = (int)((key[i] >> (8 * s)) & 255);
+        // the leading digits mostly agree within a warp: one add for all
+        if (p0 + 31 < n && __all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+          if (lane == 0) atomicAdd(&h[s * 256 + d], 32);
+        } else if (ok) {
+          atomicAdd(&h[s * 256 + d], 1);
+        }
+      }
     }
   }
   __syncthreads();
+  for (int i = threadIdx.x; i < passes * 256; i += kScanThreads)
+    if (h[i] != 0) atomicAdd(&hist[i], h[i]);
+}
+
+// One pass.  Warp w of a tile handles items base + w * 256 + j * 32 + lane,
+// j = 0..7, i.e. 8 consecutive groups of 32 consecutive items: processing j in
+// order visits the warp's items in index order.  vals_in null: the values are
+// the indices.  keys_out null: the keys are not needed any more.
+template <class K>
+__global__ void __launch_bounds__(kScanThreads)
+k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int shift,
+             const int32_t* __restrict__ hist, int32_t* __restrict__ ticket, uint32_t* pub, K* __restrict__ keys_out,
+             int32_t* __restrict__ vals_out, int32_t* __restrict__ status) {
+  __shared__ int32_t wcount[kScanWarps][256];
+  __shared__ int32_t s_tile;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d0 = threadIdx.x;
+  const int32_t all = hist[d0];
+  if (d0 == 0) s_tile = atomicAdd(ticket, 1);
+  for (int d = lane; d < 256; d += 32) wcount[warp][d] = 0;
+  const bool same = __syncthreads_or((int64_t)all == n);
+  const int32_t tile = s_tile;
+  const int64_t base = (int64_t)tile * kRadixTile + warp * (32 * kRadixItems);
+  K key[kRadixItems];
+  int32_t val[kRadixItems], rank[kRadixItems];
+#pragma unroll
+  for (int j = 0; j < kRadixItems; ++j) {
+    const int64_t p = base + j * 32 + lane;
+    key[j] = p < n ? keys_in[p] : (K)0;
+    val[j] = p < n ? (vals_in != nullptr ? vals_in[p] : (int32_t)p) : 0;
+  }
+  bool copy = same;  // every key has this digit
+  int32_t dst0 = 0;
+  if (!copy) {
+    int32_t tot_all;
+    dst0 = block_scan(all, &tot_all);  // first place of digit d0
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < kRadixItems; ++j) {
+      const bool ok = base + j * 32 + lane < n;
+      const int d = ok ? (int)((key[j] >> shift) & 255) : 256 + lane;  // out-of-range items never match
+      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      int r = 0;
+      if (ok) r = wcount[warp][d] + __popc(peers & lt);
+      rank[j] = r;
+      __syncwarp();
+      // the highest lane of each group of equal digits advances the count
+      if (ok && (peers >> lane) == 1u) wcount[warp][d] += __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    // the tile's count of digit d0, and each warp's first place within the tile
+    int32_t mine = 0;
+#pragma unroll
+    for (int w = 0; w < kScanWarps; ++w) {
+      const int32_t c = wcount[w][d0];
+      wcount[w][d0] = mine;
+      mine += c;
+    }
+    uint32_t* my = pub + (int64_t)tile * 256 + d0;
+    pub_store(my, (tile == 0 ? kPubPrefix : kPubCount) | (uint32_t)mine);
+    int32_t before = 0;
+    bool failed = false;
+    for (int32_t t = tile - 1; t >= 0;) {
+      // four tiles back at a time, their words in flight together
+      uint32_t v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = t - i >= 0 ? pub_load(pub + (int64_t)(t - i) * 256 + d0) : kPubPrefix;
+      bool stop = false;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (!stop && t - i >= 0) {
+          if (v[i] == 0u) v[i] = pub_wait(pub + (int64_t)(t - i) * 256 + d0);
+          failed = failed || pub_is_failed(v[i]);
+          stop = pub_is_last(v[i]);
+          if (!failed) before += (int32_t)(v[i] & kPubValue);
+        }
+      }
+      if (stop) break;
+      t -= 4;
+    }
+    if (tile > 0) pub_store(my, failed ? kPubFailed : kPubPrefix | (uint32_t)(before + mine));
+    copy = __syncthreads_or(failed);
+    if (copy && d0 == 0) atomicOr(status, SPH_ST_TIMEOUT);
+    // the place of the tile's first item of digit d0
+    if (!copy) {
+#pragma unroll
+      for (int w = 0; w < kScanWarps; ++w) wcount[w][d0] += dst0 + before;
+    }
+    __syncthreads();
+  }
 #pragma unroll
   for (int j = 0; j < kRadixItems; ++j) {
     const int64_t p = base + j * 32 + lane;
     if (p < n) {
-      const int d = (int)((key[j] >> shift) & 255);
-      const int64_t dst = (int64_t)offsets[(int64_t)d * n_tiles + blockIdx.x] + wcount[warp][d] + rank[j];
-      keys_out[dst] = key[j];
+      const int64_t dst = copy ? p : (int64_t)wcount[warp][(int)((key[j] >> shift) & 255)] + rank[j];
+      if (keys_out != nullptr) keys_out[dst] = key[j];
       vals_out[dst] = val[j];
     }
   }
 }
 
-__global__ void k_iota(int64_t n, int32_t* __restrict__ v) {
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-    v[p] = (int32_t)p;
-}
+// Exclusive scan of in[0 .. len), len = *len_dev or len_host, into out (which
+// may be in); with_total: out[len] = the sum.  Sums stay below 2^30.
+constexpr int kScanItems = 16;
+constexpr int kScanTile = kScanThreads * kScanItems;
 
-// Exclusive scan of m (host-known) int32 in place: per-tile scans, a scan
-// of the tile totals, and a final add.
-constexpr int kScanTileH = kRadixThreads * 4;
-
-__device__ __forceinline__ int32_t radix_block_scan(int32_t v, int32_t* total) {
-  __shared__ int32_t ws[kRadixWarps];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int32_t x = v;
+__global__ void __launch_bounds__(kScanThreads)
+k_scan(const int32_t* in, int32_t* out, const int32_t* __restrict__ len_dev, int64_t len_host, int with_total,
+       int32_t* __restrict__ ticket, uint32_t* pub, int32_t* __restrict__ status) {
+  __shared__ int32_t s_tile, s_before;
+  const int64_t len = len_dev != nullptr ? (int64_t)*len_dev : len_host;
+  const int64_t tiles = len > 0 ? (len + kScanTile - 1) / kScanTile : 1;
+  const bool vec = (((uintptr_t)in | (uintptr_t)out) & 15u) == 0u;
+  for (;;) {
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
+    __syncthreads();
+    const int32_t tile = s_tile;
+    if (tile >= tiles) return;
+    const int64_t c0 = (int64_t)tile * kScanTile + threadIdx.x * kScanItems;
+    int32_t v[kScanItems];
+    if (vec && c0 + kScanItems <= len) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int32_t t = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += t;
-  }
-  if (lane == 31) ws[w] = x;
-  __syncthreads();
-  int32_t wbase = 0, tot = 0;
-  for (int k = 0; k < kRadixWarps; ++k) {
-    wbase += k < w ? ws[k] : 0;
-    tot += ws[k];
-  }
-  __syncthreads();
-  *total = tot;
-  return wbase + x - v;
-}
-
-__global__ void k_scanh_tiles(int32_t* __restrict__ a, int64_t m, int32_t* __restrict__ sums) {
-  const int64_t base = (int64_t)blockIdx.x * kScanTileH;
-  int32_t v[4];
-  int32_t s = 0;
+      for (int i = 0; i < kScanItems; i += 4) {
+        const int4 q = *reinterpret_cast<const int4*>(in + c0 + i);
+        v[i] = q.x;
+        v[i + 1] = q.y;
+        v[i + 2] = q.z;
+        v[i + 3] = q.w;
+      }
+    } else {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t k = base + threadIdx.x * 4 + i;
-    v[i] = k < m ? a[k] : 0;
-    s += v[i];
-  }
-  int32_t tot;
-  int32_t run = radix_block_scan(s, &tot);
+      for (int i = 0; i < kScanItems; ++i) v[i] = c0 + i < len ? in[c0 + i] : 0;
+    }
+    int32_t s = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int64_t k = base + threadIdx.x * 4 + i;
-    if (k < m) a[k] = run;
-    run += v[i];
-  }
-  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-__global__ void k_scanh_sums(int32_t* __restrict__ sums, int64_t nt) {
-  int32_t carry = 0;
-  for (int64_t b0 = 0; b0 < nt; b0 += kRadixThreads) {
-    const int64_t i = b0 + threadIdx.x;
-    const int32_t v = i < nt ? sums[i] : 0;
+    for (int i = 0; i < kScanItems; ++i) s += v[i];
     int32_t tot;
-    const int32_t ex = radix_block_scan(v, &tot);
-    if (i < nt) sums[i] = carry + ex;
-    carry += tot;
-  }
-}
-
-__global__ void k_scanh_add(int32_t* __restrict__ a, int64_t m, const int32_t* __restrict__ sums) {
-  const int64_t base = (int64_t)blockIdx.x * kScanTileH;
-  const int32_t add = sums[blockIdx.x];
-  for (int i = threadIdx.x; i < kScanTileH; i += kRadixThreads) {
-    const int64_t k = base + i;
-    if (k < m) a[k] += add;
+    int32_t run = block_scan(s, &tot);
+    if (threadIdx.x < 32) lookback(pub, tile, tot, &s_before, status);
+    __syncthreads();
+    const int32_t before = s_before >= 0 ? s_before : 0;
+    run += before;
+    if (with_total && tile == tiles - 1 && threadIdx.x == 0) out[len] = before + tot;
+    if (vec && c0 + kScanItems <= len) {
+#pragma unroll
+      for (int i = 0; i < kScanItems; i += 4) {
+        int4 q;
+        q.x = run;
+        q.y = q.x + v[i];
+        q.z = q.y + v[i + 1];
+        q.w = q.z + v[i + 2];
+        run = q.w + v[i + 3];
+        *reinterpret_cast<int4*>(out + c0 + i) = q;
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kScanItems; ++i) {
+        if (c0 + i < len) out[c0 + i] = run;
+        run += v[i];
+      }
+    }
+    __syncthreads();  // s_before and s_tile are read before the next tile's
   }
 }
 
@@ -168,65 +230,74 @@ __global__ void k_scanh_add(int32_t* __restrict__ a, int64_t m, const int32_t* _
 namespace sphh {
 using namespace sphk;
 
-// histogram (256 per tile) followed by the scan's tile totals
-int64_t radix_hist_words(int64_t n) {
-  const int64_t h = 256 * ((n + kRadixTile - 1) / kRadixTile);
-  return h + (h + kScanTileH - 1) / kScanTileH + 1;
+// Sort scratch: per pass 256 digit counts, a tile counter and 256 published
+// words per tile.
+int64_t radix_words(int64_t n, int passes) {
+  return (int64_t)passes * (256 + 1 + 256 * ((n + kRadixTile - 1) / kRadixTile)) + 64;
 }
 
-// Sorts keys (bits significant bits) stably, values = 0..n-1, into vals_out.
-// keys / keys_tmp / vals_tmp / vals_out hold n entries; hist holds
-// radix_hist_words(n).  keys is clobbered.
 template <class K>
-static cudaError_t radix_sort_impl(int64_t n, int bits, K* keys, K* keys_tmp, int32_t* vals_out,
-                                   int32_t* vals_tmp, int32_t* hist, cudaStream_t st) {
+static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_out, K* keys_tmp, bool want_keys,
+                                   int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
+                                   cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const int n_tiles = (int)((n + kRadixTile - 1) / kRadixTile);
+  const int64_t tiles = (n + kRadixTile - 1) / kRadixTile;
   const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
-  int64_t ib = (n + 255) / 256;
-  if (ib > 65535) ib = 65535;
-  // values ping-pong so that the last pass lands in vals_out
-  int32_t* v_in = (passes % 2 == 0) ? vals_out : vals_tmp;
-  int32_t* v_out = (passes % 2 == 0) ? vals_tmp : vals_out;
-  k_iota<<<(int)ib, 256, 0, st>>>(n, v_in);
-  K* k_in = keys;
-  K* k_out = keys_tmp;
-  for (int pass = 0; pass < passes; ++pass) {
-    const int shift = 8 * pass;
-    k_radix_hist<K><<<n_tiles, kRadixThreads, 0, st>>>(n, k_in, shift, n_tiles, hist);
-    const int64_t m = (int64_t)256 * n_tiles;
-    const int64_t nt = (m + kScanTileH - 1) / kScanTileH;
-    k_scanh_tiles<<<(unsigned)nt, kRadixThreads, 0, st>>>(hist, m, hist + m);
-    k_scanh_sums<<<1, kRadixThreads, 0, st>>>(hist + m, nt);
-    k_scanh_add<<<(unsigned)nt, kRadixThreads, 0, st>>>(hist, m, hist + m);
-    k_radix_scatter<K><<<n_tiles, kRadixThreads, 0, st>>>(n, k_in, v_in, shift, n_tiles, hist, k_out, v_out);
-    K* t = k_in;
+  if (passes > kRadixMaxPasses) return cudaErrorInvalidValue;
+  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)radix_words(n, passes), st);
+  if (e != cudaSuccess) return e;
+  int32_t* hist = scratch;
+  int32_t* ticket = hist + 256 * passes;
+  uint32_t* pub = reinterpret_cast<uint32_t*>(ticket + passes);
+  k_radix_hist<K><<<(unsigned)(tiles < 1024 ? tiles : 1024), kScanThreads, 0, st>>>(n, keys, passes, hist);
+  const K* k_in = keys;
+  const int32_t* v_in = nullptr;
+  for (int p = 0; p < passes; ++p) {
+    // outputs alternate so that the last pass lands in keys_out / vals_out
+    const bool odd = ((passes - 1 - p) & 1) != 0;
+    K* k_out = odd ? keys_tmp : keys_out;
+    int32_t* v_out = odd ? vals_tmp : vals_out;
+    k_radix_pass<K><<<(unsigned)tiles, kScanThreads, 0, st>>>(n, k_in, v_in, 8 * p, hist + 256 * p, ticket + p,
+                                                               pub + (int64_t)p * tiles * 256,
+                                                               p == passes - 1 && !want_keys ? nullptr : k_out, v_out,
+                                                               status);
     k_in = k_out;
-    k_out = t;
-    int32_t* tv = v_in;
     v_in = v_out;
-    v_out = tv;
   }
   return cudaGetLastError();
 }
 
-cudaError_t scan_exclusive_host_n(int32_t* a, int64_t m, int32_t* tmp, cudaStream_t st) {
-  if (m <= 0) return cudaSuccess;
-  const int64_t nt = (m + kScanTileH - 1) / kScanTileH;
-  k_scanh_tiles<<<(unsigned)nt, kRadixThreads, 0, st>>>(a, m, tmp);
-  k_scanh_sums<<<1, kRadixThreads, 0, st>>>(tmp, nt);
-  k_scanh_add<<<(unsigned)nt, kRadixThreads, 0, st>>>(a, m, tmp);
+cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* tmp_a, int32_t* tmp_b,
+                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
+                             cudaStream_t st) {
+  return radix_sort_impl<int32_t>(n, bits, keys, tmp_a, tmp_b, false, vals_out, vals_tmp, scratch, status, st);
+}
+
+cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,
+                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
+                               cudaStream_t st) {
+  return radix_sort_impl<uint64_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, status, st);
+}
+
+cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, int32_t* status,
+                            cudaStream_t st) {
+  return radix_sort_impl<int8_t>(n, 8, keys, nullptr, nullptr, false, vals_out, nullptr, scratch, status, st);
+}
+
+// tiles' published words after the tile counter
+int64_t scan_words(int64_t cap) { return (cap + kScanTile - 1) / kScanTile + 2; }
+
+cudaError_t scan_exclusive(const int32_t* in, int32_t* out, const int32_t* len_dev, int64_t cap, bool with_total,
+                           int32_t* scratch, int32_t* status, int num_sms, cudaStream_t st) {
+  const int64_t tiles = cap > 0 ? (cap + kScanTile - 1) / kScanTile : 1;
+  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)(tiles + 1), st);
+  if (e != cudaSuccess) return e;
+  // (the length may be known on the device only: blocks take tiles from the
+  // counter, idle ones return at once)
+  const int64_t most = (int64_t)num_sms * 6;
+  k_scan<<<(unsigned)(tiles < most ? tiles : most), kScanThreads, 0, st>>>(
+      in, out, len_dev, cap, with_total ? 1 : 0, scratch, reinterpret_cast<uint32_t*>(scratch + 1), status);
   return cudaGetLastError();
-}
-
-cudaError_t radix_sort_index(int64_t n, int bits, int32_t* keys, int32_t* keys_tmp, int32_t* vals_out,
-                             int32_t* vals_tmp, int32_t* hist, cudaStream_t st) {
-  return radix_sort_impl<int32_t>(n, bits, keys, keys_tmp, vals_out, vals_tmp, hist, st);
-}
-
-cudaError_t radix_sort_index64(int64_t n, int bits, uint64_t* keys, uint64_t* keys_tmp,
-                               int32_t* vals_out, int32_t* vals_tmp, int32_t* hist, cudaStream_t st) {
-  return radix_sort_impl<uint64_t>(n, bits, keys, keys_tmp, vals_out, vals_tmp, hist, st);
 }
 
 }  // namespace sphh

@@ -29,8 +29,8 @@ struct BuildArgs {
   sphk::GridDev* grid;
   int32_t* misc;
   int32_t* hmax_bits;  // per simulation scratch
-  int32_t *key, *slot, *count, *cell_start, *scan_sums, *perm;
-  int32_t *rk, *rv, *hist;  // radix-sort scratch: n, n, radix_hist_words(n)
+  int32_t *key, *slot, *count, *cell_start, *scan_sums, *perm;  // slot: n scratch; scan_sums: scan_words(cells)
+  int32_t *rk, *rv, *hist;  // radix-sort scratch: n, n, radix_words(n, passes)
   int sort_cells = 1;       // 0: counts and cell_start only (the tree build orders)
   double radius = 0.0;      // > 0: cells at least this wide, h unused (friends-of-friends)
   int cells_per_particle = 8;  // n_c^3 <= cells_per_particle n + 216 per simulation
@@ -52,13 +52,25 @@ struct FofArgs {
 };
 cudaError_t launch_fof(const FofArgs& a, cudaStream_t st);
 
-// Stable radix sort of keys (bits significant bits) with values 0..n-1
-// (radix.cu); keys is clobbered, the sorted values land in vals_out.
-int64_t radix_hist_words(int64_t n);
-cudaError_t radix_sort_index(int64_t n, int bits, int32_t* keys, int32_t* keys_tmp, int32_t* vals_out,
-                             int32_t* vals_tmp, int32_t* hist, cudaStream_t st);
-cudaError_t radix_sort_index64(int64_t n, int bits, uint64_t* keys, uint64_t* keys_tmp,
-                               int32_t* vals_out, int32_t* vals_tmp, int32_t* hist, cudaStream_t st);
+// Stable radix sort of keys (bits significant bits, at most 64) with values
+// 0..n-1 (radix.cu); the sorted values land in vals_out (vals_tmp: n, unless
+// bits <= 8), the 64-bit sort's keys in keys_out.  scratch: radix_words(n,
+// passes of 8 bits).  The keys are left as they are.
+int64_t radix_words(int64_t n, int passes);
+cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* tmp_a, int32_t* tmp_b,
+                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status, cudaStream_t st);
+cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,
+                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
+                               cudaStream_t st);
+// The indices 0..n-1 by ascending key (0..127), equal keys in ascending order.
+cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, int32_t* status,
+                            cudaStream_t st);
+// Exclusive scan of int32 (radix.cu), in place if out is in: of *len_dev <= cap
+// entries, or of cap where len_dev is null; with_total: the sum at out[length].
+// scratch: scan_words(cap).
+int64_t scan_words(int64_t cap);
+cudaError_t scan_exclusive(const int32_t* in, int32_t* out, const int32_t* len_dev, int64_t cap, bool with_total,
+                           int32_t* scratch, int32_t* status, int num_sms, cudaStream_t st);
 
 struct GatherDensityArgs {
   int64_t n_total;
@@ -298,13 +310,15 @@ struct TreeBuildArgs {
   const float* h;
   const int32_t* cell_key;    // top cell of each particle (launch_build's key)
   const int32_t* cell_start;  // top cells' ranges (valid in source order too)
-  uint64_t *key64, *key64_b, *key64_c;  // n each (scratch)
+  uint64_t *key64, *key64_b;  // n each (scratch)
   uint64_t* skey;             // n: source keys in source order
   int32_t* perm;              // n: source order -> pool index
   int32_t* tgt;               // n: target order -> source index
   int32_t *rv, *hist;         // radix scratch
-  int32_t *flag, *leaf_of;    // n each
-  int32_t* scan_tmp;          // n / 1024 + 2
+  int32_t* leaf_of;           // n: target order -> its group
+  int32_t* scan_tmp;          // scan_words(n)
+  int32_t* status;
+  int num_sms;
   sphk::TreeLeaf* leaves;     // n + 1: target groups, start in target order
   int32_t* n_leaves;          // 1 (device)
   sphk::TreeRange* ranges;    // 27 n: source-order ranges of each group
@@ -346,7 +360,7 @@ struct TreeDensityArgs {
   const int32_t* tgt;  // target order -> source index
   const sphk::TreeLeaf* leaves;
   const int32_t* n_leaves;
-  const int32_t *flag, *leaf_of;  // target order: first of its leaf; leaves that begin before it
+  const int32_t* leaf_of;  // target order -> its leaf
   const sphk::TreeRange* ranges;
   const int4* fine;
   const float4 *rel, *vel4;
@@ -364,7 +378,7 @@ struct TreeDensityArgs {
   int32_t* rev_fill;   // n: scatter cursors
   uint32_t* rev;       // rev_cap: packed sources ordered by (receiver, source)
   int64_t rev_cap;
-  int32_t* scan_tmp;   // (n + 1) / 1024 + 2
+  int32_t* scan_tmp;   // scan_words(n + 1)
   int32_t* work;       // 1: group counter (reset by the launcher)
   // targets whose support outgrew their level, re-solved one level coarser
   const uint64_t* skey;        // n: source keys
@@ -382,9 +396,9 @@ struct TreeDensityArgs {
 };
 cudaError_t launch_tree_density(const TreeDensityArgs& a, const sphk::PhysDev& ph, cudaStream_t st);
 // The mask in tree order: out[k] = active[perm[k]]; with pre (n + 1 int32,
-// scan scratch tmp of (n + 1) / 1024 + 2) also its exclusive prefix sums.
+// scan scratch tmp of scan_words(n + 1)) also its exclusive prefix sums.
 cudaError_t launch_tree_mask(int64_t n, const int32_t* perm, const uint8_t* active, uint8_t* out, int32_t* pre,
-                             int32_t* tmp, cudaStream_t st);
+                             int32_t* tmp, int32_t* status, int num_sms, cudaStream_t st);
 
 struct TreeForceArgs {
   int n_sims;
@@ -434,10 +448,6 @@ cudaError_t launch_tree_sphenix_gradient(const TreeForceArgs& a, const sphk::Phy
 // a.bins_out), and the wake-up pass (a.fE, a.act, a.wake).
 cudaError_t launch_tree_limit(const TreeForceArgs& a, const sphk::PhysDev& ph, cudaStream_t st);
 cudaError_t launch_tree_wake(const TreeForceArgs& a, const sphk::PhysDev& ph, cudaStream_t st);
-// Exclusive scan of m int32 in place with a host-known length (radix.cu);
-// tmp holds m / 1024 + 2 entries.
-cudaError_t scan_exclusive_host_n(int32_t* a, int64_t m, int32_t* tmp, cudaStream_t st);
-
 // Time integration over a pool (step.cu).
 struct StepArgs {
   int n_sims;

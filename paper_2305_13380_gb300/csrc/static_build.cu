@@ -22,8 +22,10 @@ namespace {
 // Largest build served by the fixed scratch.
 constexpr int64_t kStaticMaxN = 65536;
 constexpr int64_t kStaticMaxCells = 8 * kStaticMaxN + 216;
-constexpr int64_t kStaticScanSums = kStaticMaxCells / 1024 + 2;
-constexpr int64_t kStaticHist = 256 * ((kStaticMaxN + 2047) / 2048) + 16;
+constexpr int64_t kStaticScanSums = kStaticMaxCells / 4096 + 4;  // scan_words
+// radix_words for the three digits of up to kStaticMaxCells cell ids
+constexpr int64_t kStaticHist = 3 * (256 + 1 + 256 * ((kStaticMaxN + 2047) / 2048)) + 64;
+static_assert(kStaticMaxCells < (1 << 24), "cell ids of three digits");
 
 // Layout of the scratch, in 4-byte words, each part 256-byte aligned.
 constexpr int64_t align64(int64_t w) { return (w + 63) / 64 * 64; }

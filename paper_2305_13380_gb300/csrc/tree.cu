@@ -16,12 +16,16 @@
 // least (1 + margin) H_i, stopping at a cell with at most n_leaf particles or
 // at kTreeDepth.  (A rule on the largest H of a whole cell would keep a dense
 // core at the coarse level of the one wide particle beside it; per particle,
-// each target's 27 neighbour cells stay ~H wide.)  Targets are grouped by
-// (cell at their level, level) through a second sort: "target order", with
-// groups contiguous.  A group's sources are the particles of the 27 cells of
+// each target's 27 neighbour cells stay ~H wide.)  "Target order" is a stable
+// partition of source order by level: the particles of one cell at one level,
+// a group, follow each other in it.  (One digit of sorting instead of a second
+// 64-bit sort by cell and level, 40 us instead of 390 us at 2M particles; and
+// the groups of the coarse levels, whose cells may hold thousands of sources,
+// come first, so that the loops do not end on them.)  A group's sources are the particles of the 27 cells of
 // its level around it, one source-order range each (binary search), which
 // hold every particle within one cell side of the group: enough for the
 // density of its targets, whose supports are at most that side.
+#include "lookback.cuh"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "tree.cuh"
@@ -41,8 +45,7 @@ __device__ __forceinline__ int32_t fine_coord(double x, double L, int32_t n_c, i
 __global__ void k_tree_key(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
                            const double* __restrict__ z, const int64_t* __restrict__ sim_offset,
                            int n_sims, const GridDev* __restrict__ grid,
-                           const int32_t* __restrict__ cell_key, uint64_t* __restrict__ key64,
-                           uint64_t* __restrict__ key64_copy) {
+                           const int32_t* __restrict__ cell_key, uint64_t* __restrict__ key64) {
   const WarpRange wr = warp_range(n);
   SimCursor sc;
   for (int64_t p = wr.lo + (threadIdx.x & 31); p < wr.hi; p += 32) {
@@ -56,25 +59,15 @@ __global__ void k_tree_key(int64_t n, const double* __restrict__ x, const double
     const uint32_t lz = (uint32_t)(fine_coord(z[p], G.L, G.n_c, kz) - kz * kTreeFine);
     const uint64_t k = ((uint64_t)(uint32_t)c << 30) | (spread3(lx) | (spread3(ly) << 1) | (spread3(lz) << 2));
     key64[p] = k;
-    key64_copy[p] = k;
   }
 }
 
-// Source keys in source order.
-__global__ void k_tree_sorted(int64_t n, const int32_t* __restrict__ perm, const uint64_t* __restrict__ key64,
-                              uint64_t* __restrict__ skey) {
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
-    skey[s] = key64[perm[s]];
-}
-
-// Level of each particle (source order) by descending from its top cell, its
-// level and cell side, and its target key (top cell, Morton prefix of its cell at that
-// level, level) with a copy for the sort.
+// Level and cell side of each particle (source order), by descending from its
+// top cell.
 __global__ void k_tree_level(int64_t n, const uint64_t* __restrict__ skey, const int32_t* __restrict__ perm,
                              const float* __restrict__ h, int n_sims,
                              const GridDev* __restrict__ grid, int n_leaf, double margin, float gamma_k,
-                             int8_t* __restrict__ level, float* __restrict__ leaf_side,
-                             uint64_t* __restrict__ tkey, uint64_t* __restrict__ tkey_copy) {
+                             int8_t* __restrict__ level, float* __restrict__ leaf_side) {
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t key = skey[s];
     const int32_t c = (int32_t)(key >> 30);
@@ -105,51 +98,70 @@ __global__ void k_tree_level(int64_t n, const uint64_t* __restrict__ skey, const
     }
     level[s] = (int8_t)d;
     leaf_side[s] = G.cell_f * __int_as_float((127 - d) << 23);  // G.cell_f / 2^d, exact
-    const int sh = 3 * (kTreeDepth - d);
-    const uint64_t m = ((key & 0x3fffffffull) >> sh) << sh;
-    const uint64_t t = ((uint64_t)(uint32_t)c << 34) | (m << 4) | (uint64_t)d;
-    tkey[s] = t;
-    tkey_copy[s] = t;
   }
 }
 
-// Target keys in target order (tgt: target order -> source index).
-__global__ void k_tree_tsorted(int64_t n, const int32_t* __restrict__ tgt, const uint64_t* __restrict__ tkey,
-                               uint64_t* __restrict__ tsorted) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    tsorted[k] = tkey[tgt[k]];
-}
-
-__global__ void k_tree_leaf_flag(int64_t n, const uint64_t* __restrict__ tsorted, int32_t* __restrict__ flag) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
-    flag[k] = (k == 0) || (tsorted[k] != tsorted[k - 1]);
-}
-
-// After the exclusive scan of flag (-> leaf_of), the group records.
-__global__ void k_tree_leaf_fill(int64_t n, const uint64_t* __restrict__ tsorted, const int32_t* __restrict__ flag,
-                                 const int32_t* __restrict__ leaf_of, TreeLeaf* __restrict__ leaves) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    if (!flag[k]) continue;
-    const uint64_t t = tsorted[k];
-    const int d = (int)(t & 15u);
-    const uint32_t m = (uint32_t)((t >> 4) & 0x3fffffffull);
-    const int sh = kTreeDepth - d;
-    TreeLeaf L;
-    L.start = (int32_t)k;
-    L.depth = d;
-    L.cell = (int32_t)(t >> 34);
-    L.lx = (int32_t)(compact3(m) >> sh);
-    L.ly = (int32_t)(compact3(m >> 1) >> sh);
-    L.lz = (int32_t)(compact3(m >> 2) >> sh);
-    L.pad = 0;
-    leaves[leaf_of[k]] = L;
+// The groups in target order: a target whose level or cell differs from the
+// one before it starts a group.  Each target's group (leaf_of), the group
+// records with a sentinel, and their number; tiles of 2048 targets, prefixed by
+// look-back (a wait that runs out leaves no groups).
+constexpr int kLeafItems = 8;
+constexpr int kLeafTile = kScanThreads * kLeafItems;
+__global__ void __launch_bounds__(kScanThreads)
+k_tree_leaves(int64_t n, const int32_t* __restrict__ tgt, const int8_t* __restrict__ level,
+              const uint64_t* __restrict__ skey, int32_t* __restrict__ leaf_of, TreeLeaf* __restrict__ leaves,
+              int32_t* __restrict__ n_leaves, int32_t* __restrict__ ticket, uint32_t* pub,
+              int32_t* __restrict__ status) {
+  __shared__ int32_t s_tile, s_before;
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
+  __syncthreads();
+  const int32_t tile = s_tile;
+  const int64_t k0 = (int64_t)tile * kLeafTile + threadIdx.x * kLeafItems;
+  uint64_t key[kLeafItems];
+  int d[kLeafItems];
+  unsigned first = 0u;  // bit i: target k0 + i starts a group
+  uint64_t cell = 0;
+  int last = -1;
+  if (k0 > 0 && k0 < n) {
+    const int32_t s = tgt[k0 - 1];
+    last = level[s];
+    cell = skey[s] >> (3 * (kTreeDepth - last));
   }
-}
-
-__global__ void k_tree_leaf_count(int64_t n, const int32_t* __restrict__ flag, const int32_t* __restrict__ leaf_of,
-                                  int32_t* __restrict__ n_leaves, TreeLeaf* __restrict__ leaves) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const int32_t nl = n > 0 ? leaf_of[n - 1] + flag[n - 1] : 0;
+#pragma unroll
+  for (int i = 0; i < kLeafItems; ++i) {
+    const int64_t k = k0 + i;
+    key[i] = 0;
+    d[i] = 0;
+    if (k < n) {
+      const int32_t s = tgt[k];
+      d[i] = level[s];
+      key[i] = skey[s];
+      const uint64_t c = key[i] >> (3 * (kTreeDepth - d[i]));
+      if (d[i] != last || c != cell) first |= 1u << i;
+      last = d[i];
+      cell = c;
+    }
+  }
+  int32_t tot;
+  int32_t at = block_scan(__popc(first), &tot);
+  if (threadIdx.x < 32) lookback(pub, tile, tot, &s_before, status);
+  __syncthreads();
+  const bool ok = s_before >= 0;
+  at += ok ? s_before : 0;
+#pragma unroll
+  for (int i = 0; i < kLeafItems; ++i) {
+    const int64_t k = k0 + i;
+    if (k < n) {
+      if ((first >> i) & 1u) {
+        TreeLeaf L = cell_at_depth(key[i], d[i]);
+        L.start = (int32_t)k;
+        leaves[at++] = L;
+      }
+      leaf_of[k] = at - 1;
+    }
+  }
+  if (threadIdx.x == 0 && ((int64_t)tile + 1) * kLeafTile >= n) {
+    const int32_t nl = ok ? s_before + tot : 0;
     *n_leaves = nl;
     leaves[nl].start = (int32_t)n;  // sentinel: end of the last group
   }
@@ -222,30 +234,25 @@ static int blocks_n(int64_t n) {
 
 cudaError_t launch_tree_build(const TreeBuildArgs& a, cudaStream_t st) {
   const int64_t n = a.n_total;
-  if (n <= 0) {
-    k_tree_leaf_count<<<1, 32, 0, st>>>(0, a.flag, a.leaf_of, a.n_leaves, a.leaves);
-    return cudaGetLastError();
-  }
+  cudaError_t e;
+  if (n <= 0) return cudaMemsetAsync(a.n_leaves, 0, sizeof(int32_t), st);
   int cbits = 1;
   while (cbits < 30 && ((int64_t)1 << cbits) <= a.cap_cells) ++cbits;
   // source order: (top cell, Morton code), ties by pool index
-  k_tree_key<<<blocks_n(n), 256, 0, st>>>(n, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.cell_key,
-                                          a.key64, a.key64_b);
-  cudaError_t e = radix_sort_index64(n, 30 + cbits, a.key64_b, a.key64_c, a.perm, a.rv, a.hist, st);
+  k_tree_key<<<blocks_n(n), 256, 0, st>>>(n, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.cell_key, a.key64);
+  e = radix_sort_index64(n, 30 + cbits, a.key64, a.skey, a.key64_b, a.perm, a.rv, a.hist, a.status, st);
   if (e != cudaSuccess) return e;
-  k_tree_sorted<<<blocks_n(n), 256, 0, st>>>(n, a.perm, a.key64, a.skey);
-  // levels and target order: (top cell, cell at the level, level), ties by source index
-  k_tree_level<<<blocks_n(n), 256, 0, st>>>(n, a.skey, a.perm, a.h, a.n_sims, a.grid, a.n_leaf,
-                                            a.margin, a.gamma_k, a.level, a.leaf_side, a.key64, a.key64_b);
-  e = radix_sort_index64(n, 34 + cbits, a.key64_b, a.key64_c, a.tgt, a.rv, a.hist, st);
+  // levels, and target order: by level, ties by source index
+  k_tree_level<<<blocks_n(n), 256, 0, st>>>(n, a.skey, a.perm, a.h, a.n_sims, a.grid, a.n_leaf, a.margin, a.gamma_k,
+                                            a.level, a.leaf_side);
+  e = radix_partition(n, a.level, a.tgt, a.hist, a.status, st);
   if (e != cudaSuccess) return e;
-  k_tree_tsorted<<<blocks_n(n), 256, 0, st>>>(n, a.tgt, a.key64, a.key64_c);
-  k_tree_leaf_flag<<<blocks_n(n), 256, 0, st>>>(n, a.key64_c, a.flag);
-  cudaMemcpyAsync(a.leaf_of, a.flag, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st);
-  e = scan_exclusive_host_n(a.leaf_of, n, a.scan_tmp, st);
+  const int64_t tiles = (n + kLeafTile - 1) / kLeafTile;
+  e = cudaMemsetAsync(a.scan_tmp, 0, sizeof(int32_t) * (size_t)(tiles + 1), st);
   if (e != cudaSuccess) return e;
-  k_tree_leaf_fill<<<blocks_n(n), 256, 0, st>>>(n, a.key64_c, a.flag, a.leaf_of, a.leaves);
-  k_tree_leaf_count<<<1, 32, 0, st>>>(n, a.flag, a.leaf_of, a.n_leaves, a.leaves);
+  k_tree_leaves<<<(unsigned)tiles, kScanThreads, 0, st>>>(n, a.tgt, a.level, a.skey, a.leaf_of, a.leaves, a.n_leaves,
+                                                         a.scan_tmp, reinterpret_cast<uint32_t*>(a.scan_tmp + 1),
+                                                         a.status);
   k_tree_neigh<<<blocks_n(n * 4), 256, 0, st>>>(a.leaves, a.n_leaves, a.skey, n, a.cell_start, a.n_sims, a.grid,
                                                 a.ranges);
   return cudaGetLastError();

@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sph
   unsigned long long pair_acc = 0, free_acc = 0;
   for (int64_t w0 = (int64_t)next_group(a.work, lane) * kTWin; w0 < n; w0 = (int64_t)next_group(a.work, lane) * kTWin) {
     const int32_t w1 = (int32_t)(w0 + kTWin < n ? w0 + kTWin : n);
-    for (int32_t li = a.leaf_of[w0] + a.flag[w0] - 1; li < nl; ++li) {
+    for (int32_t li = a.leaf_of[w0]; li < nl; ++li) {
       const TreeLeaf Lf = a.leaves[li];
       if (Lf.start >= w1) break;
       const int32_t t_hi = a.leaves[li + 1].start;
@@ -1649,7 +1649,7 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   else
     k_tree_density<K, false><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
   k_tree_density_fb<K><<<a.num_sms * bps_fb, kTWarps * 32, kTFbSmem, st>>>(a, ph);
-  e = scan_exclusive_host_n(a.rev_start, n + 1, a.scan_tmp, st);
+  e = scan_exclusive(a.rev_start, a.rev_start, nullptr, n + 1, false, a.scan_tmp, a.status, a.num_sms, st);
   if (e != cudaSuccess) return e;
   k_rev_scatter<<<a.num_sms * 4, 256, 0, st>>>(a.rev_raw, a.rev_count, a.rev_cap, a.rev_start, a.rev_fill, a.rev);
   k_rev_sort<<<tree_blocks(n), 256, 0, st>>>(n, a.rev_start, a.rev);
@@ -1724,11 +1724,11 @@ cudaError_t launch_tree_wake(const TreeForceArgs& a, const PhysDev& ph, cudaStre
 }
 
 cudaError_t launch_tree_mask(int64_t n, const int32_t* perm, const uint8_t* active, uint8_t* out, int32_t* pre,
-                             int32_t* tmp, cudaStream_t st) {
+                             int32_t* tmp, int32_t* status, int num_sms, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   k_tree_mask<<<tree_blocks(n + 1), 256, 0, st>>>(n, perm, active, out, pre);
   if (pre != nullptr) {
-    const cudaError_t e = scan_exclusive_host_n(pre, n + 1, tmp, st);
+    const cudaError_t e = scan_exclusive(pre, pre, nullptr, n + 1, false, tmp, status, num_sms, st);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
