@@ -170,6 +170,7 @@ struct BlockTargets {
   int32_t n;              // targets in the block
   int32_t per, tpp, lg, rounds;
   int32_t next;           // next unclaimed round
+  float hcap;             // the density's cap on h in this block
   int32_t wcount[kBlkWarps];  // active targets per warp slice (masked builds)
 };
 

@@ -92,6 +92,8 @@ __global__ void k_grid_setup(const int64_t* __restrict__ sim_offset, const doubl
     g.cell = L / (double)nc;
     g.cell_f = (float)g.cell;
     g.reach_f = g.cell_f;
+    g.hcap_f = h_cap(g.cell, 2.0 * g.cell, gamma_k);
+    g.hcap_box_f = h_cap(L, L, gamma_k);
     g.scale_f = (float)((double)nc / L);
     g.cell_base = 0;
     g.blk_base = 0;

@@ -93,7 +93,7 @@ __device__ __forceinline__ void dens_pair(const float4& pi, const float4& vi, co
                                           const float4& vj, float H, float Hinv, DensSums& s) {
   const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float q = r2 * rinv * Hinv;
   float w, g;
   kernel_w_g<K>(q, H * rinv, w, g);
@@ -157,7 +157,7 @@ __device__ __forceinline__ void fin_pair(const float4& pi, const float4& vi, con
                                          float mj, float H, float Hinv, FinSums& s) {
   const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float q = r2 * rinv * Hinv;
   float w, dw, g;
   if constexpr (K == kKernCubic) {
@@ -258,6 +258,46 @@ __device__ __forceinline__ float list_r2(const float* lr2, const uint16_t* lj, c
   return fmaf(dx, dx, fmaf(dy, dy, dz * dz));
 }
 
+// The lane's candidates of its target's nine runs into its list column: the
+// staged slots A0 + sub, A0 + sub + kTpp, ... of each run with an expanded r^2
+// within the search radius.
+template <int K, int kTpp>
+__device__ __forceinline__ void filter_runs(const BlockGeom& g, const StageTable& T, int tx, int ty, int tz, int sub,
+                                            int lane, const float4* spos, const float4& pi, float R2, uint16_t* lj,
+                                            int& cnt) {
+  const float mx = -2.0f * pi.x, my = -2.0f * pi.y, mz = -2.0f * pi.z;
+  const float cthr = fmaf(R2, 2e-5f, R2) - pi.w;
+#pragma unroll 1
+  for (int r = 0; r < 9; ++r) {
+    int32_t A0, B0;
+    warp_run(g, T, tx, ty, tz, r, A0, B0);
+    A0 += sub;
+#pragma unroll 1
+    for (; A0 < B0; A0 += 32 * kTpp) {  // (a run of more than 32 candidates a lane in pieces)
+      const int steps = min((B0 - A0 + kTpp - 1) / kTpp, 32);
+      uint32_t hits = 0;
+#pragma unroll 1
+      for (int i = 0; i < steps; i += 4) {
+        const float4* p = spos + A0 + i * kTpp;  // (may read up to 3 kTpp slots on, still in shared memory)
+        uint32_t nib = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 pj = p[j * kTpp];
+          const float tq = fmaf(mz, pj.z, fmaf(my, pj.y, fmaf(mx, pj.x, pj.w)));
+          if (tq < cthr) nib |= 1u << j;
+        }
+        hits |= nib << i;
+      }
+      if (steps < 32) hits &= (1u << steps) - 1u;
+#pragma unroll 1
+      for (; hits != 0u; hits &= hits - 1u) {
+        lj[min(cnt, list_cap<K>()) * 32 + lane] = (uint16_t)(A0 + kTpp * (__ffs((int)hits) - 1));
+        ++cnt;
+      }
+    }
+  }
+}
+
 template <int K>
 __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::DensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char dsm_raw[];
@@ -280,6 +320,8 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
   for (int32_t b = blockIdx.x; b < total; b += gridDim.x) {
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
+    // (FP64, by one thread; read after the barriers below)
+    if (threadIdx.x == 0) BT.hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
     if (nsrc > dens_cap<K>()) {
       if (threadIdx.x == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
@@ -313,7 +355,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
     else
       __syncthreads();  // the staging
 
-    const float hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
+    const float hcap = BT.hcap;
     const float R2 = g.G.cell_f * g.G.cell_f;
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
@@ -387,21 +429,14 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
         // nothing: the passes recompute r^2 exactly, and the force tests
         // its own reach)
         static_assert(!kCacheR2, "the expanded filter keeps no r^2");
-        const float mx = -2.0f * pi.x, my = -2.0f * pi.y, mz = -2.0f * pi.z;
-        const float cthr = fmaf(R2, 2e-5f, R2) - pi.w;
-#pragma unroll 1
-        for (int r = 0; r < 9; ++r) {
-          int32_t A0, B0;
-          warp_run(g, T, tx, ty, tz, r, A0, B0);
-#pragma unroll 4
-          for (int32_t k = A0 + sub; k < B0; k += tpp) {
-            const float4 pj = spos[k];
-            const float tq = fmaf(mz, pj.z, fmaf(my, pj.y, fmaf(mx, pj.x, pj.w)));
-            const int at = min(cnt, list_cap<K>()) * 32 + lane;
-            lj[at] = (uint16_t)k;
-            cnt += tq < cthr;
-          }
-        }
+        // The lane's candidates of a run (every tpp-th) set bits of a word,
+        // four at a time, and the bits are listed afterwards (1.59 ->
+        // 1.55 ms on the 2M lattice against storing every candidate with the
+        // count advanced by the hits).
+        if (tpp == 2)
+          filter_runs<K, 2>(g, T, tx, ty, tz, sub, lane, spos, pi, R2, lj, cnt);
+        else
+          filter_runs<K, 4>(g, T, tx, ty, tz, sub, lane, spos, pi, R2, lj, cnt);
       }
       bool direct = cnt > list_cap<K>();
       if (a.axis_order != nullptr) {
@@ -492,7 +527,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
         for (; e + 1 < n_l; e += 2) {
           const float r2a = list_r2(lr2, lj, spos, pi, e * 32 + lane);
           const float r2b = list_r2(lr2, lj, spos, pi, (e + 1) * 32 + lane);
-          const float ria = rsqrtf(fmaxf(r2a, 1e-30f)), rib = rsqrtf(fmaxf(r2b, 1e-30f));
+          const float ria = rsqrt_norm(fmaxf(r2a, 1e-30f)), rib = rsqrt_norm(fmaxf(r2b, 1e-30f));
           const float qa = r2a * ria * Hinv, qb = r2b * rib * Hinv;
           float wa, dwa, wb, dwb;
           newton_terms<K>(qa, wa, dwa);
@@ -504,7 +539,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
         }
         if (e < n_l) {
           const float r2a = list_r2(lr2, lj, spos, pi, e * 32 + lane);
-          const float ria = rsqrtf(fmaxf(r2a, 1e-30f));
+          const float ria = rsqrt_norm(fmaxf(r2a, 1e-30f));
           float wa, dwa;
           newton_terms<K>(r2a * ria * Hinv, wa, dwa);
           Sw0 += wa;
@@ -518,7 +553,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
               const float4 pj = spos[k];
               const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
               const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-              const float ri = rsqrtf(fmaxf(r2, 1e-30f));
+              const float ri = rsqrt_norm(fmaxf(r2, 1e-30f));
               const float q = r2 * ri * Hinv;
               float w, dw;
               newton_terms<K>(q, w, dw);

@@ -95,15 +95,15 @@ __device__ __forceinline__ void force_pair(const ForceTarget& T, const float4& A
   }
   const float dx = T.A.x - Aj.x, dy = T.A.y - Aj.y, dz = T.A.z - Aj.z;
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float r = r2 * rinv;
   const float Gi = kernel_g<K>(r * T.D.y, T.A.w * rinv) * T.Hinv5;
   const float vx = T.B.x - Bj.x, vy = T.B.y - Bj.y, vz = T.B.z - Bj.z;
   const float vdotx = fmaf(vx, dx, fmaf(vy, dy, vz * dz));
   if constexpr (kFl == kFlGradient) {
     // zero beyond H_i (G_i = 0) and for the self pair (u_i - u_j = 0)
-    s.ax = fmaf(__fdividef(Bj.w, Dj.x) * (T.E.x - Ej.x), Gi, s.ax);
-    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(__fdividef(2.0f * fabsf(T.E.z - Ej.z), T.D.x + Dj.x)));
+    s.ax = fmaf(div_norm(Bj.w, Dj.x) * (T.E.x - Ej.x), Gi, s.ax);
+    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(T.E.z - Ej.z), T.D.x + Dj.x)));
     s.vsig = counted ? fmaxf(s.vsig, vc) : s.vsig;
     s.ay = counted ? fmaxf(s.ay, Ej.y) : s.ay;
     s.npair += counted;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void force_pair(const ForceTarget& T, const float4& A
   const float mu = fminf(vdotx, 0.0f) * rinv;
   const float vs = fmaf(-ph.beta_v, mu, T.C.z + Cj.z);
   const float av = kFl == kFlSphenix ? 0.5f * (T.E.y + Ej.y) : ph.alpha_v;
-  const float nu = __fdividef(-av * (T.C.w + Cj.w) * mu * vs, T.D.x + Dj.x);
+  const float nu = div_norm(-av * (T.C.w + Cj.w) * mu * vs, T.D.x + Dj.x);
   const float piG = T.C.x * Gi;
   const float visc = fmaf(T.C.y, Gi, Cj.y * Gj);
   const float sc = Bj.w * fmaf(0.5f * nu, visc, fmaf(Cj.x, Gj, piG));
@@ -125,9 +125,9 @@ __device__ __forceinline__ void force_pair(const ForceTarget& T, const float4& A
   if constexpr (kFl == kFlSphenix) {
     // conduction: zero beyond both supports (visc = 0) and for r = 0
     const float Ps = T.E.z + Ej.z, rs = T.D.x + Dj.x;
-    const float ac = Ps > 0.0f ? __fdividef(fmaf(T.E.z, T.E.w, Ej.z * Ej.w), Ps) : 0.0f;
-    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(__fdividef(2.0f * fabsf(T.E.z - Ej.z), rs)));
-    s.du = fmaf(Bj.w * ac * vc * (T.E.x - Ej.x) * r, __fdividef(visc, rs), s.du);
+    const float ac = Ps > 0.0f ? div_norm(fmaf(T.E.z, T.E.w, Ej.z * Ej.w), Ps) : 0.0f;
+    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(T.E.z - Ej.z), rs)));
+    s.du = fmaf(Bj.w * ac * vc * (T.E.x - Ej.x) * r, div_norm(visc, rs), s.du);
   }
   s.vsig = counted ? fmaxf(s.vsig, vs) : s.vsig;
   s.npair += counted;
@@ -463,7 +463,7 @@ __device__ __forceinline__ void min_pair(const MinTarget& T, const float4& A, co
                                          float rho_j, float beta, MinSums& s) {
   const float dx = T.x - A.x, dy = T.y - A.y, dz = T.z - A.z;
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float r = r2 * rinv;
   const float qi = r * T.Hinv, qj = r * A.w;
   // q >= 0, so max(1 - q, 0) and max(1 - 2q, 0) are saturations to [0, 1]
@@ -474,7 +474,7 @@ __device__ __forceinline__ void min_pair(const MinTarget& T, const float4& A, co
   const float vdotx = fmaf(vx, dx, fmaf(vy, dy, vz * dz));
   const float mu = fminf(vdotx, 0.0f) * rinv;
   const float vs = fmaf(-beta, mu, T.c + C.z);
-  const float nu2 = __fdividef(-(T.B + C.w) * mu * vs, T.rho + rho_j);
+  const float nu2 = div_norm(-(T.B + C.w) * mu * vs, T.rho + rho_j);
   const float piT = T.P * ti;
   const float Pt = fmaf(C.x, tj, piT);
   const float Ft = fmaf(T.F, ti, C.y * tj);

@@ -42,6 +42,8 @@ struct GridDev {
   float scale_f;      // n_c / L in FP32 (estimates of cell coordinates)
   float reach_f;      // largest support the cells serve: cell_f after a build,
                       // less twice the drift since, while cells are kept
+  float hcap_f;       // the largest h whose support stays below the cell side, and ...
+  float hcap_box_f;   // ... below half the box (h_cap)
   int64_t part_base;  // first pool index of this simulation
   int64_t n;          // particles in this simulation
 };
@@ -106,44 +108,78 @@ struct SphenixDev {
 // so that with A = S_w / gamma_K^3 - eta^3 and B = 3 eta^3 - S_dw / gamma_K^3
 // the Newton step is h <- h (1 - A/B).
 //
-// The convergence test |A| <= h_tol B runs in FP64 on gamma_K^3 A and
+// The convergence test |A| <= h_tol B is decided in FP64 on gamma_K^3 A and
 // gamma_K^3 B (a positive scale changes neither the test nor the ratio A/B):
 // those are one FP64 subtraction each from the FP32 sums.  The update itself
-// runs in FP32, whose rounding (~1e-7 relative) is far below h_tol; this
-// keeps FP64 division, slow on this GPU, out of the loop.  A finished target
-// gets its last correction applied (Newton converges quadratically, so the
-// result is within ~2 (A/B)^2 of the root).  Safeguards: the step is clamped
-// to [h/2, 2h] and falls back to bisection of the bracket [lo, hi] when it
-// leaves it or B <= 0; h never exceeds hcap.  Returns true when the target
+// runs in FP32, whose rounding (~1e-7 relative) is far below h_tol.  A finished
+// target gets its last correction applied (Newton converges quadratically, so
+// the result is within ~2 (A/B)^2 of the root).  Safeguards: the step is
+// clamped to [h/2, 2h] and falls back to bisection of the bracket [lo, hi] when
+// it leaves it or B <= 0; h never exceeds hcap.  Returns true when the target
 // is done (converged, capped, or out of iterations); otherwise advances h.
+//
+// An FP64 instruction of a warp occupies this GPU's FP64 pipe for 16 cycles of
+// the SM.  So the FP64 constants are held as three FP32 parts (their sum is
+// exact), A and B come as FP32 values from an error-free difference (their FP64
+// values rounded to FP32), and FP64 decides only where |A| and h_tol B are
+// closer than that rounding can tell: the same decisions and the same h.
 struct NewtonConst {
-  double a0;  // gamma_K^3 eta^3
-  double b0;  // 3 gamma_K^3 eta^3
+  float a[3];  // gamma_K^3 eta^3
+  float b[3];  // 3 gamma_K^3 eta^3
+  float tol_f;
   double tol;
   int32_t max_it;
 };
+
+__device__ __forceinline__ void split3(double v, float (&p)[3]) {
+  p[0] = (float)v;
+  p[1] = (float)(v - (double)p[0]);
+  p[2] = (float)((v - (double)p[0]) - (double)p[1]);
+}
+
+// x - (p0 + p1 + p2): the exact x - p0 as a sum of two floats (Knuth's TwoSum),
+// then the small parts.
+__device__ __forceinline__ float diff3(float x, const float (&p)[3]) {
+  const float s = __fadd_rn(x, -p[0]);
+  const float t = __fadd_rn(s, -x);
+  const float e = __fadd_rn(__fadd_rn(x, -__fadd_rn(s, -t)), __fadd_rn(-p[0], -t));
+  return __fadd_rn(s, __fadd_rn(__fadd_rn(e, -p[1]), -p[2]));
+}
 
 template <int K = 0>
 __device__ __forceinline__ NewtonConst newton_const(const PhysDev& ph) {
   constexpr double gk = KernT<K>::gammad;
   const double g3 = gk * gk * gk;
+  const double a0 = g3 * (double)ph.eta3;
   NewtonConst c;
-  c.a0 = g3 * (double)ph.eta3;
-  c.b0 = 3.0 * c.a0;
+  split3(a0, c.a);
+  split3(3.0 * a0, c.b);
   c.tol = ph.h_tol;
+  c.tol_f = (float)ph.h_tol;
   c.max_it = ph.max_h_iter;
   return c;
+}
+
+// The FP64 test, for the few targets too close to the line.
+static __device__ __noinline__ bool newton_converged(float Sw, float Sdw, float a0, float a1, float a2, float b0, float b1,
+                                              float b2, double tol) {
+  const double A = (double)Sw - (((double)a0 + (double)a1) + (double)a2);
+  const double B = (((double)b0 + (double)b1) + (double)b2) - (double)Sdw;
+  return B > 0.0 && fabs(A) <= tol * B;
 }
 
 __device__ __forceinline__ bool newton_update(float Sw, float Sdw, const NewtonConst& nc, float hcap,
                                               float& h, float& lo, float& hi, int& it, bool& atcap,
                                               bool& conv) {
-  const double A = (double)Sw - nc.a0;
-  const double B = nc.b0 - (double)Sdw;
-  if (A < 0.0) lo = h; else hi = h;
-  conv = (B > 0.0) && (fabs(A) <= nc.tol * B);
-  atcap = (h >= hcap) && (A < 0.0);
-  const float d = (float)A / (float)B;
+  const float A = diff3(Sw, nc.a);
+  const float B = -diff3(Sdw, nc.b);
+  if (A < 0.0f) lo = h; else hi = h;
+  const float line = nc.tol_f * B, gap = fabsf(A) - line;
+  conv = B > 0.0f && gap <= 0.0f;
+  if (fabsf(gap) <= 1e-6f * fabsf(line))
+    conv = newton_converged(Sw, Sdw, nc.a[0], nc.a[1], nc.a[2], nc.b[0], nc.b[1], nc.b[2], nc.tol);
+  atcap = (h >= hcap) && (A < 0.0f);
+  const float d = A / B;
   if (conv) {
     h = h * (1.0f - d);
     if (h > hcap) {
@@ -153,9 +189,9 @@ __device__ __forceinline__ bool newton_update(float Sw, float Sdw, const NewtonC
     return true;
   }
   if (atcap || it + 1 >= nc.max_it) return true;
-  float hn = (B > 0.0) ? h * (1.0f - d) : 2.0f * h;
+  float hn = (B > 0.0f) ? h * (1.0f - d) : 2.0f * h;
   hn = fminf(fmaxf(hn, 0.5f * h), 2.0f * h);
-  if (!(B > 0.0) || !(hn > lo) || !(hn < hi)) hn = isinf(hi) ? 2.0f * h : 0.5f * (lo + hi);
+  if (!(B > 0.0f) || !(hn > lo) || !(hn < hi)) hn = isinf(hi) ? 2.0f * h : 0.5f * (lo + hi);
   if (hn > hcap) hn = hcap;
   h = hn;
   ++it;
@@ -163,9 +199,17 @@ __device__ __forceinline__ bool newton_update(float Sw, float Sdw, const NewtonC
 }
 
 // The largest h whose support gamma_K h stays below `side` (and half the box).
+__device__ __forceinline__ float h_cap(double side, double L, double gamma_k) {
+  return (float)(fmin(side, 0.5 * L) * (1.0 - 1e-5) / gamma_k);
+}
 template <int K = 0>
 __device__ __forceinline__ float h_cap(double side, double L) {
-  return (float)(fmin(side, 0.5 * L) * (1.0 - 1e-5) / KernT<K>::gammad);
+  return h_cap(side, L, KernT<K>::gammad);
+}
+// The same for cells of side G.cell / 2^depth: the halvings are exact and
+// rounding is monotonic, so the FP64 division is the build's, once.
+__device__ __forceinline__ float h_cap_depth(const GridDev& G, int depth) {
+  return fminf(G.hcap_f * __int_as_float((127 - depth) << 23), G.hcap_box_f);
 }
 
 // Simulation owning a pool index (upper bound search over sim_offset).
@@ -414,6 +458,21 @@ __device__ __forceinline__ float kernel_g(float q, float H_rinv) {
     kernel_w_g<K>(q, H_rinv, w, g);
     return g;
   }
+}
+
+// 1 / sqrt(x) of a normal x, and x / y of a normal y: the approximate
+// instructions that rsqrtf and __fdividef end in, without the scaling that
+// those put around them for subnormal operands (three instructions a pair in
+// every loop; a subnormal x counts as zero).
+__device__ __forceinline__ float rsqrt_norm(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float div_norm(float x, float y) {
+  float q;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(x), "f"(y));
+  return q;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

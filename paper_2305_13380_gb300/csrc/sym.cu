@@ -51,7 +51,7 @@ __device__ __forceinline__ bool sym_pair(const SymTarget& T, const float4& A, co
                                          float rho_j, float beta, SymSums& s, float4& pa, float& pvs) {
   const float dx = T.x - A.x, dy = T.y - A.y, dz = T.z - A.z;
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float r = r2 * rinv;
   const float qi = r * T.Hinv, qj = r * A.w;
   const float ai = __saturatef(1.0f - qi), bi = __saturatef(fmaf(-2.0f, qi, 1.0f));
@@ -61,7 +61,7 @@ __device__ __forceinline__ bool sym_pair(const SymTarget& T, const float4& A, co
   const float vdotx = fmaf(vx, dx, fmaf(vy, dy, vz * dz));
   const float mu = fminf(vdotx, 0.0f) * rinv;
   const float vs = fmaf(-beta, mu, T.c + C.z);
-  const float nu2 = __fdividef(-(T.B + C.w) * mu * vs, T.rho + rho_j);
+  const float nu2 = div_norm(-(T.B + C.w) * mu * vs, T.rho + rho_j);
   const float piT = T.P * ti, pjT = C.x * tj;
   const float Ft = fmaf(T.F, ti, C.y * tj);
   const float Bk = rinv * fmaf(nu2, Ft, piT + pjT);

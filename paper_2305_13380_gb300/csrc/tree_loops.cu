@@ -185,7 +185,7 @@ template <int K>
 __device__ __forceinline__ void tdens_pair(float dx, float dy, float dz, const float4& vi, const float4& vj,
                                            float mj, float H, float Hinv, TDSums& s) {
   const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float q = r2 * rinv * Hinv;
   float w, g;
   kernel_w_g<K>(q, H * rinv, w, g);
@@ -206,7 +206,7 @@ __device__ __forceinline__ void tdens_pair(float dx, float dy, float dz, const f
 // n-hat and its h-derivative terms of one pair (Newton passes).
 template <int K>
 __device__ __forceinline__ void tnewton_pair(float r2, float H, float Hinv, float& Sw, float& Sdw) {
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float q = r2 * rinv * Hinv;
   float w, dw;
   kernel_w_dw<K>(q, w, dw);
@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sph
         const int32_t na = lane < 27 ? a.act_pre[R.lo + (cum_next - R.cum)] - a.act_pre[R.lo] : 0;
         if (!__any_sync(0xffffffffu, na > 0)) continue;
       }
-      const float hcap = h_cap<K>(g.side_d, g.L);
+      const float hcap = h_cap_depth(G, Lf.depth);
       // few sources: the 27 ranges whole; else the children of the ranges
       // that some target of the round reaches (children are half the cell; a
       // cell at the deepest level has one child)
@@ -1081,15 +1081,15 @@ __device__ __forceinline__ void tforce_pair(float dx, float dy, float dz, const 
     s.npair += in;
     return;
   }
-  const float rinv = rsqrtf(fmaxf(r2, 1e-30f));
+  const float rinv = rsqrt_norm(fmaxf(r2, 1e-30f));
   const float r = r2 * rinv;
   const float hi2 = Hinv_i * Hinv_i;
   const float Gi = kernel_g<K>(r * Hinv_i, Hi * rinv) * (hi2 * hi2 * Hinv_i);
   const float vx = vi.x - vj.x, vy = vi.y - vj.y, vz = vi.z - vj.z;
   const float vdotx = fmaf(vx, dx, fmaf(vy, dy, vz * dz));
   if constexpr (kFl == kTGradient) {
-    s.ax = fmaf(__fdividef(vj.w, rho_j) * (ei.x - ej.x), Gi, s.ax);
-    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(__fdividef(2.0f * fabsf(ei.z - ej.z), rho_i + rho_j)));
+    s.ax = fmaf(div_norm(vj.w, rho_j) * (ei.x - ej.x), Gi, s.ax);
+    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(ei.z - ej.z), rho_i + rho_j)));
     const bool in = r2 < Hi * Hi;
     s.vsig = in ? fmaxf(s.vsig, vc) : s.vsig;
     s.ay = in ? fmaxf(s.ay, ej.y) : s.ay;
@@ -1101,7 +1101,7 @@ __device__ __forceinline__ void tforce_pair(float dx, float dy, float dz, const 
   const float mu = fminf(vdotx, 0.0f) * rinv;
   const float vs = fmaf(-ph.beta_v, mu, ci.z + cj.z);
   const float av = kFl == kTSphenix ? 0.5f * (ei.y + ej.y) : ph.alpha_v;
-  const float nu = __fdividef(-av * (ci.w + cj.w) * mu * vs, rho_i + rho_j);
+  const float nu = div_norm(-av * (ci.w + cj.w) * mu * vs, rho_i + rho_j);
   const float piG = ci.x * Gi;
   const float visc = fmaf(ci.y, Gi, cj.y * Gj);
   const float mj = vj.w;
@@ -1113,9 +1113,9 @@ __device__ __forceinline__ void tforce_pair(float dx, float dy, float dz, const 
   if constexpr (kFl == kTSphenix) {
     // conduction: zero beyond both supports (visc = 0) and for r = 0
     const float Ps = ei.z + ej.z, rs = rho_i + rho_j;
-    const float ac = Ps > 0.0f ? __fdividef(fmaf(ei.z, ei.w, ej.z * ej.w), Ps) : 0.0f;
-    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(__fdividef(2.0f * fabsf(ei.z - ej.z), rs)));
-    s.du = fmaf(mj * ac * vc * (ei.x - ej.x) * r, __fdividef(visc, rs), s.du);
+    const float ac = Ps > 0.0f ? div_norm(fmaf(ei.z, ei.w, ej.z * ej.w), Ps) : 0.0f;
+    const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(ei.z - ej.z), rs)));
+    s.du = fmaf(mj * ac * vc * (ei.x - ej.x) * r, div_norm(visc, rs), s.du);
   }
   const float Hm = fmaxf(Hi, Hj);
   const bool in = r2 < Hm * Hm;
