@@ -788,6 +788,7 @@ sphh::TreeForceArgs tree_force_args(sph_ctx* c) {
   a.tgt = c->tgt;
   a.leaves = c->leaves;
   a.n_leaves = c->n_leaves;
+  a.leaf_of = c->leaf_of;
   a.ranges = c->ranges;
   a.fine = c->fine;
   a.rel = c->rel;

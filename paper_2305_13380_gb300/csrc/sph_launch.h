@@ -407,6 +407,7 @@ struct TreeForceArgs {
   const int32_t* tgt;
   const sphk::TreeLeaf* leaves;
   const int32_t* n_leaves;
+  const int32_t* leaf_of;  // target order -> its leaf
   const sphk::TreeRange* ranges;
   const int4* fine;
   const float4* rel;

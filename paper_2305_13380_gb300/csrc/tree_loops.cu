@@ -1185,28 +1185,31 @@ __device__ __forceinline__ float3 rec_rel_to(const TGeo& g, const TRec& h, int s
   return rel_to(g, h.q0, h.q1, sc);
 }
 
+// A warp takes windows of win consecutive targets from a counter, kTPer at a
+// time with kTreeTpp lanes each, whatever their leaves (a target's lanes hold
+// its own leaf's corner): every round is full, and a large leaf is shared by
+// many warps.  Bound by the latency and the L1 wavefronts of the 64-byte record
+// gathers.
 template <int kFl, int K>
-__global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs a, PhysDev ph, SphenixDev x) {
+__global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs a, PhysDev ph, SphenixDev x,
+                                                             int win) {
   const int lane = threadIdx.x & 31;
   const int t = lane / kTreeTpp, sub = lane % kTreeTpp;
-  const int32_t nl = *a.n_leaves;
+  const int64_t n = a.n_total;
   unsigned long long pair_acc = 0;
-  for (int32_t li = next_group(a.work, lane); li < nl; li = next_group(a.work, lane)) {
-    const TreeLeaf Lf = a.leaves[li];
-    const int32_t t_lo = Lf.start, n_t = a.leaves[li + 1].start - Lf.start;
-    const int sim = sim_of_cell(a.grid, a.n_sims, Lf.cell);
-    const GridDev G = a.grid[sim];
-    const TGeo g = leaf_geo(Lf, G);
-    const float dt = kFl == kTGradient ? (float)(x.dt_dev != nullptr ? x.dt_dev[sim] : x.dt) : 0.0f;
-    if (a.act != nullptr) {
-      // masked loops: skip a group without a masked target
-      bool any = false;
-      for (int32_t k = lane; k < n_t; k += 32) any = any || a.act[a.tgt[t_lo + k]] != 0;
-      if (!__any_sync(0xffffffffu, any)) continue;
-    }
-    for (int32_t t0 = 0; t0 < n_t; t0 += kTPer) {
-      const bool valid = t0 + t < n_t;
-      const int32_t ti = a.tgt[t_lo + (valid ? t0 + t : 0)];
+  for (int64_t w0 = (int64_t)next_group(a.work, lane) * win; w0 < n;
+       w0 = (int64_t)next_group(a.work, lane) * win) {
+#pragma unroll 1
+    for (int64_t t0 = w0; t0 < w0 + win && t0 < n; t0 += kTPer) {
+      const bool valid = t0 + t < n;
+      const int64_t k = t0 + (valid ? t : 0);
+      const int32_t ti = a.tgt[k];
+      // masked loops: skip a round without a masked target
+      if (a.act != nullptr && !__any_sync(0xffffffffu, a.act[ti] != 0)) continue;
+      const TreeLeaf Lf = a.leaves[a.leaf_of[k]];
+      const int sim = sim_of_cell(a.grid, a.n_sims, Lf.cell);
+      const TGeo g = leaf_geo(Lf, a.grid[sim]);
+      const float dt = kFl == kTGradient ? (float)(x.dt_dev != nullptr ? x.dt_dev[sim] : x.dt) : 0.0f;
       TFSums s;
       s.ax = s.ay = s.az = s.du = s.vsig = 0.f;
       s.npair = 0;
@@ -1668,7 +1671,13 @@ static cudaError_t launch_tree_force_k(const TreeForceArgs& a, const PhysDev& ph
   cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_work, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  k_tree_force<kFl, K><<<a.num_sms * bps, kTWarps * 32, 0, st>>>(a, ph, x);
+  // windows of two rounds; of one while that does not fill the resident warps
+  // four times (6,000 particles 317 -> 302 us; 1M masked 1.59 -> 1.66 ms)
+  const int64_t warps = (int64_t)a.num_sms * bps * kTWarps;
+  const int win = a.n_total < warps * 4 * kTPer ? kTPer : 2 * kTPer;
+  const int64_t want = (a.n_total + (int64_t)win * kTWarps - 1) / ((int64_t)win * kTWarps);
+  const int blocks = (int)(want < (int64_t)a.num_sms * bps ? want : (int64_t)a.num_sms * bps);
+  k_tree_force<kFl, K><<<blocks < 1 ? 1 : blocks, kTWarps * 32, 0, st>>>(a, ph, x, win);
   k_tree_force_fb<kFl, K><<<a.num_sms * bps, kTWarps * 32, 0, st>>>(a, ph, x);
   return cudaGetLastError();
 }
