@@ -57,3 +57,20 @@ def test_leaves_across_windows(orc, n_leaf):
     g = run_gpu(p, tree=True, n_leaf=n_leaf)
     od, of = orc.density_force(q, q["h0"])
     compare(g, od, of)
+
+
+@pytest.mark.parametrize("case", ["short", "mid", "long"])
+def test_reverse_pairs_sorted(case):
+    # the force adds a receiver's reverse pairs in order of their source, which
+    # atomics had put in any order: segments sorted by a thread (up to 32), a
+    # warp (up to 512) or a block give the same bits in every run
+    if case == "short":
+        p = inputs.clustered(5000, n_spheres=4, seed=2, a_min=0.02, a_max=0.05)
+    elif case == "mid":
+        p = inputs.clustered(20000, n_spheres=4, seed=43)
+    else:
+        p = _core_and_shell(20000, 3000, 6000, seed=5)
+    runs = [run_gpu(p, tree=True, n_leaf=32) for _ in range(3)]
+    for r in runs[1:]:
+        for k in ("h", "rho", "ax", "ay", "az", "du_dt", "v_sig"):
+            assert np.array_equal(runs[0][k], r[k]), k
