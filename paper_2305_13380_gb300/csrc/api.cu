@@ -1712,7 +1712,13 @@ int sph_fof(sph_ctx* c, int64_t n, const double* x, const double* y, const doubl
   f.y = y;
   f.z = z;
   f.link = link_len;
-  f.rel = c->pos4;  // the sorted density copies' buffer, free between loops
+  // the sorted copies' buffers and the sort's, free between loops
+  f.rel = c->pos4;
+  f.rel0 = c->vel4;
+  f.oct = c->rk;
+  f.queue = c->rv;
+  f.queued = c->misc + sphk::kNumOverflow;
+  f.num_sms = c->num_sms;
   f.group = group;
   f.status = c->misc + sphk::kStatus;
   c->lists_valid = false;

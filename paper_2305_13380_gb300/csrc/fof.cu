@@ -13,6 +13,16 @@
 // is farther from b^2 than its rounding can reach; the rest take the FP64
 // test, so the links are exactly those of the definition.
 //
+// Dense cells.  Particles of one octant of a cell are friends as they are: an
+// octant's diagonal is 0.866 cells, below b while cells are at most 1.15 b wide.
+// A cell of at least kFofDense particles has its particles ordered by octant and
+// each octant's particles start as one set; two octants (or an octant and a
+// particle) are then linked by their first friendly pair, if they are not one
+// set yet.  A core of thousands of particles within b of each other so takes a
+// few root checks per octant instead of a union per pair, all of them contending
+// for the same root (the 1M clustered box: 7.5 ms for all pairs, 0.86 ms for the
+// octants and the rest; the call 8.2 -> 1.67 ms).
+//
 // Union-find on the caller's group array, lock-free: a set's root is its
 // smallest index, a union hooks the larger root below the smaller one with
 // one compare-and-swap (retried when the root changed meanwhile), and the
@@ -76,57 +86,251 @@ __device__ __forceinline__ bool fof_friends64(const double* x, const double* y, 
   return r2 < b2;
 }
 
-// Sorted cell-relative positions (index in .w) and singleton sets.
+constexpr int kFofDense = 16;  // particles of a cell taken by octants
+
+// Whether octants are sets as they are (with a margin far above the rounding of
+// the FP32 positions that decide the octant).
+__device__ __forceinline__ bool fof_octants(const GridDev& G, double b) { return 0.86603 * 1.0001 * G.cell < b; }
+
+// Sorted cell-relative positions (index in .w) and singleton sets; the cells
+// taken by octants are queued, their positions to `rel0` to be ordered.
 __global__ void k_fof_prep(sphh::FofArgs a) {
   const GridDev G = a.grid[0];
+  const bool oct = fof_octants(G, a.link);
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.n_total;
        s += (int64_t)gridDim.x * blockDim.x) {
     const int32_t p = a.perm[s];
-    const int32_t c = a.key[p] - G.cell_base;
+    const int32_t cg = a.key[p], c = cg - G.cell_base;
     const int32_t kx = c % G.n_c, ky = (c / G.n_c) % G.n_c, kz = c / (G.n_c * G.n_c);
-    a.rel[s] = make_float4((float)(a.x[p] - (double)kx * G.cell), (float)(a.y[p] - (double)ky * G.cell),
-                           (float)(a.z[p] - (double)kz * G.cell), __int_as_float(p));
-    a.group[p] = p;
+    const float4 r = make_float4((float)(a.x[p] - (double)kx * G.cell), (float)(a.y[p] - (double)ky * G.cell),
+                                 (float)(a.z[p] - (double)kz * G.cell), __int_as_float(p));
+    const int32_t t0 = a.cell_start[cg];
+    const bool dense = oct && a.cell_start[cg + 1] - t0 >= kFofDense;
+    (dense ? a.rel0 : a.rel)[s] = r;
+    if (dense) {
+      if (s == t0) a.queue[atomicAdd(a.queued, 1)] = cg;
+    } else {
+      a.group[p] = p;
+    }
   }
 }
 
+__device__ __forceinline__ int fof_octant(const float4& r, float half) {
+  return (r.x >= half ? 1 : 0) | (r.y >= half ? 2 : 0) | (r.z >= half ? 4 : 0);
+}
+
+// A queued cell's particles in order of octant, then index (a warp per cell);
+// an octant's particles hang from its first, the smallest index.  The octants'
+// first places go to oct[first place of the cell + octant].
+__global__ void k_fof_octants(sphh::FofArgs a) {
+  const GridDev G = a.grid[0];
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const float half = 0.5f * G.cell_f;
+  const int32_t nq = *a.queued;
+  for (int32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < nq; q += (gridDim.x * blockDim.x) >> 5) {
+    const int32_t cg = a.queue[q], t0 = a.cell_start[cg], t1 = a.cell_start[cg + 1];
+    int32_t mine = 0;  // lane o < 8: particles of octant o
+    for (int32_t t = t0; t < t1; t += 32) {
+      const int o = t + lane < t1 ? fof_octant(a.rel0[t + lane], half) : 8;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int m = __popc(__ballot_sync(0xffffffffu, o == k));
+        if (lane == k) mine += m;
+      }
+    }
+    int32_t at = mine;  // exclusive prefix: the octants' first places
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      const int32_t v = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += v;
+    }
+    at += t0 - mine;
+    if (lane < 8) a.oct[t0 + lane] = at;
+    int32_t root = 0;  // lane o < 8: octant o's first index
+    bool any = false;
+    for (int32_t t = t0; t < t1; t += 32) {
+      const bool ok = t + lane < t1;
+      const float4 r = ok ? a.rel0[t + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int o = ok ? fof_octant(r, half) : 8;
+      const int32_t p = __float_as_int(r.w);
+      int32_t to = 0, top = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned m = __ballot_sync(0xffffffffu, o == k);
+        const int32_t first = __shfl_sync(0xffffffffu, p, m != 0u ? __ffs((int)m) - 1 : 0);
+        if (lane == k && m != 0u && !any) {
+          any = true;
+          root = first;
+        }
+        const int32_t base = __shfl_sync(0xffffffffu, at, k), r0 = __shfl_sync(0xffffffffu, root, k);
+        if (o == k) {
+          to = base + __popc(m & lt);
+          top = r0;
+        }
+        if (lane == k) at += __popc(m);
+      }
+      if (ok) {
+        a.rel[to] = r;
+        a.group[p] = top;
+      }
+    }
+  }
+}
+
+// Neighbour cell o of cell (kx, ky, kz): itself (0) or along the 13 axes; its
+// range of sorted places and its offset in cells.
+struct FofCell {
+  int32_t t0, t1;
+  float ox, oy, oz;
+};
+__device__ __forceinline__ FofCell fof_cell(const sphh::FofArgs& a, const GridDev& G, int32_t kx, int32_t ky,
+                                            int32_t kz, int o) {
+  const int32_t nc = G.n_c;
+  int dx = 0, dy = 0, dz = 0;
+  if (o > 0) axis_delta(o - 1, dx, dy, dz);
+  int32_t cx = kx + dx, cy = ky + dy, cz = kz + dz;
+  cx += cx < 0 ? nc : 0;
+  cx -= cx >= nc ? nc : 0;
+  cy += cy < 0 ? nc : 0;
+  cy -= cy >= nc ? nc : 0;
+  cz += cz < 0 ? nc : 0;
+  cz -= cz >= nc ? nc : 0;
+  const int32_t cn = G.cell_base + cx + nc * (cy + nc * cz);
+  return {a.cell_start[cn], a.cell_start[cn + 1], (float)dx * G.cell_f, (float)dy * G.cell_f, (float)dz * G.cell_f};
+}
+
+// FP32 distances of cell-relative coordinates (|x| below two cells) are within
+// ~1e-6 (2 cell)^2 of the true r2: a band of that width around b^2, plus a
+// margin, goes to the FP64 test.
+struct FofTest {
+  float lo, hi;
+  double b2;
+};
+__device__ __forceinline__ FofTest fof_test(const GridDev& G, double link) {
+  const double b2 = link * link;
+  const float band = 4e-6f * (2.0f * G.cell_f) * (2.0f * G.cell_f) + 1e-5f * (float)b2;
+  return {(float)b2 - band, (float)b2 + band, b2};
+}
+__device__ __forceinline__ bool fof_friends(const sphh::FofArgs& a, const GridDev& G, const FofTest& T, const float4& p,
+                                            const float4& q, const FofCell& C) {
+  const float fx = p.x - (q.x + C.ox), fy = p.y - (q.y + C.oy), fz = p.z - (q.z + C.oz);
+  const float r2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
+  if (r2 >= T.hi) return false;
+  return r2 < T.lo || fof_friends64(a.x, a.y, a.z, __float_as_int(p.w), __float_as_int(q.w), G.L, T.b2);
+}
+
+// Gap along one axis between [p0, p1] and octant bit `bit` of a cell at offset
+// off (both in cell-relative units).
+__device__ __forceinline__ float fof_gap(float p0, float p1, float off, int bit, float half) {
+  const float lo = off + (bit ? half : 0.0f);
+  return fmaxf(fmaxf(lo - p1, p0 - (lo + half)), 0.0f);
+}
+
+// Particles of cells not taken by octants, a thread each: the later particles
+// of the cell and those of the 13 neighbours (or their octants).
 __global__ void k_fof_link(sphh::FofArgs a) {
   const GridDev G = a.grid[0];
   const int32_t nc = G.n_c;
-  const double b2 = a.link * a.link;
-  // FP32 distances of cell-relative coordinates (|x| below two cells) are
-  // within ~1e-6 (2 cell)^2 of the true r2: a band of that width around b^2,
-  // plus a margin, goes to the FP64 test
-  const float cf = G.cell_f;
-  const float band = 4e-6f * (2.0f * cf) * (2.0f * cf) + 1e-5f * (float)b2;
-  const float lo = (float)b2 - band, hi = (float)b2 + band;
+  const FofTest T = fof_test(G, a.link);
+  const int dense = fof_octants(G, a.link) ? kFofDense : INT32_MAX;
+  const float half = 0.5f * G.cell_f;
   for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.n_total;
        s += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t pi = a.perm[s];
+    const int32_t cg = a.key[pi], c = cg - G.cell_base;
+    if (a.cell_start[cg + 1] - a.cell_start[cg] >= dense) continue;
     const float4 me = a.rel[s];
-    const int32_t pi = __float_as_int(me.w);
-    const int32_t c = a.key[pi] - G.cell_base;
     const int32_t kx = c % nc, ky = (c / nc) % nc, kz = c / (nc * nc);
     for (int o = 0; o <= kAxes; ++o) {
-      int dx = 0, dy = 0, dz = 0;
-      if (o > 0) axis_delta(o - 1, dx, dy, dz);
-      int32_t cx = kx + dx, cy = ky + dy, cz = kz + dz;
-      cx += cx < 0 ? nc : 0;
-      cx -= cx >= nc ? nc : 0;
-      cy += cy < 0 ? nc : 0;
-      cy -= cy >= nc ? nc : 0;
-      cz += cz < 0 ? nc : 0;
-      cz -= cz >= nc ? nc : 0;
-      const int32_t cn = G.cell_base + cx + nc * (cy + nc * cz);
-      const int32_t t0 = o == 0 ? (int32_t)s + 1 : a.cell_start[cn];
-      const int32_t t1 = a.cell_start[cn + 1];
-      const float ox = (float)dx * cf, oy = (float)dy * cf, oz = (float)dz * cf;
-      for (int32_t t = t0; t < t1; ++t) {
+      FofCell C = fof_cell(a, G, kx, ky, kz, o);
+      if (C.t1 - C.t0 >= dense) {
+        // octants within reach that are not in this particle's set yet
+        for (int k = 0; k < 8; ++k) {
+          const int32_t u0 = a.oct[C.t0 + k], u1 = k < 7 ? a.oct[C.t0 + k + 1] : C.t1;
+          if (u0 >= u1) continue;
+          const float gx = fof_gap(me.x, me.x, C.ox, k & 1, half), gy = fof_gap(me.y, me.y, C.oy, (k >> 1) & 1, half),
+                      gz = fof_gap(me.z, me.z, C.oz, k >> 2, half);
+          if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) >= T.hi) continue;
+          const int32_t pk = __float_as_int(a.rel[u0].w);
+          if (fof_find<true>(a.group, pi, a.status) == fof_find<true>(a.group, pk, a.status)) continue;
+          for (int32_t u = u0; u < u1; ++u) {
+            if (fof_friends(a, G, T, me, a.rel[u], C)) {
+              fof_union(a.group, pi, pk, a.status);
+              break;
+            }
+          }
+        }
+        continue;
+      }
+      if (o == 0) C.t0 = (int32_t)s + 1;
+      for (int32_t t = C.t0; t < C.t1; ++t) {
         const float4 q = a.rel[t];
-        const float fx = me.x - (q.x + ox), fy = me.y - (q.y + oy), fz = me.z - (q.z + oz);
-        const float r2 = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-        if (r2 >= hi) continue;
-        const int32_t pj = __float_as_int(q.w);
-        if (r2 < lo || fof_friends64(a.x, a.y, a.z, pi, pj, G.L, b2)) fof_union(a.group, pi, pj, a.status);
+        if (fof_friends(a, G, T, me, q, C)) fof_union(a.group, pi, __float_as_int(q.w), a.status);
+      }
+    }
+  }
+}
+
+// Octants of the queued cells, a warp each: the later octants of the cell and
+// the octants or particles of the 13 neighbours.  A lane looks at one of them
+// at a time (is it within reach, and another set?); those left are tested by
+// the whole warp, pair by pair until the first friends.
+__global__ void k_fof_link_octants(sphh::FofArgs a) {
+  const GridDev G = a.grid[0];
+  const int32_t nc = G.n_c;
+  const FofTest T = fof_test(G, a.link);
+  const float half = 0.5f * G.cell_f;
+  const int lane = threadIdx.x & 31;
+  const int64_t items = 8 * (int64_t)*a.queued;
+  for (int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items;
+       it += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int32_t cg = a.queue[it >> 3], c = cg - G.cell_base;
+    const int me = (int)(it & 7);
+    const int32_t own0 = a.cell_start[cg];
+    const int32_t s0 = a.oct[own0 + me], s1 = me < 7 ? a.oct[own0 + me + 1] : a.cell_start[cg + 1];
+    if (s0 >= s1) continue;
+    const int32_t pm = __float_as_int(a.rel[s0].w);
+    const float mx = me & 1 ? half : 0.0f, my = me & 2 ? half : 0.0f, mz = me & 4 ? half : 0.0f;
+    const int32_t kx = c % nc, ky = (c / nc) % nc, kz = c / (nc * nc);
+    for (int o = 0; o <= kAxes; ++o) {
+      const FofCell C = fof_cell(a, G, kx, ky, kz, o);
+      const bool dense = C.t1 - C.t0 >= kFofDense;  // at most kFofDense - 1 particles else
+      const int nodes = dense ? 8 : C.t1 - C.t0;
+      int32_t u0 = 0, u1 = 0;
+      bool open = lane < nodes && (o > 0 || lane > me);
+      if (open) {
+        u0 = dense ? a.oct[C.t0 + lane] : C.t0 + lane;
+        u1 = dense ? (lane < 7 ? a.oct[C.t0 + lane + 1] : C.t1) : u0 + 1;
+        open = u0 < u1;
+      }
+      if (open) {
+        float gx, gy, gz;
+        const float4 q = a.rel[u0];
+        if (dense) {
+          gx = fof_gap(mx, mx + half, C.ox, lane & 1, half);
+          gy = fof_gap(my, my + half, C.oy, (lane >> 1) & 1, half);
+          gz = fof_gap(mz, mz + half, C.oz, lane >> 2, half);
+        } else {
+          gx = fof_gap(q.x + C.ox, q.x + C.ox, mx, 0, half);
+          gy = fof_gap(q.y + C.oy, q.y + C.oy, my, 0, half);
+          gz = fof_gap(q.z + C.oz, q.z + C.oz, mz, 0, half);
+        }
+        open = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < T.hi &&
+               fof_find<true>(a.group, pm, a.status) != fof_find<true>(a.group, __float_as_int(q.w), a.status);
+      }
+      for (unsigned left = __ballot_sync(0xffffffffu, open); left != 0u; left &= left - 1u) {
+        const int k = __ffs((int)left) - 1;
+        const int32_t v0 = __shfl_sync(0xffffffffu, u0, k), v1 = __shfl_sync(0xffffffffu, u1, k);
+        // 32 of this octant's particles at a time against each of the other's
+        bool found = false;
+        for (int32_t s = s0; s < s1 && !found; s += 32) {
+          const float4 p = a.rel[min(s + lane, s1 - 1)];
+          for (int32_t u = v0; u < v1 && !found; ++u)
+            found = __any_sync(0xffffffffu, fof_friends(a, G, T, p, a.rel[u], C));
+        }
+        if (found && lane == 0) fof_union(a.group, pm, __float_as_int(a.rel[v0].w), a.status);
+        __syncwarp();
       }
     }
   }
@@ -148,7 +352,11 @@ cudaError_t launch_fof(const FofArgs& a, cudaStream_t st) {
   if (a.n_total <= 0) return cudaSuccess;
   int64_t b = (a.n_total + 255) / 256;
   if (b > 65535) b = 65535;
+  cudaError_t e = cudaMemsetAsync(a.queued, 0, sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
   k_fof_prep<<<(int)b, 256, 0, st>>>(a);
+  k_fof_octants<<<a.num_sms * 8, 256, 0, st>>>(a);
+  k_fof_link_octants<<<a.num_sms * 8, 256, 0, st>>>(a);
   k_fof_link<<<(int)b, 256, 0, st>>>(a);
   k_fof_label<<<(int)b, 256, 0, st>>>(a);
   return cudaGetLastError();

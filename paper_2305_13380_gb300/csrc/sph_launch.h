@@ -47,6 +47,9 @@ struct FofArgs {
   const double *x, *y, *z;
   double link;                   // linking length b
   float4* rel;                   // n scratch: sorted cell-relative positions
+  float4* rel0;                  // n scratch: those of the dense cells before they are ordered by octant
+  int32_t *oct, *queue, *queued; // n scratch: octants' first places; the dense cells, their number
+  int num_sms;
   int32_t* group;                // n: union-find parents, then the labels
   int32_t* status;
 };
