@@ -543,7 +543,7 @@ int sph_tree_counts(sph_ctx* ctx, int64_t* out);
  * cell_start and perm.  The cells are sized for the cubic spline's support
  * H = 1.825742 h; a caller of the quartic or Wendland C2 kernel passes h
  * scaled by gamma_K(kernel) / 1.825742, or uses sph_build_cells.  All of its
- * scratch is one fixed array compiled into the library (about 3.1 MB, held
+ * scratch is one fixed array compiled into the library (about 1.2 MB, held
  * by every GPU that loads the library until the process exits); it calls no
  * allocating routine.
  *   n              particles, 0 <= n <= 65536 (more: SPH_E_CAPACITY)

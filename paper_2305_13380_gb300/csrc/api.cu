@@ -36,7 +36,7 @@ struct sph_ctx {
   double* h_box1 = nullptr;
   // grown buffers
   GridDev* grid = nullptr;
-  int32_t *key = nullptr, *slot = nullptr, *count = nullptr, *cell_start = nullptr;
+  int32_t *key = nullptr, *slot = nullptr, *cell_start = nullptr;
   int32_t *scan_sums = nullptr, *perm = nullptr, *overflow = nullptr;
   int32_t *rk = nullptr, *rv = nullptr, *rhist = nullptr;
   float4 *pos4 = nullptr, *vel4 = nullptr, *th4 = nullptr;
@@ -131,7 +131,6 @@ void free_grown(sph_ctx* c) {
   dfree(c->grid);
   dfree(c->key);
   dfree(c->slot);
-  dfree(c->count);
   dfree(c->cell_start);
   dfree(c->scan_sums);
   dfree(c->perm);
@@ -237,8 +236,8 @@ int ensure(sph_ctx* c, int64_t n, int n_sims, int cells_per_particle = 8) {
   const int cs = n_sims + n_sims / 4 + 1;
   const int64_t cc = (cells_per_particle > 8 ? cells_per_particle : 8) * cn + 216 * (int64_t)cs;
   bool ok = dalloc(c->grid, cs) && dalloc(c->key, cn) && dalloc(c->slot, cn) &&
-            dalloc(c->count, cc + 1) && dalloc(c->cell_start, cc + 1) &&
-            dalloc(c->scan_sums, sphh::scan_words(cc + 1)) && dalloc(c->perm, cn) &&
+            dalloc(c->cell_start, cc + 1) &&
+            dalloc(c->scan_sums, sphh::scan_words(cn + 1) + cn / 2048 + 2) && dalloc(c->perm, cn) &&
             dalloc(c->rk, cn) && dalloc(c->rv, cn) && dalloc(c->rhist, sphh::radix_words(cn, (c->p.flags & SPH_FLAG_TREE) ? 8 : 4)) &&
             dalloc(c->overflow, (8 * cn + 216 * (int64_t)cs) / 3 + 2) && dalloc(c->pos4, cn) &&
             dalloc(c->vel4, cn) && dalloc(c->th4, cn) && dalloc(c->hs, cn) && dalloc(c->fD, cn) &&
@@ -484,9 +483,7 @@ int do_build(sph_ctx* c, int n_sims, int64_t n_total, const int64_t* off, const 
   b.hmax_bits = c->hmax_bits;
   b.key = c->key;
   b.slot = c->slot;
-  b.count = c->count;
   b.cell_start = c->cell_start;
-  b.scan_sums = c->scan_sums;
   b.perm = c->perm;
   b.rk = c->rk;
   b.rv = c->rv;
@@ -516,6 +513,7 @@ int do_build(sph_ctx* c, int n_sims, int64_t n_total, const int64_t* off, const 
     t.h = h;
     t.cell_key = c->key;
     t.cell_start = c->cell_start;
+    t.misc = c->misc;
     t.key64 = c->key64;
     t.key64_b = c->key64_b;
     t.skey = c->skey;
@@ -1677,8 +1675,8 @@ int sph_conservation(sph_ctx* c, const sph_pool* pl, double* out) {
 // Friends-of-friends grids allow 160 cells per particle (8 for the SPH
 // loops): at the usual linking length of 0.2 mean spacings, cells of b itself
 // need 125 per particle, and cells capped wider multiply the pairs to test by
-// the cube of the widening (2.5^3 = 16 at the SPH cap).  Their counts and
-// offsets take 1.3 KB per particle.
+// the cube of the widening (2.5^3 = 16 at the SPH cap).  Their offsets take
+// 640 bytes per particle.
 constexpr int kFofCellsPerParticle = 160;
 
 int sph_fof(sph_ctx* c, int64_t n, const double* x, const double* y, const double* z, double link_len,

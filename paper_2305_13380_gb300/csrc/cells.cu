@@ -3,14 +3,16 @@
 //
 // Pipeline (all sizes that depend on the data stay on the device, so a whole
 // step can be captured in a CUDA graph):
-//   k_grid_setup   per simulation: max h -> cells per side n_c
-//   k_grid_base    prefix of n_c^3 over simulations -> global cell ids
-//   k_key_count    FP64 cell coordinates, cell id, per-cell count
-//   k_scan         exclusive scan of the counts -> cell_start (radix.cu)
+//   k_grid_hmax    max h per simulation
+//   k_grid_setup   cells per side n_c of each simulation, and the prefix of
+//                  n_c^3 over simulations -> global cell ids
+//   k_cell_key     FP64 cell coordinates, cell id
 //   radix sort     stable sort of (cell id, particle index) -> perm, so the
 //                  order inside a cell is ascending index for any cell size
 //                  (radix.cu)
+//   k_cell_bounds  cell_start from the sorted ids
 //   k_gather_*     sorted float copies relative to each particle's cell
+#include "lookback.cuh"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 
@@ -61,73 +63,67 @@ __global__ void k_grid_hmax(const int64_t* __restrict__ sim_offset, int n_sims, 
     atomicMax(&hmax_bits[cur], __float_as_int(m));
 }
 
-// One thread per simulation: cells per side from max h.
-// radius > 0: the search radius is given (friends-of-friends), not derived
-// from the smoothing lengths.
-__global__ void k_grid_setup(const int64_t* __restrict__ sim_offset, const double* __restrict__ box,
-                             const int32_t* __restrict__ hmax_bits, int n_sims, double margin,
-                             double radius, int cells_per_particle, double gamma_k,
-                             GridDev* __restrict__ grid, int32_t* __restrict__ misc) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n_sims; s += gridDim.x * blockDim.x) {
-    const int64_t a = sim_offset[s], b = sim_offset[s + 1];
-    const float m = __int_as_float(hmax_bits[s]);
-    const double L = box[s];
-    const double Hmax = radius > 0.0 ? radius : gamma_k * (double)m * (1.0 + margin);
-    const int32_t cap = cap_cells_per_side(b - a, cells_per_particle);
-    int32_t nc = cap;
-    if (Hmax > 0.0) {
-      const double t = floor(L / Hmax);
-      nc = t < (double)cap ? (int32_t)t : cap;
-    }
-    // Any n_c >= 1 gives exact sums while H <= min(cell, L/2): with fewer
-    // than 3 cells per side the 27-cell stencil visits a cell's periodic
-    // images twice, and the farther image lies at least L - H >= H away,
-    // where the kernel is exactly zero.  Supports above L/2 would break the
-    // minimum image.
-    if (Hmax > 0.5 * L) atomicOr(&misc[kStatus], SPH_ST_BOX);
-    if (nc < 1) nc = 1;
+// Cells per side of each simulation from its max h, then the first cell and
+// block of each (one block of kScanThreads threads).  radius > 0: the search
+// radius is given (friends-of-friends), not derived from the smoothing lengths.
+__global__ void __launch_bounds__(kScanThreads)
+k_grid_setup(const int64_t* __restrict__ sim_offset, const double* __restrict__ box,
+             const int32_t* __restrict__ hmax_bits, int n_sims, double margin, double radius, int cells_per_particle,
+             double gamma_k, GridDev* __restrict__ grid, int32_t* __restrict__ misc) {
+  int32_t cells = 0, blocks = 0;
+  for (int s0 = 0; s0 < n_sims; s0 += kScanThreads) {
+    const int s = s0 + threadIdx.x;
     GridDev g;
-    g.L = L;
-    g.n_c = nc;
-    g.cell = L / (double)nc;
-    g.cell_f = (float)g.cell;
-    g.reach_f = g.cell_f;
-    g.hcap_f = h_cap(g.cell, 2.0 * g.cell, gamma_k);
-    g.hcap_box_f = h_cap(L, L, gamma_k);
-    g.scale_f = (float)((double)nc / L);
-    g.cell_base = 0;
-    g.blk_base = 0;
-    g.part_base = a;
-    g.n = b - a;
-    grid[s] = g;
+    int32_t nc = 0;
+    if (s < n_sims) {
+      const int64_t a = sim_offset[s], b = sim_offset[s + 1];
+      const float m = __int_as_float(hmax_bits[s]);
+      const double L = box[s];
+      const double Hmax = radius > 0.0 ? radius : gamma_k * (double)m * (1.0 + margin);
+      const int32_t cap = cap_cells_per_side(b - a, cells_per_particle);
+      nc = cap;
+      if (Hmax > 0.0) {
+        const double t = floor(L / Hmax);
+        nc = t < (double)cap ? (int32_t)t : cap;
+      }
+      // Any n_c >= 1 gives exact sums while H <= min(cell, L/2): with fewer
+      // than 3 cells per side the 27-cell stencil visits a cell's periodic
+      // images twice, and the farther image lies at least L - H >= H away,
+      // where the kernel is exactly zero.  Supports above L/2 would break the
+      // minimum image.
+      if (Hmax > 0.5 * L) atomicOr(&misc[kStatus], SPH_ST_BOX);
+      if (nc < 1) nc = 1;
+      g.L = L;
+      g.n_c = nc;
+      g.cell = L / (double)nc;
+      g.cell_f = (float)g.cell;
+      g.reach_f = g.cell_f;
+      g.hcap_f = h_cap(g.cell, 2.0 * g.cell, gamma_k);
+      g.hcap_box_f = h_cap(L, L, gamma_k);
+      g.scale_f = (float)((double)nc / L);
+      g.part_base = a;
+      g.n = b - a;
+    }
+    const int32_t nb = (nc + 1) / 2;
+    int32_t tc, tb;
+    const int32_t c0 = block_scan(nc * nc * nc, &tc), b0 = block_scan(nb * nb * nb, &tb);
+    if (s < n_sims) {
+      g.cell_base = cells + c0;
+      g.blk_base = blocks + b0;
+      grid[s] = g;
+    }
+    cells += tc;
+    blocks += tb;
+  }
+  if (threadIdx.x == 0) {
+    misc[kTotalCells] = cells;
+    misc[kTotalBlocks] = blocks;
   }
 }
 
-__global__ void k_grid_base(GridDev* __restrict__ grid, int n_sims, int32_t* __restrict__ misc) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int64_t base = 0, bbase = 0;
-  for (int s = 0; s < n_sims; ++s) {
-    grid[s].cell_base = (int32_t)base;
-    grid[s].blk_base = (int32_t)bbase;
-    const int64_t nc = grid[s].n_c;
-    const int64_t nb = (nc + 1) / 2;
-    base += nc * nc * nc;
-    bbase += nb * nb * nb;
-  }
-  misc[kTotalCells] = (int32_t)base;
-  misc[kTotalBlocks] = (int32_t)bbase;
-}
-
-__global__ void k_zero_counts(int32_t* __restrict__ count, const int32_t* __restrict__ misc) {
-  const int32_t total = misc[kTotalCells];
-  for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c <= total; c += gridDim.x * blockDim.x)
-    count[c] = 0;
-}
-
-__global__ void k_key_count(int64_t n_total, const double* __restrict__ x, const double* __restrict__ y,
-                            const double* __restrict__ z, const int64_t* __restrict__ sim_offset,
-                            int n_sims, const GridDev* __restrict__ grid, int32_t* __restrict__ key,
-                            int32_t* __restrict__ count) {
+__global__ void k_cell_key(int64_t n_total, const double* __restrict__ x, const double* __restrict__ y,
+                           const double* __restrict__ z, const int64_t* __restrict__ sim_offset, int n_sims,
+                           const GridDev* __restrict__ grid, int32_t* __restrict__ key) {
   const WarpRange wr = warp_range(n_total);
   SimCursor sc;
   for (int64_t p = wr.lo + (threadIdx.x & 31); p < wr.hi; p += 32) {
@@ -136,12 +132,66 @@ __global__ void k_key_count(int64_t n_total, const double* __restrict__ x, const
     const int32_t kx = cell_coord_fast(x[p], G.L, G.n_c, G.scale_f);
     const int32_t ky = cell_coord_fast(y[p], G.L, G.n_c, G.scale_f);
     const int32_t kz = cell_coord_fast(z[p], G.L, G.n_c, G.scale_f);
-    const int32_t k = G.cell_base + kx + G.n_c * (ky + G.n_c * kz);
-    key[p] = k;
-    // neighbours in index order often share a cell: one atomic per distinct
-    // cell of the converged lanes
-    const unsigned peers = __match_any_sync(__activemask(), k);
-    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&count[k], __popc(peers));
+    key[p] = G.cell_base + kx + G.n_c * (ky + G.n_c * kz);
+  }
+}
+
+// cell_start[c] for c = 0 .. cells (included): the first of the n sorted keys
+// whose cell (key >> shift) is at least c.  A warp takes kChunk cells at a time:
+// the range of keys that they hold by a search of the whole warp (32 probes a
+// step), then each cell's bound within it.  kChunk is 32 where cells hold many
+// particles (the SPH loops: the searches are long, so as many warps as there
+// are), 1024, four cells a lane, where most are empty.  Cells without
+// particles cost a store: counting into every cell, scanning and adding back
+// took 1.1 of the 8.8 ms of friends-of-friends on 1M particles (160 cells per
+// particle), a one-pass scan of zeroed counts 0.58 ms, this 0.18.
+template <class K>
+__device__ __forceinline__ int32_t warp_first(const K* __restrict__ keys, int32_t lo, int32_t hi, int shift, int32_t c,
+                                              int lane) {
+  while (lo < hi) {  // the first key of cell >= c lies in [lo, hi]
+    const int32_t step = (hi - lo + 31) >> 5;
+    const int32_t p = lo + (lane + 1) * step - 1;
+    const int less = __popc(__ballot_sync(0xffffffffu, p < hi && (int32_t)(keys[p] >> shift) < c));
+    const int32_t at = lo + less * step;
+    hi = min(hi, at + step - 1);
+    lo = min(at, hi);
+  }
+  return lo;
+}
+template <class K, int kChunk>
+__global__ void k_cell_bounds(int32_t n, const K* __restrict__ keys, int shift, const int32_t* __restrict__ misc,
+                              int32_t* __restrict__ cell_start) {
+  const int32_t total = misc[kTotalCells];
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const bool vec = ((uintptr_t)cell_start & 15u) == 0u;
+  constexpr int kLane = kChunk >= 128 ? 4 : 1;  // consecutive cells of a lane
+  for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w * kChunk <= total; w += warps) {
+    const int32_t c0 = (int32_t)(w * kChunk);
+    const int32_t s0 = warp_first(keys, 0, n, shift, c0, lane);
+    const int32_t s1 = (int64_t)c0 + kChunk <= total ? warp_first(keys, s0, n, shift, c0 + kChunk, lane) : n;
+    for (int32_t c = c0 + kLane * lane; c < c0 + kChunk && c <= total; c += 32 * kLane) {
+      int32_t b[kLane], lo = s0;
+#pragma unroll
+      for (int i = 0; i < kLane; ++i) {
+        // past the keys of the cells before it: mostly none where cells are mostly empty
+        int32_t hi = s1;
+        if (i > 0 && (lo >= s1 || (int32_t)(keys[lo] >> shift) >= c + i)) hi = lo;
+        while (lo < hi) {
+          const int32_t mid = (int32_t)(((uint32_t)lo + (uint32_t)hi) >> 1);
+          if ((int32_t)(keys[mid] >> shift) < c + i) lo = mid + 1; else hi = mid;
+        }
+        b[i] = lo;
+      }
+      if (kLane == 4 && vec && c + 3 <= total) {
+        *reinterpret_cast<int4*>(cell_start + c) = make_int4(b[0], b[kLane > 1 ? 1 : 0], b[kLane > 2 ? 2 : 0],
+                                                             b[kLane > 3 ? 3 : 0]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < kLane; ++i)
+          if (c + i <= total) cell_start[c + i] = b[i];
+      }
+    }
   }
 }
 
@@ -285,6 +335,19 @@ static int grid_for(int64_t n, int threads, int max_blocks) {
   return (int)b;
 }
 
+// The cell count is known on the device only: blocks up to the capacity,
+// capped; idle warps return at once.
+template <class K>
+static void cell_bounds(int64_t n, const K* keys, int shift, int64_t cap_cells, int num_sms, const int32_t* misc,
+                        int32_t* cell_start, cudaStream_t st) {
+  if (cap_cells > 16 * n + 4096)
+    k_cell_bounds<K, 1024><<<grid_for(cap_cells + 1, 8 * 1024, num_sms * 8), 256, 0, st>>>((int32_t)n, keys, shift,
+                                                                                          misc, cell_start);
+  else
+    k_cell_bounds<K, 32><<<grid_for(cap_cells + 1, 8 * 32, num_sms * 8), 256, 0, st>>>((int32_t)n, keys, shift, misc,
+                                                                                      cell_start);
+}
+
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t st) {
   if (cudaMemsetAsync(a.hmax_bits, 0, sizeof(int32_t) * a.n_sims, st) != cudaSuccess) return cudaGetLastError();
   if (a.n_total > 0 && !(a.radius > 0.0)) {
@@ -292,26 +355,24 @@ cudaError_t launch_build(const BuildArgs& a, cudaStream_t st) {
     if (hb > (int64_t)a.num_sms * 8) hb = (int64_t)a.num_sms * 8;
     k_grid_hmax<<<(int)hb, 256, 0, st>>>(a.sim_offset, a.n_sims, a.n_total, a.h, a.hmax_bits);
   }
-  k_grid_setup<<<(a.n_sims + 127) / 128, 128, 0, st>>>(a.sim_offset, a.box, a.hmax_bits, a.n_sims,
-                                                       a.margin, a.radius, a.cells_per_particle, a.gamma_k,
-                                                       a.grid, a.misc);
-  k_grid_base<<<1, 32, 0, st>>>(a.grid, a.n_sims, a.misc);
-  // grids sized for the capacity but capped: the kernels loop up to the
-  // device-side cell count, and idle blocks would only cost launch time
-  const int zb = grid_for(a.cap_cells + 1, 256, a.num_sms * 8);
-  k_zero_counts<<<zb, 256, 0, st>>>(a.count, a.misc);
-  const int pb = grid_for(a.n_total, 256, 65535);
+  k_grid_setup<<<1, kScanThreads, 0, st>>>(a.sim_offset, a.box, a.hmax_bits, a.n_sims, a.margin, a.radius,
+                                           a.cells_per_particle, a.gamma_k, a.grid, a.misc);
   if (a.n_total > 0)
-    k_key_count<<<pb, 256, 0, st>>>(a.n_total, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.key, a.count);
-  cudaError_t e = scan_exclusive(a.count, a.cell_start, a.misc + kTotalCells, a.cap_cells, true, a.scan_sums,
-                                 a.misc + kStatus, a.num_sms, st);
+    k_cell_key<<<grid_for(a.n_total, 256, 65535), 256, 0, st>>>(a.n_total, a.x, a.y, a.z, a.sim_offset, a.n_sims,
+                                                                a.grid, a.key);
+  if (!a.sort_cells) return cudaGetLastError();  // (the nested grids sort finer keys first)
+  int bits = 1;
+  while (bits < 31 && ((int64_t)1 << bits) <= a.cap_cells) ++bits;
+  const cudaError_t e =
+      radix_sort_index(a.n_total, bits, a.key, a.rk, a.slot, a.perm, a.rv, a.hist, a.misc + kStatus, st);
   if (e != cudaSuccess) return e;
-  if (a.n_total > 0 && a.sort_cells) {
-    int bits = 1;
-    while (bits < 31 && ((int64_t)1 << bits) <= a.cap_cells) ++bits;
-    e = radix_sort_index(a.n_total, bits, a.key, a.slot, a.rk, a.perm, a.rv, a.hist, a.misc + kStatus, st);
-    if (e != cudaSuccess) return e;
-  }
+  cell_bounds(a.n_total, a.rk, 0, a.cap_cells, a.num_sms, a.misc, a.cell_start, st);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cell_bounds(int64_t n, const uint64_t* keys, int shift, int64_t cap_cells, int num_sms,
+                               const int32_t* misc, int32_t* cell_start, cudaStream_t st) {
+  cell_bounds(n, keys, shift, cap_cells, num_sms, misc, cell_start, st);
   return cudaGetLastError();
 }
 

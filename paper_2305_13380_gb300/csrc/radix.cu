@@ -267,10 +267,10 @@ static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_o
   return cudaGetLastError();
 }
 
-cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* tmp_a, int32_t* tmp_b,
+cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* keys_out, int32_t* keys_tmp,
                              int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
                              cudaStream_t st) {
-  return radix_sort_impl<int32_t>(n, bits, keys, tmp_a, tmp_b, false, vals_out, vals_tmp, scratch, status, st);
+  return radix_sort_impl<int32_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, status, st);
 }
 
 cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,

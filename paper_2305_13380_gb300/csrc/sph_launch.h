@@ -19,7 +19,7 @@ namespace sphh {
 struct BuildArgs {
   int n_sims;
   int64_t n_total;
-  int64_t cap_cells;  // upper bound of total cells (sizes count / cell_start)
+  int64_t cap_cells;  // upper bound of total cells (sizes cell_start)
   int num_sms;
   double margin;
   const int64_t* sim_offset;
@@ -29,14 +29,17 @@ struct BuildArgs {
   sphk::GridDev* grid;
   int32_t* misc;
   int32_t* hmax_bits;  // per simulation scratch
-  int32_t *key, *slot, *count, *cell_start, *scan_sums, *perm;  // slot: n scratch; scan_sums: scan_words(cells)
-  int32_t *rk, *rv, *hist;  // radix-sort scratch: n, n, radix_words(n, passes)
-  int sort_cells = 1;       // 0: counts and cell_start only (the tree build orders)
+  int32_t *key, *cell_start, *perm;
+  int32_t *slot, *rk, *rv, *hist;  // radix-sort scratch: n, n, n, radix_words(n, passes)
+  int sort_cells = 1;       // 0: cell ids only (the nested-grid build sorts and finds cell_start)
   double radius = 0.0;      // > 0: cells at least this wide, h unused (friends-of-friends)
   int cells_per_particle = 8;  // n_c^3 <= cells_per_particle n + 216 per simulation
   double gamma_k = sphk::kGammaKd;  // H / h of the kernel
 };
 cudaError_t launch_build(const BuildArgs& a, cudaStream_t st);
+// cell_start of every cell from sorted keys whose cell is key >> shift.
+cudaError_t launch_cell_bounds(int64_t n, const uint64_t* keys, int shift, int64_t cap_cells, int num_sms,
+                               const int32_t* misc, int32_t* cell_start, cudaStream_t st);
 
 // Friends-of-friends groups (fof.cu) on a uniform build whose cells are at
 // least the linking length wide: group[p] = smallest index of p's group.
@@ -56,11 +59,11 @@ struct FofArgs {
 cudaError_t launch_fof(const FofArgs& a, cudaStream_t st);
 
 // Stable radix sort of keys (bits significant bits, at most 64) with values
-// 0..n-1 (radix.cu); the sorted values land in vals_out (vals_tmp: n, unless
-// bits <= 8), the 64-bit sort's keys in keys_out.  scratch: radix_words(n,
-// passes of 8 bits).  The keys are left as they are.
+// 0..n-1 (radix.cu): the sorted keys land in keys_out, the values in vals_out
+// (keys_tmp, vals_tmp: n).  scratch: radix_words(n, passes of 8 bits).  The keys
+// are left as they are.
 int64_t radix_words(int64_t n, int passes);
-cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* tmp_a, int32_t* tmp_b,
+cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* keys_out, int32_t* keys_tmp,
                              int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status, cudaStream_t st);
 cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,
                                int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
@@ -299,8 +302,8 @@ cudaError_t launch_sphenix_alpha_v(const SphenixAlphaArgs& a, const sphk::Spheni
 cudaError_t launch_gather_sphenix(int64_t n_total, const int32_t* perm, const float* u, const float* alpha_v,
                                   const float* P, const float* alpha_c, float4* fE, cudaStream_t st);
 
-// Nested-grid build (tree.cu), after launch_build produced the top cells
-// (counts and cell_start; no cell sort).
+// Nested-grid build (tree.cu), after launch_build produced the top cells' grid
+// and ids.
 struct TreeBuildArgs {
   int n_sims;
   int64_t n_total;
@@ -312,7 +315,8 @@ struct TreeBuildArgs {
   const double *x, *y, *z;
   const float* h;
   const int32_t* cell_key;    // top cell of each particle (launch_build's key)
-  const int32_t* cell_start;  // top cells' ranges (valid in source order too)
+  int32_t* cell_start;        // top cells' ranges (written)
+  const int32_t* misc;
   uint64_t *key64, *key64_b;  // n each (scratch)
   uint64_t* skey;             // n: source keys in source order
   int32_t* perm;              // n: source order -> pool index

@@ -22,7 +22,6 @@ namespace {
 // Largest build served by the fixed scratch.
 constexpr int64_t kStaticMaxN = 65536;
 constexpr int64_t kStaticMaxCells = 8 * kStaticMaxN + 216;
-constexpr int64_t kStaticScanSums = kStaticMaxCells / 4096 + 4;  // scan_words
 // radix_words for the three digits of up to kStaticMaxCells cell ids
 constexpr int64_t kStaticHist = 3 * (256 + 1 + 256 * ((kStaticMaxN + 2047) / 2048)) + 64;
 static_assert(kStaticMaxCells < (1 << 24), "cell ids of three digits");
@@ -36,14 +35,12 @@ constexpr int64_t kOffMisc = kOffBox + 64;                                      
 constexpr int64_t kOffHmax = kOffMisc + 64;                                      // int32[1]
 constexpr int64_t kOffKey = kOffHmax + 64;
 constexpr int64_t kOffSlot = kOffKey + align64(kStaticMaxN);
-constexpr int64_t kOffCount = kOffSlot + align64(kStaticMaxN);
-constexpr int64_t kOffSums = kOffCount + align64(kStaticMaxCells + 1);
-constexpr int64_t kOffRk = kOffSums + align64(kStaticScanSums);
+constexpr int64_t kOffRk = kOffSlot + align64(kStaticMaxN);
 constexpr int64_t kOffRv = kOffRk + align64(kStaticMaxN);
 constexpr int64_t kOffHist = kOffRv + align64(kStaticMaxN);
 constexpr int64_t kWords = kOffHist + align64(kStaticHist);
 
-// The scratch.  Every GPU that loads the library holds it (about 3.1 MB)
+// The scratch.  Every GPU that loads the library holds it (about 1.2 MB)
 // until the process exits.
 static __device__ __align__(256) int32_t g_scratch[kWords];
 
@@ -123,9 +120,7 @@ extern "C" int sph_build_cells_static(int64_t n, const double* x, const double* 
   b.hmax_bits = base + kOffHmax;
   b.key = base + kOffKey;
   b.slot = base + kOffSlot;
-  b.count = base + kOffCount;
   b.cell_start = cell_start;
-  b.scan_sums = base + kOffSums;
   b.perm = perm;
   b.rk = base + kOffRk;
   b.rv = base + kOffRv;

@@ -235,12 +235,17 @@ static int blocks_n(int64_t n) {
 cudaError_t launch_tree_build(const TreeBuildArgs& a, cudaStream_t st) {
   const int64_t n = a.n_total;
   cudaError_t e;
-  if (n <= 0) return cudaMemsetAsync(a.n_leaves, 0, sizeof(int32_t), st);
+  if (n <= 0) {
+    e = cudaMemsetAsync(a.n_leaves, 0, sizeof(int32_t), st);
+    return e != cudaSuccess ? e : launch_cell_bounds(0, a.skey, 30, a.cap_cells, a.num_sms, a.misc, a.cell_start, st);
+  }
   int cbits = 1;
   while (cbits < 30 && ((int64_t)1 << cbits) <= a.cap_cells) ++cbits;
   // source order: (top cell, Morton code), ties by pool index
   k_tree_key<<<blocks_n(n), 256, 0, st>>>(n, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.cell_key, a.key64);
   e = radix_sort_index64(n, 30 + cbits, a.key64, a.skey, a.key64_b, a.perm, a.rv, a.hist, a.status, st);
+  if (e != cudaSuccess) return e;
+  e = launch_cell_bounds(n, a.skey, 30, a.cap_cells, a.num_sms, a.misc, a.cell_start, st);
   if (e != cudaSuccess) return e;
   // levels, and target order: by level, ties by source index
   k_tree_level<<<blocks_n(n), 256, 0, st>>>(n, a.skey, a.perm, a.h, a.n_sims, a.grid, a.n_leaf, a.margin, a.gamma_k,
