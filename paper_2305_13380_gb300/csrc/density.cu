@@ -74,8 +74,10 @@ __host__ __device__ constexpr size_t dens_blk_smem() {
                                 sizeof(StageTable) + sizeof(BlockTargets) +
                                 (size_t)dens_cap<K>() * (sizeof(uint16_t) + sizeof(uint8_t));
 }
-constexpr int kOvfCap = 256;  // per-warp staging of the overflow kernel
-constexpr size_t kOvfSmem = (size_t)kWarpsPerBlock * kOvfCap * 2 * sizeof(float4);
+constexpr int kOvfStage = 768;  // most sources of a cell staged at once by the overflow kernel
+constexpr int kOvfCap = 192;  // per-warp staging of the overflow kernel's streams
+static_assert(kWarpsPerBlock * kOvfCap <= kOvfStage, "the streams' buffers fit the staging");
+constexpr size_t kOvfSmem = (size_t)kOvfStage * 2 * sizeof(float4) + sizeof(OvfLists);
 
 struct DensSums {
   float w, dw, mw, mdw, div, cx, cy, cz;
@@ -618,20 +620,18 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
   }
 }
 
-// Blocks whose neighbourhood exceeded the staging buffer: one warp per target
-// cell; each lane owns a target and walks the 27 cells, streamed through a
-// per-warp shared buffer, with positions relative to the target cell.
+// Blocks whose neighbourhood exceeded the staging buffer, a CTA per target cell
+// (stencil.cuh, with what it measured), with positions relative to the target
+// cell.
 template <int K>
 __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs a, PhysDev ph) {
   extern __shared__ float4 osm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float4* spos = osm + warp * (2 * kOvfCap);
-  float4* svel = spos + kOvfCap;
   const int32_t n_items = a.misc_ro[kNumOverflow] * kBlkWarps;
+  const bool spread = n_items <= (int32_t)gridDim.x;
   const NewtonConst nwt = newton_const<K>(ph);
   unsigned long long pair_acc = 0;
-  for (int32_t item = blockIdx.x * kWarpsPerBlock + warp; item < n_items;
-       item += gridDim.x * kWarpsPerBlock) {
+  for (int32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const BlockGeom g = block_geom(a.grid, a.n_sims, a.overflow[item / kBlkWarps]);
     int tx, ty, tz;
     if (!warp_cell(g, item % kBlkWarps, tx, ty, tz)) continue;
@@ -641,6 +641,69 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
     const int32_t ts = a.cell_start[c], te = a.cell_start[c + 1];
     const NbLane nb = neighbour_lane(lane, g.G.cell_base, cx, cy, cz, nc, g.G.cell_f, a.cell_start);
     const int nsrc = warp_sum_int(nb.len);
+    const float hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
+    if (nsrc <= kOvfStage) {
+      float4* spos = osm;
+      float4* svel = osm + kOvfStage;
+      OvfLists& lists = *reinterpret_cast<OvfLists*>(osm + 2 * kOvfStage);
+      __syncthreads();  // the previous cell's sources (or streams) are done with
+      stage_all(nsrc, nb, warp, lane, [&](int slot, int32_t j, float ox, float oy, float oz) {
+        float4 p = a.pos4[j];
+        p.x += ox;
+        p.y += oy;
+        p.z += oz;
+        spos[slot] = p;
+        svel[slot] = a.vel4[j];
+      });
+      const float R2 = g.G.cell_f * g.G.cell_f * (1.0f + 1e-5f);  // any support stays below the cell side
+      for (int32_t t0 = ts; t0 < te; t0 += 32) {
+        const int nt = min(32, te - t0);
+        list_sources(nt, nsrc, R2, spos, lists, warp, lane, [&](int t) { return a.pos4[t0 + t]; });
+        const int t = walk_target(spread, nt, warp, lane);
+        const int32_t ti = t0 + t;
+        if (t >= 0 && (a.act == nullptr || a.act[ti] != 0)) {
+          const uint16_t* mine = lists.entry[t];
+          const int cnt = lists.count[t];
+          const bool all = cnt > kOvfList;
+          const int n = all ? nsrc : cnt;
+          const float4 pi = a.pos4[ti], vi = a.vel4[ti];
+          float h = start_h(a.hs[ti], hcap);
+          float lo = 0.0f, hi = INFINITY;
+          bool done = false, atcap = false, conv = false;
+          int it = 0, passes = 0;
+          while (!done) {
+            const float H = KernT<K>::gamma * h;
+            const float Hinv = 1.0f / H;
+            DensSums s;
+            sums_zero(s);
+#pragma unroll 4
+            for (int e = 0; e < n; ++e) {
+              const int k = all ? e : mine[e];
+              dens_pair<K>(pi, vi, spos[k], svel[k], H, Hinv, s);
+            }
+            passes = it + 1;
+            done = newton_update(s.w, s.dw, nwt, hcap, h, lo, hi, it, atcap, conv);
+          }
+          const float H = KernT<K>::gamma * h;
+          const float Hinv = 1.0f / H;
+          FinSums s;
+          fin_zero(s);
+#pragma unroll 2
+          for (int e = 0; e < n; ++e) {
+            const int k = all ? e : mine[e];
+            fin_pair<K>(pi, vi, spos[k], svel[k], spos[k].w, H, Hinv, s);
+          }
+          fin_scale<K>(s, H);
+          dens_write<K>(a, ph, ti, h, s, vi.w, passes, conv, atcap);
+          pair_acc += (unsigned long long)s.npair;
+        }
+        __syncthreads();  // the lists are done with
+      }
+      continue;
+    }
+    __syncthreads();  // (the streams' buffers lie in the staging)
+    float4* spos = osm + warp * (2 * kOvfCap);
+    float4* svel = spos + kOvfCap;
     auto put = [&](int slot, int32_t j, float ox, float oy, float oz) {
       float4 p = a.pos4[j];
       p.x += ox;
@@ -649,8 +712,7 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
       spos[slot] = p;
       svel[slot] = a.vel4[j];
     };
-    const float hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
-    for (int32_t t0 = ts; t0 < te; t0 += 32) {
+    for (int32_t t0 = ts + 32 * warp; t0 < te; t0 += 32 * kWarpsPerBlock) {
       const int32_t ti = t0 + lane;
       const bool valid = ti < te && (a.act == nullptr || a.act[ti] != 0);
       const float4 pi = valid ? a.pos4[ti] : make_float4(0.f, 0.f, 0.f, 0.f);

@@ -61,10 +61,12 @@ __host__ __device__ constexpr size_t force_blk_smem() {
 }
 static_assert(2 * (force_blk_smem<kFlSphenix, kKernCubic>() + 1024) <= 228 * 1024, "two SPHENIX blocks per SM");
 static_assert(2 * (force_blk_smem<kFlMinimal, kKernQuartic>() + 1024) <= 228 * 1024, "two quartic blocks per SM");
-constexpr int kFOvfCap = 160;
+constexpr int kFOvfStage = 640;  // most sources of a cell staged at once by the overflow kernel
+constexpr int kFOvfCap = 160;  // per-warp staging of the overflow kernel's streams
+static_assert(kWarpsPerBlock * kFOvfCap <= kFOvfStage, "the streams' buffers fit the staging");
 template <int kFl>
 __host__ __device__ constexpr size_t fovf_smem() {
-  return (size_t)kWarpsPerBlock * kFOvfCap * rec_bytes<kFl>();
+  return (size_t)kFOvfStage * rec_bytes<kFl>() + sizeof(OvfLists);
 }
 
 struct ForceSums {
@@ -635,24 +637,76 @@ constexpr size_t kMinSmem = (size_t)kBlkStageCap * (3 * sizeof(float4) + sizeof(
                             (size_t)kBlkStageCap * (sizeof(uint16_t) + sizeof(uint8_t));
 static_assert(kMinBlocks * (kMinSmem + 1024) <= 228 * 1024, "three k_force_min blocks per SM");
 
-// Blocks whose neighbourhood exceeded the staging buffer: one warp per target
-// cell, lane = target, the 27 cells streamed through a per-warp buffer with
-// positions relative to the target cell.
+// Blocks whose neighbourhood exceeded the staging buffer, a CTA per target cell
+// (stencil.cuh), with positions relative to the target cell.
+template <int kFl>
+struct FStage {  // staged records at `base`, room for n
+  float4 *A, *B, *C, *E;
+  float2* D;
+  __device__ FStage(unsigned char* base, int n) {
+    A = reinterpret_cast<float4*>(base);
+    B = A + n;
+    C = B + n;
+    E = C + n;  // not for the Minimal flavour
+    D = reinterpret_cast<float2*>(C + (kFl != kFlMinimal ? 2 : 1) * n);
+  }
+  __device__ void put(const sphh::ForceArgs& a, int slot, int32_t j, float ox, float oy, float oz) {
+    float4 p = a.fA[j];
+    p.x += ox;
+    p.y += oy;
+    p.z += oz;
+    A[slot] = p;
+    B[slot] = a.fB[j];
+    C[slot] = a.fC[j];
+    D[slot] = a.fD[j];
+    if (kFl != kFlMinimal) E[slot] = a.fE[j];
+  }
+};
+
+template <int kFl, int K>
+__device__ __forceinline__ void fovf_pair(const ForceTarget& Tg, const FStage<kFl>& S, int k, bool self,
+                                          const PhysDev& ph, ForceSums& s) {
+  const float4 Aj = S.A[k];
+  const float dx = Tg.A.x - Aj.x, dy = Tg.A.y - Aj.y, dz = Tg.A.z - Aj.z;
+  const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+  const float Hm = reach<kFl>(Tg.A.w, Aj.w);
+  if (r2 < Hm * Hm && !self)
+    force_pair<kFl, K>(Tg, Aj, S.B[k], S.C[k], S.D[k], kFl != kFlMinimal ? S.E[k] : Tg.E, ph, true, s);
+}
+
+template <int kFl>
+__device__ __forceinline__ ForceTarget fovf_target(const sphh::ForceArgs& a, int32_t ti) {
+  ForceTarget Tg;
+  Tg.A = a.fA[ti];
+  Tg.B = a.fB[ti];
+  Tg.C = a.fC[ti];
+  Tg.D = a.fD[ti];
+  Tg.E = kFl != kFlMinimal ? a.fE[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+  finish_target(Tg);
+  return Tg;
+}
+
+template <int kFl>
+__device__ __forceinline__ void fovf_write(const sphh::ForceArgs& a, const SphenixDev& x, float dt, int32_t ti,
+                                           const ForceTarget& Tg, const ForceSums& s) {
+  if (kFl == kFlGradient)
+    gradient_write(a, x, dt, ti, Tg, s);
+  else if (kFl == kFlLimit)
+    limit_write(a, ti, Tg, s);
+  else
+    force_write(a, ti, s);
+}
+
 template <int kFl, int K>
 __global__ void __launch_bounds__(kThreads) k_force_overflow(sphh::ForceArgs a, PhysDev ph, SphenixDev x) {
-  constexpr bool kE = kFl != kFlMinimal;
   extern __shared__ __align__(16) unsigned char fo_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* base = fo_raw + warp * (fovf_smem<kFl>() / kWarpsPerBlock);
-  float4* sA = reinterpret_cast<float4*>(base);
-  float4* sB = sA + kFOvfCap;
-  float4* sC = sB + kFOvfCap;
-  float4* sE = sC + kFOvfCap;  // SPHENIX only
-  float2* sD = reinterpret_cast<float2*>(sC + (kE ? 2 : 1) * kFOvfCap);
   const int32_t n_items = a.misc_ro[kNumOverflow] * kBlkWarps;
+  const bool spread = n_items <= (int32_t)gridDim.x;
   unsigned long long pair_acc = 0;
-  for (int32_t item = blockIdx.x * kWarpsPerBlock + warp; item < n_items;
-       item += gridDim.x * kWarpsPerBlock) {
+  const int32_t first = spread ? (int32_t)blockIdx.x : (int32_t)blockIdx.x * kWarpsPerBlock + warp;
+  const int32_t step = (int32_t)gridDim.x * (spread ? 1 : kWarpsPerBlock);
+  for (int32_t item = first; item < n_items; item += step) {
     const int32_t b = a.overflow[item / kBlkWarps];
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     int tx, ty, tz;
@@ -671,50 +725,56 @@ __global__ void __launch_bounds__(kThreads) k_force_overflow(sphh::ForceArgs a, 
     }
     const int nsrc = __shfl_sync(0xffffffffu, incl, 31);
     const int self_base = __shfl_sync(0xffffffffu, incl - nb.len, 13);
-    auto put = [&](int slot, int32_t j, float ox, float oy, float oz) {
-      float4 p = a.fA[j];
-      p.x += ox;
-      p.y += oy;
-      p.z += oz;
-      sA[slot] = p;
-      sB[slot] = a.fB[j];
-      sC[slot] = a.fC[j];
-      sD[slot] = a.fD[j];
-      if (kE) sE[slot] = a.fE[j];
-    };
-    for (int32_t t0 = ts; t0 < te; t0 += 32) {
+    if (spread) __syncthreads();  // the previous cell's sources are done with
+    if (spread && nsrc <= kFOvfStage) {
+      FStage<kFl> S(fo_raw, kFOvfStage);
+      OvfLists& lists = *reinterpret_cast<OvfLists*>(fo_raw + (size_t)kFOvfStage * rec_bytes<kFl>());
+      stage_all(nsrc, nb, warp, lane,
+                [&](int slot, int32_t j, float ox, float oy, float oz) { S.put(a, slot, j, ox, oy, oz); });
+      const float R2 = g.G.cell_f * g.G.cell_f * (1.0f + 1e-5f);  // any support stays below the cell side
+      for (int32_t t0 = ts; t0 < te; t0 += 32) {
+        const int nt = min(32, te - t0);
+        list_sources(nt, nsrc, R2, S.A, lists, warp, lane, [&](int t) { return a.fA[t0 + t]; });
+        const int t = walk_target(true, nt, warp, lane);
+        const int32_t ti = t0 + t;
+        if (t >= 0 && (a.act == nullptr || a.act[ti] != 0)) {
+          const uint16_t* mine = lists.entry[t];
+          const int cnt = lists.count[t];
+          const bool all = cnt > kOvfList;
+          const int n = all ? nsrc : cnt, me = self_base + (ti - ts);
+          const ForceTarget Tg = fovf_target<kFl>(a, ti);
+          ForceSums s;
+          fsums_zero(s);
+          if (kFl == kFlGradient) s.ay = Tg.E.y;
+#pragma unroll 2
+          for (int e = 0; e < n; ++e) {
+            const int k = all ? e : mine[e];
+            fovf_pair<kFl, K>(Tg, S, k, k == me, ph, s);
+          }
+          fovf_write<kFl>(a, x, dt, ti, Tg, s);
+          pair_acc += (unsigned long long)s.npair;
+        }
+        __syncthreads();  // the lists are done with
+      }
+      continue;
+    }
+    FStage<kFl> S(fo_raw + (size_t)warp * kFOvfCap * rec_bytes<kFl>(), kFOvfCap);
+    for (int32_t t0 = ts + (spread ? 32 * warp : 0); t0 < te; t0 += spread ? 32 * kWarpsPerBlock : 32) {
       const int32_t ti = t0 + lane;
       const bool valid = ti < te && (a.act == nullptr || a.act[ti] != 0);
-      const int32_t tl = valid ? ti : ts;
-      ForceTarget Tg;
-      Tg.A = a.fA[tl];
-      Tg.B = a.fB[tl];
-      Tg.C = a.fC[tl];
-      Tg.D = a.fD[tl];
-      Tg.E = kE ? a.fE[tl] : make_float4(0.f, 0.f, 0.f, 0.f);
-      finish_target(Tg);
+      const ForceTarget Tg = fovf_target<kFl>(a, valid ? ti : ts);
       ForceSums s;
       fsums_zero(s);
       if (kFl == kFlGradient) s.ay = Tg.E.y;
       for (int v0 = 0; v0 < nsrc; v0 += kFOvfCap) {
-        const int cnt = stage_sources(v0, kFOvfCap, nb, lane, put);
-        for (int k = 0; k < cnt; ++k) {
-          const float4 Aj = sA[k];
-          const float dx = Tg.A.x - Aj.x, dy = Tg.A.y - Aj.y, dz = Tg.A.z - Aj.z;
-          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          const float Hm = reach<kFl>(Tg.A.w, Aj.w);
-          const bool self = (v0 + k == self_base + (ti - ts));
-          if (r2 < Hm * Hm && !self) force_pair<kFl, K>(Tg, Aj, sB[k], sC[k], sD[k], kE ? sE[k] : Tg.E, ph, true, s);
-        }
+        const int cnt = stage_sources(v0, kFOvfCap, nb, lane, [&](int slot, int32_t j, float ox, float oy, float oz) {
+          S.put(a, slot, j, ox, oy, oz);
+        });
+        for (int k = 0; k < cnt; ++k) fovf_pair<kFl, K>(Tg, S, k, v0 + k == self_base + (ti - ts), ph, s);
         __syncwarp();
       }
       if (valid) {
-        if (kFl == kFlGradient)
-          gradient_write(a, x, dt, ti, Tg, s);
-        else if (kFl == kFlLimit)
-          limit_write(a, ti, Tg, s);
-        else
-          force_write(a, ti, s);
+        fovf_write<kFl>(a, x, dt, ti, Tg, s);
         pair_acc += (unsigned long long)s.npair;
       }
     }

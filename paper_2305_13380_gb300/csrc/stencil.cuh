@@ -68,4 +68,72 @@ __device__ __forceinline__ int stage_sources(int v0, int cap, const NbLane& nb, 
   return min(cum, v0 + cap) - v0;
 }
 
+// ---- cells of blocks that do not fit the loops' staging (overflow kernels) ----
+//
+// A CTA of kWarpsPerBlock warps per target cell.  The sources of the 27 cells
+// (up to 768 for the density, 640 for the force) are staged once for all its
+// targets; the warps list for each target the staged sources within the search
+// radius (a ballot per target and 32 sources, so in the sources' order), and one
+// lane per target walks its list in that order.  A source beyond the radius adds
+// exactly zero to every sum, so the sums are those of a walk of every source,
+// bit for bit.  More sources than fit are streamed through a buffer per warp,
+// 32 targets at a time.
+//
+// The walks are serial and bound by latency.  Up to one cell per resident CTA
+// ("spread") the targets are dealt to the CTA's warps.  With more cells than
+// that, issue slots count: the density's lists are walked by one warp, and the
+// force, which has one pass over the sources and no more, goes back to a warp
+// per cell that streams.  A warp per cell streaming throughout took, density +
+// force, 94 + 71 us in a step of 4096 particles (19 per cell, just past the
+// blocks' staging; few cells), this 33 + 29; in a pool of 64 lattice boxes (more
+// cells than CTAs) 304 + 151 us, this 190 + 170 (the force lists walked by one
+// warp: 208; spread there, too: 262 + 295).
+constexpr int kOvfList = 128;   // list entries per target; longer: the target walks every staged source
+struct OvfLists {
+  uint16_t entry[32][kOvfList];
+  int count[32];
+};
+
+// Stages all nsrc sources (each warp a part) through put(slot, j,
+// ox, oy, oz).  CTA-collective, ends with a barrier.
+template <class Put>
+__device__ __forceinline__ void stage_all(int nsrc, const NbLane& nb, int warp, int lane, Put put) {
+  const int part = (nsrc + kWarpsPerBlock - 1) / kWarpsPerBlock, v0 = warp * part;
+  if (v0 < nsrc)
+    stage_sources(v0, part, nb, lane, [&](int slot, int32_t j, float ox, float oy, float oz) { put(v0 + slot, j, ox, oy, oz); });
+  __syncthreads();
+}
+
+// Lists of nt <= 32 targets (positions pos(t), staged positions src[k] as x, y,
+// z): the staged slots with r^2 < R2, and their counts.  CTA-collective, ends with
+// a barrier.
+template <class Pos>
+__device__ __forceinline__ void list_sources(int nt, int nsrc, float R2, const float4* src, OvfLists& lists, int warp,
+                                             int lane, Pos pos) {
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll 1
+  for (int t = warp; t < nt; t += kWarpsPerBlock) {
+    const float4 p = pos(t);
+    int cnt = 0;
+#pragma unroll 1
+    for (int v = 0; v < nsrc; v += 32) {
+      const float4 q = src[min(v + lane, nsrc - 1)];
+      const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
+      const bool in = v + lane < nsrc && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < R2;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      const int at = cnt + __popc(m & lt);
+      if (in && at < kOvfList) lists.entry[t][at] = (uint16_t)(v + lane);
+      cnt += __popc(m);
+    }
+    if (lane == 0) lists.count[t] = cnt;
+  }
+  __syncthreads();
+}
+
+// The target of a lane's walk, or -1.
+__device__ __forceinline__ int walk_target(bool spread, int nt, int warp, int lane) {
+  const int t = spread ? lane * kWarpsPerBlock + warp : (warp == 0 ? lane : 32);
+  return t < nt ? t : -1;
+}
+
 }  // namespace sphk
