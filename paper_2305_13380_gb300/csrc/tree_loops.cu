@@ -41,7 +41,7 @@
 namespace sphk {
 
 constexpr int kTWarps = 4;             // warps per CTA
-constexpr int kTCap = 384;             // staged sources per warp and chunk (per-target kernel)
+constexpr int kTCap = 320;             // staged sources per warp and chunk (per-target kernel)
 constexpr int kTPer = 32 / kTreeTpp;   // targets per round
 constexpr int kTChildren = 27 * 8;     // children of the 27 neighbour cells
 
@@ -55,6 +55,9 @@ struct TTab {
 struct TPrune : TTab {
   int32_t hoff[kTChildren + 4];  // offsets of the target's hit children, + total
   uint8_t hch[kTChildren];       // the hit children, in order
+  // ... and their sources: item u's index is x + u, its position relative to the
+  // target's cell its fine integer position plus (y, z, w)
+  alignas(16) int4 src[kTChildren];
 };
 constexpr size_t kTPruneBytes = (sizeof(TPrune) + 15) / 16 * 16;
 constexpr size_t kTFbWarpSmem = (size_t)kTCap * (sizeof(float4) + sizeof(uint32_t)) + kTPruneBytes;
@@ -364,7 +367,8 @@ __device__ __forceinline__ float child_dist2(int ch, float side, float cside, co
 // lane sub of each eight tests child sub of the 27 cells; the hit children are
 // compacted in child order with the offsets of their sources.  Returns their
 // number and their sources.  Called by the whole warp.
-__device__ __noinline__ int2 prune_round(int lane, float3 pi, float Rb2, float side, float cside, TPrune* pr) {
+__device__ __noinline__ int2 prune_round(int lane, float3 pi, float Rb2, const TGeo& g, float cside, TPrune* pr) {
+  const float side = g.side;
   uint32_t mine = 0;
   const int sub = lane % kTreeTpp;
 #pragma unroll 1
@@ -397,7 +401,13 @@ __device__ __noinline__ int2 prune_round(int lane, float3 pi, float Rb2, float s
       const int w = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += w;
     }
-    if (k < nh) pr->hoff[k] = run + incl - v;
+    if (k < nh) {
+      const int off = run + incl - v, ch = pr->hch[k], r = ch >> 3, sc = pr->rsc[r];
+      const int sx = (sc & 3) - 1, sy = ((sc >> 2) & 3) - 1, sz = ((sc >> 4) & 3) - 1;
+      pr->hoff[k] = off;
+      pr->src[k] = make_int4(pr->rlo[r] + (pr->cv[ch] - pr->rcum[r]) - off, sx * g.nfine - g.ox, sy * g.nfine - g.oy,
+                             sz * g.nfine - g.oz);
+    }
     run += __shfl_sync(0xffffffffu, incl, 31);
   }
   if (lane == 0) pr->hoff[nh] = run;
@@ -485,67 +495,88 @@ __device__ __noinline__ int2 prune_round_fast(bool valid, int sub, int lane, flo
   return out;
 }
 
-// Stages cnt sources into spos / sidx [0, cnt) relative to the group corner (w:
-// the mass); item u is source map(u) (its index and shift code).  A lane takes
-// its items four at a time and issues their loads together, so that four L2
-// latencies overlap instead of running one after another.  Called by the whole
-// warp.
-template <class Map>
-__device__ __forceinline__ void tstage_items(int cnt, int lane, const TGeo& g, const float4* __restrict__ rel,
-                                             const int4* __restrict__ fine, float4* spos, uint32_t* sidx, Map map) {
-  for (int u0 = lane; u0 < cnt; u0 += 4 * 32) {
-    int32_t j[4];
-    int sc[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      j[i] = 0;
-      sc[i] = kNoShift;
-      if (u0 + 32 * i < cnt) map(u0 + 32 * i, j[i], sc[i]);
-    }
+// The hit child (position in the tables) of item u0 + lane of a target's hit
+// children; ci: the last child of the rows before, moved on.  The next 32
+// children's starts mark their bits of the row, a lane's child is the count of
+// the marks up to it: a search per item took most of the instructions of an
+// item.  Called by all 32 lanes.
+__device__ __forceinline__ int row_child(int u0, int nh, const TPrune* pr, int lane, int& ci) {
+  const int k = ci + 1 + lane;
+  const int d = k < nh ? pr->hoff[k] - u0 : 32;
+  const unsigned marks = __reduce_or_sync(0xffffffffu, d < 32 ? 1u << d : 0u);
+  const int c = ci + __popc(marks & (0xffffffffu >> (31 - lane)));
+  ci += __popc(marks);
+  return c;
+}
+__device__ __forceinline__ int child_shift(const TPrune* pr, int c) { return pr->rsc[pr->hch[c] >> 3]; }
+__device__ __forceinline__ float3 item_pos(const TGeo& g, const float4& rel, const int4& fine, const int4& src) {
+  return make_float3(fmaf((float)(fine.x + src.y), g.s_fine, rel.x), fmaf((float)(fine.y + src.z), g.s_fine, rel.y),
+                     fmaf((float)(fine.z + src.w), g.s_fine, rel.z));
+}
+
+// Stages items [u0, u0 + kTCap) of the target's hit children relative to its
+// cell; ci as for row_child.  Called by the whole warp.
+__device__ __noinline__ int tstage_union(int u0, int total, int nh, const TPrune* pr, int lane, const TGeo& g,
+                                         const float4* __restrict__ rel, const int4* __restrict__ fine, float4* spos,
+                                         uint32_t* sidx, int& ci) {
+  const int cnt = min(kTCap, total - u0);
+#pragma unroll 1
+  for (int v0 = 0; v0 < cnt; v0 += 4 * 32) {
     float4 rj[4];
-    int4 fj[4];
+    int4 fj[4], sj[4];
+    uint32_t je[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      rj[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      fj[i] = make_int4(0, 0, 0, 0);
-      if (u0 + 32 * i < cnt) {
-        rj[i] = rel[j[i]];
-        fj[i] = fine[j[i]];
-      }
+      const int v = v0 + 32 * i;
+      const int c = row_child(u0 + v, v < cnt ? nh : 0, pr, lane, ci);
+      sj[i] = pr->src[c];
+      const int32_t j = sj[i].x + u0 + min(v + lane, cnt - 1);
+      je[i] = pack_js(j, child_shift(pr, c));
+      rj[i] = rel[j];
+      fj[i] = fine[j];
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int u = u0 + 32 * i;
-      if (u < cnt) {
-        const float3 p = rel_to(g, rj[i], fj[i], sc[i]);
-        spos[u] = make_float4(p.x, p.y, p.z, rj[i].w);
-        sidx[u] = pack_js(j[i], sc[i]);
+      const int v = v0 + 32 * i + lane;
+      if (v < cnt) {
+        const float3 p = item_pos(g, rj[i], fj[i], sj[i]);
+        spos[v] = make_float4(p.x, p.y, p.z, rj[i].w);
+        sidx[v] = je[i];
       }
     }
   }
   __syncwarp();
+  return cnt;
 }
 
-// Stages sources [u0, u0 + kTCap) of the round's hit children (flattened)
-// relative to the group corner.  Called by the whole warp.
-__device__ __noinline__ int tstage_union(int u0, int total, int nh, const TPrune* pr, int lane,
-                                            const TGeo& g, const float4* __restrict__ rel,
-                                            const int4* __restrict__ fine, float4* spos, uint32_t* sidx) {
-  const int cnt = min(kTCap, total - u0);
-  tstage_items(cnt, lane, g, rel, fine, spos, sidx, [&](int u, int32_t& j, int& sc) {
-    const int uu = u0 + u;
-    int lo = 0, hi = nh - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (pr->hoff[mid] <= uu) lo = mid; else hi = mid - 1;
+// Newton sums of a target at pi over all items, item u by lane u % 32, straight
+// from memory: eight items' loads in flight per lane.
+template <int K>
+__device__ __noinline__ float2 tnewton_stream(int total, int nh, const TPrune* pr, int lane, const TGeo& g, float3 pi,
+                                              float H, float Hinv, const float4* __restrict__ rel,
+                                              const int4* __restrict__ fine) {
+  constexpr int kB = 8;
+  float Sw = 0.f, Sdw = 0.f;
+  int ci = 0;
+#pragma unroll 1
+  for (int u0 = 0; u0 < total; u0 += kB * 32) {
+    float4 rj[kB];
+    int4 fj[kB], sj[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      sj[i] = pr->src[row_child(u0 + 32 * i, nh, pr, lane, ci)];
+      const int32_t j = sj[i].x + min(u0 + 32 * i + lane, total - 1);
+      rj[i] = rel[j];
+      fj[i] = fine[j];
     }
-    const int ch = pr->hch[lo];
-    const int vv = pr->cv[ch] + (uu - pr->hoff[lo]);
-    const int r = ch >> 3;
-    j = pr->rlo[r] + (vv - pr->rcum[r]);
-    sc = pr->rsc[r];
-  });
-  return cnt;
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const float3 p = item_pos(g, rj[i], fj[i], sj[i]);
+      if (u0 + 32 * i + lane < total)
+        tnewton_pair<K>(r2_of(pi, make_float4(p.x, p.y, p.z, 0.f)), H, Hinv, Sw, Sdw);
+    }
+  }
+  return make_float2(Sw, Sdw);
 }
 
 // Reverse pair of target ti (support H, leaf side s_i) and source j (shift
@@ -564,6 +595,43 @@ __device__ __forceinline__ bool want_reverse(const sphh::TreeDensityArgs& a, int
   return want_reverse_t(__int_as_float(a.fine[j].w), ti, j, r2, H2, H, s_i);
 }
 
+__device__ __forceinline__ uint64_t reverse_rec(int32_t j, int32_t ti, int sc) {
+  return ((uint64_t)(uint32_t)j << 32) | pack_js(ti, mirror_s(sc));
+}
+
+// Writes record k of the reverse pairs and counts it at its receiver.
+__device__ __forceinline__ void emit_at(const sphh::TreeDensityArgs& a, unsigned long long k, uint64_t rec) {
+  if (k < (unsigned long long)a.rev_cap) {
+    a.rev_raw[k] = rec;
+    atomicAdd(&a.rev_start[(int32_t)(rec >> 32)], 1);
+  } else {
+    atomicOr(a.status, SPH_ST_CAPACITY);
+  }
+}
+
+// Appends the reverse pairs of target ti with the marked ones of a lane's four
+// sources: one counter atomic, a wait of about a microsecond, per 128 sources.
+// Called by all 32 lanes.
+__device__ __forceinline__ void emit_marked(const sphh::TreeDensityArgs& a, unsigned want, const uint32_t (&je)[4],
+                                            int32_t ti, int lane) {
+  const int mine = __popc(want);
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  const int all = __shfl_sync(0xffffffffu, incl, 31);
+  if (all == 0) return;
+  unsigned long long base = 0;
+  if (lane == 0) base = atomicAdd(a.rev_count, (unsigned long long)all);
+  unsigned long long k = __shfl_sync(0xffffffffu, base, 0) + (unsigned long long)(incl - mine);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if ((want >> i) & 1u) emit_at(a, k++, reverse_rec(unpack_j(je[i]), ti, unpack_s(je[i])));
+  }
+}
+
 // Appends the wanted records of the warp (one counter atomic per warp).
 // Called by all 32 lanes.
 __device__ __forceinline__ void emit_warp(const sphh::TreeDensityArgs& a, bool want, uint64_t rec, int lane) {
@@ -573,18 +641,8 @@ __device__ __forceinline__ void emit_warp(const sphh::TreeDensityArgs& a, bool w
   if (lane == 0) base = atomicAdd(a.rev_count, (unsigned long long)__popc(em));
   base = __shfl_sync(0xffffffffu, base, 0);
   if (want) {
-    const unsigned long long k = base + (unsigned long long)__popc(em & ((1u << lane) - 1u));
-    if (k < (unsigned long long)a.rev_cap) {
-      a.rev_raw[k] = rec;
-      atomicAdd(&a.rev_start[(int32_t)(rec >> 32)], 1);
-    } else {
-      atomicOr(a.status, SPH_ST_CAPACITY);
-    }
+    emit_at(a, base + (unsigned long long)__popc(em & ((1u << lane) - 1u)), rec);
   }
-}
-
-__device__ __forceinline__ uint64_t reverse_rec(int32_t j, int32_t ti, int sc) {
-  return ((uint64_t)(uint32_t)j << 32) | pack_js(ti, mirror_s(sc));
 }
 
 // Appends the list entries marked in each lane's mask wm (bit e: entry e of
@@ -1404,6 +1462,16 @@ __device__ __forceinline__ TRanges cell_ranges(const GridDev& G, const TreeLeaf&
   return R;
 }
 
+// The targets that left their round, a warp each: mostly low-density targets
+// beside a dense core, whose 27 cells hold thousands of sources.  There are few
+// of them (4040 of 690k particles in a pool of 48 boxes), so the kernel lasts
+// about as long as its largest target: what counts is the latency of a row of 32
+// sources.  With a search per source, four loads in flight and a counter atomic
+// per row of reverse pairs the largest of 1594 targets of 300k particles (10,000
+// sources, Wendland C2) took 550 us of the loop; row_child, loads of eight rows
+// (four with the velocities) and an atomic per four rows: 220 (the pool's 356 ->
+// 203).  Keeping the sources in reach in shared memory costs another 85 us: most
+// of these targets have more of them than fit.
 template <int K>
 __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
@@ -1443,10 +1511,11 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
       prune_tables(a.skey, Rr, Lp.depth, lane, pr);
       const float cs = Lp.depth < kTreeDepth ? 0.5f * gp.side : gp.side;
       const float H2 = H * H;
-      const int2 hp2 = prune_round(lane, pp, H2 * (1.0f + 0x1p-10f), gp.side, cs, pr);
+      const int2 hp2 = prune_round(lane, pp, H2 * (1.0f + 0x1p-10f), gp, cs, pr);
       const int nhp = hp2.x, tot = hp2.y;
+      int ci = 0;
       for (int v0 = 0; v0 < tot; v0 += kTCap) {
-        const int c = tstage_union(v0, tot, nhp, pr, lane, gp, a.rel, a.fine, spos, sidx);
+        const int c = tstage_union(v0, tot, nhp, pr, lane, gp, a.rel, a.fine, spos, sidx, ci);
         for (int k0 = 0; k0 < c; k0 += 32) {
           const int k = k0 + lane;
           bool want = false;
@@ -1488,18 +1557,20 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
     int nh = 0, total = 0;
     float Rp = 0.0f, cside = 0.0f;
     // the sources: the children of the 27 cells whose box lies within the
-    // selection radius Rp (with a margin far above the rounding of r), staged
-    // in chunks; Rp = min(cell side, 1.25 H) leaves room for the support to
-    // grow, and a support beyond it selects again (H is warp-uniform)
-#define TREE_FB_SELECT(Hsup)                                                                                   \
-  if ((Hsup) > Rp) {                                                                                           \
-    Rp = fminf(g.side, 1.25f * (Hsup));                                                                        \
-    const int2 hit = prune_round(lane, pi, Rp * Rp * (1.0f + 0x1p-10f), g.side, cside, pr);                     \
-    nh = hit.x;                                                                                                \
-    total = hit.y;                                                                                             \
-    one_chunk = total <= kTCap;                                                                                \
-    if (one_chunk) tstage_union(0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx);                         \
-  }
+    // selection radius Rp (with a margin far above the rounding of r); Rp =
+    // min(cell side, 1.25 H) leaves room for the support to grow, and a support
+    // beyond it selects again (H is warp-uniform).  Up to kTCap of them are
+    // staged for the Newton passes, more are read again by each pass
+    auto select = [&](float Hsup) {
+      if (!(Hsup > Rp)) return;
+      Rp = fminf(g.side, 1.25f * Hsup);
+      const int2 hit = prune_round(lane, pi, Rp * Rp * (1.0f + 0x1p-10f), g, cside, pr);
+      nh = hit.x;
+      total = hit.y;
+      one_chunk = total <= kTCap;
+      int ci = 0;
+      if (one_chunk) tstage_union(0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx, ci);
+    };
     for (; d >= 0; --d) {
       const TreeLeaf Lc = cell_at_depth(key, d);
       g = leaf_geo(Lc, G);
@@ -1515,13 +1586,15 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
       bool done = false;
       while (!done) {  // warp-uniform: every lane holds the same reduced sums
         const float H = KernT<K>::gamma * h;
-        TREE_FB_SELECT(H)
+        select(H);
         const float Hinv = 1.0f / H;
         float Sw = 0.f, Sdw = 0.f;
-        for (int v0 = 0; v0 < total; v0 += kTCap) {
-          const int c = one_chunk ? total : tstage_union(v0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx);
-          for (int k = lane; k < c; k += 32) tnewton_pair<K>(r2_of(pi, spos[k]), H, Hinv, Sw, Sdw);
-          if (!one_chunk) __syncwarp();
+        if (one_chunk) {
+          for (int k = lane; k < total; k += 32) tnewton_pair<K>(r2_of(pi, spos[k]), H, Hinv, Sw, Sdw);
+        } else {
+          const float2 S = tnewton_stream<K>(total, nh, pr, lane, g, pi, H, Hinv, a.rel, a.fine);
+          Sw = S.x;
+          Sdw = S.y;
         }
         Sw = wsum(Sw);
         Sdw = wsum(Sdw);
@@ -1537,33 +1610,39 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
     }
     // final pass at h, reverse pairs of this target
     const float H = KernT<K>::gamma * h;
-    TREE_FB_SELECT(H)
-#undef TREE_FB_SELECT
+    select(H);
     const float Hinv = 1.0f / H;
     const float H2 = H * H;
     TDSums s;
     tds_zero(s);
-    for (int v0 = 0; v0 < total; v0 += kTCap) {
-      const int c = one_chunk ? total : tstage_union(v0, total, nh, pr, lane, g, a.rel, a.fine, spos, sidx);
-      for (int k0 = 0; k0 < c; k0 += 32) {
-        const int k = k0 + lane;
-        bool want = false;
-        uint64_t rec = 0;
-        if (k < c) {
-          const float4 pj = spos[k];
-          const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          if (r2 < H2) {
-            const uint32_t je = sidx[k];
-            const int32_t j = unpack_j(je);
-            tdens_pair<K>(dx, dy, dz, vi, a.vel4[j], pj.w, H, Hinv, s);
-            want = want_reverse(a, ti, j, r2, H2, H, g.side);
-            rec = reverse_rec(j, ti, unpack_s(je));
-          }
-        }
-        emit_warp(a, want, rec, lane);
+    int ci = 0;
+#pragma unroll 1
+    for (int u0 = 0; u0 < total; u0 += 4 * 32) {
+      float4 rj[4], vj[4];
+      int4 fj[4], sj[4];
+      uint32_t je[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = row_child(u0 + 32 * i, nh, pr, lane, ci);
+        sj[i] = pr->src[c];
+        const int32_t j = sj[i].x + min(u0 + 32 * i + lane, total - 1);
+        je[i] = pack_js(j, child_shift(pr, c));
+        rj[i] = a.rel[j];
+        fj[i] = a.fine[j];
+        vj[i] = a.vel4[j];
       }
-      if (!one_chunk) __syncwarp();
+      unsigned want = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float3 pj = item_pos(g, rj[i], fj[i], sj[i]);
+        const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        if (u0 + 32 * i + lane < total && r2 < H2) {
+          tdens_pair<K>(dx, dy, dz, vi, vj[i], rj[i].w, H, Hinv, s);
+          if (want_reverse_t(__int_as_float(fj[i].w), ti, unpack_j(je[i]), r2, H2, H, g.side)) want |= 1u << i;
+        }
+      }
+      emit_marked(a, want, je, ti, lane);
     }
     s.w = wsum(s.w);
     s.dw = wsum(s.dw);
@@ -1585,9 +1664,19 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
   if (ph.count_pairs && lane == 0 && pair_acc) atomicAdd(a.pairs, pair_acc);
 }
 
+// The force on the targets of k_tree_density_fb, a warp each, and as there bound
+// by the latency of the largest.  The reach's sources are tested 128 at a time,
+// and those in reach gathered into full warps of pairs.  Against a walk child by
+// child with the ranges searched one after another: 229 -> 145 us in the pool of
+// 48 boxes, 189 -> 109 us for 300k particles with Wendland C2.  A CTA per target
+// (the set-up by one warp) took 183 and 105.
 template <int kFl, int K>
 __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceArgs a, PhysDev ph, SphenixDev x) {
+  __shared__ TPrune prune[kTWarps];
+  __shared__ uint32_t rings[kTWarps][64];
   const int lane = threadIdx.x & 31;
+  TPrune* pr = &prune[threadIdx.x >> 5];
+  uint32_t* ring = rings[threadIdx.x >> 5];
   const int32_t nq = min(*a.fb_count, (int32_t)a.n_total);
   unsigned long long pair_acc = 0;
   for (int32_t q = next_group(a.fb_work, lane); q < nq; q = next_group(a.fb_work, lane)) {
@@ -1617,52 +1706,76 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceA
     s.ax = s.ay = s.az = s.du = s.vsig = 0.f;
     s.npair = 0;
     if (kFl == kTGradient) s.ay = ei.y;
-    const float cside = Lc.depth < kTreeDepth ? 0.5f * g.side : g.side;
-    const float Cb2 = C2 * (1.0f + 0x1p-10f);
-    for (int r = 0; r < 27; ++r) {
-      const TreeRange Rg = neighbour_range(G, Lc, r, a.skey, a.cell_start);
-      if (Rg.hi <= Rg.lo) continue;
-      // the range's 8 children (contiguous in Morton order; a cell of the
-      // deepest level is its own single child): lane c < 8 finds child c's
-      // start and tests its box against the reach (with a margin far above
-      // the rounding of r)
-      int32_t c0 = Rg.lo;
-      if (Lc.depth < kTreeDepth && lane > 0 && lane < 8) {
-        const int sh = 3 * (kTreeDepth - Lc.depth - 1);
-        const uint64_t base = (a.skey[Rg.lo] >> (sh + 3)) << (sh + 3);
-        c0 = (int32_t)lower_bound64(a.skey, Rg.lo, Rg.hi, base + ((uint64_t)lane << sh));
-      }
-      if (Lc.depth >= kTreeDepth && lane > 0) c0 = Rg.hi;
-      const int32_t nx = __shfl_down_sync(0xffffffffu, c0, 1);  // every lane takes part
-      const int32_t c1 = lane < 7 ? nx : Rg.hi;
-      const bool hit = lane < 8 && c1 > c0 && child_dist2(r * 8 + lane, g.side, cside, pi) < Cb2;
-      unsigned hm = __ballot_sync(0xffffffffu, hit);
-      while (hm) {
-        const int ch = __ffs((int)hm) - 1;
-        hm &= hm - 1u;
-        const int32_t lo = __shfl_sync(0xffffffffu, c0, ch), hi = __shfl_sync(0xffffffffu, c1, ch);
-        for (int32_t j = lo + lane; j < hi; j += 32) {
-          if (j == ti) continue;
-          const TRec hj = trec_head(a.rec, j);
-          const float3 pj = rec_rel_to(g, hj, Rg.shift);
-          const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-          if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < C2)
-            tforce_rec<kFl, K>(dx, dy, dz, vi, ci, ei, Hi, di.y, di.x, a, j, hj, ph, s);
-        }
-      }
-    }
-    if (kFl != kTGradient) {
-      const int32_t r0 = a.rev_start[ti], r1 = a.rev_start[ti + 1];
-      for (int32_t k = r0 + lane; k < r1; k += 32) {
-        const uint32_t je = a.rev[k];
+    // the pairs in reach wait in a ring until there is one for every lane
+    int head = 0, np = 0;
+    auto walk = [&](int cnt) {
+      if (lane < cnt) {
+        const uint32_t je = ring[(head + lane) & 63];
         const int32_t j = unpack_j(je);
         const TRec hj = trec_head(a.rec, j);
         const float3 pj = rec_rel_to(g, hj, unpack_s(je));
+        tforce_rec<kFl, K>(pi.x - pj.x, pi.y - pj.y, pi.z - pj.z, vi, ci, ei, Hi, di.y, di.x, a, j, hj, ph, s);
+      }
+    };
+    auto push = [&](bool in, uint32_t je) {
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) ring[(head + np + __popc(m & ((1u << lane) - 1u))) & 63] = je;
+      np += __popc(m);
+      __syncwarp();
+      if (np >= 32) {
+        walk(32);
+        head += 32;
+        np -= 32;
+        __syncwarp();
+      }
+    };
+    const float cside = Lc.depth < kTreeDepth ? 0.5f * g.side : g.side;
+    const TRanges R = cell_ranges(G, Lc, a.skey, a.cell_start, lane);
+    prune_tables(a.skey, R, Lc.depth, lane, pr);
+    // (a margin far above the rounding of r)
+    const int2 hit = prune_round(lane, pi, C2 * (1.0f + 0x1p-10f), g, cside, pr);
+    int at = 0;
+#pragma unroll 1
+    for (int u0 = 0; u0 < hit.y; u0 += 4 * 32) {
+      uint32_t je[4];
+      bool in[4];
+      int4 sj[4];
+      TRec hj[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int c = row_child(u0 + 32 * i, hit.x, pr, lane, at);
+        sj[i] = pr->src[c];
+        const int32_t j = sj[i].x + min(u0 + 32 * i + lane, hit.y - 1);
+        je[i] = pack_js(j, child_shift(pr, c));
+        hj[i] = trec_head(a.rec, j);
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float3 pj = item_pos(g, hj[i].q0, hj[i].q1, sj[i]);
         const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-        if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= C2)
-          tforce_rec<kFl, K>(dx, dy, dz, vi, ci, ei, Hi, di.y, di.x, a, j, hj, ph, s);
+        in[i] = u0 + 32 * i + lane < hit.y && unpack_j(je[i]) != ti && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < C2;
+      }
+#pragma unroll 1
+      for (int i = 0; i < 4; ++i) push(i == 0 ? in[0] : i == 1 ? in[1] : i == 2 ? in[2] : in[3],
+                                       i == 0 ? je[0] : i == 1 ? je[1] : i == 2 ? je[2] : je[3]);
+    }
+    if (kFl != kTGradient) {
+      const int32_t r0 = a.rev_start[ti], r1 = a.rev_start[ti + 1];
+#pragma unroll 1
+      for (int32_t k0 = r0; k0 < r1; k0 += 32) {
+        bool in = false;
+        uint32_t je = 0;
+        if (k0 + lane < r1) {
+          je = a.rev[k0 + lane];
+          const float3 pj = rec_rel_to(g, trec_head(a.rec, unpack_j(je)), unpack_s(je));
+          const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
+          in = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= C2;
+        }
+        push(in, je);
       }
     }
+    walk(np);
+    __syncwarp();
     s.ax = wsum(s.ax);
     if (kFl == kTGradient) {
 #pragma unroll
