@@ -4,19 +4,21 @@
 // counting sort of the cell grid (Sec. 2.1), for any cell size.
 //
 //   k_radix_hist  the digit counts of every pass, from one read of the keys
-//   k_radix_pass  one 8-bit digit: a tile of 2048 items ranks its keys (warp
-//                 match + running per-warp counts), finds by look-back how many
-//                 equal digits the tiles before it hold (lookback.cuh, a word
-//                 per tile and digit), and scatters.  A pass whose keys all
-//                 share the digit (the bits beyond the cells in use) only
+//   k_radix_pass  one 8-bit digit: a tile of 2048 items ranks its keys (equal
+//                 digits within a warp + running per-warp counts), finds by
+//                 look-back how many equal digits the tiles before it hold
+//                 (lookback.cuh, a word per tile and digit), and writes the tile
+//                 in order of digits, equal ones as one run.  A pass whose keys
+//                 all share the digit (the bits beyond the cells in use) only
 //                 copies.
+//   k_radix_small all passes of up to 8192 items in one block
 //   k_scan        exclusive scan, tiles of 4096, the same look-back
 //
-// Both are bound by the latency of the look-back and of the scattered stores,
-// not by bandwidth.  A pass over 2M 64-bit keys takes 40 us (49 us as a
-// histogram, three scan kernels and a scatter), 8 us at 6,000 keys (23 us):
-// one launch instead of five is what small inputs pay for.  The nested-grid
-// build of 6,000 particles went from 62 launches and 310 us to 18 and 90 us.
+// They are bound by the latency of the look-back, not by bandwidth.  Seven passes
+// over 2M 64-bit keys take 203 us (277 with every item scattered by itself: its
+// sector of 32 bytes for 8; 343 as a histogram, three scan kernels and a
+// scatter).  6,000 keys, six passes: 58 us with the histogram as launches, 36 in
+// one block, which is bound by its one SM.
 //
 // A tile whose wait ran out, and those behind it, copy their items in place:
 // stale, but valid, keys and indices.
@@ -64,6 +66,27 @@ __global__ void k_radix_hist(int64_t n, const K* __restrict__ keys, int passes, 
     if (h[i] != 0) atomicAdd(&hist[i], h[i]);
 }
 
+// The lanes with ok and the digit d of this one.  A match costs as much as there
+// are distinct digits in the warp: few in cell indices and levels, where
+// neighbours in memory are mostly neighbours in space, up to 32 in the low bits
+// of 64-bit Morton keys, where eight ballots are cheaper (seven passes over 2M
+// keys: 230 -> 203 us; four over 2M cell indices: 89 -> 96 us).
+template <class K>
+__device__ __forceinline__ unsigned digit_peers(int d, bool ok) {
+  if constexpr (sizeof(K) < 8) {
+    return __match_any_sync(0xffffffffu, ok ? d : 256 + (int)(threadIdx.x & 31));  // !ok: no peers
+  } else {
+    unsigned peers = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      const bool one = (d >> b) & 1;
+      const unsigned m = __ballot_sync(0xffffffffu, one);
+      peers &= one ? m : ~m;
+    }
+    return peers;
+  }
+}
+
 // One pass.  Warp w of a tile handles items base + w * 256 + j * 32 + lane,
 // j = 0..7, i.e. 8 consecutive groups of 32 consecutive items: processing j in
 // order visits the warp's items in index order.  vals_in null: the values are
@@ -74,6 +97,9 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
              const int32_t* __restrict__ hist, int32_t* __restrict__ ticket, uint32_t* pub, K* __restrict__ keys_out,
              int32_t* __restrict__ vals_out, int32_t* __restrict__ status) {
   __shared__ int32_t wcount[kScanWarps][256];
+  __shared__ int32_t first[256];  // place of digit d's item i of the ordered tile: first[d] + i
+  __shared__ K skeys[kRadixTile];
+  __shared__ int32_t svals[kRadixTile];
   __shared__ int32_t s_tile;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d0 = threadIdx.x;
   const int32_t all = hist[d0];
@@ -99,8 +125,8 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {
       const bool ok = base + j * 32 + lane < n;
-      const int d = ok ? (int)((key[j] >> shift) & 255) : 256 + lane;  // out-of-range items never match
-      const unsigned peers = __match_any_sync(0xffffffffu, d);
+      const int d = (int)((key[j] >> shift) & 255);
+      const unsigned peers = digit_peers<K>(d, ok);
       int r = 0;
       if (ok) r = wcount[warp][d] + __popc(peers & lt);
       rank[j] = r;
@@ -120,10 +146,25 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
     }
     uint32_t* my = pub + (int64_t)tile * 256 + d0;
     pub_store(my, (tile == 0 ? kPubPrefix : kPubCount) | (uint32_t)mine);
+    // the tile in order of digits, in shared memory
+    int32_t cnt;
+    const int32_t at0 = block_scan(mine, &cnt);
+#pragma unroll
+    for (int w = 0; w < kScanWarps; ++w) wcount[w][d0] += at0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kRadixItems; ++j) {
+      if (base + j * 32 + lane < n) {
+        const int at = wcount[warp][(int)((key[j] >> shift) & 255)] + rank[j];
+        skeys[at] = key[j];
+        svals[at] = val[j];
+      }
+    }
     int32_t before = 0;
     bool failed = false;
     for (int32_t t = tile - 1; t >= 0;) {
-      // four tiles back at a time, their words in flight together
+      // four tiles back at a time, their words in flight together (eight: 230 us for
+      // the seven passes over 2M keys instead of 208, sixteen: 242)
       uint32_t v[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) v[i] = t - i >= 0 ? pub_load(pub + (int64_t)(t - i) * 256 + d0) : kPubPrefix;
@@ -141,22 +182,132 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
       t -= 4;
     }
     if (tile > 0) pub_store(my, failed ? kPubFailed : kPubPrefix | (uint32_t)(before + mine));
+    first[d0] = dst0 + before - at0;
     copy = __syncthreads_or(failed);
     if (copy && d0 == 0) atomicOr(status, SPH_ST_TIMEOUT);
-    // the place of the tile's first item of digit d0
     if (!copy) {
+      // equal digits leave as runs of consecutive places
 #pragma unroll
-      for (int w = 0; w < kScanWarps; ++w) wcount[w][d0] += dst0 + before;
+      for (int j = 0; j < kRadixItems; ++j) {
+        const int at = j * kScanThreads + d0;
+        if (at < cnt) {
+          const K k = skeys[at];
+          const int64_t dst = (int64_t)first[(int)((k >> shift) & 255)] + at;
+          if (keys_out != nullptr) keys_out[dst] = k;
+          vals_out[dst] = svals[at];
+        }
+      }
+      return;
     }
-    __syncthreads();
   }
 #pragma unroll
   for (int j = 0; j < kRadixItems; ++j) {
     const int64_t p = base + j * 32 + lane;
     if (p < n) {
-      const int64_t dst = copy ? p : (int64_t)wcount[warp][(int)((key[j] >> shift) & 255)] + rank[j];
-      if (keys_out != nullptr) keys_out[dst] = key[j];
-      vals_out[dst] = val[j];
+      if (keys_out != nullptr) keys_out[p] = key[j];
+      vals_out[p] = val[j];
+    }
+  }
+}
+
+// All passes of up to kSmallMax items in one block: the items of a warp (256
+// consecutive ones) are ranked as in k_radix_pass, the whole of them reordered in
+// shared memory, pass after pass.
+constexpr int kSmallMax = 8192;
+constexpr int kSmallItems = 8;
+template <class K>
+__host__ __device__ constexpr size_t small_smem() {
+  return (size_t)kSmallMax * (sizeof(K) + sizeof(int32_t)) + (size_t)(kSmallMax / 256) * 256 * sizeof(uint16_t);
+}
+
+template <class K>
+__global__ void __launch_bounds__(kSmallMax / kSmallItems)
+k_radix_small(int n, const K* __restrict__ keys_in, int passes, K* __restrict__ keys_out,
+              int32_t* __restrict__ vals_out) {
+  extern __shared__ __align__(16) unsigned char rsm[];
+  int32_t* svals = reinterpret_cast<int32_t*>(rsm + (size_t)kSmallMax * sizeof(K));
+  K* skeys = reinterpret_cast<K*>(rsm);
+  uint16_t* counts = reinterpret_cast<uint16_t*>(svals + kSmallMax);  // [warp][digit]
+  __shared__ int32_t ws[8];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nw = blockDim.x >> 5;
+  const int base = warp * (32 * kSmallItems);
+  const unsigned lt = (1u << lane) - 1u;
+  K key[kSmallItems];
+  int32_t val[kSmallItems], rank[kSmallItems];
+#pragma unroll
+  for (int j = 0; j < kSmallItems; ++j) {
+    const int p = base + j * 32 + lane;
+    key[j] = p < n ? keys_in[p] : (K)0;
+    val[j] = p;
+  }
+#pragma unroll 1
+  for (int pass = 0; pass < passes; ++pass) {
+    const int shift = 8 * pass;
+    uint16_t* mine = counts + warp * 256;
+    *reinterpret_cast<uint4*>(mine + 8 * lane) = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kSmallItems; ++j) {
+      const bool ok = base + j * 32 + lane < n;
+      const int d = (int)((key[j] >> shift) & 255);
+      const unsigned peers = digit_peers<K>(d, ok);
+      int r = 0;
+      if (ok) r = mine[d] + __popc(peers & lt);
+      rank[j] = r;
+      __syncwarp();
+      if (ok && (peers >> lane) == 1u) mine[d] = (uint16_t)(mine[d] + __popc(peers));
+      __syncwarp();
+    }
+    __syncthreads();
+    // digit t: its items of the warps before each warp, and its first place
+    int32_t sum = 0;
+    if (t < 256) {
+#pragma unroll 8
+      for (int w = 0; w < nw; ++w) {
+        const int32_t c = counts[w * 256 + t];
+        counts[w * 256 + t] = (uint16_t)sum;
+        sum += c;
+      }
+    }
+    if (__syncthreads_or(t < 256 && sum == n)) continue;  // every key has this digit
+    int32_t x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t v = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += v;
+    }
+    if (t < 256 && lane == 31) ws[warp] = x;
+    __syncthreads();
+    if (t < 256) {
+      int32_t first = x - sum;
+      for (int k = 0; k < warp; ++k) first += ws[k];
+      for (int w = 0; w < nw; ++w) counts[w * 256 + t] = (uint16_t)(counts[w * 256 + t] + first);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSmallItems; ++j) {
+      if (base + j * 32 + lane < n) {
+        const int at = mine[(int)((key[j] >> shift) & 255)] + rank[j];
+        skeys[at] = key[j];
+        svals[at] = val[j];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSmallItems; ++j) {
+      const int p = base + j * 32 + lane;
+      if (p < n) {
+        key[j] = skeys[p];
+        val[j] = svals[p];
+      }
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < kSmallItems; ++j) {
+    const int p = base + j * 32 + lane;
+    if (p < n) {
+      if (keys_out != nullptr) keys_out[p] = key[j];
+      vals_out[p] = val[j];
     }
   }
 }
@@ -244,6 +395,19 @@ static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_o
   const int64_t tiles = (n + kRadixTile - 1) / kRadixTile;
   const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
   if (passes > kRadixMaxPasses) return cudaErrorInvalidValue;
+  if (n <= kSmallMax) {
+    static bool set = false;
+    if (!set) {
+      const cudaError_t e = cudaFuncSetAttribute(k_radix_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)small_smem<K>());
+      if (e != cudaSuccess) return e;
+      set = true;
+    }
+    const int warps = (int)((n + 32 * kSmallItems - 1) / (32 * kSmallItems));
+    k_radix_small<K><<<1, 32 * (warps < 8 ? 8 : warps), small_smem<K>(), st>>>((int)n, keys, passes,
+                                                                               want_keys ? keys_out : nullptr, vals_out);
+    return cudaGetLastError();
+  }
   cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)radix_words(n, passes), st);
   if (e != cudaSuccess) return e;
   int32_t* hist = scratch;
