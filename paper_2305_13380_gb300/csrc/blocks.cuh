@@ -181,6 +181,15 @@ __device__ __forceinline__ int next_round(BlockTargets& B, int lane) {
   return __shfl_sync(0xffffffffu, r, 0);
 }
 
+// CTAs per block: grids with few blocks share each block's rounds between
+// several CTAs, each of which stages the sources, as far as CTAs are resident.  A
+// step of 4096 particles (27 blocks of 152 targets, two rounds a warp) lasts as
+// long as one block's rounds: 190 -> 169 us (up to 2 CTAs a block 167, 8 177).
+constexpr int kMaxParts = 4;
+__device__ __forceinline__ int block_parts(int32_t total) {
+  return max(1, min(kMaxParts, (int)gridDim.x / max(total, 1)));
+}
+
 // Block-collective; ends with __syncthreads().  Targets are dealt to warps
 // in rounds of `per` targets with tpp lanes each: 4 lanes up to 8 targets a
 // round, else 2 lanes for up to 16.  Kernels wider than the cubic spline (K)
@@ -199,7 +208,8 @@ __device__ __forceinline__ int next_round(BlockTargets& B, int lane) {
 template <int K = kKernCubic>
 __device__ __forceinline__ void build_targets(const BlockGeom& g, const StageTable& T, BlockTargets& B,
                                               uint16_t* tgt_slot, uint8_t* tgt_cell,
-                                              const uint8_t* __restrict__ act = nullptr, int lanes = 0) {
+                                              const uint8_t* __restrict__ act = nullptr, int lanes = 0,
+                                              int parts = 1) {
   if (threadIdx.x == 0) {
     int i = 0, run = 0;
     for (int z = 1; z <= g.wz; ++z)
@@ -263,6 +273,8 @@ __device__ __forceinline__ void build_targets(const BlockGeom& g, const StageTab
     if ((K != kKernCubic || lanes == 4) && per > 8) per = 8;
     const int tpp = lanes == 2 ? 2 : (per <= 8 ? 4 : 2);
     if (per > 16) per = 16;
+    // (a target's lanes, and so its sums, do not depend on the parts)
+    if (parts > 1) per = min(per, max(1, (n + kBlkWarps * parts - 1) / (kBlkWarps * parts)));
     B.per = per;
     B.tpp = tpp;
     B.lg = tpp == 4 ? 2 : 1;

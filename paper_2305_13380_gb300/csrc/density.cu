@@ -319,21 +319,24 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
   const NewtonConst nwt = newton_const<K>(ph);
   unsigned long long pair_acc = 0;
 
-  for (int32_t b = blockIdx.x; b < total; b += gridDim.x) {
+  const int parts = block_parts(total);
+  for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
+    const int32_t b = item / parts;
+    const int part = item - b * parts;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     // (FP64, by one thread; read after the barriers below)
     if (threadIdx.x == 0) BT.hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
     if (nsrc > dens_cap<K>()) {
-      if (threadIdx.x == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
+      if (threadIdx.x == 0 && part == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
       __syncthreads();
       continue;
     }
     if (a.act != nullptr) {
       // masked: the block's active targets first, and nothing to stage
       // when it has none
-      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes);
+      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);
       if (BT.n == 0) continue;
     }
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
@@ -353,7 +356,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
       svel[v] = make_float4(v4.x, v4.y, v4.z, p.w);
     }
     if (a.act == nullptr)
-      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, nullptr, ph.lanes);  // ends with a barrier
+      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, nullptr, ph.lanes, parts);  // ends with a barrier
     else
       __syncthreads();  // the staging
 
@@ -361,7 +364,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
     const float R2 = g.G.cell_f * g.G.cell_f;
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
-    for (int rd = warp; rd < BT.rounds; rd = next_round(BT, lane)) {
+    for (int rd = part + parts * warp; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);

@@ -263,25 +263,29 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
   const int32_t total = a.misc_ro[kTotalBlocks];
   unsigned long long pair_acc = 0;
 
-  for (int32_t b = blockIdx.x; b < total; b += gridDim.x) {
+  const int parts = block_parts(total);
+  for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
+    const int32_t b = item / parts;
+    const int part = item - b * parts;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
     if (nsrc > kCap) {
-      if (threadIdx.x == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
+      if (threadIdx.x == 0 && part == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
       __syncthreads();
       continue;
     }
     const float dt = kFl == kFlGradient ? block_dt(a, x, b) : 0.0f;
     // the targets' rounds first (they need only the table), so that each
     // warp's first list is in flight together with the staging loads
-    build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes);  // ends with a barrier
+    build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);  // ends with a barrier
     if (BT.n == 0) continue;  // a masked block without active targets
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
     int pre_lc = 0xffff;
     uint4 pre[kFListCap / 8];
-    if (a.lists != nullptr && warp < BT.rounds) fetch_list(a, BT, T, tgt_slot, tgt_cell, warp, lane, pre_lc, pre);
+    const int rd0 = part + parts * warp;
+    if (a.lists != nullptr && rd0 < BT.rounds) fetch_list(a, BT, T, tgt_slot, tgt_cell, rd0, lane, pre_lc, pre);
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
       const int k = staged_cell_of(T, v);
       float ox, oy, oz;
@@ -299,7 +303,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
     }
     __syncthreads();
 
-    for (int rd = warp; rd < BT.rounds; rd = next_round(BT, lane)) {
+    for (int rd = rd0; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);
@@ -310,7 +314,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
       }
       const int tx = kc % g.ex - 1, ty = (kc / g.ex) % g.ey - 1, tz = kc / (g.ex * g.ey) - 1;
       const int32_t ti = T.gstart[kc] + (self_slot - T.start[kc]);
-      if (a.lists != nullptr && rd != warp) fetch_list(a, BT, T, tgt_slot, tgt_cell, rd, lane, pre_lc, pre);
+      if (a.lists != nullptr && rd != rd0) fetch_list(a, BT, T, tgt_slot, tgt_cell, rd, lane, pre_lc, pre);
       ForceTarget Tg;
       Tg.A = sA[self_slot];
       Tg.B = sB[self_slot];
@@ -516,16 +520,19 @@ __global__ void __launch_bounds__(kBlkThreads, kMinBlocks) k_force_min(sphh::For
   const float half_alpha = 0.5f * ph.alpha_v, beta = ph.beta_v;
   unsigned long long pair_acc = 0;
 
-  for (int32_t b = blockIdx.x; b < total; b += gridDim.x) {
+  const int parts = block_parts(total);
+  for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
+    const int32_t b = item / parts;
+    const int part = item - b * parts;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
     if (nsrc > kCap) {
-      if (threadIdx.x == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
+      if (threadIdx.x == 0 && part == 0) a.overflow[atomicAdd(&a.misc[kNumOverflow], 1)] = b;
       __syncthreads();
       continue;
     }
-    build_targets<kKernCubic>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes);  // ends with a barrier
+    build_targets<kKernCubic>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);  // ends with a barrier
     if (BT.n == 0) continue;
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
       const int k = staged_cell_of(T, v);
@@ -546,7 +553,7 @@ __global__ void __launch_bounds__(kBlkThreads, kMinBlocks) k_force_min(sphh::For
 
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
-    for (int rd = warp; rd < BT.rounds; rd = next_round(BT, lane)) {
+    for (int rd = part + parts * warp; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);
