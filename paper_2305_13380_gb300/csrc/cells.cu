@@ -252,15 +252,15 @@ __global__ void k_gather_force(int64_t n_total, const int32_t* __restrict__ perm
     }
     const float H = gamma_k * h[p];
     if (rec != nullptr) {
-      // nested grids: one record per source (the arrays below are not read)
+      // nested grids: a record per source in four arrays (those below are not read)
       const float4 rl = trel[s];
       const int4 fn = tfine[s];
       const float r = rho[p];
-      float4* o = rec + 4 * s;
+      float4* o = rec + s;
       o[0] = make_float4(rl.x, rl.y, rl.z, H);
-      o[1] = make_float4(__int_as_float(fn.x), __int_as_float(fn.y), __int_as_float(fn.z), r);
-      o[2] = make_float4(vx[p], vy[p], vz[p], m[p]);
-      o[3] = make_float4(f[p] * P[p] / (r * r), f[p], c[p], B[p]);
+      o[n_total] = make_float4(__int_as_float(fn.x), __int_as_float(fn.y), __int_as_float(fn.z), r);
+      o[2 * n_total] = make_float4(vx[p], vy[p], vz[p], m[p]);
+      o[3 * n_total] = make_float4(f[p] * P[p] / (r * r), f[p], c[p], B[p]);
       continue;
     }
     if (kPos) {

@@ -107,8 +107,8 @@ struct GatherForceArgs {
   // 1: compute fA.xyz from x, y, z; 0: fA.xyz already holds them (or is not
   // read), write H only
   int positions = 1;
-  // nested grids: 64-byte records (rel, H), (fine, rho), (v, m), (fP, f, c, B)
-  // per source instead of fA..fD; rel and fine are the tree gather's copies
+  // nested grids: records (rel, H), (fine, rho), (v, m), (fP, f, c, B) per
+  // source, four arrays of n_total one after another, instead of fA..fD; rel and fine are the tree gather's copies
   const float4* rel = nullptr;
   const int4* fine = nullptr;
   float4* rec = nullptr;
@@ -420,7 +420,7 @@ struct TreeForceArgs {
   const float4* rel;
   const float *lrad, *leaf_side;
   const int32_t* perm;
-  const float4* rec;  // 4 float4 per source, as GatherForceArgs::rec
+  const float4* rec;  // 4 n_total float4, as GatherForceArgs::rec
   const uint32_t* lists;
   const uint16_t* list_cnt;
   const int32_t* rev_start;

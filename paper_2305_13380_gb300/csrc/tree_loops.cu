@@ -98,8 +98,8 @@ constexpr int32_t kFbOwnLevel = 1 << 30;
 constexpr int32_t kFbPassive = 1 << 29;
 constexpr int32_t kFbIndex = kFbPassive - 1;
 static_assert(kTreeList <= kTreeListRegion, "published lists fit their regions");
-// a target's published list: its lanes' lists packed one after another in a
-// region of kTreeTpp * kTreeListRegion entries, the count in list_cnt[target]
+// a target's published list: its lanes' first entries, then their second ones,
+// and so on, in a region of kTreeTpp * kTreeListRegion entries, the count in list_cnt[target]
 constexpr int kTreeListTarget = kTreeTpp * kTreeListRegion;
 
 struct TGeo {
@@ -933,19 +933,30 @@ __global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sph
             }
           }
           // 3. final pass at h; the list's reverse pairs are marked on the way
-          // (bit e: entry e), with j's threshold read with its fine position
+          // (bit e: entry e), with j's threshold read with its fine position.
+          // The list is published for the force loop as it is walked: entry e of
+          // every lane, lane by lane, then entry e + 1, close to the sources'
+          // order, so that the lanes of the force's targets read neighbouring
+          // sources
           const float H = KernT<K>::gamma * h;
           const float Hinv = 1.0f / H;
           const float H2 = H * H;
           TDSums s;
           tds_zero(s);
           uint32_t wm = 0;
-          if (on_now && !queued) {
+          const int mine = on_now && !queued ? cnt : 0;
+          uint32_t* dst = a.lists + (int64_t)ti * kTreeListTarget;
+          int all = 0;
 #pragma unroll 1
-            for (int e = 0; e < cnt; ++e) {
+          for (int e = 0;; ++e) {
+            const unsigned m = __ballot_sync(0xffffffffu, e < mine);
+            if (m == 0u) break;
+            const unsigned row = (m >> (t * kTreeTpp)) & kTGroup;
+            if (e < mine) {
               const float4 pk = S.pos[S.list[e][lane]];
               const uint32_t je = __float_as_uint(pk.w);
               const int32_t j = unpack_j(je);
+              dst[all + __popc(row & ((1u << sub) - 1u))] = je;
               const float4 rj = a.rel[j];
               const int4 fj = a.fine[j];
               const float3 d = pair_vec(g, reli, fi, rj, fj, unpack_s(je));
@@ -954,7 +965,10 @@ __global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sph
                   (!kMask || a.act[j] != 0))
                 wm |= 1u << e;
             }
-          } else if (kMask && act_now && !queued) {
+            all += __popc(row);
+          }
+          if (on_now && sub == 0) a.list_cnt[ti] = (uint16_t)(atcap || queued ? kListFallback : all);
+          if (kMask && act_now && !queued && !on) {
             // outside the mask: the reverse pairs to its listed (masked) sources
 #pragma unroll 1
             for (int e = 0; e < cnt; ++e) {
@@ -966,26 +980,6 @@ __global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sph
           // whole round
           emit_marked(TEmit{a.rev_count, a.rev_raw, a.rev_start, a.rev_cap, a.status}, wm, S, ti, lane);
           tcombine(s);
-          // 4. publish the list for the force loop: the target's lanes' lists
-          // packed one after another (lane sub's entries after those of the
-          // lanes below it), so that the force reads them in whole sectors
-          {
-            int incl = on_now && !queued ? cnt : 0;
-#pragma unroll
-            for (int o = 1; o < kTreeTpp; o <<= 1) {
-              const int v = __shfl_up_sync(0xffffffffu, incl, o, kTreeTpp);
-              if (sub >= o) incl += v;
-            }
-            const int all = __shfl_sync(0xffffffffu, incl, kTreeTpp - 1, kTreeTpp);
-            if (on_now) {
-              if (sub == 0) a.list_cnt[ti] = (uint16_t)(atcap || queued ? kListFallback : all);
-              if (!queued) {
-                uint32_t* dst = a.lists + (int64_t)ti * kTreeListTarget + (incl - cnt);
-#pragma unroll 1
-                for (int e = 0; e < cnt; ++e) dst[e] = __float_as_uint(S.pos[S.list[e][lane]].w);
-              }
-            }
-          }
           if (act_now && sub == 0) {
             if (queued) {
               // solved at its own level by the per-target kernel
@@ -1181,23 +1175,26 @@ struct TFSums {
   int npair;
 };
 
-// A source's force record, 64 bytes in source order (written by the force
-// gather): q0 = (rel x, y, z, H), q1 = (fine x, y, z, rho as bits),
-// q2 = (v, m), q3 = (f P / rho^2, f, c, B).  One record replaces six
-// gathers from six arrays; 1/H is recomputed (correctly rounded, the value
-// the arrays held).
+// A source's force record, in source order (written by the force gather): q0 =
+// (rel x, y, z, H), q1 = (fine x, y, z, rho as bits), q2 = (v, m), q3 =
+// (f P / rho^2, f, c, B), each in an array of its own: a target's eight lanes
+// read neighbouring sources, whose quarters share a line or two.  With 64-byte
+// records and lists in the density lanes' order the force gathers filled the L1's
+// data stage (94 % of its wavefronts): 2M clustered particles 1306 -> 1023 us.
+// 1/H is recomputed (correctly rounded, the value the arrays held).
 struct TRec {
   float4 q0;
   int4 q1;
 };
 
-__device__ __forceinline__ TRec trec_head(const float4* __restrict__ rec, int32_t j) {
-  const float4* r = rec + 4 * (int64_t)j;
+__device__ __forceinline__ TRec trec_head(const sphh::TreeForceArgs& a, int32_t j) {
   TRec t;
-  t.q0 = r[0];
-  t.q1 = *reinterpret_cast<const int4*>(r + 1);
+  t.q0 = a.rec[j];
+  t.q1 = *reinterpret_cast<const int4*>(a.rec + a.n_total + j);
   return t;
 }
+__device__ __forceinline__ float4 trec_vel(const sphh::TreeForceArgs& a, int32_t j) { return a.rec[2 * a.n_total + j]; }
+__device__ __forceinline__ float4 trec_pres(const sphh::TreeForceArgs& a, int32_t j) { return a.rec[3 * a.n_total + j]; }
 
 // Flavours of the force kernels: the "Minimal" force, the SPHENIX force and
 // the SPHENIX gradient pass (Sec. 3.3; the terms are those of force.cu's
@@ -1282,12 +1279,11 @@ __device__ __forceinline__ void tforce_rec(float dx, float dy, float dz, const f
     if (r2 < Hm * Hm && a.act[j] == 0 && w > (int)a.fE[j].x) atomicMax(a.wake + a.perm[j], w);
     return;
   }
-  const float4* r = a.rec + 4 * (int64_t)j;
   const float4 ej = kFl != kTMin ? a.fE[j] : make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (kFl == kTLimit) {
     tforce_pair<kFl, K>(dx, dy, dz, vi, ci, ei, Hi, Hinv_i, rho_i, vi, ci, ej, h.q0.w, 0.0f, 0.0f, ph, s);
   } else {
-    tforce_pair<kFl, K>(dx, dy, dz, vi, ci, ei, Hi, Hinv_i, rho_i, r[2], r[3], ej, h.q0.w, __frcp_rn(h.q0.w),
+    tforce_pair<kFl, K>(dx, dy, dz, vi, ci, ei, Hi, Hinv_i, rho_i, trec_vel(a, j), trec_pres(a, j), ej, h.q0.w, __frcp_rn(h.q0.w),
                         __int_as_float(h.q1.w), ph, s);
   }
 }
@@ -1331,8 +1327,8 @@ __device__ __forceinline__ float3 rec_rel_to(const TGeo& g, const TRec& h, int s
 // A warp takes windows of win consecutive targets from a counter, kTPer at a
 // time with kTreeTpp lanes each, whatever their leaves (a target's lanes hold
 // its own leaf's corner): every round is full, and a large leaf is shared by
-// many warps.  Bound by the latency and the L1 wavefronts of the 64-byte record
-// gathers.
+// many warps.  Bound by the L1 wavefronts of the record gathers (79 %) and by
+// instruction issue (61 %).
 template <int kFl, int K>
 __global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs a, PhysDev ph, SphenixDev x,
                                                              int win) {
@@ -1360,15 +1356,15 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs
       const bool fb = lc == kListFallback;  // written by k_tree_force_fb
       const float4 ei = kFl != kTMin ? a.fE[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
       if (kFl == kTGradient) s.ay = ei.y;  // alpha_V,max starts at the target's
-      const TRec hi = trec_head(a.rec, ti);
+      const TRec hi = trec_head(a, ti);
       const float Hi = hi.q0.w;
       const bool on = valid && !fb && (a.act == nullptr || a.act[ti] != 0);
       if (on) {
         const float4 reli = hi.q0;
         const int4 fi = hi.q1;
         const float3 pi = rel_to(g, reli, fi, kNoShift);
-        const float4 vi = a.rec[4 * (int64_t)ti + 2];
-        const float4 ci = a.rec[4 * (int64_t)ti + 3];
+        const float4 vi = trec_vel(a, ti);
+        const float4 ci = trec_pres(a, ti);
         const float2 di = make_float2(__int_as_float(hi.q1.w), __frcp_rn(hi.q0.w));
         // own reach: the list radius (a target without a complete list went
         // to the per-target kernel, kListFallback)
@@ -1379,7 +1375,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs
           const uint32_t je = lst[e];
           const int32_t j = unpack_j(je);
           if (j == ti) continue;
-          const TRec hj = trec_head(a.rec, j);
+          const TRec hj = trec_head(a, j);
           const float3 d = pair_vec(g, reli, fi, hj.q0, hj.q1, unpack_s(je));
           tforce_rec<kFl, K>(d.x, d.y, d.z, vi, ci, ei, Hi, di.y, di.x, a, j, hj, ph, s);
         }
@@ -1390,7 +1386,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force(sphh::TreeForceArgs
           for (int32_t k = r0 + sub; k < r1; k += kTreeTpp) {
             const uint32_t je = a.rev[k];
             const int32_t j = unpack_j(je);
-            const TRec hj = trec_head(a.rec, j);
+            const TRec hj = trec_head(a, j);
             const float3 pj = rec_rel_to(g, hj, unpack_s(je));
             const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
             if (fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= C2)
@@ -1689,10 +1685,10 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceA
     const TreeLeaf Lc = cell_at_depth(key, (int)a.fb_level[ti]);
     const TGeo g = leaf_geo(Lc, G);
     const float dt = kFl == kTGradient ? (float)(x.dt_dev != nullptr ? x.dt_dev[sim] : x.dt) : 0.0f;
-    const TRec hi = trec_head(a.rec, ti);
+    const TRec hi = trec_head(a, ti);
     const float3 pi = rec_rel_to(g, hi, kNoShift);
-    const float4 vi = a.rec[4 * (int64_t)ti + 2];
-    const float4 ci = a.rec[4 * (int64_t)ti + 3];
+    const float4 vi = trec_vel(a, ti);
+    const float4 ci = trec_pres(a, ti);
     const float4 ei = kFl != kTMin ? a.fE[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
     const float2 di = make_float2(__int_as_float(hi.q1.w), __frcp_rn(hi.q0.w));
     const float Hi = hi.q0.w;
@@ -1712,7 +1708,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceA
       if (lane < cnt) {
         const uint32_t je = ring[(head + lane) & 63];
         const int32_t j = unpack_j(je);
-        const TRec hj = trec_head(a.rec, j);
+        const TRec hj = trec_head(a, j);
         const float3 pj = rec_rel_to(g, hj, unpack_s(je));
         tforce_rec<kFl, K>(pi.x - pj.x, pi.y - pj.y, pi.z - pj.z, vi, ci, ei, Hi, di.y, di.x, a, j, hj, ph, s);
       }
@@ -1747,7 +1743,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceA
         sj[i] = pr->src[c];
         const int32_t j = sj[i].x + min(u0 + 32 * i + lane, hit.y - 1);
         je[i] = pack_js(j, child_shift(pr, c));
-        hj[i] = trec_head(a.rec, j);
+        hj[i] = trec_head(a, j);
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -1767,7 +1763,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_force_fb(sphh::TreeForceA
         uint32_t je = 0;
         if (k0 + lane < r1) {
           je = a.rev[k0 + lane];
-          const float3 pj = rec_rel_to(g, trec_head(a.rec, unpack_j(je)), unpack_s(je));
+          const float3 pj = rec_rel_to(g, trec_head(a, unpack_j(je)), unpack_s(je));
           const float dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
           in = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) >= C2;
         }
