@@ -71,7 +71,10 @@ constexpr int kTKept = 256;
 constexpr int kTWhole = 384;           // a leaf with at most this many sources is taken whole
 constexpr int kTSegs = 27 * 4 + 4;     // runs of hit children: at most four per range
 constexpr int kTWin = 2 * kTPer;       // targets per window (k_tree_density)
-constexpr int kTDensBlocks = 6;        // resident CTAs per SM the registers are sized for
+// resident CTAs per SM that the registers are sized for (the plain instance over
+// 2M clustered particles: 5 4.18, 6 3.85, 7 3.88 ms; the masked one, which keeps
+// more alive, over 1M: 4 734, 5 657, 6 734 us)
+constexpr int kTDensBlocks = 6, kTMaskBlocks = 5;
 struct TRound {
   float4 pos[kTKept];                  // position from the leaf corner; packed index and shift
   float4 tgt[kTPer];                   // the targets' positions and R^2
@@ -733,7 +736,8 @@ __device__ __forceinline__ void tdens_write(const sphh::TreeDensityArgs& a, cons
 // kMask: the masked loops (a.act, a.act_pre set); the plain instance carries
 // none of their tests.
 template <int K, bool kMask>
-__global__ void __launch_bounds__(kTWarps * 32, kTDensBlocks) k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
+__global__ void __launch_bounds__(kTWarps * 32, kMask ? kTMaskBlocks : kTDensBlocks)
+k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
