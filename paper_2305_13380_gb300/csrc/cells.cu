@@ -15,6 +15,7 @@
 #include "lookback.cuh"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
+#include "tree.cuh"
 
 namespace sphk {
 
@@ -101,6 +102,7 @@ k_grid_setup(const int64_t* __restrict__ sim_offset, const double* __restrict__ 
       g.hcap_f = h_cap(g.cell, 2.0 * g.cell, gamma_k);
       g.hcap_box_f = h_cap(L, L, gamma_k);
       g.scale_f = (float)((double)nc / L);
+      g.fine_scale = (double)nc * (double)kTreeFine / L;
       g.part_base = a;
       g.n = b - a;
     }

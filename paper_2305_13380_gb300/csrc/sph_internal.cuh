@@ -44,6 +44,7 @@ struct GridDev {
                       // less twice the drift since, while cells are kept
   float hcap_f;       // the largest h whose support stays below the cell side, and ...
   float hcap_box_f;   // ... below half the box (h_cap)
+  double fine_scale;  // kTreeFine n_c / L (estimates of fine coordinates)
   int64_t part_base;  // first pool index of this simulation
   int64_t n;          // particles in this simulation
 };
