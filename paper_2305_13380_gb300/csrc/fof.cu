@@ -55,19 +55,27 @@ __device__ __forceinline__ int32_t fof_find(int32_t* parent, int32_t x, int32_t*
   return x;
 }
 
-__device__ __forceinline__ void fof_union(int32_t* parent, int32_t a, int32_t b, int32_t* status) {
+// Joins the sets of a and b; returns a root that both had at some time since.
+__device__ __noinline__ int32_t fof_union(int32_t* parent, int32_t a, int32_t b, int32_t* status) {
   for (int it = 0; it < kFofMaxSteps; ++it) {
     a = fof_find<true>(parent, a, status);
     b = fof_find<true>(parent, b, status);
-    if (a == b) return;
+    if (a == b) return a;
     if (a > b) {
       const int32_t t = a;
       a = b;
       b = t;
     }
-    if (atomicCAS(parent + b, b, a) == b) return;  // b was still a root: hooked
+    if (atomicCAS(parent + b, b, a) == b) return a;  // b was still a root: hooked
   }
   atomicOr(status, SPH_ST_CAPACITY);
+  return a;
+}
+
+// Whether b is known to be in the set of ancestor `root` of another particle: one
+// load where two finds take four.
+__device__ __forceinline__ bool fof_joined(const int32_t* parent, int32_t root, int32_t b) {
+  return __ldcg(parent + b) == root;
 }
 
 // FP64 friendship test of the definition (minimum image, no contraction).
@@ -228,55 +236,114 @@ __device__ __forceinline__ float fof_gap(float p0, float p1, float off, int bit,
 }
 
 // Particles of cells not taken by octants, a thread each: the later particles
-// of the cell and those of the 13 neighbours (or their octants).
-__global__ void k_fof_link(sphh::FofArgs a) {
+// of the cell and those of the 13 neighbours (or their octants, which the warp
+// searches together).  Bound by latency: the empty rows skipped, four particles'
+// loads in flight, one load instead of two finds for a pair that is joined
+// already, and twelve blocks of 128 threads per SM took the 1M clustered box from
+// 508 to 388 us.
+__global__ void __launch_bounds__(128, 12) k_fof_link(sphh::FofArgs a) {
   const GridDev G = a.grid[0];
   const int32_t nc = G.n_c;
   const FofTest T = fof_test(G, a.link);
   const int dense = fof_octants(G, a.link) ? kFofDense : INT32_MAX;
   const float half = 0.5f * G.cell_f;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < a.n_total;
-       s += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t pi = a.perm[s];
-    const int32_t cg = a.key[pi], c = cg - G.cell_base;
-    if (a.cell_start[cg + 1] - a.cell_start[cg] >= dense) continue;
-    const float4 me = a.rel[s];
+  const int lane = threadIdx.x & 31;
+  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; w < a.n_total;
+       w += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t s = w + lane;
+    bool on = s < a.n_total;
+    const int32_t pi = on ? a.perm[s] : 0;
+    const int32_t cg = on ? a.key[pi] : G.cell_base, c = cg - G.cell_base;
+    on = on && a.cell_start[cg + 1] - a.cell_start[cg] < dense;
+    const float4 me = on ? a.rel[s] : make_float4(0.f, 0.f, 0.f, 0.f);
     const int32_t kx = c % nc, ky = (c / nc) % nc, kz = c / (nc * nc);
-    for (int o = 0; o <= kAxes; ++o) {
-      FofCell C = fof_cell(a, G, kx, ky, kz, o);
-      if (C.t1 - C.t0 >= dense) {
-        // octants within reach that are not in this particle's set yet
-        for (int k = 0; k < 8; ++k) {
-          const int32_t u0 = a.oct[C.t0 + k], u1 = k < 7 ? a.oct[C.t0 + k + 1] : C.t1;
-          if (u0 >= u1) continue;
+    int32_t root = on ? fof_find<true>(a.group, pi, a.status) : 0;  // an ancestor of pi
+    // the neighbours beyond the own row lie in four rows of three cells, one
+    // after another in memory: a row without particles is skipped (most are, of
+    // cells of the linking length), and all rows' ends are in flight together
+    unsigned todo = on ? (1u << (kAxes + 1)) - 1u : 0u;
+    if (on && kx > 0 && kx < nc - 1) {
+      int32_t r0[4], r1[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int dy = k == 0 ? 1 : k - 2, dz = k == 0 ? 0 : 1;
+        int32_t cy = ky + dy, cz = kz + dz;
+        cy += cy < 0 ? nc : 0;
+        cy -= cy >= nc ? nc : 0;
+        cz -= cz >= nc ? nc : 0;
+        const int32_t cn = G.cell_base + kx - 1 + nc * (cy + nc * cz);
+        r0[k] = a.cell_start[cn];
+        r1[k] = a.cell_start[cn + 3];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (r0[k] == r1[k]) todo &= ~(7u << (2 + 3 * k));
+    }
+    for (unsigned all = __reduce_or_sync(0xffffffffu, todo); all != 0u; all &= all - 1u) {
+      const int o = __ffs((int)all) - 1;
+      FofCell C = {0, 0, 0.f, 0.f, 0.f};
+      if ((todo >> o) & 1u) C = fof_cell(a, G, kx, ky, kz, o);
+      const bool octs = C.t1 - C.t0 >= dense;
+      if (!octs) {
+        if (o == 0) C.t0 = (int32_t)s + 1;
+        for (int32_t t = C.t0; t < C.t1; t += 4) {
+          int32_t pq[4], up[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 q = a.rel[min(t + i, C.t1 - 1)];
+            pq[i] = t + i < C.t1 && fof_friends(a, G, T, me, q, C) ? __float_as_int(q.w) : -1;
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) up[i] = pq[i] >= 0 ? __ldcg(a.group + pq[i]) : 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (pq[i] >= 0 && up[i] != root) root = fof_union(a.group, pi, pq[i], a.status);
+        }
+      }
+      if (!__any_sync(0xffffffffu, octs)) continue;
+      // octants within reach that are not in this particle's set yet, searched
+      // for a friend by the whole warp
+#pragma unroll 1
+      for (int k = 0; k < 8; ++k) {
+        int32_t u0 = 0, u1 = 0, pk = 0;
+        bool open = octs;
+        if (open) {
+          u0 = a.oct[C.t0 + k];
+          u1 = k < 7 ? a.oct[C.t0 + k + 1] : C.t1;
           const float gx = fof_gap(me.x, me.x, C.ox, k & 1, half), gy = fof_gap(me.y, me.y, C.oy, (k >> 1) & 1, half),
                       gz = fof_gap(me.z, me.z, C.oz, k >> 2, half);
-          if (fmaf(gx, gx, fmaf(gy, gy, gz * gz)) >= T.hi) continue;
-          const int32_t pk = __float_as_int(a.rel[u0].w);
-          if (fof_find<true>(a.group, pi, a.status) == fof_find<true>(a.group, pk, a.status)) continue;
-          for (int32_t u = u0; u < u1; ++u) {
-            if (fof_friends(a, G, T, me, a.rel[u], C)) {
-              fof_union(a.group, pi, pk, a.status);
-              break;
-            }
-          }
+          open = u0 < u1 && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < T.hi;
         }
-        continue;
-      }
-      if (o == 0) C.t0 = (int32_t)s + 1;
-      for (int32_t t = C.t0; t < C.t1; ++t) {
-        const float4 q = a.rel[t];
-        if (fof_friends(a, G, T, me, q, C)) fof_union(a.group, pi, __float_as_int(q.w), a.status);
+        if (open) {
+          pk = __float_as_int(a.rel[u0].w);
+          open = !fof_joined(a.group, root, pk) &&
+                 fof_find<true>(a.group, pi, a.status) != fof_find<true>(a.group, pk, a.status);
+        }
+        for (unsigned left = __ballot_sync(0xffffffffu, open); left != 0u; left &= left - 1u) {
+          const int l = __ffs((int)left) - 1;
+          const float4 p = make_float4(__shfl_sync(0xffffffffu, me.x, l), __shfl_sync(0xffffffffu, me.y, l),
+                                       __shfl_sync(0xffffffffu, me.z, l), __shfl_sync(0xffffffffu, me.w, l));
+          const int32_t v0 = __shfl_sync(0xffffffffu, u0, l), v1 = __shfl_sync(0xffffffffu, u1, l);
+          const FofCell D = {v0, v1, __shfl_sync(0xffffffffu, C.ox, l), __shfl_sync(0xffffffffu, C.oy, l),
+                             __shfl_sync(0xffffffffu, C.oz, l)};
+          bool found = false;
+          for (int32_t u = v0; u < v1 && !found; u += 32)
+            found = __any_sync(0xffffffffu, fof_friends(a, G, T, p, a.rel[min(u + lane, v1 - 1)], D));
+          if (found && lane == l) root = fof_union(a.group, pi, pk, a.status);
+          __syncwarp();
+        }
       }
     }
   }
 }
 
 // Octants of the queued cells, a warp each: the later octants of the cell and
-// the octants or particles of the 13 neighbours.  A lane looks at one of them
-// at a time (is it within reach, and another set?); those left are tested by
-// the whole warp, pair by pair until the first friends.
-__global__ void k_fof_link_octants(sphh::FofArgs a) {
+// the octants or particles of the 13 neighbours, 32 at a time.  A lane looks at
+// one of them (is it within reach, and another set?); those left are tested by
+// the whole warp, pair by pair until the first friends.  300 us of the 1M
+// clustered box, whatever the occupancy, the order of the nodes or the pairs
+// tested: bound by the finds and unions that a core's octants contend in.
+__global__ void __launch_bounds__(128) k_fof_link_octants(sphh::FofArgs a) {
   const GridDev G = a.grid[0];
   const int32_t nc = G.n_c;
   const FofTest T = fof_test(G, a.link);
@@ -293,44 +360,91 @@ __global__ void k_fof_link_octants(sphh::FofArgs a) {
     const int32_t pm = __float_as_int(a.rel[s0].w);
     const float mx = me & 1 ? half : 0.0f, my = me & 2 ? half : 0.0f, mz = me & 4 ? half : 0.0f;
     const int32_t kx = c % nc, ky = (c / nc) % nc, kz = c / (nc * nc);
-    for (int o = 0; o <= kAxes; ++o) {
-      const FofCell C = fof_cell(a, G, kx, ky, kz, o);
+    int32_t root = fof_find<true>(a.group, pm, a.status);  // an ancestor of pm
+    // lane o <= 13: cell o; its nodes (a dense one's octants, the particles of
+    // another) follow those of the cells before it
+    const FofCell M = lane <= kAxes ? fof_cell(a, G, kx, ky, kz, lane) : FofCell{0, 0, 0.f, 0.f, 0.f};
+    int32_t incl = M.t1 - M.t0 >= kFofDense ? 8 : M.t1 - M.t0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int32_t nodes = __shfl_sync(0xffffffffu, incl, 31);
+    for (int32_t n0 = 0; n0 < nodes; n0 += 32) {
+      const int32_t n = n0 + lane;
+      int o = 0;
+#pragma unroll
+      for (int step = 8; step > 0; step >>= 1)
+        if (__shfl_sync(0xffffffffu, incl, o + step - 1) <= n) o += step;
+      o = min(o, kAxes);
+      const int32_t before = __shfl_sync(0xffffffffu, incl, max(o - 1, 0));
+      const int k = n - (o > 0 ? before : 0);
+      FofCell C;
+      C.t0 = __shfl_sync(0xffffffffu, M.t0, o);
+      C.t1 = __shfl_sync(0xffffffffu, M.t1, o);
+      C.ox = __shfl_sync(0xffffffffu, M.ox, o);
+      C.oy = __shfl_sync(0xffffffffu, M.oy, o);
+      C.oz = __shfl_sync(0xffffffffu, M.oz, o);
       const bool dense = C.t1 - C.t0 >= kFofDense;  // at most kFofDense - 1 particles else
-      const int nodes = dense ? 8 : C.t1 - C.t0;
-      int32_t u0 = 0, u1 = 0;
-      bool open = lane < nodes && (o > 0 || lane > me);
+      int32_t u0 = 0, u1 = 0, pq = 0;
+      bool open = n < nodes && (o > 0 || k > me);
       if (open) {
-        u0 = dense ? a.oct[C.t0 + lane] : C.t0 + lane;
-        u1 = dense ? (lane < 7 ? a.oct[C.t0 + lane + 1] : C.t1) : u0 + 1;
+        u0 = dense ? a.oct[C.t0 + k] : C.t0 + k;
+        u1 = dense ? (k < 7 ? a.oct[C.t0 + k + 1] : C.t1) : u0 + 1;
         open = u0 < u1;
       }
       if (open) {
         float gx, gy, gz;
         const float4 q = a.rel[u0];
+        pq = __float_as_int(q.w);
         if (dense) {
-          gx = fof_gap(mx, mx + half, C.ox, lane & 1, half);
-          gy = fof_gap(my, my + half, C.oy, (lane >> 1) & 1, half);
-          gz = fof_gap(mz, mz + half, C.oz, lane >> 2, half);
+          gx = fof_gap(mx, mx + half, C.ox, k & 1, half);
+          gy = fof_gap(my, my + half, C.oy, (k >> 1) & 1, half);
+          gz = fof_gap(mz, mz + half, C.oz, k >> 2, half);
         } else {
           gx = fof_gap(q.x + C.ox, q.x + C.ox, mx, 0, half);
           gy = fof_gap(q.y + C.oy, q.y + C.oy, my, 0, half);
           gz = fof_gap(q.z + C.oz, q.z + C.oz, mz, 0, half);
         }
-        open = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < T.hi &&
-               fof_find<true>(a.group, pm, a.status) != fof_find<true>(a.group, __float_as_int(q.w), a.status);
+        open = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < T.hi && !fof_joined(a.group, root, pq) &&
+               fof_find<true>(a.group, pm, a.status) != fof_find<true>(a.group, pq, a.status);
       }
-      for (unsigned left = __ballot_sync(0xffffffffu, open); left != 0u; left &= left - 1u) {
-        const int k = __ffs((int)left) - 1;
-        const int32_t v0 = __shfl_sync(0xffffffffu, u0, k), v1 = __shfl_sync(0xffffffffu, u1, k);
+      for (unsigned left = __ballot_sync(0xffffffffu, open); left != 0u;) {
+        const int l = __ffs((int)left) - 1;
+        left &= left - 1u;
+        const int32_t v0 = __shfl_sync(0xffffffffu, u0, l), v1 = __shfl_sync(0xffffffffu, u1, l);
+        const FofCell D = {v0, v1, __shfl_sync(0xffffffffu, C.ox, l), __shfl_sync(0xffffffffu, C.oy, l),
+                           __shfl_sync(0xffffffffu, C.oz, l)};
+        // the other's box (an octant, or a particle)
+        const bool dl = __shfl_sync(0xffffffffu, dense ? 1 : 0, l) != 0;
+        const int kl = __shfl_sync(0xffffffffu, k, l);
+        const float4 f = a.rel[v0];
+        const float wx = D.ox + (dl ? (kl & 1 ? half : 0.0f) : f.x), wy = D.oy + (dl ? (kl & 2 ? half : 0.0f) : f.y),
+                    wz = D.oz + (dl ? (kl & 4 ? half : 0.0f) : f.z), ww = dl ? half : 0.0f;
         // 32 of this octant's particles at a time against each of the other's
         bool found = false;
         for (int32_t s = s0; s < s1 && !found; s += 32) {
           const float4 p = a.rel[min(s + lane, s1 - 1)];
-          for (int32_t u = v0; u < v1 && !found; ++u)
-            found = __any_sync(0xffffffffu, fof_friends(a, G, T, p, a.rel[u], C));
+          // (those beside the other octant, or particle, only)
+          const float px = fof_gap(p.x, p.x, wx, 0, ww), py = fof_gap(p.y, p.y, wy, 0, ww),
+                      pz = fof_gap(p.z, p.z, wz, 0, ww);
+          const bool near = fmaf(px, px, fmaf(py, py, pz * pz)) < T.hi;
+          if (!__any_sync(0xffffffffu, near)) continue;
+          for (int32_t u = v0; u < v1 && !found; u += 4) {
+            bool hit = false;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) hit = hit || (near && fof_friends(a, G, T, p, a.rel[min(u + i, v1 - 1)], D));
+            found = __any_sync(0xffffffffu, hit);
+          }
         }
-        if (found && lane == 0) fof_union(a.group, pm, __float_as_int(a.rel[v0].w), a.status);
-        __syncwarp();
+        if (found) {
+          if (lane == l) root = fof_union(a.group, pm, pq, a.status);
+          root = __shfl_sync(0xffffffffu, root, l);
+          // (the union may have taken in others of this batch)
+          open = open && lane > l && fof_find<true>(a.group, pm, a.status) != fof_find<true>(a.group, pq, a.status);
+          left = __ballot_sync(0xffffffffu, open);
+        }
       }
     }
   }
@@ -356,8 +470,8 @@ cudaError_t launch_fof(const FofArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   k_fof_prep<<<(int)b, 256, 0, st>>>(a);
   k_fof_octants<<<a.num_sms * 8, 256, 0, st>>>(a);
-  k_fof_link_octants<<<a.num_sms * 8, 256, 0, st>>>(a);
-  k_fof_link<<<(int)b, 256, 0, st>>>(a);
+  k_fof_link_octants<<<a.num_sms * 8, 128, 0, st>>>(a);
+  k_fof_link<<<2 * (int)b, 128, 0, st>>>(a);
   k_fof_label<<<(int)b, 256, 0, st>>>(a);
   return cudaGetLastError();
 }
