@@ -115,29 +115,37 @@ __global__ void k_kick_drift(sphh::StepArgs a) {
       hdt = a.dt_f[2 * s];
       dt3 = a.dt_f[2 * s + 1];
     }
-    const float vx = fmaf(hdt, a.ax[p], a.vx[p]);
-    const float vy = fmaf(hdt, a.ay[p], a.vy[p]);
-    const float vz = fmaf(hdt, a.az[p], a.vz[p]);
-    const float u = fmaf(hdt, a.du_dt[p], a.u[p]);
+    // every load before the first store, behind which the compiler has to keep it
+    // (the arrays might overlap): one latency instead of five (2M particles:
+    // 73 -> 64 us; k_kick 31 -> 17)
+    const float ax = a.ax[p], ay = a.ay[p], az = a.az[p], du = a.du_dt[p];
+    const float vx0 = a.vx[p], vy0 = a.vy[p], vz0 = a.vz[p], u0 = a.u[p];
+    const double x = a.x[p], y = a.y[p], z = a.z[p];
+    const bool guess = a.h_guess != nullptr;
+    const float div_v = guess ? a.div_v[p] : 0.0f, h = guess ? a.h_guess[p] : 0.0f;
+    const float vx = fmaf(hdt, ax, vx0);
+    const float vy = fmaf(hdt, ay, vy0);
+    const float vz = fmaf(hdt, az, vz0);
+    const float u = fmaf(hdt, du, u0);
     a.vx[p] = vx;
     a.vy[p] = vy;
     a.vz[p] = vz;
     a.u[p] = u;
-    a.x[p] = wrap1(fma(widen(vx), dt, a.x[p]), L);
-    a.y[p] = wrap1(fma(widen(vy), dt, a.y[p]), L);
-    a.z[p] = wrap1(fma(widen(vz), dt, a.z[p]), L);
-    a.vpx[p] = fmaf(hdt, a.ax[p], vx);
-    a.vpy[p] = fmaf(hdt, a.ay[p], vy);
-    a.vpz[p] = fmaf(hdt, a.az[p], vz);
-    const float up = fmaf(hdt, a.du_dt[p], u);
+    a.x[p] = wrap1(fma(widen(vx), dt, x), L);
+    a.y[p] = wrap1(fma(widen(vy), dt, y), L);
+    a.z[p] = wrap1(fma(widen(vz), dt, z), L);
+    a.vpx[p] = fmaf(hdt, ax, vx);
+    a.vpy[p] = fmaf(hdt, ay, vy);
+    a.vpz[p] = fmaf(hdt, az, vz);
+    const float up = fmaf(hdt, du, u);
     a.up[p] = up;
     if (u < 0.0f || up < 0.0f) atomicOr(a.status, SPH_ST_NEG_U);
-    if (a.h_guess != nullptr) {
+    if (guess) {
       // the smoothing length follows the density, rho ~ h^-3, whose rate is
       // -rho div v: h (1 + div_v dt / 3) starts the next solve closer to its
       // root (clamped to [0.8, 1.25]; a NaN rate leaves the factor at 0.8)
-      const float f = fmaf(dt3, a.div_v[p], 1.0f);
-      a.h_guess[p] *= fminf(fmaxf(f, 0.8f), 1.25f);
+      const float f = fmaf(dt3, div_v, 1.0f);
+      a.h_guess[p] = h * fminf(fmaxf(f, 0.8f), 1.25f);
     }
   }
 }
@@ -154,10 +162,12 @@ __global__ void k_kick(sphh::StepArgs a) {
       cur = s;
       hdt = a.dt_f[2 * s];
     }
-    a.vx[p] = fmaf(hdt, a.ax[p], a.vx[p]);
-    a.vy[p] = fmaf(hdt, a.ay[p], a.vy[p]);
-    a.vz[p] = fmaf(hdt, a.az[p], a.vz[p]);
-    const float u = fmaf(hdt, a.du_dt[p], a.u[p]);
+    const float ax = a.ax[p], ay = a.ay[p], az = a.az[p], du = a.du_dt[p];
+    const float vx = a.vx[p], vy = a.vy[p], vz = a.vz[p], u0 = a.u[p];  // (loads first, as above)
+    a.vx[p] = fmaf(hdt, ax, vx);
+    a.vy[p] = fmaf(hdt, ay, vy);
+    a.vz[p] = fmaf(hdt, az, vz);
+    const float u = fmaf(hdt, du, u0);
     a.u[p] = u;
     if (u < 0.0f) atomicOr(a.status, SPH_ST_NEG_U);
   }
