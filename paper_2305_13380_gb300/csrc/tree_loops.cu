@@ -27,7 +27,7 @@
 // density of j emits it as a reverse pair (receiver i, source j).  Reverse
 // pairs are grouped by receiver and sorted by source (deterministic order).
 //
-// Force, one warp per leaf: each target walks its list and its reverse pairs.
+// Force, a warp per four targets: each walks its list and its reverse pairs.
 // The same kernels run the SPHENIX force and gradient pass (Sec. 3.3) with a
 // fifth record per source (kTSphenix, kTGradient).
 // Whether a pair is the list's or a reverse pair is decided in the target's
@@ -721,9 +721,10 @@ __device__ __forceinline__ void tdens_write(const sphh::TreeDensityArgs& a, cons
 // the window, so that a leaf's rounds, and with them the order of every sum, do
 // not depend on the windows nor on what else the pool holds.
 //
-// Bound by instruction issue and fetch: 24 warps per SM, 1,670 warp
-// instructions per particle.  On the 2M clustered box the call (build, density,
-// force) went from 11.10 to 7.13 ms and the kernel from 7.9 to 4.1 ms; before,
+// Bound by instruction issue (70 % of the slots): 24 warps per SM, 1,590 warp
+// instructions per particle, 3.85 ms on the 2M clustered box.  Taken together the
+// changes here took the call (build, density, force) from 11.10 to 7.13 ms and the
+// kernel from 7.9 to 4.1 ms; before,
 // every round staged the ~290 sources of its children in shared memory (18.6 KB
 // per warp, 12 warps per SM) and filtered them from there.  What counted: the
 // filter on sources held in registers, keeping only the ~90 listed ones (11.1
