@@ -29,6 +29,7 @@
 // does not fit the staging buffer is queued for k_density_overflow, which
 // streams each target cell's 27 cells through a per-warp buffer.
 #include "blocks.cuh"
+#include "per_device.h"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "stencil.cuh"
@@ -774,25 +775,19 @@ using namespace sphk;
 
 template <int K>
 static cudaError_t launch_density_k(const DensityArgs& a, const PhysDev& ph, cudaStream_t st) {
-  static int bps = 0, bps_o = 0;
-  if (!bps) {
-    cudaError_t e = cudaFuncSetAttribute(k_density<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)dens_blk_smem<K>());
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_density<K>, kBlkThreads, dens_blk_smem<K>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_density_overflow<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kOvfSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_o, k_density_overflow<K>, kThreads, kOvfSmem);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) bps = 1;
-    if (bps_o < 1) bps_o = 1;
-  }
-  cudaError_t e = cudaMemsetAsync(a.misc + kNumOverflow, 0, sizeof(int32_t), st);
+  static PerDevice<2> known;
+  int bps[2];  // resident blocks of the main and of the overflow kernel
+  cudaError_t e = known.get(bps, [](int (&v)[2]) {
+    cudaError_t r = opt_in(k_density<K>, dens_blk_smem<K>());
+    if (r == cudaSuccess) r = opt_in(k_density_overflow<K>, kOvfSmem);
+    if (r == cudaSuccess) r = resident_blocks(k_density<K>, kBlkThreads, dens_blk_smem<K>(), &v[0]);
+    if (r == cudaSuccess) r = resident_blocks(k_density_overflow<K>, kThreads, kOvfSmem, &v[1]);
+    return r;
+  });
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.misc + kNumOverflow, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  k_density<K><<<a.num_sms * bps, kBlkThreads, dens_blk_smem<K>(), st>>>(a, ph);
-  k_density_overflow<K><<<a.num_sms * bps_o, kThreads, kOvfSmem, st>>>(a, ph);
+  k_density<K><<<a.num_sms * bps[0], kBlkThreads, dens_blk_smem<K>(), st>>>(a, ph);
+  k_density_overflow<K><<<a.num_sms * bps[1], kThreads, kOvfSmem, st>>>(a, ph);
   return cudaGetLastError();
 }
 

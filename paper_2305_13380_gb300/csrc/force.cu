@@ -34,6 +34,7 @@
 // two blocks per SM (a 2.29-lattice-points-per-cell grid stages up to ~1050);
 // larger neighbourhoods go to the overflow kernel.
 #include "blocks.cuh"
+#include "per_device.h"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "stencil.cuh"
@@ -801,40 +802,34 @@ using namespace sphk;
 
 template <int kFl, int K>
 static cudaError_t launch_force_fk(const ForceArgs& a, const PhysDev& ph, const SphenixDev& x, cudaStream_t st) {
-  static int bps = 0, bps_o = 0;
+  static PerDevice<2> known;
+  int bps[2];  // resident blocks of the main and of the overflow kernel
   // the Minimal flavour with the cubic spline runs k_force_min
   constexpr bool kMin = kFl == kFlMinimal && K == kKernCubic;
   constexpr size_t kSmem = kMin ? kMinSmem : force_blk_smem<kFl, K>(), kSmemO = fovf_smem<kFl>();
-  if (!bps) {
-    cudaError_t e;
+  cudaError_t e = known.get(bps, [](int (&v)[2]) {
+    cudaError_t r;
     if (kMin) {
-      e = cudaFuncSetAttribute(k_force_min<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-      if (e != cudaSuccess) return e;
-      e = cudaFuncSetAttribute(k_force_min<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-      if (e != cudaSuccess) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_force_min<false>, kBlkThreads, kSmem);
+      r = opt_in(k_force_min<false>, kSmem);
+      if (r == cudaSuccess) r = opt_in(k_force_min<true>, kSmem);
+      if (r == cudaSuccess) r = resident_blocks(k_force_min<false>, kBlkThreads, kSmem, &v[0]);
     } else {
-      e = cudaFuncSetAttribute(k_force<kFl, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-      if (e != cudaSuccess) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_force<kFl, K>, kBlkThreads, kSmem);
+      r = opt_in(k_force<kFl, K>, kSmem);
+      if (r == cudaSuccess) r = resident_blocks(k_force<kFl, K>, kBlkThreads, kSmem, &v[0]);
     }
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_force_overflow<kFl, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemO);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_o, k_force_overflow<kFl, K>, kThreads, kSmemO);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) bps = 1;
-    if (bps_o < 1) bps_o = 1;
-  }
-  cudaError_t e = cudaMemsetAsync(a.misc + kNumOverflow, 0, sizeof(int32_t), st);
+    if (r == cudaSuccess) r = opt_in(k_force_overflow<kFl, K>, kSmemO);
+    if (r == cudaSuccess) r = resident_blocks(k_force_overflow<kFl, K>, kThreads, kSmemO, &v[1]);
+    return r;
+  });
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.misc + kNumOverflow, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   if (kMin && ph.count_pairs)
-    k_force_min<true><<<a.num_sms * bps, kBlkThreads, kSmem, st>>>(a, ph);
+    k_force_min<true><<<a.num_sms * bps[0], kBlkThreads, kSmem, st>>>(a, ph);
   else if (kMin)
-    k_force_min<false><<<a.num_sms * bps, kBlkThreads, kSmem, st>>>(a, ph);
+    k_force_min<false><<<a.num_sms * bps[0], kBlkThreads, kSmem, st>>>(a, ph);
   else
-    k_force<kFl, K><<<a.num_sms * bps, kBlkThreads, kSmem, st>>>(a, ph, x);
-  k_force_overflow<kFl, K><<<a.num_sms * bps_o, kThreads, kSmemO, st>>>(a, ph, x);
+    k_force<kFl, K><<<a.num_sms * bps[0], kBlkThreads, kSmem, st>>>(a, ph, x);
+  k_force_overflow<kFl, K><<<a.num_sms * bps[1], kThreads, kSmemO, st>>>(a, ph, x);
   return cudaGetLastError();
 }
 

@@ -23,6 +23,7 @@
 // A tile whose wait ran out, and those behind it, copy their items in place:
 // stale, but valid, keys and indices.
 #include "lookback.cuh"
+#include "per_device.h"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 
@@ -396,13 +397,13 @@ static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_o
   const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
   if (passes > kRadixMaxPasses) return cudaErrorInvalidValue;
   if (n <= kSmallMax) {
-    static bool set = false;
-    if (!set) {
-      const cudaError_t e = cudaFuncSetAttribute(k_radix_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)small_smem<K>());
-      if (e != cudaSuccess) return e;
-      set = true;
-    }
+    static PerDevice<1> known;
+    int bytes[1];
+    const cudaError_t e = known.get(bytes, [](int (&v)[1]) {
+      v[0] = (int)small_smem<K>();
+      return opt_in(k_radix_small<K>, small_smem<K>());
+    });
+    if (e != cudaSuccess) return e;
     const int warps = (int)((n + 32 * kSmallItems - 1) / (32 * kSmallItems));
     k_radix_small<K><<<1, 32 * (warps < 8 ? 8 : warps), small_smem<K>(), st>>>((int)n, keys, passes,
                                                                                want_keys ? keys_out : nullptr, vals_out);

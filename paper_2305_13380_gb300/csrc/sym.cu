@@ -23,6 +23,7 @@
 // Blocks whose neighbourhood exceeds the staging buffer are done in place, one
 // lane per target over the 27 cells read from global memory.
 #include "blocks.cuh"
+#include "per_device.h"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "stencil.cuh"
@@ -486,25 +487,22 @@ static int grid_sym(int64_t n, int threads) {
 int64_t sym_tiles(int64_t n) { return (n + kSymScanItems - 1) / kSymScanItems; }
 
 cudaError_t launch_force_sym(const ForceArgs& a, const SymArgs& y, const PhysDev& ph, int64_t n, cudaStream_t st) {
-  static int bps = 0;
-  if (!bps) {
-    cudaError_t e = cudaFuncSetAttribute(k_force_sym<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSymSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_force_sym<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSymSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_force_sym<false>, kBlkThreads, kSymSmem);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) bps = 1;
-  }
-  cudaError_t e = cudaMemsetAsync(y.counter, 0, sizeof(int32_t), st);
+  static PerDevice<1> known;
+  int bps[1];
+  cudaError_t e = known.get(bps, [](int (&v)[1]) {
+    cudaError_t r = opt_in(k_force_sym<false>, kSymSmem);
+    if (r == cudaSuccess) r = opt_in(k_force_sym<true>, kSymSmem);
+    if (r == cudaSuccess) r = resident_blocks(k_force_sym<false>, kBlkThreads, kSymSmem, &v[0]);
+    return r;
+  });
+  if (e == cudaSuccess) e = cudaMemsetAsync(y.counter, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(y.cnt, 0, sizeof(int32_t) * (size_t)n, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(y.cursor, 0, sizeof(int32_t) * (size_t)n, st);
   if (e != cudaSuccess) return e;
   if (ph.count_pairs)
-    k_force_sym<true><<<a.num_sms * bps, kBlkThreads, kSymSmem, st>>>(a, y, ph);
+    k_force_sym<true><<<a.num_sms * bps[0], kBlkThreads, kSymSmem, st>>>(a, y, ph);
   else
-    k_force_sym<false><<<a.num_sms * bps, kBlkThreads, kSymSmem, st>>>(a, y, ph);
+    k_force_sym<false><<<a.num_sms * bps[0], kBlkThreads, kSymSmem, st>>>(a, y, ph);
   if (n > 0) {
     const int64_t tiles = sym_tiles(n);
     k_sym_scan_tiles<<<(int)tiles, kSymScanThreads, 0, st>>>(n, y.cnt, y.off, y.tile_sum);

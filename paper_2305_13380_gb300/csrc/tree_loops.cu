@@ -34,6 +34,7 @@
 // own leaf frame with the same arithmetic as the density filter, so no pair is
 // counted twice or dropped at the boundary; emission uses a margin so that the
 // reverse pairs are a superset.
+#include "per_device.h"
 #include "sph_internal.cuh"
 #include "sph_launch.h"
 #include "tree.cuh"
@@ -1864,25 +1865,18 @@ static int tree_blocks(int64_t n) {
 
 template <int K>
 static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev& ph, cudaStream_t st) {
-  static int bps = 0, bps_fb = 0;
-  if (!bps) {
-    int b = 0;
-    cudaError_t e = cudaFuncSetAttribute(k_tree_density<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kTDensSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_tree_density<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTDensSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_tree_density_fb<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTFbSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_tree_density<K, false>, kTWarps * 32, kTDensSmem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps_fb, k_tree_density_fb<K>, kTWarps * 32, kTFbSmem);
-    if (e != cudaSuccess) return e;
-    if (bps_fb < 1) bps_fb = 1;
-    bps = b < 1 ? 1 : b;
-  }
+  static PerDevice<2> known;
+  int bps[2];  // resident blocks of the main and of the per-target kernel
+  cudaError_t e = known.get(bps, [](int (&v)[2]) {
+    cudaError_t r = opt_in(k_tree_density<K, false>, kTDensSmem);
+    if (r == cudaSuccess) r = opt_in(k_tree_density<K, true>, kTDensSmem);
+    if (r == cudaSuccess) r = opt_in(k_tree_density_fb<K>, kTFbSmem);
+    if (r == cudaSuccess) r = resident_blocks(k_tree_density<K, false>, kTWarps * 32, kTDensSmem, &v[0]);
+    if (r == cudaSuccess) r = resident_blocks(k_tree_density_fb<K>, kTWarps * 32, kTFbSmem, &v[1]);
+    return r;
+  });
   const int64_t n = a.n_total;
-  cudaError_t e = cudaMemsetAsync(a.rev_count, 0, sizeof(unsigned long long), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_count, 0, sizeof(unsigned long long), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_count, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_work, 0, sizeof(int32_t), st);
@@ -1891,12 +1885,12 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
   const int64_t want = (n + (int64_t)kTWin * kTWarps - 1) / ((int64_t)kTWin * kTWarps);
-  const int blocks = (int)(want < (int64_t)a.num_sms * bps ? want : (int64_t)a.num_sms * bps);
+  const int blocks = (int)(want < (int64_t)a.num_sms * bps[0] ? want : (int64_t)a.num_sms * bps[0]);
   if (a.act != nullptr)
     k_tree_density<K, true><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
   else
     k_tree_density<K, false><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
-  k_tree_density_fb<K><<<a.num_sms * bps_fb, kTWarps * 32, kTFbSmem, st>>>(a, ph);
+  k_tree_density_fb<K><<<a.num_sms * bps[1], kTWarps * 32, kTFbSmem, st>>>(a, ph);
   e = scan_exclusive(a.rev_start, a.rev_start, nullptr, n + 1, false, a.scan_tmp, a.status, a.num_sms, st);
   if (e != cudaSuccess) return e;
   k_rev_scatter<<<a.num_sms * 4, 256, 0, st>>>(a.rev_raw, a.rev_count, a.rev_cap, a.rev_start, a.rev_fill, a.rev);
@@ -1914,23 +1908,21 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
 template <int kFl, int K>
 static cudaError_t launch_tree_force_k(const TreeForceArgs& a, const PhysDev& ph, const SphenixDev& x,
                                        cudaStream_t st) {
-  static int bps = 0;
-  if (!bps) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_tree_force<kFl, K>, kTWarps * 32, 0);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) bps = 1;
-  }
-  cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
+  static PerDevice<1> known;
+  int bps[1];
+  cudaError_t e =
+      known.get(bps, [](int (&v)[1]) { return resident_blocks(k_tree_force<kFl, K>, kTWarps * 32, 0, &v[0]); });
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_work, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   // windows of two rounds; of one while that does not fill the resident warps
   // four times (6,000 particles 317 -> 302 us; 1M masked 1.59 -> 1.66 ms)
-  const int64_t warps = (int64_t)a.num_sms * bps * kTWarps;
+  const int64_t warps = (int64_t)a.num_sms * bps[0] * kTWarps;
   const int win = a.n_total < warps * 4 * kTPer ? kTPer : 2 * kTPer;
   const int64_t want = (a.n_total + (int64_t)win * kTWarps - 1) / ((int64_t)win * kTWarps);
-  const int blocks = (int)(want < (int64_t)a.num_sms * bps ? want : (int64_t)a.num_sms * bps);
+  const int blocks = (int)(want < (int64_t)a.num_sms * bps[0] ? want : (int64_t)a.num_sms * bps[0]);
   k_tree_force<kFl, K><<<blocks < 1 ? 1 : blocks, kTWarps * 32, 0, st>>>(a, ph, x, win);
-  k_tree_force_fb<kFl, K><<<a.num_sms * bps, kTWarps * 32, 0, st>>>(a, ph, x);
+  k_tree_force_fb<kFl, K><<<a.num_sms * bps[0], kTWarps * 32, 0, st>>>(a, ph, x);
   return cudaGetLastError();
 }
 
