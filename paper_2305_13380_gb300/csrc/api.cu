@@ -237,7 +237,7 @@ int ensure(sph_ctx* c, int64_t n, int n_sims, int cells_per_particle = 8) {
   const int64_t cc = (cells_per_particle > 8 ? cells_per_particle : 8) * cn + 216 * (int64_t)cs;
   bool ok = dalloc(c->grid, cs) && dalloc(c->key, cn) && dalloc(c->slot, cn) &&
             dalloc(c->cell_start, cc + 1) &&
-            dalloc(c->scan_sums, sphh::scan_words(cn + 1) + cn / 2048 + 2) && dalloc(c->perm, cn) &&
+            dalloc(c->scan_sums, sphh::scan_words(cn + 1) + cn / 1024 + 4) && dalloc(c->perm, cn) &&
             dalloc(c->rk, cn) && dalloc(c->rv, cn) && dalloc(c->rhist, sphh::radix_words(cn, (c->p.flags & SPH_FLAG_TREE) ? 8 : 4)) &&
             dalloc(c->overflow, (8 * cn + 216 * (int64_t)cs) / 3 + 2) && dalloc(c->pos4, cn) &&
             dalloc(c->vel4, cn) && dalloc(c->th4, cn) && dalloc(c->hs, cn) && dalloc(c->fD, cn) &&

@@ -13,25 +13,44 @@ namespace sphk {
 constexpr int kScanThreads = 256;
 constexpr int kScanWarps = kScanThreads / 32;
 
-// A published word: a count below 2^30 and its state (0: not yet).
-constexpr uint32_t kPubCount = 1u << 30;   // the tile's own count
-constexpr uint32_t kPubPrefix = 2u << 30;  // the inclusive prefix up to the tile
-constexpr uint32_t kPubFailed = 3u << 30;  // a wait ran out
-constexpr uint32_t kPubValue = (1u << 30) - 1u;
-constexpr int kPollLimit = 1 << 22;        // polls of one wait (seconds)
+// A published word: a value and, in the top two bits, its state (0: not yet).  The
+// sort's are of 32 bits, a digit's items (the library takes fewer than 2^27); the
+// scans' of 64, sums up to 2^31 - 1.
+template <class W>
+struct Pub {
+  static constexpr int kShift = 8 * (int)sizeof(W) - 2;
+  static constexpr W kCount = (W)1 << kShift;   // the tile's own count
+  static constexpr W kPrefix = (W)2 << kShift;  // the inclusive prefix up to the tile
+  static constexpr W kFailed = (W)3 << kShift;  // a wait ran out
+  static constexpr W kValue = kCount - 1;
+};
+constexpr int kPollLimit = 1 << 22;  // polls of one wait (seconds)
 
-__device__ __forceinline__ uint32_t pub_load(const uint32_t* p) { return *(const volatile uint32_t*)p; }
-__device__ __forceinline__ void pub_store(uint32_t* p, uint32_t v) { *(volatile uint32_t*)p = v; }
-__device__ __forceinline__ bool pub_is_last(uint32_t v) { return (v & kPubPrefix) != 0u; }  // a prefix, or a failure
-__device__ __forceinline__ bool pub_is_failed(uint32_t v) { return (v & kPubFailed) == kPubFailed; }
+template <class W>
+__device__ __forceinline__ W pub_load(const W* p) {
+  return *(const volatile W*)p;
+}
+template <class W>
+__device__ __forceinline__ void pub_store(W* p, W v) {
+  *(volatile W*)p = v;
+}
+template <class W>
+__device__ __forceinline__ bool pub_is_last(W v) {  // a prefix, or a failure
+  return (v & Pub<W>::kPrefix) != 0;
+}
+template <class W>
+__device__ __forceinline__ bool pub_is_failed(W v) {
+  return (v & Pub<W>::kFailed) == Pub<W>::kFailed;
+}
 
-__device__ __forceinline__ uint32_t pub_wait(const uint32_t* p) {
-  uint32_t v = pub_load(p);
-  for (int it = 0; v == 0u && it < kPollLimit; ++it) {
+template <class W>
+__device__ __forceinline__ W pub_wait(const W* p) {
+  W v = pub_load(p);
+  for (int it = 0; v == 0 && it < kPollLimit; ++it) {
     if (it > 8) __nanosleep(40);
     v = pub_load(p);
   }
-  return v != 0u ? v : kPubFailed;
+  return v != 0 ? v : Pub<W>::kFailed;
 }
 
 // Exclusive scan of one value per thread over a block of kScanThreads; total in
@@ -61,24 +80,25 @@ __device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* total) {
 // Publishes tile's count tot and finds the sum of the tiles before it, into
 // *before (-1 if a wait ran out).  Called by the block's first warp; 32 tiles
 // back at a time.
-__device__ __forceinline__ void lookback(uint32_t* pub, int32_t tile, int32_t tot, int32_t* before, int32_t* status) {
+__device__ __forceinline__ void lookback(uint64_t* pub, int32_t tile, int32_t tot, int32_t* before, int32_t* status) {
+  using P = Pub<uint64_t>;
   const int lane = threadIdx.x & 31;
-  if (lane == 0) pub_store(pub + tile, (tile == 0 ? kPubPrefix : kPubCount) | (uint32_t)tot);
+  if (lane == 0) pub_store(pub + tile, (tile == 0 ? P::kPrefix : P::kCount) | (uint64_t)tot);
   int32_t sum = 0;
   bool failed = false;
   for (int32_t t = tile - 1 - lane; tile > 0; t -= 32) {
-    const uint32_t w = t >= 0 ? pub_wait(pub + t) : kPubPrefix;
+    const uint64_t w = t >= 0 ? pub_wait(pub + t) : P::kPrefix;
     const unsigned last = __ballot_sync(0xffffffffu, pub_is_last(w));
     const bool use = last == 0u || lane < __ffs((int)last);
     failed = __any_sync(0xffffffffu, use && pub_is_failed(w));
-    int32_t x = use ? (int32_t)(w & kPubValue) : 0;
+    int32_t x = use ? (int32_t)(w & P::kValue) : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     sum += x;
     if (last != 0u || failed) break;
   }
   if (lane == 0) {
-    if (tile > 0) pub_store(pub + tile, failed ? kPubFailed : kPubPrefix | (uint32_t)(sum + tot));
+    if (tile > 0) pub_store(pub + tile, failed ? P::kFailed : P::kPrefix | (uint64_t)(sum + tot));
     if (failed) atomicOr(status, SPH_ST_TIMEOUT);
     *before = failed ? -1 : sum;
   }

@@ -102,6 +102,7 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
   __shared__ K skeys[kRadixTile];
   __shared__ int32_t svals[kRadixTile];
   __shared__ int32_t s_tile;
+  using Word = Pub<uint32_t>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d0 = threadIdx.x;
   const int32_t all = hist[d0];
   if (d0 == 0) s_tile = atomicAdd(ticket, 1);
@@ -146,7 +147,7 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
       mine += c;
     }
     uint32_t* my = pub + (int64_t)tile * 256 + d0;
-    pub_store(my, (tile == 0 ? kPubPrefix : kPubCount) | (uint32_t)mine);
+    pub_store(my, (tile == 0 ? Word::kPrefix : Word::kCount) | (uint32_t)mine);
     // the tile in order of digits, in shared memory
     int32_t cnt;
     const int32_t at0 = block_scan(mine, &cnt);
@@ -168,7 +169,7 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
       // the seven passes over 2M keys instead of 208, sixteen: 242)
       uint32_t v[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = t - i >= 0 ? pub_load(pub + (int64_t)(t - i) * 256 + d0) : kPubPrefix;
+      for (int i = 0; i < 4; ++i) v[i] = t - i >= 0 ? pub_load(pub + (int64_t)(t - i) * 256 + d0) : Word::kPrefix;
       bool stop = false;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -176,13 +177,13 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
           if (v[i] == 0u) v[i] = pub_wait(pub + (int64_t)(t - i) * 256 + d0);
           failed = failed || pub_is_failed(v[i]);
           stop = pub_is_last(v[i]);
-          if (!failed) before += (int32_t)(v[i] & kPubValue);
+          if (!failed) before += (int32_t)(v[i] & Word::kValue);
         }
       }
       if (stop) break;
       t -= 4;
     }
-    if (tile > 0) pub_store(my, failed ? kPubFailed : kPubPrefix | (uint32_t)(before + mine));
+    if (tile > 0) pub_store(my, failed ? Word::kFailed : Word::kPrefix | (uint32_t)(before + mine));
     first[d0] = dst0 + before - at0;
     copy = __syncthreads_or(failed);
     if (copy && d0 == 0) atomicOr(status, SPH_ST_TIMEOUT);
@@ -314,13 +315,14 @@ k_radix_small(int n, const K* __restrict__ keys_in, int passes, K* __restrict__ 
 }
 
 // Exclusive scan of in[0 .. len), len = *len_dev or len_host, into out (which
-// may be in); with_total: out[len] = the sum.  Sums stay below 2^30.
+// may be in); with_total: out[len] = the sum.  Sums up to 2^31 - 1 (a context
+// holds that many reverse pairs of the nested grids).
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
 __global__ void __launch_bounds__(kScanThreads)
 k_scan(const int32_t* in, int32_t* out, const int32_t* __restrict__ len_dev, int64_t len_host, int with_total,
-       int32_t* __restrict__ ticket, uint32_t* pub, int32_t* __restrict__ status) {
+       int32_t* __restrict__ ticket, uint64_t* pub, int32_t* __restrict__ status) {
   __shared__ int32_t s_tile, s_before;
   const int64_t len = len_dev != nullptr ? (int64_t)*len_dev : len_host;
   const int64_t tiles = len > 0 ? (len + kScanTile - 1) / kScanTile : 1;
@@ -449,19 +451,19 @@ cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, in
   return radix_sort_impl<int8_t>(n, 8, keys, nullptr, nullptr, false, vals_out, nullptr, scratch, status, st);
 }
 
-// tiles' published words after the tile counter
-int64_t scan_words(int64_t cap) { return (cap + kScanTile - 1) / kScanTile + 2; }
+// the tile counter, and from an 8-byte boundary a published word of 64 bits per tile
+int64_t scan_words(int64_t cap) { return 2 * ((cap + kScanTile - 1) / kScanTile) + 4; }
 
 cudaError_t scan_exclusive(const int32_t* in, int32_t* out, const int32_t* len_dev, int64_t cap, bool with_total,
                            int32_t* scratch, int32_t* status, int num_sms, cudaStream_t st) {
   const int64_t tiles = cap > 0 ? (cap + kScanTile - 1) / kScanTile : 1;
-  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)(tiles + 1), st);
+  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)(2 * tiles + 2), st);
   if (e != cudaSuccess) return e;
   // (the length may be known on the device only: blocks take tiles from the
   // counter, idle ones return at once)
   const int64_t most = (int64_t)num_sms * 6;
   k_scan<<<(unsigned)(tiles < most ? tiles : most), kScanThreads, 0, st>>>(
-      in, out, len_dev, cap, with_total ? 1 : 0, scratch, reinterpret_cast<uint32_t*>(scratch + 1), status);
+      in, out, len_dev, cap, with_total ? 1 : 0, scratch, reinterpret_cast<uint64_t*>(scratch + 2), status);
   return cudaGetLastError();
 }
 

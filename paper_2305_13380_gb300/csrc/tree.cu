@@ -134,7 +134,7 @@ constexpr int kLeafTile = kScanThreads * kLeafItems;
 __global__ void __launch_bounds__(kScanThreads)
 k_tree_leaves(int64_t n, const int32_t* __restrict__ tgt, const int8_t* __restrict__ level,
               const uint64_t* __restrict__ skey, int32_t* __restrict__ leaf_of, TreeLeaf* __restrict__ leaves,
-              int32_t* __restrict__ n_leaves, int32_t* __restrict__ ticket, uint32_t* pub,
+              int32_t* __restrict__ n_leaves, int32_t* __restrict__ ticket, uint64_t* pub,
               int32_t* __restrict__ status) {
   __shared__ int32_t s_tile, s_before;
   if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
@@ -277,10 +277,10 @@ cudaError_t launch_tree_build(const TreeBuildArgs& a, cudaStream_t st) {
   e = radix_partition(n, a.level, a.tgt, a.hist, a.status, st);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (n + kLeafTile - 1) / kLeafTile;
-  e = cudaMemsetAsync(a.scan_tmp, 0, sizeof(int32_t) * (size_t)(tiles + 1), st);
+  e = cudaMemsetAsync(a.scan_tmp, 0, sizeof(int32_t) * (size_t)(2 * tiles + 2), st);
   if (e != cudaSuccess) return e;
   k_tree_leaves<<<(unsigned)tiles, kScanThreads, 0, st>>>(n, a.tgt, a.level, a.skey, a.leaf_of, a.leaves, a.n_leaves,
-                                                         a.scan_tmp, reinterpret_cast<uint32_t*>(a.scan_tmp + 1),
+                                                         a.scan_tmp, reinterpret_cast<uint64_t*>(a.scan_tmp + 2),
                                                          a.status);
   k_tree_neigh<<<blocks_n(n * 4), 256, 0, st>>>(a.leaves, a.n_leaves, a.skey, n, a.cell_start, a.n_sims, a.grid,
                                                 a.ranges);

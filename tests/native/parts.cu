@@ -1,0 +1,14 @@
+// Parts of the library behind its entry points, for the tests that drive them
+// directly (linked with libsph.so).
+#include "../../paper_2305_13380_gb300/csrc/sph_internal.cuh"
+#include "../../paper_2305_13380_gb300/csrc/sph_launch.h"
+
+extern "C" {
+
+long part_scan_words(long n) { return sphh::scan_words(n); }
+int part_scan(const int32_t* in, int32_t* out, long n, int with_total, int32_t* scratch, int32_t* status,
+              cudaStream_t st) {
+  return (int)sphh::scan_exclusive(in, out, nullptr, n, with_total != 0, scratch, status, 152, st);
+}
+
+}
