@@ -59,8 +59,7 @@ enum {
   SPH_ST_REBUILD = 2,   /* a converged H is larger than the cell size        */
   SPH_ST_BOX = 4,       /* a support larger than half the box was needed     */
   SPH_ST_CAPACITY = 8,  /* a cell held more particles than a kernel handles  */
-  SPH_ST_NEG_U = 16,    /* a kick made some internal energy negative         */
-  SPH_ST_TIMEOUT = 32   /* a bounded device wait expired                     */
+  SPH_ST_NEG_U = 16     /* a kick made some internal energy negative         */
 };
 
 /* ---- context flags ------------------------------------------------------ */

@@ -237,7 +237,7 @@ int ensure(sph_ctx* c, int64_t n, int n_sims, int cells_per_particle = 8) {
   const int64_t cc = (cells_per_particle > 8 ? cells_per_particle : 8) * cn + 216 * (int64_t)cs;
   bool ok = dalloc(c->grid, cs) && dalloc(c->key, cn) && dalloc(c->slot, cn) &&
             dalloc(c->cell_start, cc + 1) &&
-            dalloc(c->scan_sums, sphh::scan_words(cn + 1) + cn / 1024 + 4) && dalloc(c->perm, cn) &&
+            dalloc(c->scan_sums, sphh::scan_words(cn) + cn / 1024 + 4) && dalloc(c->perm, cn) &&
             dalloc(c->rk, cn) && dalloc(c->rv, cn) && dalloc(c->rhist, sphh::radix_words(cn, (c->p.flags & SPH_FLAG_TREE) ? 8 : 4)) &&
             dalloc(c->overflow, (8 * cn + 216 * (int64_t)cs) / 3 + 2) && dalloc(c->pos4, cn) &&
             dalloc(c->vel4, cn) && dalloc(c->th4, cn) && dalloc(c->hs, cn) && dalloc(c->fD, cn) &&
@@ -423,7 +423,6 @@ int cuda_code(cudaError_t e) { return e == cudaSuccess ? SPH_OK : SPH_E_CUDA; }
 
 // Maps device status bits to the most severe return code.
 int code_of_status(int32_t s) {
-  if (s & SPH_ST_TIMEOUT) return SPH_E_TIMEOUT;
   if (s & SPH_ST_BOX) return SPH_E_BOX;
   if (s & SPH_ST_CAPACITY) return SPH_E_CAPACITY;
   if (s & SPH_ST_REBUILD) return SPH_E_REBUILD;
@@ -523,7 +522,6 @@ int do_build(sph_ctx* c, int n_sims, int64_t n_total, const int64_t* off, const 
     t.hist = c->rhist;
     t.leaf_of = c->leaf_of;
     t.scan_tmp = c->scan_sums;
-    t.status = c->misc + sphk::kStatus;
     t.num_sms = c->num_sms;
     t.leaves = c->leaves;
     t.n_leaves = c->n_leaves;
@@ -627,7 +625,7 @@ int do_tree_density(sph_ctx* c, const double* x, const double* y, const double* 
     const int rc = ensure_act(c, c->built_n);
     if (rc != SPH_OK) return rc;
     if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, c->act_pre, c->scan_sums,
-                               c->misc + sphk::kStatus, c->num_sms, c->st) !=
+                               c->num_sms, c->st) !=
         cudaSuccess)
       return SPH_E_CUDA;
     d.act = c->act_s;
@@ -882,7 +880,7 @@ int do_force(sph_ctx* c, const double* x, const double* y, const double* z, cons
     if (active) {
       const int rc = ensure_act(c, c->built_n);
       if (rc != SPH_OK) return rc;
-      if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, nullptr, nullptr, nullptr, 0, c->st) != cudaSuccess)
+      if (sphh::launch_tree_mask(c->built_n, c->perm, active, c->act_s, nullptr, nullptr, 0, c->st) != cudaSuccess)
         return SPH_E_CUDA;
       a.act = c->act_s;
     }
@@ -1508,7 +1506,7 @@ int hier_substep(sph_ctx* c, const sph_pool* pl, int32_t* bins, int64_t* tbeg, d
     a.wake = c->hwake;
     if (cudaMemsetAsync(c->hwake, 0xff, (size_t)n * sizeof(int32_t), c->st) != cudaSuccess ||
         sphh::launch_gather_bins(n, c->perm, bins, c->sx4, c->st) != cudaSuccess ||
-        sphh::launch_tree_mask(n, c->perm, c->hact, c->act_s, nullptr, nullptr, nullptr, 0, c->st) != cudaSuccess ||
+        sphh::launch_tree_mask(n, c->perm, c->hact, c->act_s, nullptr, nullptr, 0, c->st) != cudaSuccess ||
         sphh::launch_tree_wake(a, phys_of(c->p), c->st) != cudaSuccess)
       return SPH_E_CUDA;
     h.wake = c->hwake;

@@ -365,8 +365,7 @@ cudaError_t launch_build(const BuildArgs& a, cudaStream_t st) {
   if (!a.sort_cells) return cudaGetLastError();  // (the nested grids sort finer keys first)
   int bits = 1;
   while (bits < 31 && ((int64_t)1 << bits) <= a.cap_cells) ++bits;
-  const cudaError_t e =
-      radix_sort_index(a.n_total, bits, a.key, a.rk, a.slot, a.perm, a.rv, a.hist, a.misc + kStatus, st);
+  const cudaError_t e = radix_sort_index(a.n_total, bits, a.key, a.rk, a.slot, a.perm, a.rv, a.hist, st);
   if (e != cudaSuccess) return e;
   cell_bounds(a.n_total, a.rk, 0, a.cap_cells, a.num_sms, a.misc, a.cell_start, st);
   return cudaGetLastError();

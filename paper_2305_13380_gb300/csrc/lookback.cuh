@@ -3,8 +3,9 @@
 // prefix when it knows it; a reader adds the counts of the tiles before it
 // until it meets a prefix.  Tiles are numbered by a counter as blocks start, so
 // every tile that a block waits for is already running; the waits are bounded
-// all the same, and one that runs out sets SPH_ST_TIMEOUT and is passed on as a
-// failure to the tiles behind it.
+// all the same, and a block whose wait runs out counts the items of all tiles
+// before its own itself (the inputs are not written while a launch reads them):
+// slower, the same prefix.
 #pragma once
 #include "sph_internal.cuh"
 
@@ -21,28 +22,29 @@ struct Pub {
   static constexpr int kShift = 8 * (int)sizeof(W) - 2;
   static constexpr W kCount = (W)1 << kShift;   // the tile's own count
   static constexpr W kPrefix = (W)2 << kShift;  // the inclusive prefix up to the tile
-  static constexpr W kFailed = (W)3 << kShift;  // a wait ran out
   static constexpr W kValue = kCount - 1;
 };
-constexpr int kPollLimit = 1 << 22;  // polls of one wait (seconds)
+// Polls of one wait (seconds).  -1: no published word is ever seen, every tile
+// counts for itself (the tests build that).
+#ifndef SPH_POLL_LIMIT
+#define SPH_POLL_LIMIT (1 << 22)
+#endif
+constexpr int kPollLimit = SPH_POLL_LIMIT;
 
 template <class W>
 __device__ __forceinline__ W pub_load(const W* p) {
-  return *(const volatile W*)p;
+  return kPollLimit < 0 ? (W)0 : *(const volatile W*)p;
 }
 template <class W>
 __device__ __forceinline__ void pub_store(W* p, W v) {
   *(volatile W*)p = v;
 }
 template <class W>
-__device__ __forceinline__ bool pub_is_last(W v) {  // a prefix, or a failure
+__device__ __forceinline__ bool pub_is_prefix(W v) {
   return (v & Pub<W>::kPrefix) != 0;
 }
-template <class W>
-__device__ __forceinline__ bool pub_is_failed(W v) {
-  return (v & Pub<W>::kFailed) == Pub<W>::kFailed;
-}
 
+// The word, or 0 if the wait ran out.
 template <class W>
 __device__ __forceinline__ W pub_wait(const W* p) {
   W v = pub_load(p);
@@ -50,7 +52,7 @@ __device__ __forceinline__ W pub_wait(const W* p) {
     if (it > 8) __nanosleep(40);
     v = pub_load(p);
   }
-  return v != 0 ? v : Pub<W>::kFailed;
+  return v;
 }
 
 // Exclusive scan of one value per thread over a block of kScanThreads; total in
@@ -77,31 +79,47 @@ __device__ __forceinline__ int32_t block_scan(int32_t v, int32_t* total) {
   return wbase + x - v;
 }
 
-// Publishes tile's count tot and finds the sum of the tiles before it, into
-// *before (-1 if a wait ran out).  Called by the block's first warp; 32 tiles
-// back at a time.
-__device__ __forceinline__ void lookback(uint64_t* pub, int32_t tile, int32_t tot, int32_t* before, int32_t* status) {
+// Publishes tile's count tot and finds the sum of the tiles before it.  Called by
+// the block's first warp; 32 tiles back at a time.  -1 if a wait ran out.
+__device__ __forceinline__ int32_t lookback(uint64_t* pub, int32_t tile, int32_t tot) {
   using P = Pub<uint64_t>;
   const int lane = threadIdx.x & 31;
   if (lane == 0) pub_store(pub + tile, (tile == 0 ? P::kPrefix : P::kCount) | (uint64_t)tot);
   int32_t sum = 0;
-  bool failed = false;
   for (int32_t t = tile - 1 - lane; tile > 0; t -= 32) {
     const uint64_t w = t >= 0 ? pub_wait(pub + t) : P::kPrefix;
-    const unsigned last = __ballot_sync(0xffffffffu, pub_is_last(w));
+    const unsigned last = __ballot_sync(0xffffffffu, pub_is_prefix(w));
     const bool use = last == 0u || lane < __ffs((int)last);
-    failed = __any_sync(0xffffffffu, use && pub_is_failed(w));
+    if (__any_sync(0xffffffffu, use && w == 0)) return -1;
     int32_t x = use ? (int32_t)(w & P::kValue) : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     sum += x;
-    if (last != 0u || failed) break;
+    if (last != 0u) break;
   }
-  if (lane == 0) {
-    if (tile > 0) pub_store(pub + tile, failed ? P::kFailed : P::kPrefix | (uint64_t)(sum + tot));
-    if (failed) atomicOr(status, SPH_ST_TIMEOUT);
-    *before = failed ? -1 : sum;
+  if (lane == 0 && tile > 0) pub_store(pub + tile, P::kPrefix | (uint64_t)(sum + tot));
+  return sum;
+}
+
+// The sum of the tiles before tile, of `items` items in all, for every thread of
+// the block: by look-back, or counted (count(i): item i's) where a wait ran out.
+// (*s_before is free again after the caller's next barrier.)
+template <class Count>
+__device__ __forceinline__ int32_t tiles_before(uint64_t* pub, int32_t tile, int32_t tot, int64_t items,
+                                                int32_t* s_before, Count count) {
+  if (threadIdx.x < 32) {
+    const int32_t b = lookback(pub, tile, tot);
+    if (threadIdx.x == 0) *s_before = b;
   }
+  __syncthreads();
+  const int32_t before = *s_before;
+  if (before >= 0) return before;
+  int32_t mine = 0, all;
+#pragma unroll 1
+  for (int64_t i = threadIdx.x; i < items; i += kScanThreads) mine += count(i);
+  block_scan(mine, &all);
+  if (threadIdx.x == 0) pub_store(pub + tile, Pub<uint64_t>::kPrefix | (uint64_t)(all + tot));
+  return all;
 }
 
 }  // namespace sphk

@@ -20,8 +20,8 @@
 // scatter).  6,000 keys, six passes: 58 us with the histogram as launches, 36 in
 // one block, which is bound by its one SM.
 //
-// A tile whose wait ran out, and those behind it, copy their items in place:
-// stale, but valid, keys and indices.
+// A tile whose wait ran out counts the digits before it itself (lookback.cuh): the
+// same order.
 #include "lookback.cuh"
 #include "per_device.h"
 #include "sph_internal.cuh"
@@ -96,7 +96,7 @@ template <class K>
 __global__ void __launch_bounds__(kScanThreads)
 k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int shift,
              const int32_t* __restrict__ hist, int32_t* __restrict__ ticket, uint32_t* pub, K* __restrict__ keys_out,
-             int32_t* __restrict__ vals_out, int32_t* __restrict__ status) {
+             int32_t* __restrict__ vals_out) {
   __shared__ int32_t wcount[kScanWarps][256];
   __shared__ int32_t first[256];  // place of digit d's item i of the ordered tile: first[d] + i
   __shared__ K skeys[kRadixTile];
@@ -118,11 +118,9 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
     key[j] = p < n ? keys_in[p] : (K)0;
     val[j] = p < n ? (vals_in != nullptr ? vals_in[p] : (int32_t)p) : 0;
   }
-  bool copy = same;  // every key has this digit
-  int32_t dst0 = 0;
-  if (!copy) {
+  if (!same) {  // (else every key has this digit)
     int32_t tot_all;
-    dst0 = block_scan(all, &tot_all);  // first place of digit d0
+    const int32_t dst0 = block_scan(all, &tot_all);  // first place of digit d0
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int j = 0; j < kRadixItems; ++j) {
@@ -163,7 +161,7 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
       }
     }
     int32_t before = 0;
-    bool failed = false;
+    bool expired = false;
     for (int32_t t = tile - 1; t >= 0;) {
       // four tiles back at a time, their words in flight together (eight: 230 us for
       // the seven passes over 2M keys instead of 208, sixteen: 242)
@@ -175,32 +173,40 @@ k_radix_pass(int64_t n, const K* __restrict__ keys_in, const int32_t* __restrict
       for (int i = 0; i < 4; ++i) {
         if (!stop && t - i >= 0) {
           if (v[i] == 0u) v[i] = pub_wait(pub + (int64_t)(t - i) * 256 + d0);
-          failed = failed || pub_is_failed(v[i]);
-          stop = pub_is_last(v[i]);
-          if (!failed) before += (int32_t)(v[i] & Word::kValue);
+          expired = v[i] == 0u;
+          stop = expired || pub_is_prefix(v[i]);
+          before += (int32_t)(v[i] & Word::kValue);
         }
       }
       if (stop) break;
       t -= 4;
     }
-    if (tile > 0) pub_store(my, failed ? Word::kFailed : Word::kPrefix | (uint32_t)(before + mine));
+    if (tile > 0 && !expired) pub_store(my, Word::kPrefix | (uint32_t)(before + mine));
     first[d0] = dst0 + before - at0;
-    copy = __syncthreads_or(failed);
-    if (copy && d0 == 0) atomicOr(status, SPH_ST_TIMEOUT);
-    if (!copy) {
-      // equal digits leave as runs of consecutive places
-#pragma unroll
-      for (int j = 0; j < kRadixItems; ++j) {
-        const int at = j * kScanThreads + d0;
-        if (at < cnt) {
-          const K k = skeys[at];
-          const int64_t dst = (int64_t)first[(int)((k >> shift) & 255)] + at;
-          if (keys_out != nullptr) keys_out[dst] = k;
-          vals_out[dst] = svals[at];
-        }
-      }
-      return;
+    if (__syncthreads_or(expired)) {
+      wcount[0][d0] = 0;
+      __syncthreads();
+#pragma unroll 1
+      for (int64_t p = d0; p < (int64_t)tile * kRadixTile; p += kScanThreads)
+        atomicAdd(&wcount[0][(int)((keys_in[p] >> shift) & 255)], 1);
+      __syncthreads();
+      before = wcount[0][d0];
+      pub_store(my, Word::kPrefix | (uint32_t)(before + mine));
+      first[d0] = dst0 + before - at0;
+      __syncthreads();
     }
+    // equal digits leave as runs of consecutive places
+#pragma unroll
+    for (int j = 0; j < kRadixItems; ++j) {
+      const int at = j * kScanThreads + d0;
+      if (at < cnt) {
+        const K k = skeys[at];
+        const int64_t dst = (int64_t)first[(int)((k >> shift) & 255)] + at;
+        if (keys_out != nullptr) keys_out[dst] = k;
+        vals_out[dst] = svals[at];
+      }
+    }
+    return;
   }
 #pragma unroll
   for (int j = 0; j < kRadixItems; ++j) {
@@ -314,18 +320,18 @@ k_radix_small(int n, const K* __restrict__ keys_in, int passes, K* __restrict__ 
   }
 }
 
-// Exclusive scan of in[0 .. len), len = *len_dev or len_host, into out (which
-// may be in); with_total: out[len] = the sum.  Sums up to 2^31 - 1 (a context
-// holds that many reverse pairs of the nested grids).
+// Exclusive scan of in[0 .. n) into out, and the sum at out[n].  out is not in (a
+// tile whose wait ran out reads what lies before it again).  Sums up to 2^31 - 1 (a
+// context holds that many reverse pairs of the nested grids).
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
+template <class T>
 __global__ void __launch_bounds__(kScanThreads)
-k_scan(const int32_t* in, int32_t* out, const int32_t* __restrict__ len_dev, int64_t len_host, int with_total,
-       int32_t* __restrict__ ticket, uint64_t* pub, int32_t* __restrict__ status) {
+k_scan(const T* __restrict__ in, int32_t* __restrict__ out, int64_t n, int32_t* __restrict__ ticket, uint64_t* pub) {
+  constexpr int kLoad = 16 / (int)sizeof(T);  // items of 16 bytes
   __shared__ int32_t s_tile, s_before;
-  const int64_t len = len_dev != nullptr ? (int64_t)*len_dev : len_host;
-  const int64_t tiles = len > 0 ? (len + kScanTile - 1) / kScanTile : 1;
+  const int64_t tiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
   const bool vec = (((uintptr_t)in | (uintptr_t)out) & 15u) == 0u;
   for (;;) {
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
@@ -334,30 +340,29 @@ k_scan(const int32_t* in, int32_t* out, const int32_t* __restrict__ len_dev, int
     if (tile >= tiles) return;
     const int64_t c0 = (int64_t)tile * kScanTile + threadIdx.x * kScanItems;
     int32_t v[kScanItems];
-    if (vec && c0 + kScanItems <= len) {
+    if (vec && c0 + kScanItems <= n) {
 #pragma unroll
-      for (int i = 0; i < kScanItems; i += 4) {
-        const int4 q = *reinterpret_cast<const int4*>(in + c0 + i);
-        v[i] = q.x;
-        v[i + 1] = q.y;
-        v[i + 2] = q.z;
-        v[i + 3] = q.w;
+      for (int i = 0; i < kScanItems; i += kLoad) {
+        const uint4 q = *reinterpret_cast<const uint4*>(in + c0 + i);
+        const uint32_t word[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int k = 0; k < kLoad; ++k)
+          v[i + k] = sizeof(T) == 4 ? (int32_t)word[k & 3] : (int32_t)((word[k >> 2] >> (8 * (k & 3))) & 255u);
       }
     } else {
 #pragma unroll
-      for (int i = 0; i < kScanItems; ++i) v[i] = c0 + i < len ? in[c0 + i] : 0;
+      for (int i = 0; i < kScanItems; ++i) v[i] = c0 + i < n ? (int32_t)in[c0 + i] : 0;
     }
     int32_t s = 0;
 #pragma unroll
     for (int i = 0; i < kScanItems; ++i) s += v[i];
     int32_t tot;
     int32_t run = block_scan(s, &tot);
-    if (threadIdx.x < 32) lookback(pub, tile, tot, &s_before, status);
-    __syncthreads();
-    const int32_t before = s_before >= 0 ? s_before : 0;
+    const int32_t before = tiles_before(pub, tile, tot, (int64_t)tile * kScanTile, &s_before,
+                                        [&](int64_t i) { return (int32_t)in[i]; });
     run += before;
-    if (with_total && tile == tiles - 1 && threadIdx.x == 0) out[len] = before + tot;
-    if (vec && c0 + kScanItems <= len) {
+    if (tile == tiles - 1 && threadIdx.x == 0) out[n] = before + tot;
+    if (vec && c0 + kScanItems <= n) {
 #pragma unroll
       for (int i = 0; i < kScanItems; i += 4) {
         int4 q;
@@ -371,7 +376,7 @@ k_scan(const int32_t* in, int32_t* out, const int32_t* __restrict__ len_dev, int
     } else {
 #pragma unroll
       for (int i = 0; i < kScanItems; ++i) {
-        if (c0 + i < len) out[c0 + i] = run;
+        if (c0 + i < n) out[c0 + i] = run;
         run += v[i];
       }
     }
@@ -392,8 +397,7 @@ int64_t radix_words(int64_t n, int passes) {
 
 template <class K>
 static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_out, K* keys_tmp, bool want_keys,
-                                   int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
-                                   cudaStream_t st) {
+                                   int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int64_t tiles = (n + kRadixTile - 1) / kRadixTile;
   const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
@@ -426,8 +430,7 @@ static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_o
     int32_t* v_out = odd ? vals_tmp : vals_out;
     k_radix_pass<K><<<(unsigned)tiles, kScanThreads, 0, st>>>(n, k_in, v_in, 8 * p, hist + 256 * p, ticket + p,
                                                                pub + (int64_t)p * tiles * 256,
-                                                               p == passes - 1 && !want_keys ? nullptr : k_out, v_out,
-                                                               status);
+                                                               p == passes - 1 && !want_keys ? nullptr : k_out, v_out);
     k_in = k_out;
     v_in = v_out;
   }
@@ -435,36 +438,41 @@ static cudaError_t radix_sort_impl(int64_t n, int bits, const K* keys, K* keys_o
 }
 
 cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* keys_out, int32_t* keys_tmp,
-                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
-                             cudaStream_t st) {
-  return radix_sort_impl<int32_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, status, st);
+                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, cudaStream_t st) {
+  return radix_sort_impl<int32_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, st);
 }
 
 cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,
-                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
-                               cudaStream_t st) {
-  return radix_sort_impl<uint64_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, status, st);
+                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, cudaStream_t st) {
+  return radix_sort_impl<uint64_t>(n, bits, keys, keys_out, keys_tmp, true, vals_out, vals_tmp, scratch, st);
 }
 
-cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, int32_t* status,
-                            cudaStream_t st) {
-  return radix_sort_impl<int8_t>(n, 8, keys, nullptr, nullptr, false, vals_out, nullptr, scratch, status, st);
+cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, cudaStream_t st) {
+  return radix_sort_impl<int8_t>(n, 8, keys, nullptr, nullptr, false, vals_out, nullptr, scratch, st);
 }
 
 // the tile counter, and from an 8-byte boundary a published word of 64 bits per tile
-int64_t scan_words(int64_t cap) { return 2 * ((cap + kScanTile - 1) / kScanTile) + 4; }
+int64_t scan_words(int64_t n) { return 2 * ((n + kScanTile - 1) / kScanTile) + 4; }
 
-cudaError_t scan_exclusive(const int32_t* in, int32_t* out, const int32_t* len_dev, int64_t cap, bool with_total,
-                           int32_t* scratch, int32_t* status, int num_sms, cudaStream_t st) {
-  const int64_t tiles = cap > 0 ? (cap + kScanTile - 1) / kScanTile : 1;
-  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)(2 * tiles + 2), st);
+template <class T>
+static cudaError_t scan_impl(const T* in, int32_t* out, int64_t n, int32_t* scratch, int num_sms, cudaStream_t st) {
+  const int64_t tiles = n > 0 ? (n + kScanTile - 1) / kScanTile : 1;
+  const cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int32_t) * (size_t)(2 * tiles + 2), st);
   if (e != cudaSuccess) return e;
-  // (the length may be known on the device only: blocks take tiles from the
-  // counter, idle ones return at once)
   const int64_t most = (int64_t)num_sms * 6;
-  k_scan<<<(unsigned)(tiles < most ? tiles : most), kScanThreads, 0, st>>>(
-      in, out, len_dev, cap, with_total ? 1 : 0, scratch, reinterpret_cast<uint64_t*>(scratch + 2), status);
+  k_scan<T><<<(unsigned)(tiles < most ? tiles : most), kScanThreads, 0, st>>>(
+      in, out, n, scratch, reinterpret_cast<uint64_t*>(scratch + 2));
   return cudaGetLastError();
+}
+
+cudaError_t scan_exclusive(const int32_t* in, int32_t* out, int64_t n, int32_t* scratch, int num_sms,
+                           cudaStream_t st) {
+  return scan_impl(in, out, n, scratch, num_sms, st);
+}
+
+cudaError_t scan_exclusive(const uint8_t* in, int32_t* out, int64_t n, int32_t* scratch, int num_sms,
+                           cudaStream_t st) {
+  return scan_impl(in, out, n, scratch, num_sms, st);
 }
 
 }  // namespace sphh

@@ -64,19 +64,18 @@ cudaError_t launch_fof(const FofArgs& a, cudaStream_t st);
 // are left as they are.
 int64_t radix_words(int64_t n, int passes);
 cudaError_t radix_sort_index(int64_t n, int bits, const int32_t* keys, int32_t* keys_out, int32_t* keys_tmp,
-                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status, cudaStream_t st);
+                             int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, cudaStream_t st);
 cudaError_t radix_sort_index64(int64_t n, int bits, const uint64_t* keys, uint64_t* keys_out, uint64_t* keys_tmp,
-                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, int32_t* status,
-                               cudaStream_t st);
+                               int32_t* vals_out, int32_t* vals_tmp, int32_t* scratch, cudaStream_t st);
 // The indices 0..n-1 by ascending key (0..127), equal keys in ascending order.
-cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, int32_t* status,
-                            cudaStream_t st);
-// Exclusive scan of int32 (radix.cu), in place if out is in: of *len_dev <= cap
-// entries, or of cap where len_dev is null; with_total: the sum at out[length].
-// scratch: scan_words(cap).
-int64_t scan_words(int64_t cap);
-cudaError_t scan_exclusive(const int32_t* in, int32_t* out, const int32_t* len_dev, int64_t cap, bool with_total,
-                           int32_t* scratch, int32_t* status, int num_sms, cudaStream_t st);
+cudaError_t radix_partition(int64_t n, const int8_t* keys, int32_t* vals_out, int32_t* scratch, cudaStream_t st);
+// Exclusive scan of n counts (radix.cu), the sum at out[n]; out is not in.
+// scratch: scan_words(n).
+int64_t scan_words(int64_t n);
+cudaError_t scan_exclusive(const int32_t* in, int32_t* out, int64_t n, int32_t* scratch, int num_sms,
+                           cudaStream_t st);
+cudaError_t scan_exclusive(const uint8_t* in, int32_t* out, int64_t n, int32_t* scratch, int num_sms,
+                           cudaStream_t st);
 
 struct GatherDensityArgs {
   int64_t n_total;
@@ -323,8 +322,7 @@ struct TreeBuildArgs {
   int32_t* tgt;               // n: target order -> source index
   int32_t *rv, *hist;         // radix scratch
   int32_t* leaf_of;           // n: target order -> its group
-  int32_t* scan_tmp;          // scan_words(n)
-  int32_t* status;
+  int32_t* scan_tmp;          // 2 n / 2048 + 4
   int num_sms;
   sphk::TreeLeaf* leaves;     // n + 1: target groups, start in target order
   int32_t* n_leaves;          // 1 (device)
@@ -381,11 +379,11 @@ struct TreeDensityArgs {
   uint16_t* list_cnt;
   uint64_t* rev_raw;   // rev_cap emitted pairs (receiver << 32 | packed source)
   unsigned long long* rev_count;  // 1: pairs emitted (may exceed rev_cap)
-  int32_t* rev_start;  // n + 1: per-receiver counts, then their exclusive scan
-  int32_t* rev_fill;   // n: scatter cursors
+  int32_t* rev_start;  // n + 1: first place of each receiver's pairs
+  int32_t* rev_fill;   // n: per-receiver counts, then scatter cursors, then the sort's queue
   uint32_t* rev;       // rev_cap: packed sources ordered by (receiver, source)
   int64_t rev_cap;
-  int32_t* scan_tmp;   // scan_words(n + 1)
+  int32_t* scan_tmp;   // scan_words(n)
   int32_t* work;       // 1: group counter (reset by the launcher)
   // targets whose support outgrew their level, re-solved one level coarser
   const uint64_t* skey;        // n: source keys
@@ -403,9 +401,9 @@ struct TreeDensityArgs {
 };
 cudaError_t launch_tree_density(const TreeDensityArgs& a, const sphk::PhysDev& ph, cudaStream_t st);
 // The mask in tree order: out[k] = active[perm[k]]; with pre (n + 1 int32,
-// scan scratch tmp of scan_words(n + 1)) also its exclusive prefix sums.
+// scan scratch tmp of scan_words(n)) also its exclusive prefix sums.
 cudaError_t launch_tree_mask(int64_t n, const int32_t* perm, const uint8_t* active, uint8_t* out, int32_t* pre,
-                             int32_t* tmp, int32_t* status, int num_sms, cudaStream_t st);
+                             int32_t* tmp, int num_sms, cudaStream_t st);
 
 struct TreeForceArgs {
   int n_sims;

@@ -128,14 +128,13 @@ __global__ void k_tree_level(int64_t n, const uint64_t* __restrict__ skey, const
 // The groups in target order: a target whose level or cell differs from the
 // one before it starts a group.  Each target's group (leaf_of), the group
 // records with a sentinel, and their number; tiles of 2048 targets, prefixed by
-// look-back (a wait that runs out leaves no groups).
+// look-back.
 constexpr int kLeafItems = 8;
 constexpr int kLeafTile = kScanThreads * kLeafItems;
 __global__ void __launch_bounds__(kScanThreads)
 k_tree_leaves(int64_t n, const int32_t* __restrict__ tgt, const int8_t* __restrict__ level,
               const uint64_t* __restrict__ skey, int32_t* __restrict__ leaf_of, TreeLeaf* __restrict__ leaves,
-              int32_t* __restrict__ n_leaves, int32_t* __restrict__ ticket, uint64_t* pub,
-              int32_t* __restrict__ status) {
+              int32_t* __restrict__ n_leaves, int32_t* __restrict__ ticket, uint64_t* pub) {
   __shared__ int32_t s_tile, s_before;
   if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1);
   __syncthreads();
@@ -168,10 +167,13 @@ k_tree_leaves(int64_t n, const int32_t* __restrict__ tgt, const int8_t* __restri
   }
   int32_t tot;
   int32_t at = block_scan(__popc(first), &tot);
-  if (threadIdx.x < 32) lookback(pub, tile, tot, &s_before, status);
-  __syncthreads();
-  const bool ok = s_before >= 0;
-  at += ok ? s_before : 0;
+  const int32_t before = tiles_before(pub, tile, tot, (int64_t)tile * kLeafTile, &s_before, [&](int64_t k) {
+    if (k == 0) return 1;
+    const int32_t s = tgt[k], r = tgt[k - 1];
+    const int sh = 3 * (kTreeDepth - level[s]);
+    return level[s] != level[r] || (skey[s] >> sh) != (skey[r] >> sh) ? 1 : 0;
+  });
+  at += before;
 #pragma unroll
   for (int i = 0; i < kLeafItems; ++i) {
     const int64_t k = k0 + i;
@@ -185,7 +187,7 @@ k_tree_leaves(int64_t n, const int32_t* __restrict__ tgt, const int8_t* __restri
     }
   }
   if (threadIdx.x == 0 && ((int64_t)tile + 1) * kLeafTile >= n) {
-    const int32_t nl = ok ? s_before + tot : 0;
+    const int32_t nl = before + tot;
     *n_leaves = nl;
     leaves[nl].start = (int32_t)n;  // sentinel: end of the last group
   }
@@ -267,21 +269,20 @@ cudaError_t launch_tree_build(const TreeBuildArgs& a, cudaStream_t st) {
   while (cbits < 30 && ((int64_t)1 << cbits) <= a.cap_cells) ++cbits;
   // source order: (top cell, Morton code), ties by pool index
   k_tree_key<<<blocks_n(n), 256, 0, st>>>(n, a.x, a.y, a.z, a.sim_offset, a.n_sims, a.grid, a.cell_key, a.key64);
-  e = radix_sort_index64(n, 30 + cbits, a.key64, a.skey, a.key64_b, a.perm, a.rv, a.hist, a.status, st);
+  e = radix_sort_index64(n, 30 + cbits, a.key64, a.skey, a.key64_b, a.perm, a.rv, a.hist, st);
   if (e != cudaSuccess) return e;
   e = launch_cell_bounds(n, a.skey, 30, a.cap_cells, a.num_sms, a.misc, a.cell_start, st);
   if (e != cudaSuccess) return e;
   // levels, and target order: by level, ties by source index
   k_tree_level<<<blocks_n(n), 256, 0, st>>>(n, a.skey, a.perm, a.h, a.n_sims, a.grid, a.n_leaf, a.margin, a.gamma_k,
                                             a.level, a.leaf_side);
-  e = radix_partition(n, a.level, a.tgt, a.hist, a.status, st);
+  e = radix_partition(n, a.level, a.tgt, a.hist, st);
   if (e != cudaSuccess) return e;
   const int64_t tiles = (n + kLeafTile - 1) / kLeafTile;
   e = cudaMemsetAsync(a.scan_tmp, 0, sizeof(int32_t) * (size_t)(2 * tiles + 2), st);
   if (e != cudaSuccess) return e;
   k_tree_leaves<<<(unsigned)tiles, kScanThreads, 0, st>>>(n, a.tgt, a.level, a.skey, a.leaf_of, a.leaves, a.n_leaves,
-                                                         a.scan_tmp, reinterpret_cast<uint64_t*>(a.scan_tmp + 2),
-                                                         a.status);
+                                                         a.scan_tmp, reinterpret_cast<uint64_t*>(a.scan_tmp + 2));
   k_tree_neigh<<<blocks_n(n * 4), 256, 0, st>>>(a.leaves, a.n_leaves, a.skey, n, a.cell_start, a.n_sims, a.grid,
                                                 a.ranges);
   return cudaGetLastError();

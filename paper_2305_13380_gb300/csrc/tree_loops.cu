@@ -607,7 +607,7 @@ __device__ __forceinline__ uint64_t reverse_rec(int32_t j, int32_t ti, int sc) {
 __device__ __forceinline__ void emit_at(const sphh::TreeDensityArgs& a, unsigned long long k, uint64_t rec) {
   if (k < (unsigned long long)a.rev_cap) {
     a.rev_raw[k] = rec;
-    atomicAdd(&a.rev_start[(int32_t)(rec >> 32)], 1);
+    atomicAdd(&a.rev_fill[(int32_t)(rec >> 32)], 1);
   } else {
     atomicOr(a.status, SPH_ST_CAPACITY);
   }
@@ -657,7 +657,7 @@ __device__ __forceinline__ void emit_warp(const sphh::TreeDensityArgs& a, bool w
 struct TEmit {
   unsigned long long* count;
   uint64_t* raw;
-  int32_t* start;
+  int32_t* per_receiver;
   int64_t cap;
   int32_t* status;
 };
@@ -680,7 +680,7 @@ __device__ __noinline__ void emit_marked(TEmit o, uint32_t wm, const TRound& S, 
       const int32_t j = unpack_j(je);
       if (k < (unsigned long long)o.cap) {
         o.raw[k] = reverse_rec(j, ti, unpack_s(je));
-        atomicAdd(&o.start[j], 1);
+        atomicAdd(&o.per_receiver[j], 1);
       } else {
         atomicOr(o.status, SPH_ST_CAPACITY);
       }
@@ -984,7 +984,7 @@ k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
           }
           // reverse pairs from the lists: the warp takes one slot range for the
           // whole round
-          emit_marked(TEmit{a.rev_count, a.rev_raw, a.rev_start, a.rev_cap, a.status}, wm, S, ti, lane);
+          emit_marked(TEmit{a.rev_count, a.rev_raw, a.rev_fill, a.rev_cap, a.status}, wm, S, ti, lane);
           tcombine(s);
           if (act_now && sub == 0) {
             if (queued) {
@@ -1850,12 +1850,9 @@ namespace sphh {
 using namespace sphk;
 
 __global__ void k_tree_mask(int64_t n, const int32_t* __restrict__ perm, const uint8_t* __restrict__ active,
-                            uint8_t* __restrict__ out, int32_t* __restrict__ pre) {
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k <= n; k += (int64_t)gridDim.x * blockDim.x) {
-    const uint8_t v = k < n && active[perm[k]] != 0 ? 1 : 0;
-    if (k < n) out[k] = v;
-    if (pre != nullptr) pre[k] = v;
-  }
+                            uint8_t* __restrict__ out) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+    out[k] = active[perm[k]] != 0 ? 1 : 0;
 }
 
 static int tree_blocks(int64_t n) {
@@ -1880,7 +1877,6 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   if (e == cudaSuccess) e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_count, 0, sizeof(int32_t), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_work, 0, sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_start, 0, sizeof(int32_t) * (n + 1), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_fill, 0, sizeof(int32_t) * (n > 0 ? n : 1), st);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
@@ -1891,7 +1887,8 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   else
     k_tree_density<K, false><<<blocks, kTWarps * 32, kTDensSmem, st>>>(a, ph);
   k_tree_density_fb<K><<<a.num_sms * bps[1], kTWarps * 32, kTFbSmem, st>>>(a, ph);
-  e = scan_exclusive(a.rev_start, a.rev_start, nullptr, n + 1, false, a.scan_tmp, a.status, a.num_sms, st);
+  e = scan_exclusive(a.rev_fill, a.rev_start, n, a.scan_tmp, a.num_sms, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_fill, 0, sizeof(int32_t) * n, st);
   if (e != cudaSuccess) return e;
   k_rev_scatter<<<a.num_sms * 4, 256, 0, st>>>(a.rev_raw, a.rev_count, a.rev_cap, a.rev_start, a.rev_fill, a.rev);
   // (the scatter's cursors and the work counters are free again: the queue of
@@ -1977,11 +1974,11 @@ cudaError_t launch_tree_wake(const TreeForceArgs& a, const PhysDev& ph, cudaStre
 }
 
 cudaError_t launch_tree_mask(int64_t n, const int32_t* perm, const uint8_t* active, uint8_t* out, int32_t* pre,
-                             int32_t* tmp, int32_t* status, int num_sms, cudaStream_t st) {
+                             int32_t* tmp, int num_sms, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_tree_mask<<<tree_blocks(n + 1), 256, 0, st>>>(n, perm, active, out, pre);
+  k_tree_mask<<<tree_blocks(n), 256, 0, st>>>(n, perm, active, out);
   if (pre != nullptr) {
-    const cudaError_t e = scan_exclusive(pre, pre, nullptr, n + 1, false, tmp, status, num_sms, st);
+    const cudaError_t e = scan_exclusive(out, pre, n, tmp, num_sms, st);
     if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();

@@ -30,7 +30,6 @@ SPH_ST_REBUILD = 2
 SPH_ST_BOX = 4
 SPH_ST_CAPACITY = 8
 SPH_ST_NEG_U = 16
-SPH_ST_TIMEOUT = 32
 
 SPH_FLAG_SYNC = 1
 SPH_FLAG_COUNT_PAIRS = 2

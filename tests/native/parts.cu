@@ -6,9 +6,11 @@
 extern "C" {
 
 long part_scan_words(long n) { return sphh::scan_words(n); }
-int part_scan(const int32_t* in, int32_t* out, long n, int with_total, int32_t* scratch, int32_t* status,
-              cudaStream_t st) {
-  return (int)sphh::scan_exclusive(in, out, nullptr, n, with_total != 0, scratch, status, 152, st);
+int part_scan(const int32_t* in, int32_t* out, long n, int32_t* scratch, cudaStream_t st) {
+  return (int)sphh::scan_exclusive(in, out, n, scratch, 152, st);
+}
+int part_scan_bytes(const uint8_t* in, int32_t* out, long n, int32_t* scratch, cudaStream_t st) {
+  return (int)sphh::scan_exclusive(in, out, n, scratch, 152, st);
 }
 
 }

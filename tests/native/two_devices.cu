@@ -19,9 +19,9 @@ int main() {
     auto report = [&](const char* name, cudaError_t e) { std::printf("%s %d %d\n", name, device, (int)e); };
     static uint64_t keys[8];
     static int8_t levels[8];
-    report("radix_sort_index", radix_sort_index(5000, 20, words, words, words, words, words, words, words, nullptr));
-    report("radix_sort_index64", radix_sort_index64(8192, 50, keys, keys, keys, words, words, words, words, nullptr));
-    report("radix_partition", radix_partition(100, levels, words, words, words, nullptr));
+    report("radix_sort_index", radix_sort_index(5000, 20, words, words, words, words, words, words, nullptr));
+    report("radix_sort_index64", radix_sort_index64(8192, 50, keys, keys, keys, words, words, words, nullptr));
+    report("radix_partition", radix_partition(100, levels, words, words, nullptr));
     for (int k = 0; k < sphk::kNumKernels; ++k) {
       ph.kernel = k;
       DensityArgs d{};

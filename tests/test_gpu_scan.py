@@ -17,24 +17,25 @@ def parts(tmp_path_factory):
     return native_parts.load(tmp_path_factory.mktemp("parts"))
 
 
-def _scan(parts, v):
+def _scan(parts, v, dtype="int32"):
     import torch
     n = len(v)
-    a = torch.as_tensor(v, dtype=torch.int32, device="cuda")
+    a = torch.as_tensor(v, device="cuda").to(getattr(torch, dtype))
     out = torch.full((n + 1,), -1, dtype=torch.int32, device="cuda")
-    status = torch.zeros(1, dtype=torch.int32, device="cuda")
     scratch = torch.empty(parts.part_scan_words(n), dtype=torch.int32, device="cuda")
-    rc = parts.part_scan(native_parts.ptr(a), native_parts.ptr(out), ctypes.c_long(n), 1, native_parts.ptr(scratch),
-                         native_parts.ptr(status), native_parts.stream())
+    f = parts.part_scan if dtype == "int32" else parts.part_scan_bytes
+    rc = f(native_parts.ptr(a), native_parts.ptr(out), ctypes.c_long(n), native_parts.ptr(scratch),
+           native_parts.stream())
     torch.cuda.synchronize()
-    assert rc == 0 and int(status[0]) == 0
+    assert rc == 0
     return out.cpu().numpy()
 
 
+@pytest.mark.parametrize("dtype", ["int32", "uint8"])
 @pytest.mark.parametrize("n", [1, 15, 16, 4095, 4096, 4097, 100000, 4096 * 1100 + 3])
-def test_lengths(parts, n):
-    v = np.random.default_rng(n).integers(0, 400, n)
-    assert np.array_equal(_scan(parts, v), np.concatenate([[0], np.cumsum(v)]))
+def test_lengths(parts, n, dtype):
+    v = np.random.default_rng(n).integers(0, 256, n)
+    assert np.array_equal(_scan(parts, v, dtype), np.concatenate([[0], np.cumsum(v)]))
 
 
 @pytest.mark.parametrize("total", [2 ** 30 - 1, 2 ** 30, 2 ** 30 + 1, 2 ** 31 - 1])
