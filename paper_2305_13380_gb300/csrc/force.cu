@@ -128,7 +128,7 @@ __device__ __forceinline__ void force_pair(const ForceTarget& T, const float4& A
   if constexpr (kFl == kFlSphenix) {
     // conduction: zero beyond both supports (visc = 0) and for r = 0
     const float Ps = T.E.z + Ej.z, rs = T.D.x + Dj.x;
-    const float ac = Ps > 0.0f ? div_norm(fmaf(T.E.z, T.E.w, Ej.z * Ej.w), Ps) : 0.0f;
+    const float ac = Ps > 0.0f ? __fdividef(fmaf(T.E.z, T.E.w, Ej.z * Ej.w), Ps) : 0.0f;
     const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(T.E.z - Ej.z), rs)));
     s.du = fmaf(Bj.w * ac * vc * (T.E.x - Ej.x) * r, div_norm(visc, rs), s.du);
   }

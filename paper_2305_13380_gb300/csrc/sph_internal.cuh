@@ -461,19 +461,21 @@ __device__ __forceinline__ float kernel_g(float q, float H_rinv) {
   }
 }
 
-// 1 / sqrt(x) of a normal x, and x / y of a normal y: the approximate
-// instructions that rsqrtf and __fdividef end in, without the scaling that
-// those put around them for subnormal operands (three instructions a pair in
-// every loop; a subnormal x counts as zero).
+// 1 / sqrt(x) of a normal x, and x / y of a normal y (densities: a subnormal one
+// has overflowed in f P / rho^2 before): the approximate instructions without the
+// scaling that rsqrtf and __fdividef put around them for a subnormal operand (three
+// instructions a pair in every loop).  Same bits as those: x / y is x (1 / y), the
+// product rounded as any other, so a subnormal x or quotient stays one (kernel
+// gradients go with H^-5, below 2^-126 from H = 4e7 length units on).
 __device__ __forceinline__ float rsqrt_norm(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
 __device__ __forceinline__ float div_norm(float x, float y) {
-  float q;
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(q) : "f"(x), "f"(y));
-  return q;
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(y));
+  return __fmul_rn(x, r);
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -1305,7 +1305,7 @@ __device__ __forceinline__ void tforce_pair(float dx, float dy, float dz, const 
   if constexpr (kFl == kTSphenix) {
     // conduction: zero beyond both supports (visc = 0) and for r = 0
     const float Ps = ei.z + ej.z, rs = rho_i + rho_j;
-    const float ac = Ps > 0.0f ? div_norm(fmaf(ei.z, ei.w, ej.z * ej.w), Ps) : 0.0f;
+    const float ac = Ps > 0.0f ? __fdividef(fmaf(ei.z, ei.w, ej.z * ej.w), Ps) : 0.0f;
     const float vc = fmaf(fabsf(vdotx), rinv, sqrtf(div_norm(2.0f * fabsf(ei.z - ej.z), rs)));
     s.du = fmaf(mj * ac * vc * (ei.x - ej.x) * r, div_norm(visc, rs), s.du);
   }
