@@ -662,7 +662,8 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
       const float R2 = g.G.cell_f * g.G.cell_f * (1.0f + 1e-5f);  // any support stays below the cell side
       for (int32_t t0 = ts; t0 < te; t0 += 32) {
         const int nt = min(32, te - t0);
-        list_sources(nt, nsrc, R2, spos, lists, warp, lane, [&](int t) { return a.pos4[t0 + t]; });
+        list_sources(nt, nsrc, spos, lists, warp, lane, [&](int t) { return a.pos4[t0 + t]; },
+                     [&](float, float) { return R2; });
         const int t = walk_target(spread, nt, warp, lane);
         const int32_t ti = t0 + t;
         if (t >= 0 && (a.act == nullptr || a.act[ti] != 0)) {

@@ -739,10 +739,12 @@ __global__ void __launch_bounds__(kThreads) k_force_overflow(sphh::ForceArgs a, 
       OvfLists& lists = *reinterpret_cast<OvfLists*>(fo_raw + (size_t)kFOvfStage * rec_bytes<kFl>());
       stage_all(nsrc, nb, warp, lane,
                 [&](int slot, int32_t j, float ox, float oy, float oz) { S.put(a, slot, j, ox, oy, oz); });
-      const float R2 = g.G.cell_f * g.G.cell_f * (1.0f + 1e-5f);  // any support stays below the cell side
       for (int32_t t0 = ts; t0 < te; t0 += 32) {
         const int nt = min(32, te - t0);
-        list_sources(nt, nsrc, R2, S.A, lists, warp, lane, [&](int t) { return a.fA[t0 + t]; });
+        list_sources(nt, nsrc, S.A, lists, warp, lane, [&](int t) { return a.fA[t0 + t]; }, [](float Hi, float Hj) {
+          const float Hm = reach<kFl>(Hi, Hj);
+          return Hm * Hm;
+        });
         const int t = walk_target(true, nt, warp, lane);
         const int32_t ti = t0 + t;
         if (t >= 0 && (a.act == nullptr || a.act[ti] != 0)) {

@@ -72,11 +72,12 @@ __device__ __forceinline__ int stage_sources(int v0, int cap, const NbLane& nb, 
 //
 // A CTA of kWarpsPerBlock warps per target cell.  The sources of the 27 cells
 // (up to 768 for the density, 640 for the force) are staged once for all its
-// targets; the warps list for each target the staged sources within the search
-// radius (a ballot per target and 32 sources, so in the sources' order), and one
-// lane per target walks its list in that order.  A source beyond the radius adds
-// exactly zero to every sum, so the sums are those of a walk of every source,
-// bit for bit.  More sources than fit are streamed through a buffer per warp,
+// targets; the warps list for each target the staged sources that can count (the
+// density: within the cell side, which caps every support; the force: within the
+// pair's reach, whatever the supports are), a ballot per target and 32 sources, so
+// in the sources' order, and one lane per target walks its list in that order.  A
+// source not listed adds exactly zero to every sum, so the sums are those of a walk
+// of every source, bit for bit.  More sources than fit are streamed through a buffer per warp,
 // 32 targets at a time.
 //
 // The walks are serial and bound by latency.  Up to one cell per resident CTA
@@ -104,12 +105,12 @@ __device__ __forceinline__ void stage_all(int nsrc, const NbLane& nb, int warp, 
   __syncthreads();
 }
 
-// Lists of nt <= 32 targets (positions pos(t), staged positions src[k] as x, y,
-// z): the staged slots with r^2 < R2, and their counts.  CTA-collective, ends with
-// a barrier.
-template <class Pos>
-__device__ __forceinline__ void list_sources(int nt, int nsrc, float R2, const float4* src, OvfLists& lists, int warp,
-                                             int lane, Pos pos) {
+// Lists of nt <= 32 targets (pos(t) and the staged src[k]: x, y, z and a value):
+// the staged slots with r^2 < reach2(pos(t).w, src[k].w), and their counts.
+// CTA-collective, ends with a barrier.
+template <class Pos, class Reach2>
+__device__ __forceinline__ void list_sources(int nt, int nsrc, const float4* src, OvfLists& lists, int warp, int lane,
+                                             Pos pos, Reach2 reach2) {
   const unsigned lt = (1u << lane) - 1u;
 #pragma unroll 1
   for (int t = warp; t < nt; t += kWarpsPerBlock) {
@@ -119,7 +120,7 @@ __device__ __forceinline__ void list_sources(int nt, int nsrc, float R2, const f
     for (int v = 0; v < nsrc; v += 32) {
       const float4 q = src[min(v + lane, nsrc - 1)];
       const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z;
-      const bool in = v + lane < nsrc && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < R2;
+      const bool in = v + lane < nsrc && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < reach2(p.w, q.w);
       const unsigned m = __ballot_sync(0xffffffffu, in);
       const int at = cnt + __popc(m & lt);
       if (in && at < kOvfList) lists.entry[t][at] = (uint16_t)(v + lane);
