@@ -400,6 +400,10 @@ struct TreeDensityArgs {
   const int32_t* act_pre = nullptr;
 };
 cudaError_t launch_tree_density(const TreeDensityArgs& a, const sphk::PhysDev& ph, cudaStream_t st);
+// Each receiver's segment rev[start[i] .. start[i + 1]), i < n, into ascending
+// order.  Scratch: queue n, n_mid and n_long 1 each.
+cudaError_t sort_reverse_pairs(int64_t n, const int32_t* start, uint32_t* rev, int32_t* queue, int32_t* n_mid,
+                               int32_t* n_long, int num_sms, cudaStream_t st);
 // The mask in tree order: out[k] = active[perm[k]]; with pre (n + 1 int32,
 // scan scratch tmp of scan_words(n)) also its exclusive prefix sums.
 cudaError_t launch_tree_mask(int64_t n, const int32_t* perm, const uint8_t* active, uint8_t* out, int32_t* pre,

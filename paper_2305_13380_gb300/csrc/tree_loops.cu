@@ -1860,6 +1860,17 @@ static int tree_blocks(int64_t n) {
   return (int)(b < 1 ? 1 : (b > 65535 ? 65535 : b));
 }
 
+cudaError_t sort_reverse_pairs(int64_t n, const int32_t* start, uint32_t* rev, int32_t* queue, int32_t* n_mid,
+                               int32_t* n_long, int num_sms, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(n_mid, 0, sizeof(int32_t), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(n_long, 0, sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+  k_rev_sort<<<tree_blocks(n), kRevThreads, 0, st>>>(n, start, rev, queue, n_mid, n_long);
+  k_rev_mid<<<num_sms * 6, kRevThreads, 0, st>>>(start, rev, queue, n_mid);
+  k_rev_long<<<num_sms * 4, kRevThreads, 0, st>>>(n, start, rev, queue, n_long);
+  return cudaGetLastError();
+}
+
 template <int K>
 static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev& ph, cudaStream_t st) {
   static PerDevice<2> known;
@@ -1891,15 +1902,8 @@ static cudaError_t launch_tree_density_k(const TreeDensityArgs& a, const PhysDev
   if (e == cudaSuccess) e = cudaMemsetAsync(a.rev_fill, 0, sizeof(int32_t) * n, st);
   if (e != cudaSuccess) return e;
   k_rev_scatter<<<a.num_sms * 4, 256, 0, st>>>(a.rev_raw, a.rev_count, a.rev_cap, a.rev_start, a.rev_fill, a.rev);
-  // (the scatter's cursors and the work counters are free again: the queue of
-  // longer segments and its two lengths)
-  e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(a.fb_work, 0, sizeof(int32_t), st);
-  if (e != cudaSuccess) return e;
-  k_rev_sort<<<tree_blocks(n), kRevThreads, 0, st>>>(n, a.rev_start, a.rev, a.rev_fill, a.work, a.fb_work);
-  k_rev_mid<<<a.num_sms * 6, kRevThreads, 0, st>>>(a.rev_start, a.rev, a.rev_fill, a.work);
-  k_rev_long<<<a.num_sms * 4, kRevThreads, 0, st>>>(n, a.rev_start, a.rev, a.rev_fill, a.fb_work);
-  return cudaGetLastError();
+  // (the scatter's cursors and the work counters are free again)
+  return sort_reverse_pairs(n, a.rev_start, a.rev, a.rev_fill, a.work, a.fb_work, a.num_sms, st);
 }
 
 template <int kFl, int K>

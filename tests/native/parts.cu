@@ -12,5 +12,9 @@ int part_scan(const int32_t* in, int32_t* out, long n, int32_t* scratch, cudaStr
 int part_scan_bytes(const uint8_t* in, int32_t* out, long n, int32_t* scratch, cudaStream_t st) {
   return (int)sphh::scan_exclusive(in, out, n, scratch, 152, st);
 }
+int part_sort_reverse_pairs(long n, const int32_t* start, uint32_t* rev, int32_t* queue, int32_t* counts,
+                            cudaStream_t st) {
+  return (int)sphh::sort_reverse_pairs(n, start, rev, queue, counts, counts + 1, 152, st);
+}
 
 }
