@@ -76,9 +76,9 @@ __host__ __device__ constexpr size_t dens_blk_smem() {
                                 (size_t)dens_cap<K>() * (sizeof(uint16_t) + sizeof(uint8_t));
 }
 constexpr int kOvfStage = 768;  // most sources of a cell staged at once by the overflow kernel
-constexpr int kOvfCap = 192;  // per-warp staging of the overflow kernel's streams
-static_assert(kWarpsPerBlock * kOvfCap <= kOvfStage, "the streams' buffers fit the staging");
+constexpr int kOvfCap = 256;  // per-warp staging of the overflow kernel's streams (over the lists, too)
 constexpr size_t kOvfSmem = (size_t)kOvfStage * 2 * sizeof(float4) + sizeof(OvfLists);
+static_assert(kWarpsPerBlock * kOvfCap * 2 * sizeof(float4) <= kOvfSmem, "the streams' buffers fit");
 
 struct DensSums {
   float w, dw, mw, mdw, div, cx, cy, cz;
@@ -624,34 +624,142 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
   }
 }
 
+// A target cell of an overflow block and its sources (by a whole warp).
+struct OvfCell {
+  int32_t ts, te;  // targets
+  NbLane nb;
+  int nsrc;
+  float hcap, cell;
+  bool exists;
+};
+template <int K>
+__device__ __forceinline__ OvfCell ovf_cell(const sphh::DensityArgs& a, int32_t item, int lane) {
+  const BlockGeom g = block_geom(a.grid, a.n_sims, a.overflow[item / kBlkWarps]);
+  OvfCell C;
+  int tx, ty, tz;
+  C.exists = warp_cell(g, item % kBlkWarps, tx, ty, tz);
+  if (!C.exists) return C;
+  const int32_t nc = g.G.n_c;
+  const int32_t cx = g.c0x + tx, cy = g.c0y + ty, cz = g.c0z + tz;
+  const int32_t c = g.G.cell_base + cx + nc * (cy + nc * cz);
+  C.ts = a.cell_start[c];
+  C.te = a.cell_start[c + 1];
+  C.nb = neighbour_lane(lane, g.G.cell_base, cx, cy, cz, nc, g.G.cell_f, a.cell_start);
+  C.nsrc = warp_sum_int(C.nb.len);
+  C.hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
+  C.cell = g.G.cell_f;
+  return C;
+}
+
+// Targets t0 .. t0 + 31 of a streamed cell, a lane each, by one warp; buf: its
+// staging.  Returns the lane's pairs.
+template <int K>
+__device__ __forceinline__ int ovf_stream(const sphh::DensityArgs& a, const PhysDev& ph, const NewtonConst& nwt,
+                                          const OvfCell& C, int32_t t0, float4* spos, int lane) {
+  float4* svel = spos + kOvfCap;
+  auto put = [&](int slot, int32_t j, float ox, float oy, float oz) {
+    float4 p = a.pos4[j];
+    p.x += ox;
+    p.y += oy;
+    p.z += oz;
+    spos[slot] = p;
+    svel[slot] = a.vel4[j];
+  };
+  int pairs = 0;
+  const int32_t ti = t0 + lane;
+  const bool valid = ti < C.te && (a.act == nullptr || a.act[ti] != 0);
+  const float4 pi = valid ? a.pos4[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 vi = valid ? a.vel4[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
+  float h = valid ? start_h(a.hs[ti], C.hcap) : C.hcap;
+  float lo = 0.0f, hi = INFINITY;
+  bool done = !valid, atcap = false, conv = false;
+  int it = 0;
+  int passes = 0;
+  while (__any_sync(0xffffffffu, !done)) {
+    const float H = KernT<K>::gamma * h;
+    const float Hinv = 1.0f / H;
+    DensSums s;
+    sums_zero(s);
+    for (int v0 = 0; v0 < C.nsrc; v0 += kOvfCap) {
+      const int cnt = stage_sources(v0, kOvfCap, C.nb, lane, put);
+      // (four, here and below: with two the walks of dense cells took 1.3 times as long)
+#pragma unroll 4
+      for (int k = 0; k < cnt; ++k) dens_pair<K>(pi, vi, spos[k], svel[k], H, Hinv, s);
+      __syncwarp();
+    }
+    if (!done) {
+      passes = it + 1;
+      if (newton_update(s.w, s.dw, nwt, C.hcap, h, lo, hi, it, atcap, conv)) done = true;
+    }
+  }
+  // final pass at the converged h
+  {
+    const float H = KernT<K>::gamma * h;
+    const float Hinv = 1.0f / H;
+    FinSums s;
+    fin_zero(s);
+    for (int v0 = 0; v0 < C.nsrc; v0 += kOvfCap) {
+      const int cnt = stage_sources(v0, kOvfCap, C.nb, lane, put);
+#pragma unroll 4
+      for (int k = 0; k < cnt; ++k) fin_pair<K>(pi, vi, spos[k], svel[k], spos[k].w, H, Hinv, s);
+      __syncwarp();
+    }
+    fin_scale<K>(s, H);
+    if (valid) {
+      dens_write<K>(a, ph, ti, h, s, vi.w, passes, conv, atcap);
+      pairs = s.npair;
+    }
+  }
+  return pairs;
+}
+
 // Blocks whose neighbourhood exceeded the staging buffer, a CTA per target cell
 // (stencil.cuh, with what it measured), with positions relative to the target
-// cell.
+// cell.  A streamed cell keeps a warp busy per 32 targets, so streamed cells are put
+// off, and the warps then deal their 32s among themselves: a cell of 30 targets does
+// not hold up three warps, one of thousands keeps all four.  (Lattices of 100^3
+// particles with 31, 41, 72 per cell: a warp per streamed cell 6.8, 9.6, 13.4 ms, a
+// CTA per cell 9.1, 12.0, 13.9, this 6.7, 8.5, 12.2; 30,000 clustered particles 210,
+// 51 and 49 ms.)
 template <int K>
 __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs a, PhysDev ph) {
   extern __shared__ float4 osm[];
+  __shared__ int32_t off_item[32], off_first[32];  // cells put off, the number of 32s before each
+  __shared__ int dealt;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t n_items = a.misc_ro[kNumOverflow] * kBlkWarps;
   const bool spread = n_items <= (int32_t)gridDim.x;
   const NewtonConst nwt = newton_const<K>(ph);
   unsigned long long pair_acc = 0;
-  for (int32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const BlockGeom g = block_geom(a.grid, a.n_sims, a.overflow[item / kBlkWarps]);
-    int tx, ty, tz;
-    if (!warp_cell(g, item % kBlkWarps, tx, ty, tz)) continue;
-    const int32_t nc = g.G.n_c;
-    const int32_t cx = g.c0x + tx, cy = g.c0y + ty, cz = g.c0z + tz;
-    const int32_t c = g.G.cell_base + cx + nc * (cy + nc * cz);
-    const int32_t ts = a.cell_start[c], te = a.cell_start[c + 1];
-    const NbLane nb = neighbour_lane(lane, g.G.cell_base, cx, cy, cz, nc, g.G.cell_f, a.cell_start);
-    const int nsrc = warp_sum_int(nb.len);
-    const float hcap = h_cap<K>((double)g.G.reach_f, g.G.L);
+  int n_off = 0, n_units = 0;
+  for (int32_t item = blockIdx.x;; item += gridDim.x) {
+    if (n_off == 32 || (item >= n_items && n_off > 0)) {
+      if (threadIdx.x == 0) dealt = kWarpsPerBlock;
+      __syncthreads();  // (the streams' buffers lie in the staging)
+      const int first = lane < n_off ? off_first[lane] : INT32_MAX;
+      for (int u = warp; u < n_units;) {
+        const int k = __popc(__ballot_sync(0xffffffffu, first <= u)) - 1;
+        const OvfCell C = ovf_cell<K>(a, off_item[k], lane);
+        pair_acc += (unsigned long long)ovf_stream<K>(a, ph, nwt, C, C.ts + 32 * (u - off_first[k]),
+                                                      osm + warp * (2 * kOvfCap), lane);
+        int next = 0;
+        if (lane == 0) next = atomicAdd(&dealt, 1);
+        u = __shfl_sync(0xffffffffu, next, 0);
+      }
+      __syncthreads();
+      n_off = n_units = 0;
+    }
+    if (item >= n_items) break;
+    const OvfCell C = ovf_cell<K>(a, item, lane);
+    if (!C.exists) continue;
+    const int32_t ts = C.ts, te = C.te;
+    const int nsrc = C.nsrc;
     if (nsrc <= kOvfStage) {
       float4* spos = osm;
       float4* svel = osm + kOvfStage;
       OvfLists& lists = *reinterpret_cast<OvfLists*>(osm + 2 * kOvfStage);
       __syncthreads();  // the previous cell's sources (or streams) are done with
-      stage_all(nsrc, nb, warp, lane, [&](int slot, int32_t j, float ox, float oy, float oz) {
+      stage_all(nsrc, C.nb, warp, lane, [&](int slot, int32_t j, float ox, float oy, float oz) {
         float4 p = a.pos4[j];
         p.x += ox;
         p.y += oy;
@@ -659,7 +767,7 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
         spos[slot] = p;
         svel[slot] = a.vel4[j];
       });
-      const float R2 = g.G.cell_f * g.G.cell_f * (1.0f + 1e-5f);  // any support stays below the cell side
+      const float R2 = C.cell * C.cell * (1.0f + 1e-5f);  // any support stays below the cell side
       for (int32_t t0 = ts; t0 < te; t0 += 32) {
         const int nt = min(32, te - t0);
         list_sources(nt, nsrc, spos, lists, warp, lane, [&](int t) { return a.pos4[t0 + t]; },
@@ -672,7 +780,7 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
           const bool all = cnt > kOvfList;
           const int n = all ? nsrc : cnt;
           const float4 pi = a.pos4[ti], vi = a.vel4[ti];
-          float h = start_h(a.hs[ti], hcap);
+          float h = start_h(a.hs[ti], C.hcap);
           float lo = 0.0f, hi = INFINITY;
           bool done = false, atcap = false, conv = false;
           int it = 0, passes = 0;
@@ -687,7 +795,7 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
               dens_pair<K>(pi, vi, spos[k], svel[k], H, Hinv, s);
             }
             passes = it + 1;
-            done = newton_update(s.w, s.dw, nwt, hcap, h, lo, hi, it, atcap, conv);
+            done = newton_update(s.w, s.dw, nwt, C.hcap, h, lo, hi, it, atcap, conv);
           }
           const float H = KernT<K>::gamma * h;
           const float Hinv = 1.0f / H;
@@ -706,59 +814,13 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
       }
       continue;
     }
-    __syncthreads();  // (the streams' buffers lie in the staging)
-    float4* spos = osm + warp * (2 * kOvfCap);
-    float4* svel = spos + kOvfCap;
-    auto put = [&](int slot, int32_t j, float ox, float oy, float oz) {
-      float4 p = a.pos4[j];
-      p.x += ox;
-      p.y += oy;
-      p.z += oz;
-      spos[slot] = p;
-      svel[slot] = a.vel4[j];
-    };
-    for (int32_t t0 = ts + 32 * warp; t0 < te; t0 += 32 * kWarpsPerBlock) {
-      const int32_t ti = t0 + lane;
-      const bool valid = ti < te && (a.act == nullptr || a.act[ti] != 0);
-      const float4 pi = valid ? a.pos4[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 vi = valid ? a.vel4[ti] : make_float4(0.f, 0.f, 0.f, 0.f);
-      float h = valid ? start_h(a.hs[ti], hcap) : hcap;
-      float lo = 0.0f, hi = INFINITY;
-      bool done = !valid, atcap = false, conv = false;
-      int it = 0;
-      int passes = 0;
-      while (__any_sync(0xffffffffu, !done)) {
-        const float H = KernT<K>::gamma * h;
-        const float Hinv = 1.0f / H;
-        DensSums s;
-        sums_zero(s);
-        for (int v0 = 0; v0 < nsrc; v0 += kOvfCap) {
-          const int cnt = stage_sources(v0, kOvfCap, nb, lane, put);
-          for (int k = 0; k < cnt; ++k) dens_pair<K>(pi, vi, spos[k], svel[k], H, Hinv, s);
-          __syncwarp();
-        }
-        if (!done) {
-          passes = it + 1;
-          if (newton_update(s.w, s.dw, nwt, hcap, h, lo, hi, it, atcap, conv)) done = true;
-        }
+    if (ts < te) {
+      if (threadIdx.x == 0) {
+        off_item[n_off] = item;
+        off_first[n_off] = n_units;
       }
-      // final pass at the converged h
-      {
-        const float H = KernT<K>::gamma * h;
-        const float Hinv = 1.0f / H;
-        FinSums s;
-        fin_zero(s);
-        for (int v0 = 0; v0 < nsrc; v0 += kOvfCap) {
-          const int cnt = stage_sources(v0, kOvfCap, nb, lane, put);
-          for (int k = 0; k < cnt; ++k) fin_pair<K>(pi, vi, spos[k], svel[k], spos[k].w, H, Hinv, s);
-          __syncwarp();
-        }
-        fin_scale<K>(s, H);
-        if (valid) {
-          dens_write<K>(a, ph, ti, h, s, vi.w, passes, conv, atcap);
-          pair_acc += (unsigned long long)s.npair;
-        }
-      }
+      ++n_off;
+      n_units += (te - ts + 31) / 32;
     }
   }
   if (ph.count_pairs) {

@@ -77,8 +77,8 @@ __device__ __forceinline__ int stage_sources(int v0, int cap, const NbLane& nb, 
 // pair's reach, whatever the supports are), a ballot per target and 32 sources, so
 // in the sources' order, and one lane per target walks its list in that order.  A
 // source not listed adds exactly zero to every sum, so the sums are those of a walk
-// of every source, bit for bit.  More sources than fit are streamed through a buffer per warp,
-// 32 targets at a time.
+// of every source, bit for bit.  More sources than fit are streamed through a buffer
+// per warp, 32 targets at a time.
 //
 // The walks are serial and bound by latency.  Up to one cell per resident CTA
 // ("spread") the targets are dealt to the CTA's warps.  With more cells than
