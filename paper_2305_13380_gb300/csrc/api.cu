@@ -411,11 +411,10 @@ PhysDev phys_of(const sph_params& p) {
   ph.alpha_v = (float)p.alpha_v;
   ph.beta_v = (float)p.beta_v;
   ph.eps_balsara = (float)p.eps_balsara;
-  ph.h_tol = p.h_tol;
-  ph.max_h_iter = p.max_h_iter;
   ph.count_pairs = (p.flags & SPH_FLAG_COUNT_PAIRS) ? 1 : 0;
   ph.kernel = p.kernel;
   ph.lanes = p.lanes_per_target;
+  ph.newton = sphk::newton_const(sphk::kernel_gamma(p.kernel), ph.eta3, p.h_tol, p.max_h_iter);
   return ph;
 }
 

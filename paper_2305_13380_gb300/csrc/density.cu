@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
   float* lr2 = lr2_all + warp * (list_rows<K>() * 32);
   uint16_t* lj = lj_all + warp * (list_rows<K>() * 32);
   const int32_t total = a.misc_ro[kTotalBlocks];
-  const NewtonConst nwt = newton_const<K>(ph);
+  const NewtonConst& nwt = ph.newton;
   unsigned long long pair_acc = 0;
 
   const int parts = block_parts(total);
@@ -729,7 +729,7 @@ __global__ void __launch_bounds__(kThreads) k_density_overflow(sphh::DensityArgs
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int32_t n_items = a.misc_ro[kNumOverflow] * kBlkWarps;
   const bool spread = n_items <= (int32_t)gridDim.x;
-  const NewtonConst nwt = newton_const<K>(ph);
+  const NewtonConst& nwt = ph.newton;
   unsigned long long pair_acc = 0;
   int n_off = 0, n_units = 0;
   for (int32_t item = blockIdx.x;; item += gridDim.x) {

@@ -77,6 +77,15 @@ __host__ __device__ inline double kernel_gamma(int k) {
                            : (k == kKernWendlandC2 ? KernT<kKernWendlandC2>::gammad : KernT<kKernCubic>::gammad);
 }
 
+// Constants of the Newton-Raphson update (below): FP64 values as three FP32 parts.
+struct NewtonConst {
+  float a[3];  // gamma_K^3 eta^3
+  float b[3];  // 3 gamma_K^3 eta^3
+  float tol_f;
+  double tol;
+  int32_t max_it;
+};
+
 // Physics constants passed by value to the loop kernels.
 struct PhysDev {
   float gamma;
@@ -84,11 +93,10 @@ struct PhysDev {
   float alpha_v;
   float beta_v;
   float eps_balsara;
-  double h_tol;
-  int32_t max_h_iter;
   int32_t count_pairs;
   int32_t kernel;  // kKern*
   int32_t lanes;   // lanes per target of the uniform loops (0: automatic)
+  NewtonConst newton;
 };
 
 // Constants of the SPHENIX flavour (Sec. 3.3) and the step dt over which its
@@ -124,18 +132,23 @@ struct SphenixDev {
 // exact), A and B come as FP32 values from an error-free difference (their FP64
 // values rounded to FP32), and FP64 decides only where |A| and h_tol B are
 // closer than that rounding can tell: the same decisions and the same h.
-struct NewtonConst {
-  float a[3];  // gamma_K^3 eta^3
-  float b[3];  // 3 gamma_K^3 eta^3
-  float tol_f;
-  double tol;
-  int32_t max_it;
-};
-
-__device__ __forceinline__ void split3(double v, float (&p)[3]) {
+inline void split3(double v, float (&p)[3]) {
   p[0] = (float)v;
   p[1] = (float)(v - (double)p[0]);
   p[2] = (float)((v - (double)p[0]) - (double)p[1]);
+}
+
+// (on the host: some twenty FP64 instructions a warp were 3 us of every launch of the
+// density kernels, the overflow kernel's with an empty queue included)
+inline NewtonConst newton_const(double gamma_k, float eta3, double h_tol, int32_t max_h_iter) {
+  const double a0 = gamma_k * gamma_k * gamma_k * (double)eta3;
+  NewtonConst c;
+  split3(a0, c.a);
+  split3(3.0 * a0, c.b);
+  c.tol = h_tol;
+  c.tol_f = (float)h_tol;
+  c.max_it = max_h_iter;
+  return c;
 }
 
 // x - (p0 + p1 + p2): the exact x - p0 as a sum of two floats (Knuth's TwoSum),
@@ -145,20 +158,6 @@ __device__ __forceinline__ float diff3(float x, const float (&p)[3]) {
   const float t = __fadd_rn(s, -x);
   const float e = __fadd_rn(__fadd_rn(x, -__fadd_rn(s, -t)), __fadd_rn(-p[0], -t));
   return __fadd_rn(s, __fadd_rn(__fadd_rn(e, -p[1]), -p[2]));
-}
-
-template <int K = 0>
-__device__ __forceinline__ NewtonConst newton_const(const PhysDev& ph) {
-  constexpr double gk = KernT<K>::gammad;
-  const double g3 = gk * gk * gk;
-  const double a0 = g3 * (double)ph.eta3;
-  NewtonConst c;
-  split3(a0, c.a);
-  split3(3.0 * a0, c.b);
-  c.tol = ph.h_tol;
-  c.tol_f = (float)ph.h_tol;
-  c.max_it = ph.max_h_iter;
-  return c;
 }
 
 // The FP64 test, for the few targets too close to the line.

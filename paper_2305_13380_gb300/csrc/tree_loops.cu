@@ -743,7 +743,7 @@ k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const NewtonConst nwt = newton_const<K>(ph);
+  const NewtonConst& nwt = ph.newton;
   TRound& S = *reinterpret_cast<TRound*>(tsm + (size_t)(threadIdx.x >> 5) * kTRoundBytes);
   const int t = lane / kTreeTpp, sub = lane % kTreeTpp;
   const int32_t nl = *a.n_leaves;
@@ -1524,7 +1524,7 @@ template <int K>
 __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const NewtonConst nwt = newton_const<K>(ph);
+  const NewtonConst& nwt = ph.newton;
   unsigned char* base = tsm + (size_t)warp * kTFbWarpSmem;
   float4* spos = reinterpret_cast<float4*>(base);
   uint32_t* sidx = reinterpret_cast<uint32_t*>(spos + kTCap);
