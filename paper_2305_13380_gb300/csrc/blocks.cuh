@@ -169,6 +169,7 @@ struct BlockTargets {
   int32_t cell_first[9];  // prefix of the block cells' particle counts
   int32_t n;              // targets in the block
   int32_t per, tpp, lg, rounds;
+  int32_t parts;          // CTAs that share the rounds (the others have none)
   int32_t next;           // next unclaimed round
   float hcap;             // the density's cap on h in this block
   int32_t wcount[kBlkWarps];  // active targets per warp slice (masked builds)
@@ -181,10 +182,11 @@ __device__ __forceinline__ int next_round(BlockTargets& B, int lane) {
   return __shfl_sync(0xffffffffu, r, 0);
 }
 
-// CTAs per block: grids with few blocks share each block's rounds between
-// several CTAs, each of which stages the sources, as far as CTAs are resident.  A
-// step of 4096 particles (27 blocks of 152 targets, two rounds a warp) lasts as
-// long as one block's rounds: 190 -> 169 us (up to 2 CTAs a block 167, 8 177).
+// CTAs per block, at most: grids with few blocks share each block's rounds between
+// several CTAs, each of which stages the sources, as far as CTAs are resident and a
+// warp alone would have more than one round (B.parts: a round takes as long for
+// fewer targets).  A step of 4096 particles (27 blocks of 152 targets, two rounds a
+// warp) lasts as long as one block's rounds: 190 -> 169 us.
 constexpr int kMaxParts = 4;
 __device__ __forceinline__ int block_parts(int32_t total) {
   return max(1, min(kMaxParts, (int)gridDim.x / max(total, 1)));
@@ -274,7 +276,11 @@ __device__ __forceinline__ void build_targets(const BlockGeom& g, const StageTab
     const int tpp = lanes == 2 ? 2 : (per <= 8 ? 4 : 2);
     if (per > 16) per = 16;
     // (a target's lanes, and so its sums, do not depend on the parts)
-    if (parts > 1) per = min(per, max(1, (n + kBlkWarps * parts - 1) / (kBlkWarps * parts)));
+    if (parts > 1) {
+      parts = max(1, min(parts, (n + per * kBlkWarps - 1) / (per * kBlkWarps)));
+      per = min(per, max(1, (n + kBlkWarps * parts - 1) / (kBlkWarps * parts)));
+    }
+    B.parts = parts;
     B.per = per;
     B.tpp = tpp;
     B.lg = tpp == 4 ? 2 : 1;

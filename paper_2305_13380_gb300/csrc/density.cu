@@ -322,8 +322,8 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
 
   const int parts = block_parts(total);
   for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
-    const int32_t b = item / parts;
-    const int part = item - b * parts;
+    const int part = parts == 1 ? 0 : item / total;  // (part by part: the CTAs without rounds come last)
+    const int32_t b = item - part * total;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     // (FP64, by one thread; read after the barriers below)
@@ -334,11 +334,11 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
       __syncthreads();
       continue;
     }
-    if (a.act != nullptr) {
-      // masked: the block's active targets first, and nothing to stage
-      // when it has none
+    if (a.act != nullptr || parts > 1) {
+      // masked, or shared: the block's targets first, and nothing to stage when
+      // it has none, or none for this CTA
       build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);
-      if (BT.n == 0) continue;
+      if (BT.n == 0 || (part > 0 && part >= BT.parts)) continue;
     }
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
       const int k = staged_cell_of(T, v);
@@ -356,8 +356,8 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
       spos[v] = make_float4(p.x, p.y, p.z, fmaf(p.x, p.x, fmaf(p.y, p.y, p.z * p.z)));
       svel[v] = make_float4(v4.x, v4.y, v4.z, p.w);
     }
-    if (a.act == nullptr)
-      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, nullptr, ph.lanes, parts);  // ends with a barrier
+    if (a.act == nullptr && parts == 1)
+      build_targets<K>(g, T, BT, tgt_slot, tgt_cell, nullptr, ph.lanes);  // ends with a barrier
     else
       __syncthreads();  // the staging
 
@@ -365,7 +365,8 @@ __global__ void __launch_bounds__(kBlkThreads, kDensMinBlocks) k_density(sphh::D
     const float R2 = g.G.cell_f * g.G.cell_f;
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
-    for (int rd = part + parts * warp; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
+    const int sharing = parts == 1 ? 1 : BT.parts;
+    for (int rd = part + sharing * warp; rd < BT.rounds; rd = part + sharing * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);

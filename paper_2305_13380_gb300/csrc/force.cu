@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
 
   const int parts = block_parts(total);
   for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
-    const int32_t b = item / parts;
-    const int part = item - b * parts;
+    const int part = parts == 1 ? 0 : item / total;  // (part by part: the CTAs without rounds come last)
+    const int32_t b = item - part * total;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
@@ -280,12 +280,12 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
     // the targets' rounds first (they need only the table), so that each
     // warp's first list is in flight together with the staging loads
     build_targets<K>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);  // ends with a barrier
-    if (BT.n == 0) continue;  // a masked block without active targets
+    if (BT.n == 0 || (part > 0 && part >= BT.parts)) continue;  // no (active) targets, or none for this CTA
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
     int pre_lc = 0xffff;
     uint4 pre[kFListCap / 8];
-    const int rd0 = part + parts * warp;
+    const int sharing = parts == 1 ? 1 : BT.parts, rd0 = part + sharing * warp;
     if (a.lists != nullptr && rd0 < BT.rounds) fetch_list(a, BT, T, tgt_slot, tgt_cell, rd0, lane, pre_lc, pre);
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
       const int k = staged_cell_of(T, v);
@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kBlkThreads, 2) k_force(sphh::ForceArgs a, Phy
     }
     __syncthreads();
 
-    for (int rd = rd0; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
+    for (int rd = rd0; rd < BT.rounds; rd = part + sharing * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);
@@ -523,8 +523,8 @@ __global__ void __launch_bounds__(kBlkThreads, kMinBlocks) k_force_min(sphh::For
 
   const int parts = block_parts(total);
   for (int32_t item = blockIdx.x; item < total * parts; item += gridDim.x) {
-    const int32_t b = item / parts;
-    const int part = item - b * parts;
+    const int part = parts == 1 ? 0 : item / total;  // (part by part: the CTAs without rounds come last)
+    const int32_t b = item - part * total;
     if (a.blk_any != nullptr && a.blk_any[b] == 0) continue;  // no active target
     const BlockGeom g = block_geom(a.grid, a.n_sims, b);
     const int32_t nsrc = build_stage_table(g, a.cell_start, T);
@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(kBlkThreads, kMinBlocks) k_force_min(sphh::For
       continue;
     }
     build_targets<kKernCubic>(g, T, BT, tgt_slot, tgt_cell, a.act, ph.lanes, parts);  // ends with a barrier
-    if (BT.n == 0) continue;
+    if (BT.n == 0 || (part > 0 && part >= BT.parts)) continue;
     for (int32_t v = threadIdx.x; v < nsrc; v += kBlkThreads) {
       const int k = staged_cell_of(T, v);
       float ox, oy, oz;
@@ -554,7 +554,8 @@ __global__ void __launch_bounds__(kBlkThreads, kMinBlocks) k_force_min(sphh::For
 
     const int tpp = BT.tpp, lg = BT.lg, per = BT.per;
     const int sub = lane & (tpp - 1);
-    for (int rd = part + parts * warp; rd < BT.rounds; rd = part + parts * next_round(BT, lane)) {
+    const int sharing = parts == 1 ? 1 : BT.parts;
+    for (int rd = part + sharing * warp; rd < BT.rounds; rd = part + sharing * next_round(BT, lane)) {
       const int t = lane >> lg;
       const int32_t e_t = rd * per + t;
       const bool valid = (t < per) && (e_t < BT.n);
