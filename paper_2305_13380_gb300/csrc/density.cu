@@ -15,7 +15,7 @@
 //     iteration of the paper, h <- h - f/f' with f = n_hat - (eta/h)^3 and
 //     f' = dn_hat/dh + 3 eta^3 / h^4, is h <- h (1 - A/B) with
 //     A = S_w/gamma_K^3 - eta^3, B = 3 eta^3 - S_dw/gamma_K^3 (newton_update:
-//     the convergence test in FP64, the update in FP32); a target stops when
+//     FP64 decides where FP32 cannot tell, the update is in FP32); a target stops when
 //     |A/B| <= h_tol, with that last correction applied (or at the cell cap
 //     / max_h_iter);
 //  3. a final pass at the converged h accumulates, in FP32,
@@ -27,7 +27,7 @@
 // fixed order, so results do not depend on scheduling.  A target whose list
 // overflows walks the staged sources directly.  A block whose neighbourhood
 // does not fit the staging buffer is queued for k_density_overflow, which
-// streams each target cell's 27 cells through a per-warp buffer.
+// stages each target cell's 27 cells by themselves, or streams them.
 #include "blocks.cuh"
 #include "per_device.h"
 #include "sph_internal.cuh"

@@ -20,15 +20,15 @@
 // particle) are then linked by their first friendly pair, if they are not one
 // set yet.  A core of thousands of particles within b of each other so takes a
 // few root checks per octant instead of a union per pair, all of them contending
-// for the same root (the 1M clustered box: 7.5 ms for all pairs, 0.86 ms for the
-// octants and the rest; the call 8.2 -> 1.67 ms).
+// for the same root (the 1M clustered box: 7.5 ms for all pairs, 0.73 ms for the
+// octants and the rest; the call 8.2 -> 1.15 ms, cell_start and the sort included).
 //
 // Union-find on the caller's group array, lock-free: a set's root is its
 // smallest index, a union hooks the larger root below the smaller one with
 // one compare-and-swap (retried when the root changed meanwhile), and the
-// link pass's finds halve their paths.  Every parent pointer only ever moves to an ancestor,
-// so concurrent halving and hooking keep a valid forest, and the final roots
-// are the groups' smallest indices whatever the order of the unions.  The
+// link pass's finds halve their paths.  Every parent pointer only ever moves to an
+// ancestor, so concurrent halving and hooking keep a valid forest, and the final
+// roots are the groups' smallest indices whatever the order of the unions.  The
 // parent loads bypass L1 (other SMs write them).  Loops are bounded; a
 // bound that is hit sets SPH_ST_CAPACITY.
 #include "sph_internal.cuh"

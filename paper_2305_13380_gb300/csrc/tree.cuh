@@ -38,19 +38,10 @@ struct TreeRange {
 // measured on the 2M clustered box with the per-target kernel: 1.01-1.03
 // within 1 % of each other, 1.05 10 % and 1.1 15 % slower per step, 1.0 (every
 // growing support queued) four times slower.
-#ifndef SPH_TREE_LIST
-#define SPH_TREE_LIST 32
-#endif
-#ifndef SPH_TREE_LIST_REACH
-#define SPH_TREE_LIST_REACH 1.02f
-#endif
-#ifndef SPH_TREE_TPP
-#define SPH_TREE_TPP 8
-#endif
-constexpr int kTreeTpp = SPH_TREE_TPP;  // a power of two dividing 8
-constexpr int kTreeList = SPH_TREE_LIST;
-constexpr int kTreeListRegion = SPH_TREE_LIST;
-constexpr float kTreeListReach = SPH_TREE_LIST_REACH;
+constexpr int kTreeTpp = 8;
+constexpr int kTreeList = 32;
+constexpr int kTreeListRegion = kTreeList;
+constexpr float kTreeListReach = 1.02f;
 
 __device__ __forceinline__ uint32_t spread3(uint32_t v) {
   // 10 bits -> every third bit of 30

@@ -616,8 +616,8 @@ __device__ __forceinline__ void emit_at(const sphh::TreeDensityArgs& a, unsigned
 // Appends the reverse pairs of target ti with the marked ones of a lane's four
 // sources: one counter atomic, a wait of about a microsecond, per 128 sources.
 // Called by all 32 lanes.
-__device__ __forceinline__ void emit_marked(const sphh::TreeDensityArgs& a, unsigned want, const uint32_t (&je)[4],
-                                            int32_t ti, int lane) {
+__device__ __forceinline__ void emit_rows(const sphh::TreeDensityArgs& a, unsigned want, const uint32_t (&je)[4],
+                                          int32_t ti, int lane) {
   const int mine = __popc(want);
   int incl = mine;
 #pragma unroll
@@ -723,17 +723,13 @@ __device__ __forceinline__ void tdens_write(const sphh::TreeDensityArgs& a, cons
 // not depend on the windows nor on what else the pool holds.
 //
 // Bound by instruction issue (70 % of the slots): 24 warps per SM, 1,590 warp
-// instructions per particle, 3.85 ms on the 2M clustered box.  Taken together the
-// changes here took the call (build, density, force) from 11.10 to 7.13 ms and the
-// kernel from 7.9 to 4.1 ms; before,
-// every round staged the ~290 sources of its children in shared memory (18.6 KB
-// per warp, 12 warps per SM) and filtered them from there.  What counted: the
-// filter on sources held in registers, keeping only the ~90 listed ones (11.1
-// -> 9.8 ms with windows of 32 targets); the loops and warp functions that are
-// not expanded in place, as fetch stalls were the largest (63 -> 43 KB of code,
-// 10.0 -> 7.3 ms); windows of two rounds, as a round beside a dense core tests
-// up to 23,000 sources (32 targets 7.32 ms, 12 7.02, 8 7.13, 4 7.61; but the
-// pool of 48 uneven boxes 4.45, 3.73, 3.64 and 3.59 ms).
+// instructions per particle, 3.85 ms on the 2M clustered box (7.9 when every round
+// staged its ~290 sources in shared memory, 12 warps per SM, and filtered them from
+// there).  The filter works on sources held in registers and keeps only the ~90
+// listed ones; the loops and warp functions are not expanded in place (fetch stalls
+// were the largest at 63 KB of code); windows are of two rounds, as a round beside a
+// dense core tests up to 23,000 sources (with 32 targets per window the pool of 48
+// uneven boxes took 1.2 times as long).
 //
 // kMask: the masked loops (a.act, a.act_pre set); the plain instance carries
 // none of their tests.
@@ -1690,7 +1686,7 @@ __global__ void __launch_bounds__(kTWarps * 32) k_tree_density_fb(sphh::TreeDens
           if (want_reverse_t(__int_as_float(fj[i].w), ti, unpack_j(je[i]), r2, H2, H, g.side)) want |= 1u << i;
         }
       }
-      emit_marked(a, want, je, ti, lane);
+      emit_rows(a, want, je, ti, lane);
     }
     s.w = wsum(s.w);
     s.dw = wsum(s.dw);
