@@ -132,7 +132,7 @@ struct SphenixDev {
 // exact), A and B come as FP32 values from an error-free difference (their FP64
 // values rounded to FP32), and FP64 decides only where |A| and h_tol B are
 // closer than that rounding can tell: the same decisions and the same h.
-inline void split3(double v, float (&p)[3]) {
+__host__ __device__ inline void split3(double v, float (&p)[3]) {
   p[0] = (float)v;
   p[1] = (float)(v - (double)p[0]);
   p[2] = (float)((v - (double)p[0]) - (double)p[1]);
@@ -140,7 +140,7 @@ inline void split3(double v, float (&p)[3]) {
 
 // (on the host: some twenty FP64 instructions a warp were 3 us of every launch of the
 // density kernels, the overflow kernel's with an empty queue included)
-inline NewtonConst newton_const(double gamma_k, float eta3, double h_tol, int32_t max_h_iter) {
+__host__ __device__ inline NewtonConst newton_const(double gamma_k, float eta3, double h_tol, int32_t max_h_iter) {
   const double a0 = gamma_k * gamma_k * gamma_k * (double)eta3;
   NewtonConst c;
   split3(a0, c.a);

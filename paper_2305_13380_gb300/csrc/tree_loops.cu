@@ -739,7 +739,11 @@ k_tree_density(sphh::TreeDensityArgs a, PhysDev ph) {
   extern __shared__ __align__(16) unsigned char tsm[];
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const NewtonConst& nwt = ph.newton;
+  // (the quartic instance is scheduled worse around constants from the parameters:
+  // 96k clustered particles 1.93 -> 1.98 ms)
+  const NewtonConst nwt = K == kKernQuartic
+                              ? newton_const(KernT<K>::gammad, ph.eta3, ph.newton.tol, ph.newton.max_it)
+                              : ph.newton;
   TRound& S = *reinterpret_cast<TRound*>(tsm + (size_t)(threadIdx.x >> 5) * kTRoundBytes);
   const int t = lane / kTreeTpp, sub = lane % kTreeTpp;
   const int32_t nl = *a.n_leaves;
