@@ -32,40 +32,6 @@
 
 namespace sphk {
 
-// Fine coordinate on one axis: g = floor(1024 fl(fl(x n_c) / L)), clamped to
-// the top cell k (the same product and quotient that define k).
-__device__ __forceinline__ int32_t fine_coord(double x, double L, int32_t n_c, int32_t k) {
-  const double s = __ddiv_rn(__dmul_rn(x, (double)n_c), L);
-  int64_t g = (int64_t)floor(s * (double)kTreeFine);
-  const int64_t lo = (int64_t)k * kTreeFine, hi = lo + kTreeFine - 1;
-  g = g < lo ? lo : (g > hi ? hi : g);
-  return (int32_t)g;
-}
-
-// The same g with FP64 work only near the faces of sub-cells (FP64 runs at 1/64
-// of the integer rate here).  The leading 64 bits P of the product of the
-// mantissas of x and of fl(1024 n_c / L) hold 1024 x n_c / L as fixed point, its
-// sh fraction bits below.  P and the quotient that defines g are each within
-// 2^-51 of the exact value, so within 2^-20 of each other for g < 2^31: a
-// fraction farther than 2^-18 from 0 and 1 gives the same floor.  Otherwise, and
-// for an x that is not positive, not a number, huge, or below half a sub-cell,
-// the exact path decides.  (2M particles: 132 -> 32 us.)
-__device__ __forceinline__ int32_t fine_coord_fast(double x, const GridDev& G, int32_t k) {
-  const uint64_t xb = (uint64_t)__double_as_longlong(x), cb = (uint64_t)__double_as_longlong(G.fine_scale);
-  constexpr uint64_t kOne = 1ull << 52, kFrac = kOne - 1ull;
-  const int ex = (int)(xb >> 52), ec = (int)(cb >> 52);  // (the sign is bit 11)
-  const int sh = 2108 - ex - ec;
-  if (ex > 0 && ex < 2047 && sh >= 33 && sh <= 63) {
-    const uint64_t P = __umul64hi(((xb & kFrac) | kOne) << 11, ((cb & kFrac) | kOne) << 11);
-    const uint32_t frac = (uint32_t)(P >> (sh - 32));
-    if (frac - (1u << 14) < 0u - (1u << 15)) {
-      const int32_t g = (int32_t)(P >> sh), lo = k * kTreeFine, hi = lo + kTreeFine - 1;
-      return g < lo ? lo : (g > hi ? hi : g);
-    }
-  }
-  return fine_coord(x, G.L, G.n_c, k);
-}
-
 __global__ void k_tree_key(int64_t n, const double* __restrict__ x, const double* __restrict__ y,
                            const double* __restrict__ z, const int64_t* __restrict__ sim_offset,
                            int n_sims, const GridDev* __restrict__ grid,
